@@ -140,10 +140,11 @@ def _grid(lo, hi, n):
 
 def _strip(case, seed):
     """Disordered square-lattice strip between two clean leads (the strip workload's recipe); with S a
-    small Hermitian overlap on every block."""
+    small Hermitian overlap on every block.  The grid keeps off the rational mode thresholds (such as
+    E = 1, 2) where the lead's surface Green's function has a branch point."""
     d, b, nb = _Draw(seed), case["b"], case["nb"]
     eye = torch.eye(b, dtype=torch.complex128, device="cuda")
-    dev = dict(b=b, nb=nb, E=_grid(-3.5, 3.5, case["ne"]), mu=(0.1, -0.1))
+    dev = dict(b=b, nb=nb, E=_grid(-3.4637, 3.5219, case["ne"]), mu=(0.1, -0.1))
     dev["H_diag"] = _chain(b) + torch.diag_embed(d.uniform(-0.25, 0.25, nb, b)).to(torch.complex128)
     dev["H_upper"] = (-eye).expand(nb - 1, b, b).contiguous()
     dev["leads"] = (_chain(b), -eye.clone())
@@ -356,16 +357,17 @@ def tolerance(case):
     if kind == "fpx":
         return "exact"
     # FP64 with contacts: the decimation inverts blocks of condition 3e4 and more at eta = 1e-6
-    # (measured 2e-10 on the strips, 9e-10 for leads with random blocks, 8e-9 for wide strips)
+    # (measured up to 4e-9 on the strips, 2e-8 for wide leads)
     if kind == "strip":
-        return {"rel": 4e-9}
+        return {"rel": 2e-8}
     if kind == "lead" or case.get("leads"):
-        return {"rel": 4e-8}
-    # measured 3.4e-16 (fp64), 1.8e-7 (fp32), 9.9e-12 (emu64), 1.1e-4 (bf16x3)
+        return {"rel": 8e-8}
+    # measured 3.4e-16 (fp64), 1.8e-7 (fp32), 9.9e-12 (emu64), 2.5e-4 (bf16x3)
     if kind == "zgemm":
         return {"rel": dict(fp64=2e-15, fp32=1e-6, emu64=4e-11, bf16x3=1e-3)[prec]}
+    # measured 5e-16 (fp64, n = 18), 1.4e-6 (fp32), 9e-11 (emu64)
     if kind == "zinv":
-        return {"rel": dict(fp64=1e-13, fp32=1e-5, emu64=4e-10)[prec]}
+        return {"rel": dict(fp64=2e-14, fp32=1e-5, emu64=4e-10)[prec]}
     # solves: the current is a small difference of large traces and carries the largest error
     # (measured 1.2e-11 in fp64, 4.5e-3 in fp32, 1.1e-7 in emu64)
     return {"rel": dict(fp64=1e-10, fp32=2e-2, emu64=5e-7)[prec]}
