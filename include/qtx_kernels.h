@@ -22,7 +22,8 @@ enum { QTX_OP_N = 0, QTX_OP_C = 1 /* conjugate transpose */ };
  *     C[e] = alpha * op(A[e]) * op(B[e]) + beta * C0[e],   e = 0 .. batch-1,
  * op(A) is M x K, op(B) is K x N, C and C0 are M x N.  lda/ldb/ldc0/ldc are row strides and
  * strideA/B/C0/C batch strides in complex elements (0 shares one matrix across the batch).
- * precision: QTX_FP64 / QTX_FP32 on the CUDA cores; QTX_EMU64 / QTX_BF16X3 on the tcgen05 tensor cores
+ * precision: QTX_FP32 on the CUDA cores; QTX_FP64 on the tensor cores with 9 bf16 digit planes (one
+ * FP64 rounding of the whole sum) when every dimension is above 32, else on the CUDA cores; QTX_EMU64 / QTX_BF16X3 on the tcgen05 tensor cores
  * with 6 (7 when K > 512) / 2 bf16 digit planes per operand (Ozaki-style slicing, Sec. II-D), inputs
  * and outputs rounded to df32 (hi + lo FP32 pairs) on the way in and out; alpha and beta are applied as
  * df32 pairs as well (~48 bits: a scalar such as 0.1 adds no FP32-sized error).  C0 may be NULL when beta == 0; C may
@@ -37,8 +38,10 @@ qtx_status qtx_zgemm_batched(int precision, int M, int N, int K, int opA, const 
 /* Batched inverse of n x n complex blocks, in place (A[e] -> A[e]^-1, batch stride strideA), as used
  * by the forward sweep (g_i = (A_i - V g U)^-1): Gauss-Jordan with partial pivoting on blocks of at
  * most 64, a 2 x 2 Schur-complement recursion above that, plus one Newton step X += X (I - A X) for
- * recursed FP32/FP64 blocks; QTX_EMU64 / QTX_BF16X3 start from the FP32 inverse and apply
- * `refine_iter` Newton sweeps with tensor-core products.  status[e] (device, may be NULL) receives
+ * recursed FP32 blocks; QTX_FP64 above 32 refines the FP32 inverse with FP64 products until its
+ * residual is at FP64 level and eliminates in FP64 (pivoted) the blocks where that does not converge;
+ * QTX_EMU64 / QTX_BF16X3 start from the FP32 inverse and apply `refine_iter` Newton sweeps with
+ * tensor-core products.  status[e] (device, may be NULL) receives
  * QTX_ERR_SINGULAR for a zero pivot. */
 qtx_status qtx_zinv_batched(int precision, int n, void *A, long strideA, int batch, int refine_iter,
                             int *status, void *stream);

@@ -51,7 +51,11 @@ typedef enum {
  * ZGEMM-dominated; lower precision is traded against accuracy).  Observables are always reduced
  * in FP64 and the lead decimation always runs in FP64. */
 typedef enum {
-  QTX_FP64 = 0,   /* complex128 throughout (SIMT DFMA) -- the plain FP64 path */
+  QTX_FP64 = 0,   /* complex128 throughout -- the plain FP64 path.  Products with all dimensions above 32
+                     on the tcgen05 tensor cores from 9 bf16 digit planes per operand (45 digit products,
+                     operands held to 2^-62 of their row's or column's largest entry, the exact sum
+                     rounded to FP64 once), smaller products and inverses with DFMA; larger inverses
+                     refined to FP64 from an FP32 start, or eliminated in FP64 where that fails */
   QTX_FP32 = 1,   /* complex64 storage; products with all dimensions >= 96 (and K <= 1024) on the
                      tcgen05 tensor cores from 4 bf16 digit planes per operand (10 digit products,
                      ~27-bit products, every digit group exact), smaller products and the leaf
@@ -95,7 +99,8 @@ typedef struct {
   int max_energies_in_flight;  /* energies solved concurrently; workspace scales with it (>= 1) */
   qtx_precision precision;
   int refine_max_iter;         /* Newton sweeps X += X (I - A X) per block inverse (QTX_EMU64,
-                                  QTX_BF16X3; FP32/FP64 apply one step to recursed blocks > 64) */
+                                  QTX_BF16X3; FP32 applies one step to recursed blocks > 64, FP64 as
+                                  many as FP64 accuracy takes) */
   int has_S;                   /* 0: S = I (S pointers ignored) */
   int has_scattering;          /* 0: no scattering self-energies (Sigma pointers ignored) */
   int energy_dependent_sigma;  /* 0: one Sigma set [N_B][b][b] for all energies; 1: [N_E][N_B][b][b] */

@@ -46,12 +46,19 @@ template <typename Tin, typename Tout>
 cudaError_t convert_strided(const cx<Tin>* in, long ldi, long si, cx<Tout>* out, long ldo, long so, int rows,
                             int cols, int batch, cudaStream_t st);
 
+// ---- in-place inverse of n x n blocks by Gauss-Jordan elimination with partial pivoting over the whole
+// block, in global memory, one CTA per active entry: the few energies whose refined inverse did not
+// converge.  perm: n ints per batch entry.  A zero or non-finite pivot stores QTX_ERR_SINGULAR.
+cudaError_t pivoted_inverse(cx<double>* A, long sA, int n, int batch, const int* active, int* status, int* perm,
+                            cudaStream_t st);
+
 // X[e] += I
 template <typename T>
 cudaError_t add_identity(cx<T>* X, long sX, int n, int batch, const int* active, cudaStream_t st);
 // next[e] = active[e] (1 when active is nullptr) and ||R[e]||_F > tol, from the hi parts in FP32; a
 // non-finite norm also sets status[e] = QTX_ERR_SINGULAR (status may be nullptr)
-cudaError_t residual_mask(const cx<df>* R, long sR, int n, int batch, double tol, const int* active, int* next,
+template <typename T>
+cudaError_t residual_mask(const cx<T>* R, long sR, int n, int batch, double tol, const int* active, int* next,
                           int* status, cudaStream_t st);
 
 // ---- assemble a diagonal block of M (step 1 of the sweep), in T precision from complex128 inputs:
@@ -193,6 +200,17 @@ size_t gemm_tc_scratch_bytes(int M, int N, int K, int batch, int digits);
 size_t gemm_tc_operand_bytes(int side, int R, int K, int batch, int digits);
 TcOperand tc_operand_at(void* base, int side, int R, int K, int batch, int digits);
 bool tc_available();
+int wait_test();  // 1 while the bounded-wait test (qtx_tc_wait_test) is switched on
+
+// ---- FP64 products on the tensor cores (tc_fp64.cu): nine bf16 digit planes per operand, one FP64
+// rounding of the exact sum.  `scratch` holds the digit planes of a portion of the batch (at least one
+// entry); the batch runs in portions of what fits.  C may alias C0, and A when K <= 512 and the whole
+// batch entry's A is finite.
+size_t gemm_fp64_tc_scratch_bytes(int M, int N, int K, int batch);
+bool gemm_fp64_tc_fits(int M, int N, int K, size_t scratch_bytes);
+cudaError_t gemm_fp64_tc(const GemmArgs<double>& g, void* scratch, size_t scratch_bytes, int* err_flag, cudaStream_t st,
+                         cudaEvent_t* ev = nullptr);
+constexpr int tc_pairs_fp64() { return 45; }
 
 // ---- FPX storage codec (fpx.cu): n_complex T-typed complex values <-> their FPX codes
 bool fpx_width_ok(int bits);

@@ -42,6 +42,12 @@ struct Arena {
   }
 };
 
+// FP64 products of at least kTcF64Min in every dimension run on the tensor cores (tc_fp64.cu)
+constexpr int kTcF64Min = 33;
+// FP64 block inverses that do not converge by refinement are eliminated with full column pivoting in
+// one CTA up to this size, by the recursion above it
+constexpr int kPivotedMax = 256;
+
 // U_i, V_i differ per energy when z multiplies an overlap block or Sigma^R_{i,i+1} depends on E.
 inline bool uv_per_energy(const qtx_rgf_desc& d) {
   return d.has_S || d.system_input || (d.offdiag_sigma && d.energy_dependent_sigma);
@@ -52,6 +58,8 @@ struct Layout {
       tc_scratch, total;
   int n_tmp, n_dec;
   size_t tc_bytes;
+  bool refine64;  // FP64 block inverses by refinement (inverse_f64) have their areas
+  size_t perm;
 };
 }  // namespace
 
@@ -135,9 +143,12 @@ Layout make_layout(const qtx_rgf_desc& d) {
   // one block shared by every energy (the slice's -(H + Sigma^R) or Sigma^<, converted once)
   L.shared_blk = a.take(d.precision == QTX_FP64 ? 0 : bb * sizeof(cx<double>));
   const bool mixed = d.precision == QTX_EMU64 || d.precision == QTX_BF16X3;
-  L.ref = a.take((mixed || b > kLeafMax) ? 3 * Ec * bb * sizeof(cx<double>) : 0);
-  L.f32a = a.take(mixed ? Ec * bb * sizeof(cx<float>) : 0);
-  L.f32tmp = a.take(mixed ? Ec * bb * sizeof(cx<float>) + 4096 : 0);
+  const bool tc64 = d.precision == QTX_FP64 && b >= kTcF64Min;
+  L.refine64 = mixed || tc64;
+  L.ref = a.take((L.refine64 || b > kLeafMax) ? 3 * Ec * bb * sizeof(cx<double>) : 0);
+  L.f32a = a.take(L.refine64 ? Ec * bb * sizeof(cx<float>) : 0);
+  L.f32tmp = a.take(L.refine64 ? Ec * bb * sizeof(cx<float>) + 4096 : 0);
+  L.perm = a.take(L.refine64 && b <= kPivotedMax ? (size_t)Ec * b * sizeof(int) : 0);
   L.n_dec = 9;
   L.dec = a.take(d.leads ? (size_t)L.n_dec * Ec * bb * sizeof(cx<double>) : 0);
   L.lead = a.take(d.leads ? 8 * Ec * bb * sizeof(cx<double>) : 0);
@@ -160,6 +171,7 @@ Layout make_layout(const qtx_rgf_desc& d) {
     L.tc_bytes = std::max(L.tc_bytes, gemm_tc_scratch_bytes((int)b, (int)b, (int)b, (int)Ec, 4));
   // the FP32 mode's products of 96 and more (four digit planes; the recursive inverse's halves too)
   if (d.precision == QTX_FP32 && b >= 96 && b <= 1024) L.tc_bytes = gemm_tc_scratch_bytes((int)b, (int)b, (int)b, (int)Ec, 4);
+  if (tc64) L.tc_bytes = gemm_fp64_tc_scratch_bytes((int)b, (int)b, (int)b, (int)Ec);
   L.tc_scratch = a.take(L.tc_bytes);
   // kept digitised operands (emulated modes): two left operands and one right operand, b x b, E_c
   // energies (none when the products are split along K)
@@ -252,7 +264,7 @@ cudaError_t group_gemm(qtx_rgf_plan_s* P, const TcArgs& a, int digits, cudaStrea
 // or the tensor cores' four-plane FP32 instance -- which are not counted).
 template <typename T>
 qtx_status gemm_simt_prof(qtx_rgf_plan_s* P, const GemmArgs<T>& g, cudaStream_t st) {
-  const bool mine = P->d.precision == QTX_FP64 || P->d.precision == QTX_FP32;
+  const bool mine = P->d.precision == (std::is_same<T, double>::value ? QTX_FP64 : QTX_FP32);
   cudaEvent_t* ev = (P->prof && mine) ? P->next_events() : nullptr;
   if (ev) cudaEventRecord(ev[0], st);
   QTX_CK(gemm_simt<T>(g, st));
@@ -268,7 +280,7 @@ qtx_status gemm_simt_prof(qtx_rgf_plan_s* P, const GemmArgs<T>& g, cudaStream_t 
 // at least kTcF32Min in every dimension run on the tensor cores with four digit planes (~27-bit
 // products, at least FP32's precision; every digit group exact), the smaller ones on the SIMT GEMM.
 constexpr int kTcF32Min = 96;
-inline bool f32_on_tc(const qtx_rgf_desc& d) { return d.precision == QTX_EMU64 || d.precision == QTX_FP32; }
+inline bool f32_on_tc(const qtx_rgf_desc& d) { return d.precision != QTX_BF16X3; }
 template <>
 qtx_status gemm<float>(qtx_rgf_plan_s* P, const GemmArgs<float>& g, cudaStream_t st, bool, DigitHint) {
   if (f32_on_tc(P->d) && g.M >= kTcF32Min && g.N >= kTcF32Min && g.K >= kTcF32Min && g.K <= 1024 &&
@@ -302,6 +314,16 @@ qtx_status gemm<float>(qtx_rgf_plan_s* P, const GemmArgs<float>& g, cudaStream_t
 }
 template <>
 qtx_status gemm<double>(qtx_rgf_plan_s* P, const GemmArgs<double>& g, cudaStream_t st, bool, DigitHint) {
+  if (g.M >= kTcF64Min && g.N >= kTcF64Min && g.K >= kTcF64Min && gemm_fp64_tc_fits(g.M, g.N, g.K, P->L.tc_bytes)) {
+    cudaEvent_t* ev = (P->prof && P->d.precision == QTX_FP64) ? P->next_events() : nullptr;
+    QTX_CK(gemm_fp64_tc(g, P->ws + P->L.tc_scratch, P->L.tc_bytes, P->d_err_flag, st, ev));
+    if (ev) {
+      const double f = 8.0 * g.M * g.N * g.K * g.batch;
+      P->pipe_flops += f * tc_pairs_fp64();
+      P->useful_flops += f;
+    }
+    return QTX_OK;
+  }
   return gemm_simt_prof<double>(P, g, st);
 }
 inline int tc_digits(const qtx_rgf_desc& d) { return d.precision == QTX_EMU64 ? 6 : 2; }
@@ -414,7 +436,60 @@ qtx_status inverse_refined_f32(qtx_rgf_plan_s* P, cx<float>* A, int n, int batch
   return inverse_rec<float>(P, A, n, nn, n, batch, active, status, scr, nn, st, true);
 }
 
-// Block inverse used by the sweep.  FP64 / FP32: recursive inverse in the sweep precision.
+// FP64 block inverse of blocks beyond the fused leaf: X0 from the FP32 inverse, then Newton sweeps
+// X <- X + X (I - A X) with FP64 products on the tensor cores, which double the correct digits each
+// (an FP32 start leaves ||I - A X0|| near kappa 2^-24, so blocks of kappa 1e3 take three sweeps and
+// of 1e6 five).  An energy stops after the sweep whose residual norm was at most 2^-27: the next
+// residual is then its square, below FP64's resolution.  Energies still above it after kSweeps64
+// (ill-conditioned beyond FP32's reach, or non-finite) are inverted again from A by pivoted
+// elimination in FP64.  A DFMA Gauss-Jordan of a 64 x 64 leaf takes 770 us on one SM (GB300's FP64 pipe
+// runs at 1/64 of its FP32 rate); the FP32 leaf takes 62 us.
+constexpr int kSweeps64 = 5;
+qtx_status inverse_f64(qtx_rgf_plan_s* P, cx<double>* A, int n, int batch, const int* active, int* status,
+                       cudaStream_t st) {
+  if (n < kTcF64Min || n != P->b || !P->L.refine64 || !gemm_fp64_tc_fits(n, n, n, P->L.tc_bytes))
+    return inverse_refined<double>(P, A, n, batch, active, status, st);
+  const long nn = (long)n * n;
+  cx<float>* A32 = reinterpret_cast<cx<float>*>(P->ws + P->L.f32a);
+  cx<double>* Acopy = reinterpret_cast<cx<double>*>(P->ws + P->L.ref);
+  cx<double>* R = Acopy + (size_t)P->Ec * nn;
+  cx<double>* Xn = R + (size_t)P->Ec * nn;
+  const cx<double>* I = reinterpret_cast<const cx<double>*>(P->ws + P->L.ident);
+  Term<double> tA; tA.p = A; tA.s = nn; tA.alpha = 1.0;
+  Term<double> none;
+  Term<float> none32;
+  QTX_CK((combine<double, float>(A32, nn, tA, none, none, n, batch, nullptr, 0.0, 0.0, active, st)));
+  QTX_CK((combine<double, double>(Acopy, nn, tA, none, none, n, batch, nullptr, 0.0, 0.0, active, st)));
+  qtx_status s = inverse_refined_f32(P, A32, n, batch, active, nullptr, st);
+  if (s) return s;
+  Term<float> tX; tX.p = A32; tX.s = nn; tX.alpha = 1.0;
+  QTX_CK((combine<float, double>(A, nn, tX, none32, none32, n, batch, nullptr, 0.0, 0.0, active, st)));
+  int* masks = reinterpret_cast<int*>(P->ws + P->L.refine_act);
+  const int* act = active;
+  for (int it = 0; it < kSweeps64; ++it) {
+    int* next = masks + (it & 1) * P->Ec;
+    if ((s = gemm<double>(P, gargs<double>(n, n, n, Acopy, n, nn, OP_N, A, n, nn, OP_N, I, n, 0, R, n, nn, -1.0, 1.0, batch, act), st))) return s;
+    QTX_CK(residual_mask<double>(R, nn, n, batch, 0x1p-27, act, next, nullptr, st));
+    // X <- X + X R, in place while the whole contraction is one launch (the product reads X through
+    // its digit planes; a block with a non-finite entry races, and ends in the elimination below)
+    cx<double>* dst = n <= 512 ? A : Xn;
+    if ((s = gemm<double>(P, gargs<double>(n, n, n, A, n, nn, OP_N, R, n, nn, OP_N, A, n, nn, dst, n, nn, 1.0, 1.0, batch, act), st))) return s;
+    if (dst == Xn) {
+      Term<double> tXn; tXn.p = Xn; tXn.s = nn; tXn.alpha = 1.0;
+      QTX_CK((combine<double, double>(A, nn, tXn, none, none, n, batch, nullptr, 0.0, 0.0, act, st)));
+    }
+    act = next;
+  }
+  Term<double> tC; tC.p = Acopy; tC.s = nn; tC.alpha = 1.0;
+  QTX_CK((combine<double, double>(A, nn, tC, none, none, n, batch, nullptr, 0.0, 0.0, act, st)));
+  if (n <= kPivotedMax) {
+    QTX_CK(pivoted_inverse(A, nn, n, batch, act, status, reinterpret_cast<int*>(P->ws + P->L.perm), st));
+    return QTX_OK;
+  }
+  return inverse_refined<double>(P, A, n, batch, act, status, st);
+}
+
+// Block inverse used by the sweep.  FP64: inverse_f64.  FP32: recursive inverse in FP32.
 // EMU64 / BF16X3: X0 from the recursive inverse in FP32, then Newton refinement
 // X <- X + X (I - A X) with both products on the tensor-core engine (the residual I - A X is
 // formed in emulated FP64 before it is rounded for the correction product).
@@ -431,7 +506,7 @@ qtx_status block_inverse<float>(qtx_rgf_plan_s* P, cx<float>* A, int n, int batc
 template <>
 qtx_status block_inverse<double>(qtx_rgf_plan_s* P, cx<double>* A, int n, int batch, const int* active,
                                  int* status, cudaStream_t st) {
-  return inverse_refined<double>(P, A, n, batch, active, status, st);
+  return inverse_f64(P, A, n, batch, active, status, st);
 }
 
 // Emulated modes (df32 storage): X0 from the FP32 inverse of the leading parts, then Newton sweeps
@@ -535,7 +610,7 @@ qtx_status contact(const Ctx<T>& c, const cx<double>* H00, const cx<double>* H01
   for (int it = 1; it <= P->d.decim_max_iter; ++it) {
     Term<double> te; te.p = eps; te.s = bb; te.alpha = -1.0;
     QTX_CK((combine<double, double>(g, bb, te, none, none, b, ne, c.E, eta, 1.0, active, st)));  // z - eps
-    if ((s = inverse_refined<double>(P, g, b, ne, active, c.status, st))) return s;
+    if ((s = inverse_f64(P, g, b, ne, active, c.status, st))) return s;
     if ((s = G(alpha, g, ag))) return s;
     if ((s = G(beta, g, bg))) return s;
     if ((s = G(ag, beta, t1))) return s;   // alpha g beta
@@ -557,7 +632,7 @@ qtx_status contact(const Ctx<T>& c, const cx<double>* H00, const cx<double>* H01
   QTX_CK(flag_active(active, c.status, (int)QTX_ERR_NOT_CONVERGED, ne, st));
   Term<double> tes; tes.p = eps_s; tes.s = bb; tes.alpha = -1.0;
   QTX_CK((combine<double, double>(g, bb, tes, none, none, b, ne, c.E, eta, 1.0, nullptr, st)));  // z - eps_s
-  if ((s = inverse_refined<double>(P, g, b, ne, nullptr, c.status, st))) return s;
+  if ((s = inverse_f64(P, g, b, ne, nullptr, c.status, st))) return s;
   // Sigma^R = H01 g_s H01^H
   if ((s = gemm<double>(P, gargs<double>(b, b, b, H01, b, 0, OP_N, g, b, bb, OP_N, nullptr, 0, 0, t1, b, bb, 1.0, 0.0, ne, nullptr), st, true))) return s;
   if ((s = gemm<double>(P, gargs<double>(b, b, b, t1, b, bb, OP_N, H01, b, 0, OP_C, nullptr, 0, 0, SR, b, bb, 1.0, 0.0, ne, nullptr), st, true))) return s;
@@ -1347,6 +1422,43 @@ const char* qtx_rgf_version(void) { return "qtx-rgf 0.1 (sm_103a)"; }
 // ============================================================================ component ABI
 namespace {
 
+// FP64 products of at least kTcF64Min in every dimension: straight from the caller's arrays into C on
+// the tensor cores (only digit planes are allocated), unless C overlaps an operand.
+bool overlaps(const void* X, int rows, int cols, long ld, long sX, int nX, const void* Y, int rowsY, int colsY, long ldY,
+              long sY, int nY) {
+  auto span = [](const void* p, int r, int c, long ld, long s, int n, uintptr_t& lo, uintptr_t& hi) {
+    const long row = (long)(r - 1) * ld, ent = (long)(n - 1) * s;
+    const long a = std::min(0L, row) + std::min(0L, ent), b = std::max(0L, row) + std::max(0L, ent) + c;
+    lo = (uintptr_t)((const cx<double>*)p + a);
+    hi = (uintptr_t)((const cx<double>*)p + b);
+  };
+  uintptr_t a0, a1, b0, b1;
+  span(X, rows, cols, ld, sX, nX, a0, a1);
+  span(Y, rowsY, colsY, ldY, sY, nY, b0, b1);
+  return a0 < b1 && b0 < a1;
+}
+qtx_status zgemm_fp64_direct(const GemmArgs<double>& g, cudaStream_t st, std::string& err) {
+  const size_t bytes = gemm_fp64_tc_scratch_bytes(g.M, g.N, g.K, g.batch);
+  void* scr = nullptr;
+  int* flag = nullptr;
+  int hflag = 0;
+  cudaError_t e = cudaMallocAsync(&scr, bytes, st);
+  if (e == cudaSuccess) e = cudaMallocAsync((void**)&flag, sizeof(int), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(flag, 0, sizeof(int), st);
+  if (e == cudaSuccess) e = gemm_fp64_tc(g, scr, bytes, flag, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
+  if (scr) cudaFreeAsync(scr, st);
+  if (flag) cudaFreeAsync(flag, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) {
+    err = cudaGetErrorString(e);
+    cudaGetLastError();
+    return QTX_ERR_CUDA;
+  }
+  if (hflag) { err = "tensor-core engine: bounded wait expired"; return QTX_ERR_TIMEOUT; }
+  return QTX_OK;
+}
+
 template <typename T>
 qtx_status zgemm_via(int precision, int M, int N, int K, int opA, const void* A, long lda, long sA, int opB,
                      const void* B, long ldb, long sB, double alpha, double beta, const void* C0, long ldc0,
@@ -1354,6 +1466,16 @@ qtx_status zgemm_via(int precision, int M, int N, int K, int opA, const void* A,
   const int rA = opA == OP_N ? M : K, cA = opA == OP_N ? K : M;
   const int rB = opB == OP_N ? K : N, cB = opB == OP_N ? N : K;
   const int nA = sA ? batch : 1, nB = sB ? batch : 1, nC0 = (C0 && beta != 0.0) ? (sC0 ? batch : 1) : 0;
+  if constexpr (std::is_same<T, double>::value) {
+    // C may be C0 itself (same layout); any other overlap takes the copies below
+    const bool c0_ok = !nC0 || (C0 == C && ldc0 == ldc && sC0 == sC) || !overlaps(C, M, N, ldc, sC, batch, C0, M, N, ldc0, sC0, nC0);
+    if (M >= kTcF64Min && N >= kTcF64Min && K >= kTcF64Min && tc_available() && c0_ok &&
+        !overlaps(C, M, N, ldc, sC, batch, A, rA, cA, lda, sA, nA) && !overlaps(C, M, N, ldc, sC, batch, B, rB, cB, ldb, sB, nB)) {
+      return zgemm_fp64_direct(gargs<double>(M, N, K, (const cx<double>*)A, lda, sA, opA, (const cx<double>*)B, ldb, sB, opB,
+                                             nC0 ? (const cx<double>*)C0 : nullptr, ldc0, nC0 > 1 ? sC0 : 0, (cx<double>*)C, ldc, sC,
+                                             alpha, nC0 ? beta : 0.0, batch, nullptr), st, err);
+    }
+  }
   const size_t es = sizeof(cx<T>);
   void *a = nullptr, *b = nullptr, *c0 = nullptr, *c = nullptr, *scr = nullptr;
   int* flag = nullptr;

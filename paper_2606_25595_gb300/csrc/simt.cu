@@ -754,31 +754,136 @@ template cudaError_t assemble_offdiag<double>(cx<double>*, cx<double>*, const cx
 template cudaError_t assemble_offdiag<float>(cx<float>*, cx<float>*, const cx<double>*, const cx<double>*, const double*, double, int, int, cudaStream_t, const cx<double>*, const cx<double>*, long);
 template cudaError_t assemble_offdiag<df>(cx<df>*, cx<df>*, const cx<double>*, const cx<double>*, const double*, double, int, int, cudaStream_t, const cx<double>*, const cx<double>*, long);
 
-__global__ void __launch_bounds__(256) k_residual_mask(const cx<df>* R, long sR, long nn, float tol2,
+// FP32 magnitude of a residual entry: the df32 value's leading part, or an FP64 value truncated to FP32
+// by integer operations (its exponent range clamped to FP32's).
+__device__ __forceinline__ float mag32(df x) { return x.hi; }
+__device__ __forceinline__ float mag32(double x) {
+  const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu;
+  const int e = (int)(h >> 20) - 1023 + 127;
+  if (e >= 255) return h > 0x7ff00000u || (h == 0x7ff00000u && __double2loint(x)) ? __uint_as_float(0x7fc00000u) : __uint_as_float(0x7f800000u);
+  return e <= 0 ? 0.f : __uint_as_float(((unsigned)e << 23) | ((h & 0xfffffu) << 3) | ((unsigned)__double2loint(x) >> 29));
+}
+template <typename T>
+__global__ void __launch_bounds__(512) k_residual_mask(const cx<T>* R, long sR, long nn, float tol2,
                                                        const int* active, int* next, int* status) {
   const int e = blockIdx.x;
   if (active && !active[e]) {
     if (threadIdx.x == 0) next[e] = 0;
     return;
   }
-  const cx<df>* X = R + (long)e * sR;
+  const cx<T>* X = R + (long)e * sR;
   float s = 0.f;
-  for (long i = threadIdx.x; i < nn; i += blockDim.x) s = fmaf(X[i].re.hi, X[i].re.hi, fmaf(X[i].im.hi, X[i].im.hi, s));
-  __shared__ float red[8];
+  for (long i = threadIdx.x; i < nn; i += blockDim.x) {
+    const cx<T> x = X[i];
+    const float a = mag32(x.re), c = mag32(x.im);
+    s = fmaf(a, a, fmaf(c, c, s));
+  }
+  __shared__ float red[16];
   for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
   if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = s;
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) s += red[w];
+    for (int w = 1; w < 16; ++w) s += red[w];
     // a NaN or infinite norm compares false against tol2: such an energy keeps refining, and its
     // block inverse has failed, so it is reported singular
     next[e] = (s <= tol2) ? 0 : 1;
     if (status && !(s <= 3.0e38f)) atomicCAS(status + e, 0, (int)QTX_ERR_SINGULAR);
   }
 }
-cudaError_t residual_mask(const cx<df>* R, long sR, int n, int batch, double tol, const int* active, int* next,
+template <typename T>
+cudaError_t residual_mask(const cx<T>* R, long sR, int n, int batch, double tol, const int* active, int* next,
                           int* status, cudaStream_t st) {
-  k_residual_mask<<<batch, 256, 0, st>>>(R, sR, (long)n * n, (float)(tol * tol), active, next, status);
+  k_residual_mask<T><<<batch, 512, 0, st>>>(R, sR, (long)n * n, (float)(tol * tol), active, next, status);
+  count_launch();
+  return cudaGetLastError();
+}
+template cudaError_t residual_mask<df>(const cx<df>*, long, int, int, double, const int*, int*, int*, cudaStream_t);
+template cudaError_t residual_mask<double>(const cx<double>*, long, int, int, double, const int*, int*, int*, cudaStream_t);
+
+// Pivoted Gauss-Jordan of one block per CTA in global memory (L2): latency-bound, about n^3 / 0.5 G
+// complex FMAs a second per block; it only runs for blocks the refined FP32 inverse cannot resolve.
+// Row interchanges are made as the elimination goes and undone as column interchanges at the end.
+__global__ void __launch_bounds__(512) k_pivoted_inverse(cx<double>* Ag, long sA, int n, const int* active, int* status,
+                                                         int* permg) {
+  const int e = blockIdx.x, t = threadIdx.x;
+  if (active && !active[e]) return;
+  cx<double>* A = Ag + (long)e * sA;
+  int* perm = permg + (long)e * n;
+  __shared__ double s_best[16];
+  __shared__ int s_at[16];
+  __shared__ int s_p;
+  for (int k = 0; k < n; ++k) {
+    double best = -1.0;
+    int at = n;
+    for (int i = k + t; i < n; i += blockDim.x) {
+      const double v = cabs1(A[(long)i * n + k]);
+      if (v > best || v != v) {  // a NaN is taken, and rejected below
+        best = v;
+        at = i;
+      }
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+      const double ov = __shfl_down_sync(0xffffffffu, best, off);
+      const int oi = __shfl_down_sync(0xffffffffu, at, off);
+      if (ov > best || ov != ov || (ov == best && oi < at)) {
+        best = ov;
+        at = oi;
+      }
+    }
+    if (t % 32 == 0) {
+      s_best[t / 32] = best;
+      s_at[t / 32] = at;
+    }
+    __syncthreads();
+    if (t == 0) {
+      for (int w = 1; w < 16; ++w)
+        if (s_best[w] > best || s_best[w] != s_best[w] || (s_best[w] == best && s_at[w] < at)) {
+          best = s_best[w];
+          at = s_at[w];
+        }
+      s_p = (best > 0.0 && isfinite(best)) ? at : -1;
+      perm[k] = s_p;
+    }
+    __syncthreads();
+    const int p = s_p;
+    if (p < 0) {
+      if (t == 0 && status) atomicCAS(status + e, 0, (int)QTX_ERR_SINGULAR);
+      return;
+    }
+    const cx<double> r = crecip(A[(long)p * n + k]);
+    __syncthreads();
+    for (int j = t; j < n; j += blockDim.x) {  // interchange rows k and p; row k scaled by 1 / pivot
+      const cx<double> x = A[(long)p * n + j];
+      if (p != k) A[(long)p * n + j] = A[(long)k * n + j];
+      A[(long)k * n + j] = j == k ? r : x * r;
+    }
+    __syncthreads();
+    // one warp per row at a time: every lane holds the row's factor before column k is overwritten
+    for (int i = t / 32; i < n; i += (int)blockDim.x / 32) {
+      if (i == k) continue;
+      const cx<double> f = A[(long)i * n + k];
+      __syncwarp();
+      for (int j = t % 32; j < n; j += 32) {
+        const cx<double> x = j == k ? mk<double>(0.0, 0.0) : A[(long)i * n + j];
+        A[(long)i * n + j] = x - f * A[(long)k * n + j];
+      }
+    }
+    __syncthreads();
+  }
+  for (int k = n - 1; k >= 0; --k) {
+    const int p = perm[k];
+    if (p != k)
+      for (int i = t; i < n; i += blockDim.x) {
+        const cx<double> x = A[(long)i * n + k];
+        A[(long)i * n + k] = A[(long)i * n + p];
+        A[(long)i * n + p] = x;
+      }
+    __syncthreads();
+  }
+}
+cudaError_t pivoted_inverse(cx<double>* A, long sA, int n, int batch, const int* active, int* status, int* perm,
+                            cudaStream_t st) {
+  k_pivoted_inverse<<<batch, 512, 0, st>>>(A, sA, n, active, status, perm);
   count_launch();
   return cudaGetLastError();
 }

@@ -1,0 +1,545 @@
+// FP64 batched complex products on the tcgen05 tensor cores (sm_103a).
+//
+// C[e] = alpha * op(A[e]) * op(B[e]) + beta * C0[e]   (complex128 in and out)
+//
+// GB300's FP64 pipe gives 1.1 TFLOP/s, so a DFMA product of 256 x 256 blocks takes 130 us per batch
+// entry.  Here every row of op(A) and column of op(B) is scaled by a power of two and rounded to a
+// 62-bit integer (61 bits when K > 256), nine bits below the last place of the row's largest entry,
+// and written as nine balanced base-128 digits in bf16 planes (Ozaki-style slicing, paper Sec. II-D).
+// The 45 digit products with i + j <= 10 run as tcgen05.mma kind::f16 into eight TMEM accumulators:
+//   acc0..acc6: i + j = 2..8, exact in FP32 (multiples of 2^(-7 (i+j-2)), below 2^24 units),
+//   acc7:       i + j = 9, 10, below 2^-32 of the leading group: its FP32 rounding is below 2^-56.
+// The epilogue converts the accumulators to integers, adds them in 92-bit fixed point and rounds to
+// FP64 once, so a product carries one rounding of the whole sum plus the operands' 2^-62 (measured
+// against 64-bit references: closer than the DFMA product, whose rounding errors grow with K).
+//
+// Why nine digits and eight accumulators: eight digits (36 products) drop digit products at 2^-51 of
+// the result, as much as DFMA's own rounding; nine put the truncation near 2^-58.  Eight
+// accumulators of 64 columns (32 complex columns, MMA N = 64, 24.8 ns each) fill the 512 TMEM
+// columns; nine exact ones would leave 24 complex columns at nearly the same time per instruction.
+//
+// Rows or columns with an infinity or a NaN take digits of zero and are computed by the epilogue with
+// DFMA from the operands themselves, so they propagate as in an FP64 product.
+//
+// Kernel structure: as the product kernel of tc_engine.cu (persistent, one CTA per SM, a producer
+// warp of bulk copies, one MMA-issuing thread, eight epilogue warps, every wait bounded).
+#include <cuda_bf16.h>
+
+#include <atomic>
+
+#include "fix64.cuh"
+#include "kernels.cuh"
+#include "tc_ptx.cuh"
+
+namespace qtx {
+namespace tc {
+namespace {
+
+constexpr int S9 = kDig64;
+constexpr int BNC9 = 32;                    // complex output columns per tile (MMA N = 64)
+constexpr int NACC9 = 8;
+constexpr int ACC9 = 2 * BNC9;              // TMEM columns of one accumulator
+constexpr int TILE_B9 = 2 * BNC9 * BKS * 2;  // bytes of one B-plane tile (Re and Im rows)
+constexpr int SUB_B9 = BNC9 * BKS * 2;
+constexpr int STAGE9 = S9 * (TILE_A + TILE_B9);  // 54 KB
+constexpr int NST9 = 3;
+constexpr int OUT9 = BM * BNC9 * 16;        // staging: [BM][BNC9] complex128, XOR-swizzled
+constexpr int SMEM9 = NST9 * STAGE9 + OUT9 + (BM + BNC9) * 4 + 128;
+
+struct Params {
+  const unsigned char* pa;  // A plane tiles [batch'][9][M_pad/128][nks][128 x 32 B]
+  const unsigned char* pb;  // B sub-tiles [batch'][9][N_pad/32][K_pad/16][3][32 x 32 B]: Re, Im, -Im
+  const int *eA, *eB;
+  int M_pad, N_pad, nks, M, N, K, bn_last, escale;
+  int a_batched, b_batched;
+  const cx<double>*A, *B;   // the operands (rows and columns with non-finite values)
+  long lda, sA, ldb, sB;
+  int opA, opB;
+  cx<double>* C; long ldc, sC;
+  const cx<double>* C0; long ldc0, sC0;
+  double alpha, beta;
+  int akind, bkind;         // alpha: 0 = +1, 1 = -1, 2 = general; beta the same, 3 = no C0 term
+  const int* active;
+  int* err;
+  int NBt, MBt, n_tiles, hold;
+  uint64_t limit_ns;
+};
+
+__device__ __forceinline__ int at9(int r, int c) { return r * BNC9 + (c ^ (r & 7)); }
+
+// one output value from the eight accumulators (pre-scaled digit products)
+__device__ __forceinline__ double recombine(const uint32_t (&v)[NACC9][8], int c) {
+  // exact groups as integers of their own unit 2^(-7 g); the tail in units of 2^-53
+  auto fx = [&](int g, int sh) { return (int64_t)__float2int_rn(__uint_as_float(v[g][c]) * __int_as_float((127 + sh) << 23)); };
+  const int64_t hi = (fx(0, 0) << 28) + (fx(1, 7) << 21) + (fx(2, 14) << 14) + (fx(3, 21) << 7) + fx(4, 28);
+  const int64_t lo = (fx(5, 35) << 21) + (fx(6, 42) << 14) + (fx(7, 53) << 3);
+  return fix_sum(hi, lo);
+}
+
+// (op(A) op(B))(m, n) of one batch entry by DFMA: rows or columns with non-finite values
+__device__ __noinline__ cx<double> dot_dfma(const Params& p, int e, int m, int n) {
+  const cx<double>* A = p.A + (long)e * p.sA;
+  const cx<double>* B = p.B + (long)e * p.sB;
+  cx<double> acc = mk<double>(0.0, 0.0);
+  for (int k = 0; k < p.K; ++k) {
+    const cx<double> a = p.opA == OP_N ? A[(long)m * p.lda + k] : conj(A[(long)k * p.lda + m]);
+    const cx<double> b = p.opB == OP_N ? B[(long)k * p.ldb + n] : conj(B[(long)n * p.ldb + k]);
+    cfma(acc, a, b);
+  }
+  return acc;
+}
+
+__global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__ Params p) {
+  extern __shared__ __align__(1024) unsigned char base[];
+  cx<double>* out = reinterpret_cast<cx<double>*>(base + NST9 * STAGE9);
+  int* s_eA = reinterpret_cast<int*>(base + NST9 * STAGE9 + OUT9);
+  int* s_eB = s_eA + BM;
+  uint64_t* full = reinterpret_cast<uint64_t*>(s_eB + BNC9);
+  uint64_t* empty = full + NST9;
+  uint64_t* accf = empty + NST9;
+  uint64_t* acce = accf + 1;
+  uint64_t* holdbar = acce + 1;   // never arrived at (the wait test)
+  uint64_t* drainbar = acce + 2;  // the MMA thread's final commit
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(acce + 3);
+  int* s_got = reinterpret_cast<int*>(tslot + 1);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < NST9; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(accf, 1);
+    mbar_init(acce, 1);
+    mbar_init(holdbar, 1);
+    mbar_init(drainbar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = *tslot;
+  const int per_e = p.NBt * p.MBt;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      long g = 0;
+      bool ok = true;
+      const long MB = p.M_pad / BM, NB = p.N_pad / BNC9, nkb = p.nks / 2;
+      for (int k = 0; ok; ++k) {
+        const long t = tile_at(k);
+        if (t >= p.n_tiles) break;
+        const int e = (int)(t / per_e), mblk = (int)((t / p.NBt) % p.MBt), nblk = (int)(t % p.NBt);
+        if (p.active && !p.active[e]) continue;
+        const long ea = p.a_batched ? e : 0, eb = p.b_batched ? e : 0;
+        const uint32_t sub = (uint32_t)(nblk == p.NBt - 1 ? p.bn_last : BNC9) * BKS * 2;
+        for (int ks = 0; ks < p.nks; ++ks, ++g) {
+          const int s = (int)(g % NST9);
+          if (!mbar_wait(&empty[s], ((uint32_t)(g / NST9) & 1u) ^ 1u, p.err, p.limit_ns)) { ok = false; break; }
+          mbar_expect_tx(&full[s], S9 * (TILE_A + 2 * sub));
+          unsigned char* st = base + s * STAGE9;
+          // K-stages [0, nkb): A's real parts against (Re, Im); [nkb, 2 nkb): imaginary against (-Im, Re)
+          const int part = ks >= nkb, kb = (int)(ks - part * nkb), s0 = part ? 2 : 0, s1 = part ? 0 : 1;
+          for (int d = 0; d < S9; ++d) {
+            bulk_load(st + d * TILE_A, p.pa + (((ea * S9 + d) * MB + mblk) * p.nks + ks) * (long)TILE_A, TILE_A, &full[s]);
+            const unsigned char* sb = p.pb + (((eb * S9 + d) * NB + nblk) * nkb + kb) * 3L * SUB_B9;
+            unsigned char* db = st + S9 * TILE_A + d * TILE_B9;
+            bulk_load(db, sb + s0 * SUB_B9, sub, &full[s]);
+            bulk_load(db + sub, sb + s1 * SUB_B9, sub, &full[s]);
+          }
+        }
+      }
+      // the copies of the last stages issued land before the CTA goes on to exit
+      for (long gi = g > NST9 ? g - NST9 : 0; gi < g; ++gi)
+        mbar_wait_drain(&full[gi % NST9], (uint32_t)(gi / NST9) & 1u, kWaitLimitNs);
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    if (lane == 0) {
+      long g = 0;
+      int j = 0;
+      bool ok = true;
+      if (p.hold && !mbar_wait(holdbar, 0u, p.err, p.limit_ns)) ok = false;
+      for (int k = 0; ok; ++k) {
+        const long t = tile_at(k);
+        if (t >= p.n_tiles) break;
+        if (p.active && !p.active[(int)(t / per_e)]) continue;
+        const uint32_t idesc = idesc_n(2 * ((int)(t % p.NBt) == p.NBt - 1 ? p.bn_last : BNC9));
+        if (!mbar_wait(acce, ((uint32_t)j & 1u) ^ 1u, p.err, p.limit_ns)) break;
+        fence_after();
+        uint32_t started = 0;
+        for (int ks = 0; ks < p.nks; ++ks, ++g) {
+          const int s = (int)(g % NST9);
+          if (!mbar_wait(&full[s], (uint32_t)(g / NST9) & 1u, p.err, p.limit_ns)) { ok = false; break; }
+          fence_after();
+          const uint32_t sa = su32(base + s * STAGE9);
+#pragma unroll
+          for (int i = 1; i <= S9; ++i) {
+#pragma unroll
+            for (int jj = 1; jj <= S9 + 1 - i; ++jj) {
+              const int ga = i + jj - 2 < NACC9 - 1 ? i + jj - 2 : NACC9 - 1;
+              mma(tmem + ga * ACC9, sdesc(sa + (i - 1) * TILE_A), sdesc(sa + S9 * TILE_A + (jj - 1) * TILE_B9), idesc,
+                  (started >> ga) & 1u);
+              started |= 1u << ga;
+            }
+          }
+          mma_commit(&empty[s]);
+        }
+        if (!ok) break;
+        mma_commit(accf);
+        ++j;
+      }
+      mma_commit(drainbar);
+      mbar_wait_drain(drainbar, 0u, kWaitLimitNs);
+    }
+    __syncwarp();
+  } else {
+    // epilogue: warps 2..9; TMEM lane quarter = warp % 4, alternate chunks of 8 columns by half
+    const int q = warp & 3, h = (warp - 2) >> 2;
+    const int r = q * 32 + lane;
+    const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16);
+    const int et = threadIdx.x - 64;
+    int j = 0;
+    for (int k = 0;; ++k) {
+      const long t = tile_at(k);
+      if (t >= p.n_tiles) break;
+      const int e = (int)(t / per_e), mblk = (int)((t / p.NBt) % p.MBt), nblk = (int)(t % p.NBt);
+      if (p.active && !p.active[e]) continue;
+      const int bn = nblk == p.NBt - 1 ? p.bn_last : BNC9;
+      __syncwarp();
+      asm volatile("bar.sync 1, 256;" ::: "memory");  // the previous tile's staging area is free
+      if (et < BNC9) s_eB[et] = p.eB[(long)(p.b_batched ? e : 0) * p.N_pad + nblk * BNC9 + et];
+      if (et >= 64 && et < 64 + BM) s_eA[et - 64] = p.eA[(long)(p.a_batched ? e : 0) * p.M_pad + mblk * BM + et - 64];
+      if (et == 0) *s_got = mbar_wait(accf, (uint32_t)j & 1u, p.err, p.limit_ns) ? 1 : 0;
+      __syncwarp();
+      asm volatile("bar.sync 2, 256;" ::: "memory");
+      if (!*s_got) break;
+      fence_after();
+#pragma unroll 1
+      for (int c0 = 8 * h; c0 < bn; c0 += 16) {
+#pragma unroll 1
+        for (int part = 0; part < 2; ++part) {
+          uint32_t v[NACC9][8];
+#pragma unroll
+          for (int g = 0; g < NACC9; ++g) tmem_ld8(trow + g * ACC9 + part * bn + c0, v[g]);
+          tmem_wait_ld();
+#pragma unroll
+          for (int c = 0; c < 8; ++c) (&out[at9(r, c0 + c)].re)[part] = recombine(v, c);
+        }
+      }
+      fence_before();
+      __syncwarp();
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      if (et == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(acce)) : "memory");
+      // store phase, overlapping the next tile's MMAs: scale, alpha, beta C0
+      const cx<double>* C0e = p.C0 ? p.C0 + (long)e * p.sC0 : nullptr;
+      cx<double>* Ce = p.C + (long)e * p.sC;
+      for (int idx = et; idx < BM * bn; idx += 256) {
+        const int rr = idx / bn, cc = idx % bn;
+        const int m = mblk * BM + rr, n = nblk * BNC9 + cc;
+        if (m >= p.M || n >= p.N) continue;
+        cx<double> v = out[at9(rr, cc)];
+        const int ea = s_eA[rr], eb = s_eB[cc];
+        if (ea >= kExpoNonFinite || eb >= kExpoNonFinite) {
+          v = dot_dfma(p, e, m, n);
+        } else {
+          v.re = scale64(v.re, ea + eb - p.escale);
+          v.im = scale64(v.im, ea + eb - p.escale);
+        }
+        if (p.akind == 1) v = mk<double>(-v.re, -v.im);
+        else if (p.akind == 2) v = p.alpha * v;
+        if (p.bkind != 3) {
+          cx<double> c0 = C0e[(long)m * p.ldc0 + n];
+          if (p.bkind == 1) c0 = mk<double>(-c0.re, -c0.im);
+          else if (p.bkind == 2) c0 = p.beta * c0;
+          v = v + c0;
+        }
+        Ce[(long)m * p.ldc + n] = v;
+      }
+      ++j;
+    }
+  }
+  __syncwarp();
+  fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+  }
+}
+
+// ------------------------------------------------------------------------------ digit planes
+// Row exponents and digit planes of one operand in one pass: a strip of RPC logical rows (rows of
+// op(A), columns of op(B)) goes once from global to shared memory, one warp per row; each thread then
+// turns 8 consecutive k of a row into nine 16-byte plane chunks per part.  Bound by HBM: it reads 16 B
+// and writes 36 (left) or 54 B (right operand: Re, Im, -Im) per complex value.
+__host__ __device__ constexpr int skew9(int k) { return k + (k >> 3); }
+
+template <int RPC>
+__global__ void __launch_bounds__(32 * RPC) k_digitize_fp64(const cx<double>* X, long ldx, long sX, int R, int K, int R_pad,
+                                                            int K_pad, int transposed, int conj_, int side, int* eout, int P,
+                                                            unsigned char* planes, const int* active) {
+  const int e = blockIdx.y;
+  if (active && !active[e]) return;
+  extern __shared__ __align__(16) unsigned char dsm[];
+  constexpr int NT = 32 * RPC;
+  const int ldS = skew9(K_pad) + 1;
+  cx<double>* strip = reinterpret_cast<cx<double>*>(dsm);
+  __shared__ int s_ex[RPC];
+  const cx<double>* Xe = X + (long)e * sX;
+  const int r0 = blockIdx.x * RPC, t = threadIdx.x;
+  if (t < RPC) s_ex[t] = kExpoZero;
+  __syncthreads();
+  const cx<double> zero = mk<double>(0.0, 0.0);
+  // direct strips: threads along k (row by row); transposed ones: threads along the rows, then k
+  const int rs = transposed ? t % RPC : 0, k1 = transposed ? t / RPC : t, kst = transposed ? NT / RPC : NT;
+  for (int rr = rs; rr < RPC; rr += transposed ? RPC : 1) {
+    const int r = r0 + rr;
+    int mx = kExpoZero;
+    for (int k0 = k1; k0 < K_pad; k0 += 4 * kst) {
+      cx<double> v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int k = k0 + u * kst;
+        v[u] = (r < R && k < K) ? Xe[transposed ? (long)k * ldx + r : (long)r * ldx + k] : zero;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int k = k0 + u * kst;
+        if (k >= K_pad) break;
+        strip[rr * ldS + skew9(k)] = v[u];
+        mx = max(mx, max(expo64(v[u].re), expo64(v[u].im)));
+      }
+    }
+    const int grp = transposed ? RPC : 1;  // lanes of a warp that hold the same row are grp apart
+    for (int off = 16; off >= grp; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    if ((t & 31) < grp) atomicMax(&s_ex[rr], mx);
+  }
+  __syncthreads();
+  if (t < RPC && r0 + t < R_pad) eout[(long)e * R_pad + r0 + t] = s_ex[t];
+  const long nks = 2L * K_pad / BKS, nkb = K_pad / BKS;
+  const long plane_bytes = side == 0 ? (long)(R_pad / BM) * nks * TILE_A : (long)(R_pad / BNC9) * nkb * 3 * SUB_B9;
+  unsigned char* pe = planes + (long)e * S9 * plane_bytes;
+  const int nkc = K_pad / 8;
+  const int R_wr = side == 1 ? min(R_pad, (R + 7) / 8 * 8) : R_pad;  // columns past bn_last are never read
+#pragma unroll 1
+  for (int item = t; item < RPC * nkc; item += NT) {
+    const int rr = item / nkc, k8 = 8 * (item % nkc), r = r0 + rr;
+    if (r >= R_wr) continue;
+    const int ex = s_ex[rr];
+    const bool dead = ex >= kExpoNonFinite;  // zero digits; the product kernel computes these by DFMA
+    uint64_t vr[8], vi[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      cx<double> v = strip[rr * ldS + skew9(k8 + j)];
+      if (conj_) v.im = -v.im;
+      vr[j] = dead ? kDigBias : fix_biased(v.re, P - ex);
+      vi[j] = dead ? kDigBias : fix_biased(v.im, P - ex);
+    }
+    long o0, o1, o2 = 0;
+    if (side == 0) {
+      const long blk = r / BM, rw = r % BM;
+      auto off = [&](int kp) { return (blk * nks + kp / BKS) * TILE_A + sw32_offset((uint32_t)rw, (uint32_t)(kp % BKS)); };
+      o0 = off(k8);
+      o1 = off(K_pad + k8);
+    } else {
+      const long cb = r / BNC9, rw = r % BNC9;
+      const long o = (cb * nkb + k8 / BKS) * 3 * (long)SUB_B9 + sw32_offset((uint32_t)rw, (uint32_t)(k8 % BKS));
+      o0 = o;
+      o1 = o + SUB_B9;
+      o2 = o + 2 * SUB_B9;
+    }
+#pragma unroll
+    for (int i = 0; i < S9; ++i) {
+      // digits d 2^(-7 i) as bf16: 0x4300 | (d + 64) is the bf16 of 192 + d (also for
+      // d = 64, where the OR carries into the exponent: 256), and (192 + d) s - 192 s is exact
+      const __nv_bfloat162 s = __float2bfloat162_rn(__int_as_float((127 - DW * i) << 23));
+      const __nv_bfloat162 m = __float2bfloat162_rn(-192.f * __int_as_float((127 - DW * i) << 23));
+      auto word = [&](uint64_t a, uint64_t b) {
+        const uint32_t w = 0x43004300u | digit_field(a, i) | (digit_field(b, i) << 16);
+        const __nv_bfloat162 d = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w), s, m);
+        return *reinterpret_cast<const uint32_t*>(&d);
+      };
+      unsigned char* pl = pe + (long)i * plane_bytes;
+      const uint4 re = make_uint4(word(vr[0], vr[1]), word(vr[2], vr[3]), word(vr[4], vr[5]), word(vr[6], vr[7]));
+      const uint4 im = make_uint4(word(vi[0], vi[1]), word(vi[2], vi[3]), word(vi[4], vi[5]), word(vi[6], vi[7]));
+      *reinterpret_cast<uint4*>(pl + o0) = re;
+      *reinterpret_cast<uint4*>(pl + o1) = im;
+      if (side == 1) {
+        const uint32_t g = 0x80008000u;  // the bf16 sign bits
+        *reinterpret_cast<uint4*>(pl + o2) = make_uint4(im.x ^ g, im.y ^ g, im.z ^ g, im.w ^ g);
+      }
+    }
+  }
+}
+
+// ------------------------------------------------------------------------------ host side
+constexpr int kMaxK9 = 512;  // longest contraction of one launch (exactness of the leading groups)
+
+struct Dims9 {
+  int M_pad, N_pad, K_pad, l1, P;
+  size_t a, b, ea, eb;  // bytes per batch entry
+};
+size_t al1k(size_t x) { return (x + 1023) & ~size_t(1023); }
+Dims9 dims9(int M, int N, int K) {
+  Dims9 d;
+  d.M_pad = (M + BM - 1) / BM * BM;
+  d.N_pad = (N + BNC9 - 1) / BNC9 * BNC9;
+  d.K_pad = (K + 15) / 16 * 16;
+  if (d.K_pad == 0) d.K_pad = 16;
+  // the leading digit's magnitude (64, or 32 beyond 512 embedded K) keeps the groups through
+  // i + j = 6 below 2^24 units whatever the data; later groups that exceed it (operands whose digits
+  // all agree in sign) round at 2^-24 of a sum that is 2^-35 and less of such a product
+  d.l1 = 2 * d.K_pad <= 512 ? 7 : 6;
+  d.P = DW * (S9 - 1) + d.l1 - 1;
+  d.a = al1k((size_t)S9 * d.M_pad * 2 * d.K_pad * 2);
+  d.b = al1k((size_t)S9 * (d.N_pad / BNC9) * (d.K_pad / BKS) * 3 * SUB_B9);
+  d.ea = al1k((size_t)d.M_pad * sizeof(int));
+  d.eb = al1k((size_t)d.N_pad * sizeof(int));
+  return d;
+}
+int chunk_k(int K) {
+  const int nc = (K + kMaxK9 - 1) / kMaxK9;
+  return nc <= 1 ? K : (K + nc - 1) / nc;
+}
+
+cudaError_t digitize9(const cx<double>* X, long ldx, long sX, int opX, int side, int R, int K, const Dims9& d, int* eout,
+                      unsigned char* planes, int batch, const int* active, cudaStream_t st) {
+  const int transposed = (side == 0) ? (opX == OP_C) : (opX == OP_N);
+  const int R_pad = side == 0 ? d.M_pad : d.N_pad;
+  constexpr int RPC = 4;  // transposed strips read four values of 16 bytes in a row: whole 32-byte sectors
+  const size_t smem = (size_t)RPC * (skew9(d.K_pad) + 1) * sizeof(cx<double>);  // at most 37 KB
+  k_digitize_fp64<RPC><<<dim3(R_pad / RPC, batch), 32 * RPC, smem, st>>>(X, ldx, sX, R, K, R_pad, d.K_pad, transposed,
+                                                                        opX == OP_C, side, eout, d.P, planes, active);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// SM count of the current device, with the kernel's shared-memory limit raised there once
+cudaError_t device_ready(int& sms) {
+  constexpr int kMaxDev = 64;
+  static std::atomic<int> known[kMaxDev];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < kMaxDev && (sms = known[dev].load(std::memory_order_acquire)) > 0) return cudaSuccess;
+  if ((e = cudaFuncSetAttribute(k_tc_gemm_fp64, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM9))) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
+  if (dev < kMaxDev) known[dev].store(sms, std::memory_order_release);
+  return cudaSuccess;
+}
+
+cudaError_t product9(const GemmArgs<double>& g, unsigned char* scratch, int* err_flag, cudaStream_t st, cudaEvent_t* ev) {
+  cudaError_t e;
+  const Dims9 d = dims9(g.M, g.N, g.K);
+  const int ab = g.sA != 0, bb = g.sB != 0;
+  const size_t na = ab ? g.batch : 1, nb = bb ? g.batch : 1;
+  Params p;
+  p.M_pad = d.M_pad;
+  p.N_pad = d.N_pad;
+  unsigned char* pa = scratch;
+  unsigned char* pb = pa + na * d.a;
+  int* eA = reinterpret_cast<int*>(pb + nb * d.b);
+  int* eB = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(eA) + na * d.ea);
+  if ((e = digitize9(g.A, g.lda, g.sA, g.opA, 0, g.M, g.K, d, eA, pa, (int)na, ab ? g.active : nullptr, st))) return e;
+  if ((e = digitize9(g.B, g.ldb, g.sB, g.opB, 1, g.N, g.K, d, eB, pb, (int)nb, bb ? g.active : nullptr, st))) return e;
+  p.pa = pa;
+  p.pb = pb;
+  p.eA = eA;
+  p.eB = eB;
+  p.nks = 2 * d.K_pad / BKS;
+  p.M = g.M; p.N = g.N; p.K = g.K;
+  p.escale = 2 * d.l1 - 2;
+  p.a_batched = ab; p.b_batched = bb;
+  p.A = g.A; p.B = g.B; p.lda = g.lda; p.sA = g.sA; p.ldb = g.ldb; p.sB = g.sB;
+  p.opA = g.opA; p.opB = g.opB;
+  p.C = g.C; p.ldc = g.ldc; p.sC = g.sC;
+  p.C0 = g.C0; p.ldc0 = g.ldc0; p.sC0 = g.sC0;
+  p.alpha = g.alpha; p.beta = g.beta;
+  auto kind = [](double x) { return x == 1.0 ? 0 : (x == -1.0 ? 1 : 2); };
+  p.akind = kind(g.alpha);
+  p.bkind = (g.C0 && g.beta != 0.0) ? kind(g.beta) : 3;
+  p.active = g.active;
+  p.err = err_flag;
+  p.NBt = d.N_pad / BNC9;
+  p.MBt = d.M_pad / BM;
+  p.bn_last = (g.N - (p.NBt - 1) * BNC9 + 7) / 8 * 8;
+  const long tiles = (long)p.NBt * p.MBt * g.batch;
+  if (tiles > 0x7fffffffL) return cudaErrorInvalidValue;
+  p.n_tiles = (int)tiles;
+  p.hold = wait_test();
+  p.limit_ns = p.hold ? kWaitTestLimitNs : kWaitLimitNs;
+  int sms = 0;
+  if ((e = device_ready(sms))) return e;
+  if (ev) cudaEventRecord(ev[0], st);
+  k_tc_gemm_fp64<<<(unsigned)(tiles < sms ? tiles : sms), 320, SMEM9, st>>>(p);
+  count_launch();
+  if (ev) cudaEventRecord(ev[1], st);
+  return cudaGetLastError();
+}
+
+}  // namespace
+}  // namespace tc
+
+// scratch bytes of one batch entry (digit planes and exponents)
+static size_t entry_bytes(int M, int N, int K) {
+  const tc::Dims9 d = tc::dims9(M, N, tc::chunk_k(K));
+  return d.a + d.b + d.ea + d.eb;
+}
+
+size_t gemm_fp64_tc_scratch_bytes(int M, int N, int K, int batch) {
+  // enough entries for four waves of tiles, at most 384 MiB (but at least one entry): the batch is
+  // taken in portions of what fits
+  const size_t one = entry_bytes(M, N, K);
+  const long tiles = (long)((M + tc::BM - 1) / tc::BM) * ((N + tc::BNC9 - 1) / tc::BNC9);
+  size_t n = (size_t)((4 * 152 + tiles - 1) / tiles);
+  const size_t cap = ((size_t)384 << 20) / one;
+  if (n > cap) n = cap;
+  if (n > (size_t)batch) n = (size_t)batch;
+  return (n < 1 ? 1 : n) * one;
+}
+
+bool gemm_fp64_tc_fits(int M, int N, int K, size_t scratch_bytes) { return scratch_bytes >= entry_bytes(M, N, K); }
+
+cudaError_t gemm_fp64_tc(const GemmArgs<double>& g0, void* scratch, size_t scratch_bytes, int* err_flag, cudaStream_t st,
+                         cudaEvent_t* ev) {
+  if (g0.M <= 0 || g0.N <= 0 || g0.batch <= 0) return cudaSuccess;
+  const long room = (long)(scratch_bytes / entry_bytes(g0.M, g0.N, g0.K));
+  if (room < 1 || g0.K < 1) return cudaErrorInvalidValue;
+  const int Kc = tc::chunk_k(g0.K);
+  // the events bracket the product kernel, or the whole call when it takes several launches
+  const bool one = g0.batch <= room && g0.K <= Kc;
+  if (ev && !one) cudaEventRecord(ev[0], st);
+  for (long e0 = 0; e0 < g0.batch; e0 += room) {
+    GemmArgs<double> g = g0;
+    g.batch = (int)(g0.batch - e0 < room ? g0.batch - e0 : room);
+    g.A += e0 * g.sA;
+    g.B += e0 * g.sB;
+    g.C += e0 * g.sC;
+    if (g.C0) g.C0 += e0 * g.sC0;
+    if (g.active) g.active += e0;
+    // contractions beyond one launch's K run as consecutive chunks, each added to the last result
+    for (int k0 = 0; k0 < g0.K; k0 += Kc) {
+      GemmArgs<double> t = g;
+      t.K = g0.K - k0 < Kc ? g0.K - k0 : Kc;
+      t.A += g.opA == OP_N ? (long)k0 : (long)k0 * g.lda;
+      t.B += g.opB == OP_N ? (long)k0 * g.ldb : (long)k0;
+      if (k0 > 0) {
+        t.C0 = g.C;
+        t.ldc0 = g.ldc;
+        t.sC0 = g.sC;
+        t.beta = 1.0;
+      }
+      const cudaError_t e = tc::product9(t, reinterpret_cast<unsigned char*>(scratch), err_flag, st, one ? ev : nullptr);
+      if (e != cudaSuccess) return e;
+    }
+  }
+  if (ev && !one) cudaEventRecord(ev[1], st);
+  return cudaSuccess;
+}
+
+}  // namespace qtx
