@@ -15,7 +15,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 SRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libqtx_rgf.so")
-SOURCES = ["simt.cu", "rgf.cu", "tc_engine.cu", "tc_fp64.cu", "noalloc.cu", "fpx.cu", "decim.cu"]
+SOURCES = ["simt.cu", "rgf.cu", "tc_engine.cu", "tc_fp64.cu", "noalloc.cu", "fpx.cu", "decim.cu",
+           "small.cu", "leaf64.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-Xptxas", "-warn-spills"]

@@ -193,6 +193,14 @@ struct GemmArgs {
   const int* active;
 };
 
+// Up to four products of one shape and batch in a launch.
+template <typename T>
+struct GemmMulti {
+  static constexpr int kMax = 4;
+  int n;
+  GemmArgs<T> g[kMax];
+};
+
 // A digitised operand kept across products (digit planes and scale exponents in caller-owned
 // memory of gemm_tc_operand_bytes): mode 1 digitises the operand into it, mode 2 uses the planes
 // already there (the operand, its op and shape unchanged since the mode-1 product).

@@ -10,185 +10,247 @@
 //     until max |alpha|, |beta| < tol max |H01|;  then g_s = (z - eps_s)^-1 and
 //     Sigma^R = H01 g_s H01^H  (the device's end slice couples to the first lead cell by H01).
 //
-// k_decimate: the whole iteration of one energy in one CTA, every block in shared memory (b <= 32:
-// eight b x b complex128 blocks, at most 128 KB).  The inverses are in-place Gauss-Jordan elimination
-// with partial (row) pivoting on |re| + |im| (first maximum on ties), the row interchanges undone as
-// column interchanges at the end.  The sweep count, the convergence test and the status are kept on
-// the device: a contact costs one launch, and a solve with contacts makes no host synchronisation
-// (so it can be captured in a CUDA graph).
+// k_decimate: the whole iteration of one energy and contact in one cluster of 1, 2, 4 or 8 CTAs, every block in
+// shared memory (b <= 32: eight b x b complex128 blocks a CTA), both contacts of a device in one launch.
+// Products are DFMA sums in ascending k.  Near a mode threshold the iteration amplifies a rounding
+// error by 1e6 and more, so these stay in FP64 arithmetic in a fixed order rather than on the tensor
+// cores: any other rounding moves the self-energies there by as much as their own error.
+//
+// What bounds it is GB300's FP64 pipe (two DFMA a cycle and SM): six products and an elimination of
+// 16 x 16 blocks are 115,000 DFMA a sweep, 57,000 cycles on one SM.  Few energies leave SMs idle, so a cluster
+// splits the products' rows (each CTA writes its rows into every CTA's copy through distributed shared
+// memory; two cluster barriers a sweep) while every CTA eliminates for itself.  In the elimination one
+// warp finds the pivot and forms its reciprocal once -- 1/d and r/d as one division in two lanes -- and
+// scales the pivot row; the rows then update from one copy of the block into another.
+#include <cooperative_groups.h>
+
+#include "gj64.cuh"
 #include "kernels.cuh"
 
 namespace qtx {
 
 namespace {
 
-constexpr int kDecThreads = 256;
+namespace cg = cooperative_groups;
+constexpr int kThreads = 256;
 
-// C = A B for n x n blocks in shared memory with row stride NM (all threads; the caller syncs)
-template <int NM>
-__device__ __forceinline__ void mm_s(const cx<double>* A, const cx<double>* B, cx<double>* C, int n) {
-  for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
-    const int r = idx / n, c = idx % n;
-    cx<double> acc = mk<double>(0.0, 0.0);
-    for (int k = 0; k < n; ++k) cfma(acc, A[r * NM + k], B[k * NM + c]);
-    C[r * NM + c] = acc;
-  }
-}
+struct Lead {
+  const cx<double>*H00, *H01;
+  cx<double>* SR;  // [ne][n][n]
+};
+struct DecimArgs {
+  Lead lead[2];
+  const double* E;
+  double eta, tol_rel;
+  int max_iter, n;
+  int* status;
+};
 
-// In-place inverse of the n x n block A (row stride NM) by Gauss-Jordan elimination with partial
-// pivoting.  colk[NM] and perm[NM] are shared scratch.  Returns false (uniformly) for a zero pivot.
 template <int NM>
-__device__ bool inv_s(cx<double>* A, int n, cx<double>* colk, int* perm, int* s_piv) {
-  const int t = threadIdx.x;
+struct DSmem {
+  static constexpr int LD = NM + 1;  // odd stride: row and column reads free of bank conflicts
+  cx<double> m[8][NM * LD];
+  cx<double> rowk[NM];
+  int perm[NM], from[NM];
+  int piv;
+  unsigned hi;
+  double red[kThreads / 32];
+};
+
+// Gauss-Jordan inverse with partial (row) pivoting on |re| + |im|, first maximum on ties, from block A
+// (destroyed) with B as the other copy; the result is the returned block (A or B), nullptr (uniformly)
+// for a zero pivot.  The order of every rounding is written out: with f the row's factor and a the scaled
+// pivot row, an entry becomes x - f a with re = fma(f.re, a.re, -(f.im a.im)), im = fma(f.im, a.re, f.re a.im);
+// the pivot column 0 - f a (a = 1 / pivot) with the two products' roles exchanged.
+template <int NM>
+__device__ cx<double>* eliminate(DSmem<NM>& s, cx<double>* A, cx<double>* B, const gj::FastDiv& fd) {
+  constexpr int LD = DSmem<NM>::LD;
+  const int t = threadIdx.x, n = fd.n;
   for (int k = 0; k < n; ++k) {
     if (t < 32) {
-      double best = -1.0;
-      int bi = -1;
-      for (int i = k + t; i < n; i += 32) {
-        const double v = cabs1(A[i * NM + k]);
-        if (v > best) {
-          best = v;
-          bi = i;
-        }
-      }
-      for (int off = 16; off > 0; off >>= 1) {
-        const double ov = __shfl_down_sync(0xffffffffu, best, off);
-        const int oi = __shfl_down_sync(0xffffffffu, bi, off);
-        if (ov > best || (ov == best && oi >= 0 && (bi < 0 || oi < bi))) {
-          best = ov;
-          bi = oi;
-        }
-      }
+      const unsigned long long key = (t >= k && t < n) ? gj::pivot_key(A[t * LD + k]) : 0ull;
+      const unsigned long long best = gj::warp_max(key);
+      const int p = best ? __ffs((int)__ballot_sync(0xffffffffu, key == best)) - 1 : -1;
       if (t == 0) {
-        *s_piv = best > 0.0 ? bi : -1;
-        perm[k] = bi;
+        s.piv = p;
+        s.perm[k] = p;
+      }
+      if (p >= 0) {
+        const cx<double> r = gj::crecip_warp(A[p * LD + k]);
+        if (t < n) {
+          const cx<double> x = A[p * LD + t];
+          const cx<double> y = mk<double>(__fma_rn(x.re, r.re, -__dmul_rn(x.im, r.im)), __fma_rn(x.re, r.im, __dmul_rn(x.im, r.re)));
+          s.rowk[t] = t == k ? r : y;
+        }
       }
     }
     __syncthreads();
-    const int p = *s_piv;
-    if (p < 0) return false;
-    if (p != k)
-      for (int j = t; j < n; j += blockDim.x) {
-        const cx<double> x = A[k * NM + j];
-        A[k * NM + j] = A[p * NM + j];
-        A[p * NM + j] = x;
-      }
-    __syncthreads();
-    const cx<double> r = crecip(A[k * NM + k]);
-    for (int i = t; i < n; i += blockDim.x) colk[i] = A[i * NM + k];
-    __syncthreads();
-    for (int j = t; j < n; j += blockDim.x) A[k * NM + j] = (j == k) ? r : A[k * NM + j] * r;
-    __syncthreads();
-    for (int idx = t; idx < n * n; idx += blockDim.x) {
-      const int i = idx / n, j = idx % n;
-      if (i == k) continue;
-      const cx<double> f = colk[i];
-      if (j == k) A[i * NM + k] = mk<double>(0.0, 0.0) - f * r;
-      else A[i * NM + j] = A[i * NM + j] - f * A[k * NM + j];
+    const int p = s.piv;
+    if (p < 0) return nullptr;
+    for (int idx = t; idx < n * n; idx += kThreads) {
+      const int i = fd.div(idx), j = idx - i * n;
+      const int src = i == p ? k : i;  // rows k and p interchanged
+      const bool kc = j == k;
+      const cx<double> f = A[src * LD + k], a = s.rowk[j], y = kc ? mk<double>(0.0, 0.0) : A[src * LD + j];
+      const double re = __fma_rn(kc ? -f.im : f.re, kc ? a.im : a.re, __dmul_rn(kc ? f.re : -f.im, kc ? a.re : a.im));
+      const double im = __fma_rn(kc ? f.re : f.im, kc ? a.im : a.re, __dmul_rn(kc ? f.im : f.re, kc ? a.re : a.im));
+      const cx<double> v = mk<double>(__dsub_rn(y.re, re), __dsub_rn(y.im, im));
+      B[i * LD + j] = i == k ? a : v;
     }
     __syncthreads();
+    cx<double>* x = A;
+    A = B;
+    B = x;
   }
-  for (int k = n - 1; k >= 0; --k) {
-    const int p = perm[k];
-    if (p != k)
-      for (int i = t; i < n; i += blockDim.x) {
-        const cx<double> x = A[i * NM + k];
-        A[i * NM + k] = A[i * NM + p];
-        A[i * NM + p] = x;
-      }
-    __syncthreads();
+  // the row interchanges undone as column interchanges, k = n - 1 .. 0: where result column j comes from
+  if (t < n) {
+    int c = t;
+    for (int k = 0; k < n; ++k) {
+      const int p = s.perm[k];
+      c = c == k ? p : (c == p ? k : c);
+    }
+    s.from[t] = c;
   }
-  return true;
+  __syncthreads();
+  for (int idx = t; idx < n * n; idx += kThreads) {
+    const int i = fd.div(idx), j = idx - i * n;
+    B[i * LD + j] = A[i * LD + s.from[j]];
+  }
+  __syncthreads();
+  return B;
 }
 
 // largest modulus over the n x n blocks X and Y (all threads get it)
 template <int NM>
-__device__ double max_mod2(const cx<double>* X, const cx<double>* Y, int n, double* red) {
+__device__ double max_mod(DSmem<NM>& s, const cx<double>* X, const cx<double>* Y, int n) {
+  constexpr int LD = DSmem<NM>::LD;
   double m = 0.0;
-  for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
-    const int r = idx / n, c = idx % n;
-    const cx<double> x = X[r * NM + c], y = Y[r * NM + c];
+  for (int idx = threadIdx.x; idx < n * n; idx += kThreads) {
+    const cx<double> x = X[(idx / n) * LD + idx % n], y = Y[(idx / n) * LD + idx % n];
     m = fmax(m, fmax(hypot(x.re, x.im), hypot(y.re, y.im)));
   }
   for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
-  if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = m;
+  if (threadIdx.x % 32 == 0) s.red[threadIdx.x / 32] = m;
   __syncthreads();
-  double r = red[0];
-  for (int w = 1; w < (int)blockDim.x / 32; ++w) r = fmax(r, red[w]);
+  double r = s.red[0];
+  for (int w = 1; w < kThreads / 32; ++w) r = fmax(r, s.red[w]);
   __syncthreads();
   return r;
 }
+// whether that modulus is below tol (tol < 2^500): the largest |re|, |im| decides by its high word unless it
+// lies within sqrt(2) of tol
+template <int NM>
+__device__ bool below(DSmem<NM>& s, const cx<double>* X, const cx<double>* Y, int n, double tol) {
+  constexpr int LD = DSmem<NM>::LD;
+  unsigned h = 0;
+  auto hw = [](double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; };
+  for (int idx = threadIdx.x; idx < n * n; idx += kThreads) {
+    const cx<double> x = X[(idx / n) * LD + idx % n], y = Y[(idx / n) * LD + idx % n];
+    h = max(h, max(max(hw(x.re), hw(x.im)), max(hw(y.re), hw(y.im))));
+  }
+  h = __reduce_max_sync(0xffffffffu, h);
+  if (threadIdx.x == 0) s.hi = 0;
+  __syncthreads();
+  if (threadIdx.x % 32 == 0) atomicMax(&s.hi, h);
+  __syncthreads();
+  h = s.hi;
+  __syncthreads();
+  if (h < 0x7ff00000u) {  // NaN: fmax skips it, so the exact maximum decides
+    if (__hiloint2double((int)h, 0) >= tol) return false;
+    if (__hiloint2double((int)h + 1, 0) * 1.4142135623731 < tol) return true;
+  }
+  return max_mod<NM>(s, X, Y, n) < tol;
+}
 
 template <int NM>
-__global__ void __launch_bounds__(kDecThreads) k_decimate(const cx<double>* H00, const cx<double>* H01,
-                                                         const double* E, double eta, double tol_rel,
-                                                         int max_iter, int n, cx<double>* SR, int* status) {
+__device__ __forceinline__ cx<double> dot(const cx<double>* A, const cx<double>* B, int r, int c, int n) {
+  constexpr int LD = DSmem<NM>::LD;
+  cx<double> acc = mk<double>(0.0, 0.0);
+  for (int k = 0; k < n; ++k) cfma(acc, A[r * LD + k], B[k * LD + c]);
+  return acc;
+}
+
+template <int NM>
+__global__ void __launch_bounds__(kThreads) k_decimate(const DecimArgs a) {
   extern __shared__ __align__(16) unsigned char dsm[];
-  cx<double>* al = reinterpret_cast<cx<double>*>(dsm);
-  cx<double>* be = al + NM * NM;
-  cx<double>* ep = be + NM * NM;
-  cx<double>* es = ep + NM * NM;
-  cx<double>* G = es + NM * NM;
-  cx<double>* AG = G + NM * NM;
-  cx<double>* BG = AG + NM * NM;
-  cx<double>* T = BG + NM * NM;
-  cx<double>* colk = T + NM * NM;
-  __shared__ int perm[NM];
-  __shared__ int s_piv;
-  __shared__ double red[kDecThreads / 32];
-  const int e = blockIdx.x, t = threadIdx.x;
-  const cx<double> z = mk<double>(E[e], eta);
-  for (int idx = t; idx < n * n; idx += blockDim.x) {
+  DSmem<NM>& s = *reinterpret_cast<DSmem<NM>*>(dsm);
+  constexpr int LD = DSmem<NM>::LD;
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const Lead& L = a.lead[blockIdx.y];
+  const int e = blockIdx.x / C, n = a.n, t = threadIdx.x;
+  const gj::FastDiv fd(n);
+  // this CTA's rows of the products
+  const int r0 = rank * n / C, rows = (rank + 1) * n / C - r0;
+  cx<double>*al = s.m[0], *be = s.m[1], *ep = s.m[2], *es = s.m[3], *G = s.m[4], *T = s.m[5], *AG = s.m[6], *BG = s.m[7];
+  const cx<double> z = mk<double>(a.E[e], a.eta);
+  auto sync = [&]() {
+    if (C > 1) cl.sync();
+    else __syncthreads();
+  };
+  // v at (r, c) of block D in every CTA of the cluster
+  auto put = [&](cx<double>* D, int r, int c, cx<double> v) {
+    if (C == 1) {
+      D[r * LD + c] = v;
+      return;
+    }
+    for (int q = 0; q < C; ++q) *cl.map_shared_rank(&D[r * LD + c], q) = v;
+  };
+  for (int idx = t; idx < n * n; idx += kThreads) {
     const int r = idx / n, c = idx % n;
-    al[r * NM + c] = H01[idx];
-    be[r * NM + c] = conj(H01[(long)c * n + r]);
-    ep[r * NM + c] = H00[idx];
-    es[r * NM + c] = H00[idx];
+    al[r * LD + c] = L.H01[idx];
+    be[r * LD + c] = conj(L.H01[(long)c * n + r]);
+    ep[r * LD + c] = L.H00[idx];
+    es[r * LD + c] = L.H00[idx];
   }
-  __syncthreads();
+  sync();  // from here on a CTA may write into another's copies
   // tolerance relative to the coupling's largest modulus (al holds H01, be its adjoint)
-  double scale = max_mod2<NM>(al, al, n, red);
-  const double tol = tol_rel * (scale > 0.0 ? scale : 1.0);
-  bool converged = false, singular = false;
-  for (int it = 1; it <= max_iter; ++it) {
-    for (int idx = t; idx < n * n; idx += blockDim.x) {
+  const double scale = max_mod<NM>(s, al, al, n);
+  const double tol = a.tol_rel * (scale > 0.0 ? scale : 1.0);
+  auto shifted = [&](const cx<double>* X) {  // AG = z - X
+    for (int idx = t; idx < n * n; idx += kThreads) {
       const int r = idx / n, c = idx % n;
-      const cx<double> x = ep[r * NM + c];
-      G[r * NM + c] = mk<double>((r == c ? z.re : 0.0) - x.re, (r == c ? z.im : 0.0) - x.im);
+      const cx<double> x = X[r * LD + c];
+      AG[r * LD + c] = mk<double>((r == c ? z.re : 0.0) - x.re, (r == c ? z.im : 0.0) - x.im);
     }
     __syncthreads();
-    if (!inv_s<NM>(G, n, colk, perm, &s_piv)) {
+  };
+  bool converged = false, singular = false;
+  for (int it = 1; it <= a.max_iter; ++it) {
+    shifted(ep);
+    cx<double>* g = eliminate<NM>(s, AG, BG, fd);
+    if (!g) {
       singular = true;
       break;
     }
-    mm_s<NM>(al, G, AG, n);
-    mm_s<NM>(be, G, BG, n);
-    __syncthreads();
-    mm_s<NM>(AG, be, T, n);  // alpha g beta
-    __syncthreads();
-    for (int idx = t; idx < n * n; idx += blockDim.x) {
-      const int r = idx / n, c = idx % n;
-      es[r * NM + c] = es[r * NM + c] + T[r * NM + c];
-      ep[r * NM + c] = ep[r * NM + c] + T[r * NM + c];
+    // g moves to G: AG and BG take the products
+    for (int idx = t; idx < n * n; idx += kThreads) G[(idx / n) * LD + idx % n] = g[(idx / n) * LD + idx % n];
+    sync();  // also: every CTA is done with its AG, BG
+    for (int idx = t; idx < 2 * rows * n; idx += kThreads) {
+      const int w = idx >= rows * n, o = idx - w * rows * n, r = r0 + fd.div(o), c = o - fd.div(o) * n;
+      put(w ? BG : AG, r, c, dot<NM>(w ? be : al, G, r, c, n));  // alpha g, beta g
     }
-    __syncthreads();
-    mm_s<NM>(BG, al, T, n);  // beta g alpha
-    __syncthreads();
-    for (int idx = t; idx < n * n; idx += blockDim.x) {
-      const int r = idx / n, c = idx % n;
-      ep[r * NM + c] = ep[r * NM + c] + T[r * NM + c];
+    sync();
+    // every CTA has its G copy free now: alpha' -> G, beta' -> T; eps, eps_s in place (owned rows)
+    for (int idx = t; idx < 3 * rows * n; idx += kThreads) {
+      const int w = idx >= 2 * rows * n ? 2 : idx >= rows * n, o = idx - w * rows * n, r = r0 + fd.div(o), c = o - fd.div(o) * n;
+      if (w == 0) {
+        const cx<double> x = dot<NM>(AG, be, r, c, n);             // alpha g beta
+        const cx<double> y = dot<NM>(BG, al, r, c, n);             // beta g alpha
+        es[r * LD + c] = es[r * LD + c] + x;
+        put(ep, r, c, (ep[r * LD + c] + x) + y);
+      } else {
+        put(w == 1 ? G : T, r, c, dot<NM>(w == 1 ? AG : BG, w == 1 ? al : be, r, c, n));
+      }
     }
-    __syncthreads();
-    mm_s<NM>(AG, al, T, n);  // alpha g alpha
-    mm_s<NM>(BG, be, G, n);  // beta g beta (G is free now)
-    __syncthreads();
-    for (int idx = t; idx < n * n; idx += blockDim.x) {
-      const int r = idx / n, c = idx % n;
-      al[r * NM + c] = T[r * NM + c];
-      be[r * NM + c] = G[r * NM + c];
-    }
-    __syncthreads();
-    if (max_mod2<NM>(al, be, n, red) < tol) {
+    sync();
+    cx<double>* x = al;
+    al = G;
+    G = x;
+    x = be;
+    be = T;
+    T = x;
+    if (below<NM>(s, al, be, n, tol)) {
       converged = true;
       break;
     }
@@ -196,57 +258,76 @@ __global__ void __launch_bounds__(kDecThreads) k_decimate(const cx<double>* H00,
   int st = 0;
   if (singular) st = (int)QTX_ERR_SINGULAR;
   else if (!converged) st = (int)QTX_ERR_NOT_CONVERGED;
+  // every CTA's rows of eps_s to the first, which finishes alone
+  if (C > 1) {
+    if (rank)
+      for (int idx = t; idx < rows * n; idx += kThreads) {
+        const int r = r0 + idx / n, c = idx % n;
+        *cl.map_shared_rank(&es[r * LD + c], 0) = es[r * LD + c];
+      }
+    cl.sync();
+    if (rank) return;
+  }
+  cx<double>* out = L.SR + (long)e * n * n;
   // g_s = (z - eps_s)^-1 (also after a capped iteration, as the launched path does)
+  cx<double>* g = nullptr;
   if (!singular) {
-    for (int idx = t; idx < n * n; idx += blockDim.x) {
+    shifted(es);
+    for (int idx = t; idx < n * n; idx += kThreads) {
       const int r = idx / n, c = idx % n;
-      const cx<double> x = es[r * NM + c];
-      G[r * NM + c] = mk<double>((r == c ? z.re : 0.0) - x.re, (r == c ? z.im : 0.0) - x.im);
-      al[r * NM + c] = H01[idx];
-      be[r * NM + c] = conj(H01[(long)c * n + r]);
+      al[r * LD + c] = L.H01[idx];
+      be[r * LD + c] = conj(L.H01[(long)c * n + r]);
     }
     __syncthreads();
-    if (!inv_s<NM>(G, n, colk, perm, &s_piv)) singular = true;
+    g = eliminate<NM>(s, AG, BG, fd);
+    if (!g) singular = true;
   }
-  cx<double>* out = SR + (long)e * n * n;
   if (singular) {
     st = (int)QTX_ERR_SINGULAR;
-    for (int idx = t; idx < n * n; idx += blockDim.x) out[idx] = mk<double>(0.0, 0.0);
+    for (int idx = t; idx < n * n; idx += kThreads) out[idx] = mk<double>(0.0, 0.0);
   } else {
-    mm_s<NM>(al, G, T, n);  // H01 g_s
+    for (int idx = t; idx < n * n; idx += kThreads) T[(idx / n) * LD + idx % n] = dot<NM>(al, g, idx / n, idx % n, n);  // H01 g_s
     __syncthreads();
-    mm_s<NM>(T, be, AG, n);  // (H01 g_s) H01^H
-    __syncthreads();
-    for (int idx = t; idx < n * n; idx += blockDim.x) out[idx] = AG[(idx / n) * NM + idx % n];
+    for (int idx = t; idx < n * n; idx += kThreads) out[idx] = dot<NM>(T, be, idx / n, idx % n, n);  // (H01 g_s) H01^H
   }
-  if (t == 0 && st && status) atomicCAS(status + e, 0, st);
+  if (t == 0 && st && a.status) atomicCAS(a.status + e, 0, st);
 }
 
 template <int NM>
-constexpr size_t decim_smem() {
-  return (size_t)(8 * NM * NM + NM) * sizeof(cx<double>);
+cudaError_t launch(const DecimArgs& a, int batch, int leads, cudaStream_t st) {
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e = allow_smem(k_decimate<NM>, (int)sizeof(DSmem<NM>), done);
+  if (e != cudaSuccess) return e;
+  // CTAs of a cluster: as many as leave every energy and contact resident at once on 152 SMs
+  int C = 1;
+  while (C < 8 && (long)batch * leads * C * 2 <= 152 && 4 * C <= a.n) C *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(batch * C, leads);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = sizeof(DSmem<NM>);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if ((e = cudaLaunchKernelEx(&cfg, k_decimate<NM>, a)) != cudaSuccess) return e;
+  count_launch();
+  return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t decimate_small(const cx<double>* H00, const cx<double>* H01, const double* E, double eta,
-                           double tol_rel, int max_iter, int n, int batch, cx<double>* SR, int* status,
+cudaError_t decimate_small(int leads, const cx<double>* const* H00, const cx<double>* const* H01, cx<double>* const* SR,
+                           const double* E, double eta, double tol_rel, int max_iter, int n, int batch, int* status,
                            cudaStream_t st) {
-  if (n < 1 || n > kDecimSmallMax) return cudaErrorInvalidValue;
-  if (n <= 16) {
-    k_decimate<16><<<batch, kDecThreads, decim_smem<16>(), st>>>(H00, H01, E, eta, tol_rel, max_iter, n, SR, status);
-  } else {
-    static bool attr = false;
-    if (!attr) {
-      const cudaError_t e = cudaFuncSetAttribute(k_decimate<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)decim_smem<32>());
-      if (e != cudaSuccess) return e;
-      attr = true;
-    }
-    k_decimate<32><<<batch, kDecThreads, decim_smem<32>(), st>>>(H00, H01, E, eta, tol_rel, max_iter, n, SR, status);
-  }
-  count_launch();
-  return cudaGetLastError();
+  if (n < 1 || n > kDecimSmallMax || leads < 1 || leads > 2) return cudaErrorInvalidValue;
+  DecimArgs a;
+  for (int k = 0; k < 2; ++k) a.lead[k] = Lead{H00[k < leads ? k : 0], H01[k < leads ? k : 0], SR[k < leads ? k : 0]};
+  a.E = E; a.eta = eta; a.tol_rel = tol_rel; a.max_iter = max_iter; a.n = n; a.status = status;
+  return n <= 16 ? launch<16>(a, batch, leads, st) : launch<32>(a, batch, leads, st);
 }
 
 }  // namespace qtx

@@ -8,6 +8,7 @@
 namespace qtx {
 
 constexpr int kDig64 = 9;          // digits per FP64 operand value
+constexpr int kFix62 = 62;         // P of nine digits with a leading one of at most 64
 constexpr int kExpoNonFinite = 1 << 20;  // row exponent of a row that holds an infinity or a NaN
 constexpr int kExpoZero = -4000;         // row exponent of a row of zeros
 
@@ -63,45 +64,46 @@ __host__ __device__ inline uint32_t digit_field(uint64_t biased, int i) {
   return (uint32_t)(biased >> (7 * (kDig64 - 1 - i))) & (i == 0 ? 255u : 127u);
 }
 
-// RN((A 2^28 + B) 2^-56) for |A| < 2^62, |B| < 2^62: the sum aligned to a 64-bit significand with a
-// sticky bit, rounded to 53 bits, ties to even.
-__host__ __device__ inline double fix_sum(int64_t A, int64_t B) {
-  int64_t hi = A + (B >> 28);
-  uint32_t lo = (uint32_t)(B & ((1ll << 28) - 1)) << 4;  // 28 fraction bits at the top of a word
-  if (hi == 0 && lo == 0) return 0.0;
-  const uint64_t sgn = hi < 0 ? 1ull << 63 : 0;
-  if (sgn) {  // two's-complement negation of (hi, lo)
-    hi = ~hi + (lo == 0);
-    lo = 0u - lo;
-  }
-  uint64_t m;       // leading 64 bits
-  bool sticky;
-  int e;            // exponent of the leading bit, in units of 2^-28
-  if (hi == 0) {
+// bf16 pairs of 2^(-7 i) and -192 2^(-7 i): 0x4300 | (d + 64) is the bf16 of 192 + d (also for d = 64, where
+// the OR carries into the exponent: 256), and (192 + d) s - 192 s = d s is exact in one bf16 FMA
+__host__ __device__ constexpr uint32_t digit_scale(int i) { return (uint32_t)(127 - 7 * i) << 7 | (uint32_t)(127 - 7 * i) << 23; }
+__host__ __device__ constexpr uint32_t digit_shift(int i) {
+  return 0x80408040u | (uint32_t)(134 - 7 * i) << 7 | (uint32_t)(134 - 7 * i) << 23;
+}
+
+// RN((A 2^28 + B) 2^(Es - 56)) for |A| < 2^62, |B| < 2^62: the sum aligned to a 64-bit significand with a
+// sticky bit, rounded to 53 bits, ties to even.  Free of branches, so that several sums interleave; `bad`
+// is raised when the result is not a normal number (the caller then takes fix_sum and scale64).
+__host__ __device__ inline double fix_sum_scaled(int64_t A, int64_t B, int Es, bool& bad) {
+  const int64_t h0 = A + (B >> 28);
+  const uint32_t l0 = (uint32_t)B << 4;  // 28 fraction bits at the top of a word
+  const int64_t s = h0 >> 63;            // all ones if negative: (h0, l0) negated in two's complement
+  const uint32_t l1 = (l0 ^ (uint32_t)s) - (uint32_t)s;
+  const uint64_t h1 = (uint64_t)(h0 ^ s) - (uint64_t)(l0 == 0 ? s : 0);
+  const bool small = h1 == 0;
+  const uint64_t h = small ? (uint64_t)l1 << 32 : h1;
+  const uint64_t l = small ? 0 : (uint64_t)l1 << 32;
+  const bool zero = h == 0;
 #ifdef __CUDA_ARCH__
-    const int lz = __clz((int)lo);
+  const int lz = __clzll((long long)(h | 1));
 #else
-    const int lz = __builtin_clz(lo);
+  const int lz = __builtin_clzll((unsigned long long)(h | 1));
 #endif
-    m = (uint64_t)lo << (32 + lz);
-    sticky = false;
-    e = -1 - lz;
-  } else {
-#ifdef __CUDA_ARCH__
-    const int lz = __clzll(hi);
-#else
-    const int lz = __builtin_clzll((unsigned long long)hi);
-#endif
-    const uint64_t lo64 = (uint64_t)lo << 32;
-    m = ((uint64_t)hi << lz) | (lz ? lo64 >> (64 - lz) : 0);
-    sticky = (lo64 << lz) != 0;
-    e = 63 - lz;
-  }
-  uint64_t r = m >> 11;
-  const uint32_t rem = (uint32_t)m & 0x7ffu;
-  if (rem > 0x400u || (rem == 0x400u && (sticky || (r & 1)))) ++r;
+  const uint64_t m = (h << lz) | ((l >> 1) >> (63 - lz));
+  const uint64_t r = m >> 11;
+  const uint32_t odd = ((l << lz) != 0) | ((uint32_t)r & 1u);
+  const uint32_t up = ((uint32_t)m & 0x7ffu) + odd > 0x400u;
+  // exponent of the leading bit in units of 2^-28: 63 - lz, or -1 - lz when the word came from l1
+  const int E = (small ? -1 : 63) - lz - 28 + 1022 + Es;
+  bad |= !zero && (E < 0 || E > 2044);
   // r in [2^52, 2^53]: adding it to the exponent field minus one carries into the exponent
-  return double_of(sgn | (((uint64_t)(e - 28 + 1022) << 52) + r));
+  const uint64_t u = ((uint64_t)(int64_t)E << 52) + r + up;
+  return double_of(zero ? 0 : (u | ((uint64_t)s & 0x8000000000000000ull)));
+}
+// RN((A 2^28 + B) 2^-56)
+__host__ __device__ inline double fix_sum(int64_t A, int64_t B) {
+  bool bad = false;
+  return fix_sum_scaled(A, B, 0, bad);
 }
 
 // x 2^E by its exponent field; results outside the normal range by two exact-or-rounding-once steps

@@ -11,9 +11,24 @@ namespace qtx {
 extern std::atomic<long long> g_launches;
 inline void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
+// Raise a kernel's dynamic shared-memory limit once per device (`done`: the kernel's bit per device).
+template <typename F>
+inline cudaError_t allow_smem(F* kernel, int bytes, std::atomic<unsigned long long>& done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess) return e;
+  done.fetch_or(bit, std::memory_order_release);
+  return cudaSuccess;
+}
+
 // ---- batched complex GEMM on the CUDA cores (T = double: DFMA, T = float: FFMA)
 template <typename T>
 cudaError_t gemm_simt(const GemmArgs<T>& g, cudaStream_t st);
+template <typename T>
+cudaError_t gemm_simt_multi(const GemmMulti<T>& m, cudaStream_t st);
 
 // ---- in-place inverse of n x n blocks (n <= kLeafMax) by Gauss-Jordan elimination with partial
 // (row) pivoting, one CTA per block.  A zero pivot stores QTX_ERR_SINGULAR into status[e].
@@ -21,6 +36,9 @@ constexpr int kLeafMax = 64;
 template <typename T>
 cudaError_t leaf_inverse(cx<T>* A, long lda, long sA, int n, int batch, const int* active,
                          int* status, cudaStream_t st);
+template <>
+cudaError_t leaf_inverse<double>(cx<double>* A, long lda, long sA, int n, int batch, const int* active, int* status,
+                                 cudaStream_t st);
 
 // ---- elementwise combination of b x b blocks (batched over energies):
 //   out[e] = sum_t alpha_t * op_t(X_t[e])  +  diag_coef * (E[e] + i eta) * I
@@ -124,21 +142,44 @@ cudaError_t continuity(const double* cur, long ldc, const double* J, const doubl
 // ---- lead post-processing: from Sigma^R (complex128) build Gamma, Sigma^<, Sigma^>
 cudaError_t lead_sigmas(const cx<double>* SR, cx<double>* Gam, cx<double>* SL, cx<double>* SG,
                         const double* E, double mu, double kT, int b, int batch, cudaStream_t st);
-// per batch entry: if the largest modulus over X and Y is < tol_rel * max(*scale, or 1 if 0), clear
-// active[e]; count sweeps (scale is a device scalar, e.g. from max_modulus)
-cudaError_t decim_converged(const cx<double>* X, const cx<double>* Y, int b, double tol_rel,
-                            const double* scale, int* active, int* sweeps, int batch, cudaStream_t st);
+// one sweep's sums of the launched decimation (es += x, ep = (ep + x) + y) and, per active batch entry, its
+// convergence: active[e] = 0 once the largest modulus over al and be is < tol_rel * (*scale, or 1 if 0)
+// (scale is a device scalar, e.g. from max_modulus)
+cudaError_t decim_update(cx<double>* es, cx<double>* ep, const cx<double>* x, const cx<double>* y, const cx<double>* al,
+                         const cx<double>* be, int b, double tol_rel, const double* scale, int* active, int batch,
+                         cudaStream_t st);
 // out[0] = largest modulus of the n complex values X[0..n) (device scalar)
 cudaError_t max_modulus(const cx<double>* X, long n, double* out, cudaStream_t st);
 // p[0..n) = v
 cudaError_t fill_int(int* p, int v, int n, cudaStream_t st);
-// The whole decimation of a lead block of size n <= kDecimSmallMax per energy in one CTA (decim.cu):
-// SR[e] = H01 g_s(E[e] + i eta) H01^H; status[e] = QTX_ERR_NOT_CONVERGED / QTX_ERR_SINGULAR (only
-// raised from 0).  No host synchronisation.
+// The whole decimation of lead blocks of size n <= kDecimSmallMax per energy and contact in one CTA
+// (decim.cu), one launch for 1 or 2 contacts: SR[k][e] = H01[k] g_s(E[e] + i eta) H01[k]^H; status[e] =
+// QTX_ERR_NOT_CONVERGED / QTX_ERR_SINGULAR (only raised from 0).  No host synchronisation.
 constexpr int kDecimSmallMax = 32;
-cudaError_t decimate_small(const cx<double>* H00, const cx<double>* H01, const double* E, double eta,
-                           double tol_rel, int max_iter, int n, int batch, cx<double>* SR, int* status,
+cudaError_t decimate_small(int leads, const cx<double>* const* H00, const cx<double>* const* H01, cx<double>* const* SR,
+                           const double* E, double eta, double tol_rel, int max_iter, int n, int batch, int* status,
                            cudaStream_t st);
+
+// ---- the FP64 sweeps of a device with blocks of at most kSmallMax, one CTA per energy (small.cu).
+// Input blocks and strides as qtx_rgf_inputs (per-energy Sigma advance by sSig); contact blocks
+// [ne][b][b] or null; g, gl [nb], z, x [nb - 1] workspace blocks with `slot` elements per slice; block
+// outputs [ne][nb or nb - 1][b][b] or null; cur [ne][ldcur], den [ne][nb], con [ne][2], tra [ne].
+constexpr int kSmallMax = 32;
+struct SmallArgs {
+  int b, nb;
+  const cx<double>*Hd, *Hu, *Sd, *Su, *SRd, *SLd;
+  long sSig;
+  const double* E;
+  double eta;
+  const cx<double>*SR_L, *Gam_L, *SL_L, *SG_L, *SR_R, *SL_R, *SG_R;
+  cx<double>*g, *gl, *z, *x;
+  long slot;
+  cx<double>*GR_diag, *GR_upper, *GR_lower, *GL_diag, *GL_upper, *GG_diag, *GG_upper;
+  double *cur, *den, *con, *tra;
+  long ldcur;
+  int* status;
+};
+cudaError_t rgf_small(const SmallArgs& a, int batch, cudaStream_t st);
 // set status[e] = code for entries still active (decimation not converged)
 cudaError_t flag_active(const int* active, int* status, int code, int batch, cudaStream_t st);
 

@@ -149,7 +149,7 @@ Layout make_layout(const qtx_rgf_desc& d) {
   L.f32a = a.take(L.refine64 ? Ec * bb * sizeof(cx<float>) : 0);
   L.f32tmp = a.take(L.refine64 ? Ec * bb * sizeof(cx<float>) + 4096 : 0);
   L.perm = a.take(L.refine64 && b <= kPivotedMax ? (size_t)Ec * b * sizeof(int) : 0);
-  L.n_dec = 9;
+  L.n_dec = 10;
   L.dec = a.take(d.leads ? (size_t)L.n_dec * Ec * bb * sizeof(cx<double>) : 0);
   L.lead = a.take(d.leads ? 8 * Ec * bb * sizeof(cx<double>) : 0);
   // per-energy observables: current, density, contact(2), transmission, scratch(2)
@@ -313,8 +313,8 @@ qtx_status gemm<float>(qtx_rgf_plan_s* P, const GemmArgs<float>& g, cudaStream_t
   return gemm_simt_prof<float>(P, g, st);
 }
 template <>
-qtx_status gemm<double>(qtx_rgf_plan_s* P, const GemmArgs<double>& g, cudaStream_t st, bool, DigitHint) {
-  if (g.M >= kTcF64Min && g.N >= kTcF64Min && g.K >= kTcF64Min && gemm_fp64_tc_fits(g.M, g.N, g.K, P->L.tc_bytes)) {
+qtx_status gemm<double>(qtx_rgf_plan_s* P, const GemmArgs<double>& g, cudaStream_t st, bool force_simt, DigitHint) {
+  if (!force_simt && g.M >= kTcF64Min && g.N >= kTcF64Min && g.K >= kTcF64Min && gemm_fp64_tc_fits(g.M, g.N, g.K, P->L.tc_bytes)) {
     cudaEvent_t* ev = (P->prof && P->d.precision == QTX_FP64) ? P->next_events() : nullptr;
     QTX_CK(gemm_fp64_tc(g, P->ws + P->L.tc_scratch, P->L.tc_bytes, P->d_err_flag, st, ev));
     if (ev) {
@@ -580,16 +580,14 @@ qtx_status contact(const Ctx<T>& c, const cx<double>* H00, const cx<double>* H01
   const long bb = c.bb;
   cudaStream_t st = c.st;
   if (b <= kDecimSmallMax) {
-    QTX_CK(decimate_small(H00, H01, c.E, eta, P->d.decim_tol, P->d.decim_max_iter, b, ne, SR, c.status, st));
+    QTX_CK(decimate_small(1, &H00, &H01, &SR, c.E, eta, P->d.decim_tol, P->d.decim_max_iter, b, ne, c.status, st));
     return QTX_OK;
   }
   cx<double>* D = reinterpret_cast<cx<double>*>(P->ws + P->L.dec);
   auto buf = [&](int k) { return D + (size_t)k * P->Ec * bb; };
   cx<double>*alpha = buf(0), *beta = buf(1), *eps = buf(2), *eps_s = buf(3), *g = buf(4), *ag = buf(5),
-  *bg = buf(6), *t1 = buf(7), *t2 = buf(8);
-  int* flags = reinterpret_cast<int*>(P->ws + P->L.flags);
-  int* active = flags;
-  int* sweeps = flags + P->Ec;
+  *bg = buf(6), *t1 = buf(7), *t2 = buf(8), *t3 = buf(9);
+  int* active = reinterpret_cast<int*>(P->ws + P->L.flags);
   double* scale = reinterpret_cast<double*>(P->ws + P->L.dscale);
   QTX_CK(max_modulus(H01, bb, scale, st));
 
@@ -602,37 +600,35 @@ qtx_status contact(const Ctx<T>& c, const cx<double>* H00, const cx<double>* H01
   QTX_CK((combine<double, double>(eps, bb, t00, none, none, b, ne, nullptr, 0, 0, nullptr, st)));
   QTX_CK((combine<double, double>(eps_s, bb, t00, none, none, b, ne, nullptr, 0, 0, nullptr, st)));
   QTX_CK(fill_int(active, 1, ne, st));
-  QTX_CK(cudaMemsetAsync(sweeps, 0, ne * sizeof(int), st));
   qtx_status s;
   auto G = [&](const cx<double>* A, const cx<double>* B, cx<double>* C) {
-    return gemm<double>(P, gargs<double>(b, b, b, A, b, bb, OP_N, B, b, bb, OP_N, nullptr, 0, 0, C, b, bb, 1.0, 0.0, ne, active), st, true);
+    return gargs<double>(b, b, b, A, b, bb, OP_N, B, b, bb, OP_N, nullptr, 0, 0, C, b, bb, 1.0, 0.0, ne, active);
   };
   for (int it = 1; it <= P->d.decim_max_iter; ++it) {
+    // four launches a sweep beside the inverse's: a converged energy's CTAs return at once
     Term<double> te; te.p = eps; te.s = bb; te.alpha = -1.0;
     QTX_CK((combine<double, double>(g, bb, te, none, none, b, ne, c.E, eta, 1.0, active, st)));  // z - eps
-    if ((s = inverse_f64(P, g, b, ne, active, c.status, st))) return s;
-    if ((s = G(alpha, g, ag))) return s;
-    if ((s = G(beta, g, bg))) return s;
-    if ((s = G(ag, beta, t1))) return s;   // alpha g beta
-    if ((s = G(bg, alpha, t2))) return s;  // beta g alpha
-    Term<double> ts; ts.p = eps_s; ts.s = bb; ts.alpha = 1.0;
-    Term<double> ta; ta.p = t1; ta.s = bb; ta.alpha = 1.0;
-    Term<double> tb; tb.p = t2; tb.s = bb; tb.alpha = 1.0;
-    Term<double> tep; tep.p = eps; tep.s = bb; tep.alpha = 1.0;
-    QTX_CK((combine<double, double>(eps_s, bb, ts, ta, none, b, ne, nullptr, 0, 0, active, st)));
-    QTX_CK((combine<double, double>(eps, bb, tep, ta, tb, b, ne, nullptr, 0, 0, active, st)));
-    if ((s = G(ag, alpha, t1))) return s;  // alpha g alpha
-    if ((s = G(bg, beta, t2))) return s;   // beta g beta
-    Term<double> tt1; tt1.p = t1; tt1.s = bb; tt1.alpha = 1.0;
-    Term<double> tt2; tt2.p = t2; tt2.s = bb; tt2.alpha = 1.0;
-    QTX_CK((combine<double, double>(alpha, bb, tt1, none, none, b, ne, nullptr, 0, 0, active, st)));
-    QTX_CK((combine<double, double>(beta, bb, tt2, none, none, b, ne, nullptr, 0, 0, active, st)));
-    QTX_CK(decim_converged(alpha, beta, b, P->d.decim_tol, scale, active, sweeps, ne, st));
+    if ((s = inverse_refined<double>(P, g, b, ne, active, c.status, st))) return s;
+    GemmMulti<double> m;
+    m.n = 2;
+    m.g[0] = G(alpha, g, ag);
+    m.g[1] = G(beta, g, bg);
+    QTX_CK(gemm_simt_multi<double>(m, st));
+    m.n = 4;
+    m.g[0] = G(ag, beta, t1);   // alpha g beta
+    m.g[1] = G(bg, alpha, t2);  // beta g alpha
+    m.g[2] = G(ag, alpha, t3);  // alpha g alpha
+    m.g[3] = G(bg, beta, g);    // beta g beta
+    QTX_CK(gemm_simt_multi<double>(m, st));
+    // converged energies leave stale blocks in the exchanged buffers, which nothing reads again
+    std::swap(alpha, t3);
+    std::swap(beta, g);
+    QTX_CK(decim_update(eps_s, eps, t1, t2, alpha, beta, b, P->d.decim_tol, scale, active, ne, st));
   }
   QTX_CK(flag_active(active, c.status, (int)QTX_ERR_NOT_CONVERGED, ne, st));
   Term<double> tes; tes.p = eps_s; tes.s = bb; tes.alpha = -1.0;
   QTX_CK((combine<double, double>(g, bb, tes, none, none, b, ne, c.E, eta, 1.0, nullptr, st)));  // z - eps_s
-  if ((s = inverse_f64(P, g, b, ne, nullptr, c.status, st))) return s;
+  if ((s = inverse_refined<double>(P, g, b, ne, nullptr, c.status, st))) return s;
   // Sigma^R = H01 g_s H01^H
   if ((s = gemm<double>(P, gargs<double>(b, b, b, H01, b, 0, OP_N, g, b, bb, OP_N, nullptr, 0, 0, t1, b, bb, 1.0, 0.0, ne, nullptr), st, true))) return s;
   if ((s = gemm<double>(P, gargs<double>(b, b, b, t1, b, bb, OP_N, H01, b, 0, OP_C, nullptr, 0, 0, SR, b, bb, 1.0, 0.0, ne, nullptr), st, true))) return s;
@@ -650,6 +646,70 @@ qtx_status emit(qtx_rgf_plan_s* P, void* out, long nslices, long slice, int e0, 
   Term<T> t1; t1.p = plus; t1.s = bb; t1.alpha = 1.0;
   Term<T> t2; t2.p = minus_h; t2.s = bb; t2.alpha = -1.0; t2.op = OP_C;
   QTX_CK((combine<T, double>(o, nslices * bb, t0, t1, t2, b, ne, nullptr, 0.0, 0.0, nullptr, st)));
+  return QTX_OK;
+}
+
+// Per-energy observables of the chunk in the workspace.
+struct ObsBufs {
+  int ncur;
+  double *cur, *den, *con, *tra;         // [ne][ncur], [ne][nb], [ne][2], [ne]
+  double *bal, *bscale, *bgn, *bhn;      // [ne][nb] each (continuity check)
+  explicit ObsBufs(qtx_rgf_plan_s* P) {
+    const int nb = P->nb;
+    ncur = nb > 1 ? nb - 1 : 1;
+    cur = reinterpret_cast<double*>(P->ws + P->L.obs);
+    den = cur + (size_t)P->Ec * ncur;
+    con = den + (size_t)P->Ec * nb;
+    tra = con + (size_t)P->Ec * 2;
+    bal = reinterpret_cast<double*>(P->ws + P->L.bal);
+    bscale = reinterpret_cast<double*>(P->ws + P->L.bscale);
+    bgn = reinterpret_cast<double*>(P->ws + P->L.bgn);
+    bhn = reinterpret_cast<double*>(P->ws + P->L.bhn);
+  }
+};
+inline bool wants_balance(const qtx_rgf_desc& d) { return (d.outputs & QTX_OUT_CONTINUITY) || d.escalate_tol > 0; }
+
+// After a chunk's sweeps: the continuity check, the per-energy outputs and the energy integrals.
+template <typename T>
+qtx_status finish_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rgf_outputs* out, int e0, int ne,
+                        cudaStream_t st) {
+  const qtx_rgf_desc& d = P->d;
+  const int nb = P->nb;
+  const unsigned m = d.outputs;
+  const ObsBufs ob(P);
+  const int ncur = ob.ncur;
+  double *cur = ob.cur, *den = ob.den, *con = ob.con, *tra = ob.tra;
+  auto want = [&](unsigned bit, const void* p) { return (m & bit) && p; };
+  // ---- continuity residual per energy (and the escalation flags)
+  if (wants_balance(d)) {
+    double* cres = reinterpret_cast<double*>(P->ws + P->L.cres);
+    int* cflag = reinterpret_cast<int*>(P->ws + P->L.cflag);
+    // unit error of the products in this mode (Eq. 6: error ~ kappa eps): 6 (7) bf16 digits ~41 bits,
+    // 2 digits ~13 bits, complex64 24 bits, FP64 53
+    const double eps_mode = std::is_same<T, double>::value ? 0x1p-53
+                            : std::is_same<T, float>::value  ? 0x1p-24
+                            : (d.precision == QTX_BF16X3 ? 0x1p-13 : 0x1p-40);
+    QTX_CK(continuity(cur, ncur, ob.bal, ob.bscale, ob.bgn, ob.bhn, nb, d.leads ? con : nullptr, in->energies + e0, nb, ne,
+                      d.escalate_tol > 0 ? d.escalate_tol : 1e300, eps_mode, cres, cflag, st));
+    if (want(QTX_OUT_CONTINUITY, out->continuity))
+      QTX_CK(cudaMemcpyAsync(out->continuity + e0, cres, (size_t)ne * sizeof(double), cudaMemcpyDeviceToDevice, st));
+  }
+  // ---- 4. outputs of the per-energy observables and their integrals
+  const int nbm1 = nb - 1;
+  if (want(QTX_OUT_CURRENT, out->current) && nbm1 > 0)
+    QTX_CK(cudaMemcpyAsync(out->current + (size_t)e0 * nbm1, cur, (size_t)ne * nbm1 * sizeof(double), cudaMemcpyDeviceToDevice, st));
+  if (want(QTX_OUT_DENSITY, out->density))
+    QTX_CK(cudaMemcpyAsync(out->density + (size_t)e0 * nb, den, (size_t)ne * nb * sizeof(double), cudaMemcpyDeviceToDevice, st));
+  if (d.leads && want(QTX_OUT_CONTACT, out->contact))
+    QTX_CK(cudaMemcpyAsync(out->contact + (size_t)e0 * 2, con, (size_t)ne * 2 * sizeof(double), cudaMemcpyDeviceToDevice, st));
+  if (d.leads && want(QTX_OUT_TRANSMISSION, out->transmission))
+    QTX_CK(cudaMemcpyAsync(out->transmission + e0, tra, (size_t)ne * sizeof(double), cudaMemcpyDeviceToDevice, st));
+  if (m & QTX_OUT_INTEGRALS) {
+    if (out->current_int && nbm1 > 0)
+      QTX_CK(integrate_add(out->current_int, cur, nbm1, nbm1, in->weights, in->energies, e0, in->n_energies, ne, 1.0, st));
+    if (out->density_int)
+      QTX_CK(integrate_add(out->density_int, den, nb, nb, in->weights, in->energies, e0, in->n_energies, ne, 1.0 / (2.0 * 3.14159265358979323846), st));
+  }
   return QTX_OK;
 }
 
@@ -701,10 +761,55 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
   cx<double>*SR_L = lb(0), *Gam_L = lb(1), *SL_L = lb(2), *SG_L = lb(3);
   cx<double>*SR_R = lb(4), *Gam_R = lb(5), *SL_R = lb(6), *SG_R = lb(7);
   if (d.leads) {
-    if ((s = contact<T>(c, (const cx<double>*)in->lead_H00_L, (const cx<double>*)in->lead_H01_L, eta, SR_L))) return s;
-    if ((s = contact<T>(c, (const cx<double>*)in->lead_H00_R, (const cx<double>*)in->lead_H01_R, eta, SR_R))) return s;
+    const cx<double>* H00[2] = {(const cx<double>*)in->lead_H00_L, (const cx<double>*)in->lead_H00_R};
+    const cx<double>* H01[2] = {(const cx<double>*)in->lead_H01_L, (const cx<double>*)in->lead_H01_R};
+    cx<double>* SR[2] = {SR_L, SR_R};
+    if (b <= kDecimSmallMax) {  // both contacts of every energy in one launch
+      QTX_CK(decimate_small(2, H00, H01, SR, c.E, eta, d.decim_tol, d.decim_max_iter, b, ne, status, st));
+    } else {
+      for (int k = 0; k < 2; ++k)
+        if ((s = contact<T>(c, H00[k], H01[k], eta, SR[k]))) return s;
+    }
     QTX_CK(lead_sigmas(SR_L, Gam_L, SL_L, SG_L, c.E, in->mu_L, in->kT, b, ne, st));
     QTX_CK(lead_sigmas(SR_R, Gam_R, SL_R, SG_R, c.E, in->mu_R, in->kT, b, ne, st));
+  }
+
+  // ---- FP64 devices of small blocks: the sweeps of each energy in one CTA
+  const unsigned m = d.outputs;
+  auto want = [&](unsigned bit, const void* p) { return (m & bit) && p; };
+  if constexpr (std::is_same<T, double>::value) {
+    // the options beyond the plain sweeps (block-tridiagonal Sigma, M given, FPX storage, streamed Sigma,
+    // current balances) stay on the launched path
+    if (b <= kSmallMax && !d.offdiag_sigma && !d.system_input && !d.storage_bits && !d.sigma_stream && !wants_balance(d)) {
+      const ObsBufs ob(P);
+      SmallArgs a{};
+      a.b = b; a.nb = nb;
+      a.Hd = Hd; a.Hu = Hu; a.Sd = Sd; a.Su = Su; a.SRd = sigR(0); a.SLd = sigL(0);
+      a.sSig = sSig;
+      a.E = c.E; a.eta = eta;
+      if (d.leads) {
+        a.SR_L = SR_L; a.Gam_L = Gam_L; a.SL_L = SL_L; a.SG_L = SG_L;
+        a.SR_R = SR_R; a.SL_R = SL_R; a.SG_R = SG_R;
+      }
+      a.slot = (long)P->Ec * bb;
+      a.g = c.g(0); a.gl = c.gl(0);
+      if (nb > 1) { a.z = c.zk(0); a.x = c.xk(0, 0); }
+      auto blocks = [&](unsigned bit, void* p, long n) {
+        return want(bit, p) ? reinterpret_cast<cx<double>*>(p) + (long)e0 * n * bb : nullptr;
+      };
+      a.GR_diag = blocks(QTX_OUT_GR_DIAG, out->GR_diag, nb);
+      a.GR_upper = blocks(QTX_OUT_GR_UPPER, out->GR_upper, nb - 1);
+      a.GR_lower = blocks(QTX_OUT_GR_LOWER, out->GR_lower, nb - 1);
+      a.GL_diag = blocks(QTX_OUT_GL_DIAG, out->GL_diag, nb);
+      a.GL_upper = blocks(QTX_OUT_GL_UPPER, out->GL_upper, nb - 1);
+      a.GG_diag = blocks(QTX_OUT_GG_DIAG, out->GG_diag, nb);
+      a.GG_upper = blocks(QTX_OUT_GG_UPPER, out->GG_upper, nb - 1);
+      a.cur = ob.cur; a.den = ob.den; a.con = ob.con; a.tra = ob.tra;
+      a.ldcur = ob.ncur;
+      a.status = status;
+      QTX_CK(rgf_small(a, ne, st));
+      return finish_chunk<T>(P, in, out, e0, ne, st);
+    }
   }
 
   // ---- off-diagonal blocks of M
@@ -845,20 +950,12 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
   //   K = P G_{i+1,i+1} Q = -G_{i,i+1} Q   (block-tridiagonal Sigma^<: Q += (g_i Sigma^<_{i,i+1})^H)
   //   G^<_ii = g^<_i + (P G^<_{i+1,i+1}) P^H + K - K^H
   //   G^<_{i,i+1} = -P G^<_{i+1,i+1} + (G_{i+1,i+1} Q)^H     [= -P G^< - g^< V^H G^A]
-  double* obs = reinterpret_cast<double*>(P->ws + P->L.obs);
-  const int ncur = nb > 1 ? nb - 1 : 1;
-  double* cur = obs;                           // [ne][nb-1]
-  double* den = cur + (size_t)P->Ec * ncur;    // [ne][nb]
-  double* con = den + (size_t)P->Ec * nb;      // [ne][2]
-  double* tra = con + (size_t)P->Ec * 2;       // [ne]
-  const unsigned m = d.outputs;
-  auto want = [&](unsigned bit, const void* p) { return (m & bit) && p; };
+  const ObsBufs ob(P);
+  const int ncur = ob.ncur;
+  double *cur = ob.cur, *den = ob.den, *con = ob.con, *tra = ob.tra;
   // current conservation (Sec. II-B): per-slice balances J_i, checked after the sweep
-  const bool cont = (m & QTX_OUT_CONTINUITY) || d.escalate_tol > 0;
-  double* bal = reinterpret_cast<double*>(P->ws + P->L.bal);        // [ne][nb]
-  double* bscale = reinterpret_cast<double*>(P->ws + P->L.bscale);  // [ne][nb]
-  double* bgn = reinterpret_cast<double*>(P->ws + P->L.bgn);        // [ne][nb]
-  double* bhn = reinterpret_cast<double*>(P->ws + P->L.bhn);        // [ne][nb]
+  const bool cont = wants_balance(d);
+  double *bal = ob.bal, *bscale = ob.bscale, *bgn = ob.bgn, *bhn = ob.bhn;
   {
     const int i = nb - 1;
     if (want(QTX_OUT_GR_DIAG, out->GR_diag) && (s = emit<T>(P, out->GR_diag, nb, i, e0, c.g(i), b, ne, st))) return s;
@@ -991,37 +1088,7 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
     if ((s = gemm<double>(P, gargs<double>(b, b, b, G64, b, bb, OP_N, Gam_L, b, bb, OP_N, nullptr, 0, 0, X2, b, bb, 1.0, 0.0, ne, nullptr), st, true))) return s;
     QTX_CK(obs_frob_dot(tra, 1, X1, bb, X2, bb, -1.0, b, ne, st));
   }
-  // ---- continuity residual per energy (and the escalation flags)
-  if (cont) {
-    double* cres = reinterpret_cast<double*>(P->ws + P->L.cres);
-    int* cflag = reinterpret_cast<int*>(P->ws + P->L.cflag);
-    // unit error of the products in this mode (Eq. 6: error ~ kappa eps): 6 (7) bf16 digits ~41 bits,
-    // 2 digits ~13 bits, complex64 24 bits, FP64 53
-    const double eps_mode = std::is_same<T, double>::value ? 0x1p-53
-                            : std::is_same<T, float>::value  ? 0x1p-24
-                            : (d.precision == QTX_BF16X3 ? 0x1p-13 : 0x1p-40);
-    QTX_CK(continuity(cur, ncur, bal, bscale, bgn, bhn, nb, d.leads ? con : nullptr, c.E, nb, ne,
-                      d.escalate_tol > 0 ? d.escalate_tol : 1e300, eps_mode, cres, cflag, st));
-    if (want(QTX_OUT_CONTINUITY, out->continuity))
-      QTX_CK(cudaMemcpyAsync(out->continuity + e0, cres, (size_t)ne * sizeof(double), cudaMemcpyDeviceToDevice, st));
-  }
-  // ---- 4. outputs of the per-energy observables and their integrals
-  const int nbm1 = nb - 1;
-  if (want(QTX_OUT_CURRENT, out->current) && nbm1 > 0)
-    QTX_CK(cudaMemcpyAsync(out->current + (size_t)e0 * nbm1, cur, (size_t)ne * nbm1 * sizeof(double), cudaMemcpyDeviceToDevice, st));
-  if (want(QTX_OUT_DENSITY, out->density))
-    QTX_CK(cudaMemcpyAsync(out->density + (size_t)e0 * nb, den, (size_t)ne * nb * sizeof(double), cudaMemcpyDeviceToDevice, st));
-  if (d.leads && want(QTX_OUT_CONTACT, out->contact))
-    QTX_CK(cudaMemcpyAsync(out->contact + (size_t)e0 * 2, con, (size_t)ne * 2 * sizeof(double), cudaMemcpyDeviceToDevice, st));
-  if (d.leads && want(QTX_OUT_TRANSMISSION, out->transmission))
-    QTX_CK(cudaMemcpyAsync(out->transmission + e0, tra, (size_t)ne * sizeof(double), cudaMemcpyDeviceToDevice, st));
-  if (m & QTX_OUT_INTEGRALS) {
-    if (out->current_int && nbm1 > 0)
-      QTX_CK(integrate_add(out->current_int, cur, nbm1, nbm1, in->weights, in->energies, e0, in->n_energies, ne, 1.0, st));
-    if (out->density_int)
-      QTX_CK(integrate_add(out->density_int, den, nb, nb, in->weights, in->energies, e0, in->n_energies, ne, 1.0 / (2.0 * 3.14159265358979323846), st));
-  }
-  return QTX_OK;
+  return finish_chunk<T>(P, in, out, e0, ne, st);
 }
 
 template <typename T>

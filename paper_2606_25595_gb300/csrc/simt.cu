@@ -17,14 +17,12 @@ std::atomic<long long> g_launches{0};
 // the other buffer after them, one barrier per stage); each thread owns a TM x TN sub-grid
 // interleaved with stride (BM/TM, BN/TN) so smem reads of a warp are contiguous.
 template <typename T, int BM, int BN, int BK, int TM, int TN>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN))
-    k_gemm(GemmArgs<T> g) {
+__device__ __forceinline__ void gemm_tile(const GemmArgs<T>& g, const int e) {
   // FP32: two stage buffers (load latency hidden behind the FMAs); FP64 is bound by the FP64 pipe,
   // where one buffer with twice the K per stage (half the barriers) is faster
   constexpr int NBUF = sizeof(T) == 4 ? 2 : 1;
   constexpr int TX = BN / TN, TY = BM / TM, NT = TX * TY;
   constexpr int LA = (BM * BK + NT - 1) / NT, LB = (BK * BN + NT - 1) / NT;  // loads per thread
-  const int e = blockIdx.z;
   if (g.active && !g.active[e]) return;
   __shared__ cx<T> As[NBUF][BK][BM + 1];
   __shared__ cx<T> Bs[NBUF][BK][BN + 1];
@@ -136,21 +134,73 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 }
 
 template <typename T, int BM, int BN, int BK, int TM, int TN>
-static cudaError_t launch_gemm(const GemmArgs<T>& g, cudaStream_t st) {
-  dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.batch);
-  k_gemm<T, BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, st>>>(g);
+__global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_gemm(GemmArgs<T> g) {
+  gemm_tile<T, BM, BN, BK, TM, TN>(g, blockIdx.z);
+}
+// several products of the same M, N and batch in one launch (blockIdx.z: product, then batch entry)
+template <typename T, int BM, int BN, int BK, int TM, int TN>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_gemm_multi(const __grid_constant__ GemmMulti<T> m) {
+  const int q = blockIdx.z / m.g[0].batch;
+  gemm_tile<T, BM, BN, BK, TM, TN>(m.g[q], blockIdx.z - q * m.g[0].batch);
+}
+
+template <typename T, int BM, int BN, int BK, int TM, int TN>
+static cudaError_t launch_gemm(const GemmMulti<T>& m, cudaStream_t st) {
+  const GemmArgs<T>& g = m.g[0];
+  dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.batch * m.n);
+  if (m.n == 1) k_gemm<T, BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, st>>>(g);
+  else k_gemm_multi<T, BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, st>>>(m);
   count_launch();
   return cudaGetLastError();
 }
 
+// FP64 tile by the FP64 pipe's work: tiles beyond M and N multiply zeros, and few tiles leave SMs idle, so
+// the tile with the least tile area times rounds of 152 SMs is taken (the sums' order is the same in all).
+// 48 x 48 products of 12 entries: 216 us in 64 x 64 tiles (12 CTAs), 13 us in 16 x 16 (108 CTAs).
+static int fp64_tile(int M, int N, long batch) {
+  int best = 64;
+  long least = 0;
+  for (int t : {64, 32, 16}) {
+    const long ctas = (long)((M + t - 1) / t) * ((N + t - 1) / t) * batch;
+    const long cost = (ctas + 151) / 152 * t * t;
+    if (t == 64 || cost < least) {
+      best = t;
+      least = cost;
+    }
+  }
+  return best;
+}
+
+template <typename T>
+cudaError_t gemm_simt_multi(const GemmMulti<T>& m, cudaStream_t st) {
+  const GemmArgs<T>& g = m.g[0];
+  if (m.n < 1 || m.n > GemmMulti<T>::kMax) return cudaErrorInvalidValue;
+  if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
+  if (m.n > 1 && (long)g.batch * m.n > 65535) {  // beyond a grid's z extent: one launch each
+    for (int q = 0; q < m.n; ++q)
+      if (const cudaError_t e = gemm_simt<T>(m.g[q], st)) return e;
+    return cudaSuccess;
+  }
+  if constexpr (sizeof(T) == 8) {
+    switch (fp64_tile(g.M, g.N, (long)g.batch * m.n)) {
+      case 16: return launch_gemm<T, 16, 16, 16, 1, 1>(m, st);
+      case 32: return launch_gemm<T, 32, 32, 16, 2, 2>(m, st);
+      default: return launch_gemm<T, 64, 64, 16, 4, 4>(m, st);
+    }
+  } else {
+    if (g.M <= 32 && g.N <= 32) return launch_gemm<T, 32, 32, 16, 2, 2>(m, st);
+    if (g.M >= 128 && g.N >= 128) return launch_gemm<T, 128, 128, 8, 8, 8>(m, st);
+    return launch_gemm<T, 64, 64, 16, 4, 4>(m, st);
+  }
+}
+template cudaError_t gemm_simt_multi<double>(const GemmMulti<double>&, cudaStream_t);
+
 template <typename T>
 cudaError_t gemm_simt(const GemmArgs<T>& g, cudaStream_t st) {
-  if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
-  if (g.M <= 32 && g.N <= 32) return launch_gemm<T, 32, 32, 16, 2, 2>(g, st);
-  if constexpr (sizeof(T) == 4) {
-    if (g.M >= 128 && g.N >= 128) return launch_gemm<T, 128, 128, 8, 8, 8>(g, st);
-  }
-  return launch_gemm<T, 64, 64, 16, 4, 4>(g, st);
+  GemmMulti<T> m;
+  m.n = 1;
+  m.g[0] = g;
+  return gemm_simt_multi<T>(m, st);
 }
 template cudaError_t gemm_simt<double>(const GemmArgs<double>&, cudaStream_t);
 template cudaError_t gemm_simt<float>(const GemmArgs<float>&, cudaStream_t);
@@ -317,7 +367,7 @@ __global__ void __launch_bounds__(NMAX * 4) k_leaf_inverse(cx<T>* Ag, long lda, 
 
 template <typename T>
 cudaError_t leaf_inverse(cx<T>* A, long lda, long sA, int n, int batch, const int* active, int* status,
-                         cudaStream_t st) {
+                         cudaStream_t st) {  // T = double: leaf64.cu
   if (n <= 0 || n > kLeafMax) return cudaErrorInvalidValue;
   if (n <= 32)
     k_leaf_inverse<T, 32><<<batch, 128, 0, st>>>(A, lda, sA, n, active, status);
@@ -326,7 +376,6 @@ cudaError_t leaf_inverse(cx<T>* A, long lda, long sA, int n, int batch, const in
   count_launch();
   return cudaGetLastError();
 }
-template cudaError_t leaf_inverse<double>(cx<double>*, long, long, int, int, const int*, int*, cudaStream_t);
 template cudaError_t leaf_inverse<float>(cx<float>*, long, long, int, int, const int*, int*, cudaStream_t);
 
 // ============================================================================ elementwise
@@ -1300,32 +1349,51 @@ cudaError_t fill_int(int* p, int v, int n, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(256) k_decim_converged(const cx<double>* X, const cx<double>* Y, int b,
-                                                         double tol_rel, const double* scale, int* active,
-                                                         int* sweeps) {
+// One sweep's sums of the launched decimation and its convergence test: es += x, ep = (ep + x) + y, then
+// active[e] = 0 once the largest modulus over alpha and beta is below tol_rel * (*scale, or 1 if 0).
+__global__ void __launch_bounds__(512) k_decim_update(cx<double>* es, cx<double>* ep, const cx<double>* x, const cx<double>* y,
+                                                      const cx<double>* al, const cx<double>* be, int b, double tol_rel,
+                                                      const double* scale, int* active) {
   const int e = blockIdx.x;
   if (!active[e]) return;
   const double tol = tol_rel * (*scale > 0.0 ? *scale : 1.0);
-  const long bb = (long)b * b;
-  double m = 0.0;
-  for (long idx = threadIdx.x; idx < bb; idx += blockDim.x) {
-    const cx<double> x = X[(long)e * bb + idx], y = Y[(long)e * bb + idx];
-    m = fmax(m, fmax(hypot(x.re, x.im), hypot(y.re, y.im)));
+  const long bb = (long)b * b, o = (long)e * bb;
+  unsigned h = 0;
+  auto hw = [](double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; };
+  for (long i = o + threadIdx.x; i < o + bb; i += blockDim.x) {
+    es[i] = es[i] + x[i];
+    ep[i] = (ep[i] + x[i]) + y[i];
+    h = max(h, max(max(hw(al[i].re), hw(al[i].im)), max(hw(be[i].re), hw(be[i].im))));
   }
+  // the largest |re|, |im| decides by its high word unless it lies within sqrt(2) of tol or is not a number
+  __shared__ unsigned s_h;
+  __shared__ double red[16];
+  if (threadIdx.x == 0) s_h = 0;
+  __syncthreads();
+  h = __reduce_max_sync(0xffffffffu, h);
+  if (threadIdx.x % 32 == 0) atomicMax(&s_h, h);
+  __syncthreads();
+  h = s_h;
+  if (h < 0x7ff00000u && __hiloint2double((int)h, 0) >= tol) return;
+  if (h < 0x7ff00000u && __hiloint2double((int)h + 1, 0) * 1.4142135623731 < tol) {
+    if (threadIdx.x == 0) active[e] = 0;
+    return;
+  }
+  double m = 0.0;
+  for (long i = o + threadIdx.x; i < o + bb; i += blockDim.x)
+    m = fmax(m, fmax(hypot(al[i].re, al[i].im), hypot(be[i].re, be[i].im)));
   for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
-  __shared__ double red[8];
   if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = m;
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int i = 1; i < (int)blockDim.x / 32; ++i) m = fmax(m, red[i]);
-    m = fmax(m, red[0]);
-    sweeps[e] += 1;
     if (m < tol) active[e] = 0;
   }
 }
-cudaError_t decim_converged(const cx<double>* X, const cx<double>* Y, int b, double tol_rel, const double* scale,
-                            int* active, int* sweeps, int batch, cudaStream_t st) {
-  k_decim_converged<<<batch, 256, 0, st>>>(X, Y, b, tol_rel, scale, active, sweeps);
+cudaError_t decim_update(cx<double>* es, cx<double>* ep, const cx<double>* x, const cx<double>* y, const cx<double>* al,
+                         const cx<double>* be, int b, double tol_rel, const double* scale, int* active, int batch,
+                         cudaStream_t st) {
+  k_decim_update<<<batch, 512, 0, st>>>(es, ep, x, y, al, be, b, tol_rel, scale, active);
   count_launch();
   return cudaGetLastError();
 }

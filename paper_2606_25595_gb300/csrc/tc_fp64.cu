@@ -67,13 +67,15 @@ struct Params {
 
 __device__ __forceinline__ int at9(int r, int c) { return r * BNC9 + (c ^ (r & 7)); }
 
-// one output value from the eight accumulators (pre-scaled digit products)
-__device__ __forceinline__ double recombine(const uint32_t (&v)[NACC9][8], int c) {
+// one output value from the eight accumulators (pre-scaled digit products), times 2^Es
+__device__ __forceinline__ double recombine(const uint32_t (&v)[NACC9][8], int c, int Es) {
   // exact groups as integers of their own unit 2^(-7 g); the tail in units of 2^-53
   auto fx = [&](int g, int sh) { return (int64_t)__float2int_rn(__uint_as_float(v[g][c]) * __int_as_float((127 + sh) << 23)); };
   const int64_t hi = (fx(0, 0) << 28) + (fx(1, 7) << 21) + (fx(2, 14) << 14) + (fx(3, 21) << 7) + fx(4, 28);
   const int64_t lo = (fx(5, 35) << 21) + (fx(6, 42) << 14) + (fx(7, 53) << 3);
-  return fix_sum(hi, lo);
+  bool bad = false;
+  const double x = fix_sum_scaled(hi, lo, Es, bad);
+  return bad ? scale64(fix_sum(hi, lo), Es) : x;
 }
 
 // (op(A) op(B))(m, n) of one batch entry by DFMA: rows or columns with non-finite values
@@ -219,6 +221,7 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__
       asm volatile("bar.sync 2, 256;" ::: "memory");
       if (!*s_got) break;
       fence_after();
+      const int er = s_eA[r] - p.escale;  // a non-finite row's or column's values are replaced below
 #pragma unroll 1
       for (int c0 = 8 * h; c0 < bn; c0 += 16) {
 #pragma unroll 1
@@ -228,14 +231,14 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__
           for (int g = 0; g < NACC9; ++g) tmem_ld8(trow + g * ACC9 + part * bn + c0, v[g]);
           tmem_wait_ld();
 #pragma unroll
-          for (int c = 0; c < 8; ++c) (&out[at9(r, c0 + c)].re)[part] = recombine(v, c);
+          for (int c = 0; c < 8; ++c) (&out[at9(r, c0 + c)].re)[part] = recombine(v, c, er + s_eB[c0 + c]);
         }
       }
       fence_before();
       __syncwarp();
       asm volatile("bar.sync 1, 256;" ::: "memory");
       if (et == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(acce)) : "memory");
-      // store phase, overlapping the next tile's MMAs: scale, alpha, beta C0
+      // store phase, overlapping the next tile's MMAs: alpha, beta C0
       const cx<double>* C0e = p.C0 ? p.C0 + (long)e * p.sC0 : nullptr;
       cx<double>* Ce = p.C + (long)e * p.sC;
       for (int idx = et; idx < BM * bn; idx += 256) {
@@ -244,12 +247,7 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__
         if (m >= p.M || n >= p.N) continue;
         cx<double> v = out[at9(rr, cc)];
         const int ea = s_eA[rr], eb = s_eB[cc];
-        if (ea >= kExpoNonFinite || eb >= kExpoNonFinite) {
-          v = dot_dfma(p, e, m, n);
-        } else {
-          v.re = scale64(v.re, ea + eb - p.escale);
-          v.im = scale64(v.im, ea + eb - p.escale);
-        }
+        if (ea >= kExpoNonFinite || eb >= kExpoNonFinite) v = dot_dfma(p, e, m, n);
         if (p.akind == 1) v = mk<double>(-v.re, -v.im);
         else if (p.akind == 2) v = p.alpha * v;
         if (p.bkind != 3) {
@@ -355,13 +353,11 @@ __global__ void __launch_bounds__(32 * RPC) k_digitize_fp64(const cx<double>* X,
     }
 #pragma unroll
     for (int i = 0; i < S9; ++i) {
-      // digits d 2^(-7 i) as bf16: 0x4300 | (d + 64) is the bf16 of 192 + d (also for
-      // d = 64, where the OR carries into the exponent: 256), and (192 + d) s - 192 s is exact
-      const __nv_bfloat162 s = __float2bfloat162_rn(__int_as_float((127 - DW * i) << 23));
-      const __nv_bfloat162 m = __float2bfloat162_rn(-192.f * __int_as_float((127 - DW * i) << 23));
+      const uint32_t sc = digit_scale(i), sh = digit_shift(i);
       auto word = [&](uint64_t a, uint64_t b) {
         const uint32_t w = 0x43004300u | digit_field(a, i) | (digit_field(b, i) << 16);
-        const __nv_bfloat162 d = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w), s, m);
+        const __nv_bfloat162 d = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w), *reinterpret_cast<const __nv_bfloat162*>(&sc),
+                                         *reinterpret_cast<const __nv_bfloat162*>(&sh));
         return *reinterpret_cast<const uint32_t*>(&d);
       };
       unsigned char* pl = pe + (long)i * plane_bytes;
@@ -419,18 +415,11 @@ cudaError_t digitize9(const cx<double>* X, long ldx, long sX, int opX, int side,
   return cudaGetLastError();
 }
 
-// SM count of the current device, with the kernel's shared-memory limit raised there once
-cudaError_t device_ready(int& sms) {
-  constexpr int kMaxDev = 64;
-  static std::atomic<int> known[kMaxDev];
+// SM count of the current device
+cudaError_t sm_count(int& sms) {
   int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < kMaxDev && (sms = known[dev].load(std::memory_order_acquire)) > 0) return cudaSuccess;
-  if ((e = cudaFuncSetAttribute(k_tc_gemm_fp64, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM9))) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
-  if (dev < kMaxDev) known[dev].store(sms, std::memory_order_release);
-  return cudaSuccess;
+  const cudaError_t e = cudaGetDevice(&dev);
+  return e != cudaSuccess ? e : cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
 }
 
 cudaError_t product9(const GemmArgs<double>& g, unsigned char* scratch, int* err_flag, cudaStream_t st, cudaEvent_t* ev) {
@@ -474,7 +463,8 @@ cudaError_t product9(const GemmArgs<double>& g, unsigned char* scratch, int* err
   p.hold = wait_test();
   p.limit_ns = p.hold ? kWaitTestLimitNs : kWaitLimitNs;
   int sms = 0;
-  if ((e = device_ready(sms))) return e;
+  static std::atomic<unsigned long long> done{0};
+  if ((e = allow_smem(k_tc_gemm_fp64, SMEM9, done)) || (e = sm_count(sms))) return e;
   if (ev) cudaEventRecord(ev[0], st);
   k_tc_gemm_fp64<<<(unsigned)(tiles < sms ? tiles : sms), 320, SMEM9, st>>>(p);
   count_launch();
