@@ -50,52 +50,75 @@ template <int NM>
 struct DSmem {
   static constexpr int LD = NM + 1;  // odd stride: row and column reads free of bank conflicts
   cx<double> m[8][NM * LD];
-  cx<double> rowk[NM];
+  cx<double> rowk[NM], recip;
   int perm[NM], from[NM];
   int piv;
   unsigned hi;
   double red[kThreads / 32];
 };
 
+// One entry of the update: x - f a with a the scaled pivot row, its roundings written out.
+__device__ __forceinline__ cx<double> upd(cx<double> x, cx<double> f, cx<double> a) {
+  return mk<double>(__dsub_rn(x.re, __fma_rn(f.re, a.re, -__dmul_rn(f.im, a.im))),
+                    __dsub_rn(x.im, __fma_rn(f.im, a.re, __dmul_rn(f.re, a.im))));
+}
+// ... of the pivot column, 0 - f r with r = 1 / pivot: the two products' roles exchanged
+__device__ __forceinline__ cx<double> upd_col(cx<double> f, cx<double> r) {
+  return mk<double>(__dsub_rn(0.0, __fma_rn(-f.im, r.im, __dmul_rn(f.re, r.re))),
+                    __dsub_rn(0.0, __fma_rn(f.re, r.im, __dmul_rn(f.im, r.re))));
+}
+
 // Gauss-Jordan inverse with partial (row) pivoting on |re| + |im|, first maximum on ties, from block A
 // (destroyed) with B as the other copy; the result is the returned block (A or B), nullptr (uniformly)
-// for a zero pivot.  The order of every rounding is written out: with f the row's factor and a the scaled
-// pivot row, an entry becomes x - f a with re = fma(f.re, a.re, -(f.im a.im)), im = fma(f.im, a.re, f.re a.im);
-// the pivot column 0 - f a (a = 1 / pivot) with the two products' roles exchanged.
+// for a zero pivot.  Step k's chain -- the column's update, its pivot and the reciprocal (two divisions of
+// 520 cycles) -- runs in warp 0 while the other warps make step k - 1's update of the remaining columns.
 template <int NM>
 __device__ cx<double>* eliminate(DSmem<NM>& s, cx<double>* A, cx<double>* B, const gj::FastDiv& fd) {
-  constexpr int LD = DSmem<NM>::LD;
+  constexpr int LD = DSmem<NM>::LD, kUpd = kThreads - 32;
   const int t = threadIdx.x, n = fd.n;
-  for (int k = 0; k < n; ++k) {
-    if (t < 32) {
-      const unsigned long long key = (t >= k && t < n) ? gj::pivot_key(A[t * LD + k]) : 0ull;
-      const unsigned long long best = gj::warp_max(key);
-      const int p = best ? __ffs((int)__ballot_sync(0xffffffffu, key == best)) - 1 : -1;
-      if (t == 0) {
-        s.piv = p;
-        s.perm[k] = p;
-      }
-      if (p >= 0) {
-        const cx<double> r = gj::crecip_warp(A[p * LD + k]);
-        if (t < n) {
-          const cx<double> x = A[p * LD + t];
-          const cx<double> y = mk<double>(__fma_rn(x.re, r.re, -__dmul_rn(x.im, r.im)), __fma_rn(x.re, r.im, __dmul_rn(x.im, r.re)));
-          s.rowk[t] = t == k ? r : y;
-        }
-      }
+  // pivot row of column k of block X and the reciprocal of its entry (warp 0)
+  auto pivot = [&](const cx<double>* X, int k) {
+    const unsigned long long key = (t >= k && t < n) ? gj::pivot_key(X[t * LD + k]) : 0ull;
+    const unsigned long long best = gj::warp_max(key);
+    const int p = best ? __ffs((int)__ballot_sync(0xffffffffu, key == best)) - 1 : -1;
+    cx<double> r = mk<double>(0.0, 0.0);
+    if (p >= 0) r = gj::crecip_warp(X[p * LD + k]);
+    if (t == 0) {
+      s.piv = p;
+      s.perm[k] = p;
+      s.recip = r;
     }
-    __syncthreads();
+  };
+  if (t < 32) pivot(A, 0);
+  __syncthreads();
+  for (int k = 0; k < n; ++k) {
     const int p = s.piv;
     if (p < 0) return nullptr;
-    for (int idx = t; idx < n * n; idx += kThreads) {
-      const int i = fd.div(idx), j = idx - i * n;
-      const int src = i == p ? k : i;  // rows k and p interchanged
-      const bool kc = j == k;
-      const cx<double> f = A[src * LD + k], a = s.rowk[j], y = kc ? mk<double>(0.0, 0.0) : A[src * LD + j];
-      const double re = __fma_rn(kc ? -f.im : f.re, kc ? a.im : a.re, __dmul_rn(kc ? f.re : -f.im, kc ? a.re : a.im));
-      const double im = __fma_rn(kc ? f.re : f.im, kc ? a.im : a.re, __dmul_rn(kc ? f.im : f.re, kc ? a.re : a.im));
-      const cx<double> v = mk<double>(__dsub_rn(y.re, re), __dsub_rn(y.im, im));
-      B[i * LD + j] = i == k ? a : v;
+    const cx<double> r = s.recip;
+    if (t < n) {  // the pivot row scaled
+      const cx<double> x = A[p * LD + t];
+      const cx<double> y = mk<double>(__fma_rn(x.re, r.re, -__dmul_rn(x.im, r.im)), __fma_rn(x.re, r.im, __dmul_rn(x.im, r.re)));
+      s.rowk[t] = t == k ? r : y;
+    }
+    __syncthreads();
+    // rows k and p interchanged: row i of the update comes from row src
+    auto src = [&](int i) { return i == p ? k : i; };
+    const int c1 = k + 1;
+    if (t < 32) {
+      if (c1 < n) {
+        if (t < n) B[t * LD + c1] = t == k ? s.rowk[c1] : upd(A[src(t) * LD + c1], A[src(t) * LD + k], s.rowk[c1]);
+        __syncwarp();
+        pivot(B, c1);
+      }
+    } else {
+      for (int idx = t - 32; idx < n * n; idx += kUpd) {
+        const int i = fd.div(idx), j = idx - i * n;
+        if (j != k && j != c1) B[i * LD + j] = i == k ? s.rowk[j] : upd(A[src(i) * LD + j], A[src(i) * LD + k], s.rowk[j]);
+      }
+      if (t >= kUpd) {
+        const int i = t - kUpd;
+        if (i < n) B[i * LD + k] = i == k ? s.rowk[k] : upd_col(A[src(i) * LD + k], s.rowk[k]);
+      }
     }
     __syncthreads();
     cx<double>* x = A;

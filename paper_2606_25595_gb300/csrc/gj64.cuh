@@ -1,6 +1,6 @@
 // Pivot search and reciprocal of the FP64 Gauss-Jordan eliminations (leaf64.cu, decim.cu).  GB300's FP64
-// pipe takes 64 cycles for a warp's instruction whatever its lanes do (measured), a division 520, so one
-// warp searches with integer compares and forms the reciprocal for its CTA, in two divisions.
+// pipe takes 64 cycles for a warp's instruction whatever its lanes do (measured), so one warp searches
+// with integer compares and forms the reciprocal for its CTA, in two divisions (520 cycles each).
 #pragma once
 #include "common.cuh"
 
@@ -17,8 +17,8 @@ struct FastDiv {
 
 // |re| + |im| as an integer that orders like it (NaN below everything)
 __device__ __forceinline__ unsigned long long pivot_key(cx<double> a) {
-  const double v = cabs1(a);
-  return v == v ? (unsigned long long)__double_as_longlong(v) : 0ull;
+  const unsigned long long v = (unsigned long long)__double_as_longlong(cabs1(a));
+  return v <= 0x7ff0000000000000ull ? v : 0ull;
 }
 // largest key over the warp's lanes
 __device__ __forceinline__ unsigned long long warp_max(unsigned long long key) {
@@ -31,7 +31,7 @@ __device__ __forceinline__ unsigned long long warp_max(unsigned long long key) {
 // two lanes.  Called by a whole warp with the same a.
 __device__ __forceinline__ cx<double> crecip_warp(cx<double> a) {
   const int lane = threadIdx.x & 31;
-  const bool tall = fabs(a.re) >= fabs(a.im);
+  const bool tall = ((unsigned long long)__double_as_longlong(a.re) << 1) >= ((unsigned long long)__double_as_longlong(a.im) << 1);
   const double p = tall ? a.im : a.re, q = tall ? a.re : a.im;
   const double r = p / q, d = __fma_rn(p, r, q);
   const double num = tall ? (lane ? -r : 1.0) : (lane ? -1.0 : r);

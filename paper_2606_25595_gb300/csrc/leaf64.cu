@@ -6,7 +6,8 @@
 // chain of about 1,700 cycles for the pivot, its reciprocal and the scaled row.  Holding the rows in the
 // registers of fixed warps and letting every warp form its own candidate's reciprocal took 640 us for a
 // 48 x 48 block: eight reciprocals a step share the pipe, and lanes beyond n work on zeros.  Here one warp
-// forms them and the threads share the n^2 entries evenly.  The order of every rounding is that of the
+// forms them, and the threads share the n^2 entries evenly (in registers, with a copy in shared memory for
+// the pivot search and the factors).  The order of every rounding is that of the
 // FP32 kernel's source and is written out.
 #include "gj64.cuh"
 #include "kernels.cuh"
@@ -15,31 +16,35 @@ namespace qtx {
 
 namespace {
 
-constexpr int kT = 256;
+constexpr int kT = 512;
 
 // LARGE: blocks above 32, whose pivot row's imaginary parts round the other product first
 template <bool LARGE>
 __global__ void __launch_bounds__(kT) k_leaf_fp64(cx<double>* Ag, long lda, long sA, const gj::FastDiv fd, const int* active,
                                                   int* status) {
+  constexpr int NMAX = LARGE ? 64 : 32, PER = NMAX * NMAX / kT;
   const int e = blockIdx.x;
   if (active && !active[e]) return;
   extern __shared__ __align__(16) unsigned char dsm[];
-  __shared__ cx<double> rowk[kLeafMax];
-  __shared__ int s_step[kLeafMax], s_piv[kLeafMax], s_p;
+  __shared__ cx<double> rowk[NMAX];
+  __shared__ int s_step[NMAX], s_piv[NMAX], s_p;
   const int n = fd.n, LD = n | 1, t = threadIdx.x;
   cx<double>* A = reinterpret_cast<cx<double>*>(dsm);
   cx<double>* B = A + n * LD;
   cx<double>* G = Ag + (long)e * sA;
-  for (int idx = t; idx < n * n; idx += kT) {
-    const int i = fd.div(idx), j = idx - i * n;
-    A[i * LD + j] = G[(long)i * lda + j];
+  cx<double> x[PER];  // this thread's entries idx = t + kT m
+#pragma unroll
+  for (int m = 0; m < PER; ++m) {
+    const int idx = t + kT * m, i = fd.div(idx), j = idx - i * n;
+    if (idx < n * n) A[i * LD + j] = x[m] = G[(long)i * lda + j];
   }
   __syncthreads();
   unsigned long long used = 0;
   for (int k = 0; k < n; ++k) {
     if (t < 32) {
       const unsigned long long k0 = (t < n && !((used >> t) & 1)) ? gj::pivot_key(A[t * LD + k]) : 0ull;
-      const unsigned long long k1 = (t + 32 < n && !((used >> (t + 32)) & 1)) ? gj::pivot_key(A[(t + 32) * LD + k]) : 0ull;
+      unsigned long long k1 = 0;
+      if (LARGE) k1 = (t + 32 < n && !((used >> (t + 32)) & 1)) ? gj::pivot_key(A[(t + 32) * LD + k]) : 0ull;
       const unsigned long long best = gj::warp_max(k0 > k1 ? k0 : k1);
       const unsigned b0 = __ballot_sync(0xffffffffu, k0 == best), b1 = __ballot_sync(0xffffffffu, k1 == best);
       const bool ok = best != 0 && best < 0x7ff0000000000000ull;
@@ -47,10 +52,12 @@ __global__ void __launch_bounds__(kT) k_leaf_fp64(cx<double>* Ag, long lda, long
       if (t == 0) s_p = p;
       if (ok) {
         const cx<double> r = gj::crecip_warp(A[p * LD + k]);
-        for (int j = t; j < n; j += 32) {
-          const cx<double> x = A[p * LD + j];
-          const double im = LARGE ? __fma_rn(x.re, r.im, __dmul_rn(x.im, r.re)) : __fma_rn(x.im, r.re, __dmul_rn(x.re, r.im));
-          rowk[j] = j == k ? r : mk<double>(__fma_rn(x.re, r.re, -__dmul_rn(x.im, r.im)), im);
+#pragma unroll
+        for (int j = t; j < NMAX; j += 32) {
+          if (j >= n) break;
+          const cx<double> y = A[p * LD + j];
+          const double im = LARGE ? __fma_rn(y.re, r.im, __dmul_rn(y.im, r.re)) : __fma_rn(y.im, r.re, __dmul_rn(y.re, r.im));
+          rowk[j] = j == k ? r : mk<double>(__fma_rn(y.re, r.re, -__dmul_rn(y.im, r.im)), im);
         }
         if (t == 0) {
           s_step[p] = k;
@@ -65,25 +72,46 @@ __global__ void __launch_bounds__(kT) k_leaf_fp64(cx<double>* Ag, long lda, long
       return;
     }
     used |= 1ull << p;
-    for (int idx = t; idx < n * n; idx += kT) {
-      const int i = fd.div(idx), j = idx - i * n;
-      const bool kc = j == k;  // pivot column: -(f r), rounded as a product; elsewhere x - f a by four FMAs
-      const cx<double> f = A[i * LD + k], a = rowk[j], x = A[i * LD + j];
-      const double re1 = __fma_rn(kc ? f.im : -f.re, kc ? a.im : a.re, kc ? -0.0 : x.re);
-      const double re2 = __fma_rn(kc ? f.re : f.im, kc ? a.re : a.im, kc ? -re1 : re1);
-      const double im1 = __fma_rn(kc ? f.im : -f.re, kc ? a.re : a.im, kc ? -0.0 : x.im);
-      const double im2 = __fma_rn(kc ? f.re : -f.im, kc ? a.im : a.re, im1);
-      const cx<double> v = mk<double>(kc ? -re2 : re2, kc ? -im2 : im2);
-      B[i * LD + j] = i == p ? a : v;
+    // the pivot column -(f r), by the last warps
+    cx<double> col = mk<double>(0.0, 0.0);
+    const int ci = t - (kT - NMAX);
+    if (ci >= 0 && ci < n) {
+      const cx<double> f = A[ci * LD + k], r = rowk[k];
+      col = mk<double>(-__fma_rn(f.re, r.re, -__dmul_rn(f.im, r.im)), -__fma_rn(f.re, r.im, __dmul_rn(f.im, r.re)));
     }
+#pragma unroll
+    for (int m = 0; m < PER; ++m) {
+      const int idx = t + kT * m;
+      if (idx - t >= n * n) break;  // uniform: whole rounds only
+      if (idx < n * n) {
+        const int i = fd.div(idx), j = idx - i * n;
+        const cx<double> f = A[i * LD + k], a = rowk[j];
+        cx<double> v = x[m];
+        v.re = __fma_rn(-f.re, a.re, v.re);
+        v.re = __fma_rn(f.im, a.im, v.re);
+        v.im = __fma_rn(-f.re, a.im, v.im);
+        v.im = __fma_rn(-f.im, a.re, v.im);
+        x[m] = i == p ? a : v;
+        if (j != k) B[i * LD + j] = x[m];
+      }
+    }
+    if (ci >= 0 && ci < n) B[ci * LD + k] = ci == p ? rowk[k] : col;
     __syncthreads();
+    // the column's owners take it back
+#pragma unroll
+    for (int m = 0; m < PER; ++m) {
+      const int idx = t + kT * m;
+      if (idx - t >= n * n) break;
+      if (idx < n * n && idx - fd.div(idx) * n == k) x[m] = B[fd.div(idx) * LD + k];
+    }
     cx<double>* q = A;
     A = B;
     B = q;
   }
-  for (int idx = t; idx < n * n; idx += kT) {
-    const int i = fd.div(idx), j = idx - i * n;
-    G[(long)s_step[i] * lda + s_piv[j]] = A[i * LD + j];
+#pragma unroll
+  for (int m = 0; m < PER; ++m) {
+    const int idx = t + kT * m, i = fd.div(idx), j = idx - i * n;
+    if (idx < n * n) G[(long)s_step[i] * lda + s_piv[j]] = x[m];
   }
 }
 
