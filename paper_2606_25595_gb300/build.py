@@ -16,7 +16,7 @@ SRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libqtx_rgf.so")
 SOURCES = ["simt.cu", "rgf.cu", "tc_engine.cu", "tc_fp64.cu", "noalloc.cu", "fpx.cu", "decim.cu",
-           "small.cu", "leaf64.cu"]
+           "small.cu", "leaf64.cu", "lesser.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-Xptxas", "-warn-spills"]

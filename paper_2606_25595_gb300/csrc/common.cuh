@@ -220,8 +220,7 @@ struct TcArgs {
   double alpha, beta;          // applied in df32 (split into hi + lo FP32 parts by the launcher)
   int batch;
   const int* active;
-  TcOperand* opndA = nullptr;  // optional kept / reused digit planes of op(A), op(B)
-  TcOperand* opndB = nullptr;
+  TcOperand* opndA = nullptr;  // optional kept / reused digit planes of op(A)
   bool f32 = false;            // A, B, C0, C point to cx<float> arrays (four digit planes only)
   int stages = 0;              // schedule: pipeline stages of the product kernel (0 = the variant's
                                // default; only sizes its shared memory allows are taken)

@@ -102,12 +102,17 @@ cudaError_t assemble_offdiag(cx<T>* U, cx<T>* V, const cx<double>* Hup, const cx
                              const cx<double>* SRu = nullptr, const cx<double>* SRl = nullptr, long sSR = 0);
 
 // ---- observables, FP64 accumulation
-// cur[e * ldcur] = 2 Re Tr[(H_up - E S_up) G^<_{i+1,i}],  G^<_{i+1,i} = -(GLu)^H.  With a device
-// scratch of scratch_doubles doubles, one energy's trace may be split over several CTAs.
+// The backward sweep's elementwise passes (lesser.cu).  lesser_offdiag: GLu = X2^H - PGL (GLu may be null),
+// X2 <- X2 - PGL^H / 2, and, with Hup given, the partial sums of Re Tr[(Hup - E Sup) GLu^H] into `scratch`.
+// lesser_diag: gl <- gl + X - X^H, out64 (may be null; batch stride so) a complex128 copy, den[e * ldden] = Im Tr gl,
+// and cur[e * ldcur] = -2 times lesser_offdiag's sums (cur may be null).  scratch: lesser_scratch_bytes.
+size_t lesser_scratch_bytes(int b, int batch);
 template <typename T>
-cudaError_t obs_current(double* cur, long ldcur, const cx<double>* Hup, const cx<double>* Sup,
-                        const cx<T>* GLu, long sG, const double* E, int b, int batch,
-                        cudaStream_t st, double* scratch = nullptr, long scratch_doubles = 0);
+cudaError_t lesser_offdiag(const cx<T>* PGL, cx<T>* X2, cx<T>* GLu, const cx<double>* Hup, const cx<double>* Sup,
+                           const double* E, int b, int batch, void* scratch, cudaStream_t st);
+template <typename T>
+cudaError_t lesser_diag(cx<T>* gl, const cx<T>* X, cx<double>* out64, long so, double* cur, long ldcur, double* den,
+                        long ldden, int b, int batch, void* scratch, cudaStream_t st);
 // den[e * ldden] = Im Tr GL[e]
 template <typename T>
 cudaError_t obs_density(double* den, long ldden, const cx<T>* GL, long sG, int b, int batch,
@@ -236,10 +241,10 @@ cudaError_t gemm_tc_launch(const TcPrepared* const* p, int n, cudaStream_t st, c
 // digit products (pairs i + j <= digits + 1) the engine issues per real product
 inline int tc_pairs(int digits) { return digits * (digits + 1) / 2; }
 size_t gemm_tc_scratch_bytes(int M, int N, int K, int batch, int digits);
-// Bytes of a TcOperand for op(A) (side 0, R = M rows) or op(B) (side 1, R = N columns) of K; 0 when
-// the product would be split along K (operands cannot be kept then).  tc_operand_at carves one.
-size_t gemm_tc_operand_bytes(int side, int R, int K, int batch, int digits);
-TcOperand tc_operand_at(void* base, int side, int R, int K, int batch, int digits);
+// Bytes of a TcOperand for op(A) (R = M rows) of K; 0 when the product would be split along K (operands
+// cannot be kept then).  tc_operand_at carves one.
+size_t gemm_tc_operand_bytes(int R, int K, int batch, int digits);
+TcOperand tc_operand_at(void* base, int R, int K, int batch, int digits);
 bool tc_available();
 int wait_test();  // 1 while the bounded-wait test (qtx_tc_wait_test) is switched on
 

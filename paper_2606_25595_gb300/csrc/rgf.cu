@@ -54,7 +54,7 @@ inline bool uv_per_energy(const qtx_rgf_desc& d) {
 }
 
 struct Layout {
-  size_t g, gl, gl2, zk, xk, gfx, glfx, fx_slot, sig_stage, opnd[3], opnd_bytes[3], refine_act, tmp, inv_tmp, U, V, ident, ident_df, shared_blk, ref, f32a, f32tmp, dec, lead, obs, flags, dscale, bal, bscale, bgn, bhn, cres, cflag,
+  size_t g, gl, gl2, zk, xk, gfx, glfx, fx_slot, sig_stage, opnd[2], opnd_bytes[2], refine_act, tmp, inv_tmp, U, V, ident, ident_df, shared_blk, ref, f32a, f32tmp, dec, lead, obs, flags, dscale, bal, bscale, bgn, bhn, cres, cflag,
       tc_scratch, total;
   int n_tmp, n_dec;
   size_t tc_bytes;
@@ -173,10 +173,10 @@ Layout make_layout(const qtx_rgf_desc& d) {
   if (d.precision == QTX_FP32 && b >= 96 && b <= 1024) L.tc_bytes = gemm_tc_scratch_bytes((int)b, (int)b, (int)b, (int)Ec, 4);
   if (tc64) L.tc_bytes = gemm_fp64_tc_scratch_bytes((int)b, (int)b, (int)b, (int)Ec);
   L.tc_scratch = a.take(L.tc_bytes);
-  // kept digitised operands (emulated modes): two left operands and one right operand, b x b, E_c
-  // energies (none when the products are split along K)
-  for (int k = 0; k < 3; ++k) {
-    L.opnd_bytes[k] = mixed ? gemm_tc_operand_bytes(k < 2 ? 0 : 1, (int)b, (int)b, (int)Ec, d.precision == QTX_EMU64 ? 6 : 2) : 0;
+  // kept digitised operands (emulated modes): two left operands, b x b, E_c energies (none when the
+  // products are split along K)
+  for (int k = 0; k < 2; ++k) {
+    L.opnd_bytes[k] = mixed ? gemm_tc_operand_bytes((int)b, (int)b, (int)Ec, d.precision == QTX_EMU64 ? 6 : 2) : 0;
     L.opnd[k] = a.take(L.opnd_bytes[k]);
   }
   L.total = a.off;
@@ -238,17 +238,16 @@ GemmArgs<T> gargs(int M, int N, int K, const cx<T>* A, long lda, long sA, int op
 }
 
 // GEMM dispatch by the plan's precision (FP32 and FP64: SIMT; EMU64 / BF16X3: tensor-core engine).
-// Which kept digitised operands (tensor-core modes) a product uses: slot 0, 1 (left operands) or
-// 2 (right operand), mode KEEP (digitise into the slot) or REUSE (take the slot's planes: the operand,
-// its op and its shape are unchanged since the KEEP product).  Ignored by the SIMT modes.
+// Which kept digitised left operand (tensor-core modes) a product uses: slot 0 or 1, mode KEEP (digitise into
+// the slot) or REUSE (take the slot's planes: the operand, its op and its shape are unchanged since the KEEP
+// product).  Ignored by the other modes.
 enum { DG_NONE = 0, DG_KEEP = 1, DG_REUSE = 2 };
 struct DigitHint {
-  int a_slot = -1, a_mode = DG_NONE, b_slot = -1, b_mode = DG_NONE;
+  int a_slot = -1, a_mode = DG_NONE;
   int digits = 0;  // digit planes of a tensor-core product (0: the plan's)
 };
 inline DigitHint keepA(int slot) { DigitHint h; h.a_slot = slot; h.a_mode = DG_KEEP; return h; }
 inline DigitHint reuseA(int slot) { DigitHint h; h.a_slot = slot; h.a_mode = DG_REUSE; return h; }
-inline DigitHint keepB(int slot) { DigitHint h; h.b_slot = slot; h.b_mode = DG_KEEP; return h; }
 inline DigitHint planes(int digits) { DigitHint h; h.digits = digits; return h; }
 
 template <typename T>
@@ -332,17 +331,12 @@ qtx_status gemm<df>(qtx_rgf_plan_s* P, const GemmArgs<df>& g, cudaStream_t st, b
   TcArgs a;
   const int digits = hint.digits > 0 ? hint.digits : tc_digits(P->d);
   // kept operands: only for the plan's b x b x b products at the plan's digit count, when slots exist
-  TcOperand oa, ob;
+  TcOperand oa;
   const bool square = g.M == P->b && g.N == P->b && g.K == P->b && g.batch <= P->Ec && digits == tc_digits(P->d);
   if (square && hint.a_mode != DG_NONE && P->L.opnd_bytes[hint.a_slot]) {
-    oa = tc_operand_at(P->ws + P->L.opnd[hint.a_slot], 0, P->b, P->b, P->Ec, tc_digits(P->d));
+    oa = tc_operand_at(P->ws + P->L.opnd[hint.a_slot], P->b, P->b, P->Ec, tc_digits(P->d));
     oa.mode = hint.a_mode;
     a.opndA = &oa;
-  }
-  if (square && hint.b_mode != DG_NONE && P->L.opnd_bytes[hint.b_slot]) {
-    ob = tc_operand_at(P->ws + P->L.opnd[hint.b_slot], 1, P->b, P->b, P->Ec, tc_digits(P->d));
-    ob.mode = hint.b_mode;
-    a.opndB = &ob;
   }
   a.M = g.M; a.N = g.N; a.K = g.K;
   a.A = g.A; a.lda = g.lda; a.sA = g.sA; a.opA = g.opA;
@@ -947,15 +941,19 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
 
   // ---- 3. backward sweep.  With P = g_i U_i, Z = V_i g_i, Q = V_i g^<_i:
   //   G_{i+1,i} = -G_{i+1,i+1} Z,  G_{i,i+1} = -P G_{i+1,i+1},  G_ii = g_i - P G_{i+1,i}
-  //   K = P G_{i+1,i+1} Q = -G_{i,i+1} Q   (block-tridiagonal Sigma^<: Q += (g_i Sigma^<_{i,i+1})^H)
-  //   G^<_ii = g^<_i + (P G^<_{i+1,i+1}) P^H + K - K^H
-  //   G^<_{i,i+1} = -P G^<_{i+1,i+1} + (G_{i+1,i+1} Q)^H     [= -P G^< - g^< V^H G^A]
+  //   X2 = G_{i+1,i+1} Q   (block-tridiagonal Sigma^<: Q += (g_i Sigma^<_{i,i+1})^H)
+  //   G^<_{i,i+1} = -P G^<_{i+1,i+1} + X2^H     [= -P G^< - g^< V^H G^A]
+  //   G^<_ii = g^<_i + T - T^H,  T = P (X2 - (P G^<_{i+1,i+1})^H / 2)
+  // The last line is g^<_i + P G^<_{i+1,i+1} P^H + P X2 - (P X2)^H with G^<_{i+1,i+1} anti-Hermitian: its
+  // congruence is (Y - Y^H) / 2 with Y = -P (P G^<)^H, so one product P (..) serves both terms: 12 products a
+  // slice (13 with G_{i,i+1}) instead of 14, and the current's error against 64 bits falls to a third.
   const ObsBufs ob(P);
   const int ncur = ob.ncur;
   double *cur = ob.cur, *den = ob.den, *con = ob.con, *tra = ob.tra;
   // current conservation (Sec. II-B): per-slice balances J_i, checked after the sweep
   const bool cont = wants_balance(d);
   double *bal = ob.bal, *bscale = ob.bscale, *bgn = ob.bgn, *bhn = ob.bhn;
+  double* spare = tra;  // the second right-hand side's traces, which nothing reads (no contacts then)
   {
     const int i = nb - 1;
     if (want(QTX_OUT_GR_DIAG, out->GR_diag) && (s = emit<T>(P, out->GR_diag, nb, i, e0, c.g(i), b, ne, st))) return s;
@@ -984,7 +982,7 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
     cx<T>* GRl = c.tmp(4);
     cx<T>* GRu = c.tmp(5);
     cx<T>* Qw = c.tmp(6);
-    cx<T>* K = c.tmp(7);
+    cx<T>* Tm = c.tmp(7);
     cx<T>* PGL = c.tmp(8);
     cx<T>* X2 = c.tmp(9);
     cx<T>* GLu = c.tmp(10);
@@ -997,10 +995,8 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
                   DigitHint h = DigitHint{}) {
       return gemm<T>(P, gargs<T>(b, b, b, A, b, sA_, opA, B, b, sB_, opB, C0, b, bb, C, b, bb, al, be, ne, nullptr), st, false, h);
     };
-    // kept digit planes (tensor-core modes): slot 0 = P (left operand of three products), slot 1 =
-    // G_{i+1,i+1} (left operand of two), slot 2 = Q (right operand of two)
-    DigitHint x2;
-    x2.a_slot = 1; x2.a_mode = DG_REUSE; x2.b_slot = 2; x2.b_mode = DG_REUSE;
+    // kept digit planes (tensor-core modes): slot 0 = P (left operand of three or four products), slot 1 =
+    // G_{i+1,i+1} (left operand of two)
     if ((s = MM(gi, bb, OP_N, U(i), sUV, OP_N, nullptr, Pm, 1.0, 0.0))) return s;
     if (!c.keep_z() && (s = MM(V(i), sUV, OP_N, gi, bb, OP_N, nullptr, Z, 1.0, 0.0))) return s;
     // block-tridiagonal right-hand side k: g_i L_k with L_k its upper block (g_i still left-connected)
@@ -1013,8 +1009,10 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
       }
     }
     if ((s = MM(GRn, bb, OP_N, Z, bb, OP_N, nullptr, GRl, -1.0, 0.0, keepA(1)))) return s;
-    if ((s = MM(Pm, bb, OP_N, GRn, bb, OP_N, nullptr, GRu, -1.0, 0.0, keepA(0)))) return s;
-    if ((s = MM(Pm, bb, OP_N, GRl, bb, OP_N, gi, gi, -1.0, 1.0, reuseA(0)))) return s;   // g_i <- G_ii
+    // G_{i,i+1} only where it is an output (itself, or in G^>_{i,i+1}) or the balance check's K needs it
+    const bool want_u = want(QTX_OUT_GR_UPPER, out->GR_upper) || (!d.second_rhs && want(QTX_OUT_GG_UPPER, out->GG_upper)) || cont;
+    if (want_u && (s = MM(Pm, bb, OP_N, GRn, bb, OP_N, nullptr, GRu, -1.0, 0.0, keepA(0)))) return s;
+    if ((s = MM(Pm, bb, OP_N, GRl, bb, OP_N, gi, gi, -1.0, 1.0, want_u ? reuseA(0) : keepA(0)))) return s;   // g_i <- G_ii
     if (want(QTX_OUT_GR_DIAG, out->GR_diag) && (s = emit<T>(P, out->GR_diag, nb, i, e0, gi, b, ne, st))) return s;
     if (want(QTX_OUT_GR_UPPER, out->GR_upper) && (s = emit<T>(P, out->GR_upper, nb - 1, i, e0, GRu, b, ne, st))) return s;
     if (want(QTX_OUT_GR_LOWER, out->GR_lower) && (s = emit<T>(P, out->GR_lower, nb - 1, i, e0, GRl, b, ne, st))) return s;
@@ -1030,34 +1028,37 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
         Term<T> t1; t1.p = Rl(k); t1.s = bb; t1.alpha = 1.0; t1.op = OP_C;
         QTX_CK((combine<T, T>(Q, bb, t0, t1, none, b, ne, nullptr, 0, 0, nullptr, st)));
       }
-      if ((s = MM(GRu, bb, OP_N, Q, bb, OP_N, nullptr, K, -1.0, 0.0, keepB(2)))) return s;
+      if ((s = MM(GRn, bb, OP_N, Q, bb, OP_N, nullptr, X2, 1.0, 0.0, reuseA(1)))) return s;
       if ((s = MM(Pm, bb, OP_N, GLn, bb, OP_N, nullptr, PGL, 1.0, 0.0, reuseA(0)))) return s;
-      if ((s = MM(PGL, bb, OP_N, Pm, bb, OP_C, gli, gli, 1.0, 1.0))) return s;   // g^<_i + PGL P^H
-      if ((s = MM(GRn, bb, OP_N, Q, bb, OP_N, nullptr, X2, 1.0, 0.0, x2))) return s;
-      {
-        Term<T> t0; t0.p = gli; t0.s = bb; t0.alpha = 1.0;
-        Term<T> t1; t1.p = K; t1.s = bb; t1.alpha = 1.0;
-        Term<T> t2; t2.p = K; t2.s = bb; t2.alpha = -1.0; t2.op = OP_C;
-        QTX_CK((combine<T, T>(gli, bb, t0, t1, t2, b, ne, nullptr, 0, 0, nullptr, st)));   // G^<_ii
-        Term<T> u0; u0.p = PGL; u0.s = bb; u0.alpha = -1.0;
-        Term<T> u1; u1.p = X2; u1.s = bb; u1.alpha = 1.0; u1.op = OP_C;
-        QTX_CK((combine<T, T>(GLu, bb, u0, u1, none, b, ne, nullptr, 0, 0, nullptr, st)));  // G^<_{i,i+1}
+      // G^<_{i,i+1} is written where an output or the balance reads it; its current trace comes with it
+      const bool up_k = k ? want(QTX_OUT_GG_UPPER, out->GG_upper)
+                          : want(QTX_OUT_GL_UPPER, out->GL_upper) || (!d.second_rhs && want(QTX_OUT_GG_UPPER, out->GG_upper)) || cont;
+      const bool cur_k = k == 0 && !d.system_input;
+      void* traces = c.tmp(0);  // (tmp 0 and 1: lesser_scratch_bytes exceeds one block for b = 1)
+      QTX_CK(lesser_offdiag<T>(PGL, X2, up_k ? GLu : nullptr, cur_k ? Hu + (long)i * bb : nullptr,
+                               cur_k && Su ? Su + (long)i * bb : nullptr, c.E, b, ne, traces, st));
+      if (cont) {
+        // plans that check the current balance form K and the congruence apart: T - T^H is anti-Hermitian
+        // whatever the rounding, so the balance would no longer see the part of it that the check measures
+        if ((s = MM(GRu, bb, OP_N, Q, bb, OP_N, nullptr, Tm, -1.0, 0.0))) return s;
+        if ((s = MM(PGL, bb, OP_N, Pm, bb, OP_C, gli, gli, 1.0, 1.0))) return s;
+      } else if ((s = MM(Pm, bb, OP_N, X2, bb, OP_N, nullptr, Tm, 1.0, 0.0, reuseA(0)))) {
+        return s;
       }
+      const long o64 = ((long)e0 * nb + i) * bb;
+      void* gd = k ? (want(QTX_OUT_GG_DIAG, out->GG_diag) ? out->GG_diag : nullptr)
+                   : (want(QTX_OUT_GL_DIAG, out->GL_diag) ? out->GL_diag : nullptr);
+      QTX_CK(lesser_diag<T>(gli, Tm, gd ? reinterpret_cast<cx<double>*>(gd) + o64 : nullptr, (long)nb * bb,
+                            cur_k ? cur + i : nullptr, ncur, k ? spare : den + i, k ? 1 : nb, b, ne, traces, st));   // G^<_ii
       if (k == 1) {  // the second right-hand side's blocks are the GG outputs
-        if (want(QTX_OUT_GG_DIAG, out->GG_diag) && (s = emit<T>(P, out->GG_diag, nb, i, e0, gli, b, ne, st))) return s;
-        if (want(QTX_OUT_GG_UPPER, out->GG_upper) && (s = emit<T>(P, out->GG_upper, nb - 1, i, e0, GLu, b, ne, st))) return s;
+        if (up_k && (s = emit<T>(P, out->GG_upper, nb - 1, i, e0, GLu, b, ne, st))) return s;
         continue;
       }
-      if (want(QTX_OUT_GL_DIAG, out->GL_diag) && (s = emit<T>(P, out->GL_diag, nb, i, e0, gli, b, ne, st))) return s;
       if (want(QTX_OUT_GL_UPPER, out->GL_upper) && (s = emit<T>(P, out->GL_upper, nb - 1, i, e0, GLu, b, ne, st))) return s;
       if (!d.second_rhs) {
         if (want(QTX_OUT_GG_DIAG, out->GG_diag) && (s = emit<T>(P, out->GG_diag, nb, i, e0, gli, b, ne, st, gi, gi))) return s;
         if (want(QTX_OUT_GG_UPPER, out->GG_upper) && (s = emit<T>(P, out->GG_upper, nb - 1, i, e0, GLu, b, ne, st, GRu, GRl))) return s;
       }
-      if (!d.system_input)
-        QTX_CK(obs_current<T>(cur + i, ncur, Hu + (long)i * bb, Su ? Su + (long)i * bb : nullptr, GLu, bb, c.E, b, ne, st,
-                              reinterpret_cast<double*>(c.tmp(0)), (long)ne * bb * (long)sizeof(cx<T>) / (long)sizeof(double)));
-      QTX_CK(obs_density<T>(den + i, nb, gli, bb, b, ne, st));
       if (cont)
         QTX_CK(obs_balance<T>(bal + i, bscale + i, bgn + i, bhn + i, nb, sigL(i), sigR(i), sSig, gi, gli, bb, eta, b,
                               ne, st, Hd + (long)i * bb, Hu + (long)i * bb, Su ? Su + (long)i * bb : nullptr, c.E, GLu));

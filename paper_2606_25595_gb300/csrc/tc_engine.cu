@@ -679,16 +679,15 @@ cudaError_t prepare(const TcArgs& a, void* scratch, size_t scratch_bytes, int* e
   if (sc.bytes > scratch_bytes) return cudaErrorInvalidValue;
   cudaError_t e;
   const int ab = a.sA != 0, bb_ = a.sB != 0;
-  // digit planes and exponents of each operand: in the scratch, or in a kept operand (digitised
-  // there now, or reused as they are)
+  // digit planes and exponents of each operand: in the scratch, or (left operand) in a kept operand,
+  // digitised there now or reused as they are
   unsigned char* pa = a.opndA ? a.opndA->planes : sc.pa;
-  unsigned char* pb = a.opndB ? a.opndB->planes : sc.pb;
+  unsigned char* pb = sc.pb;
   int* ea = a.opndA ? a.opndA->expo : sc.ea;
-  int* eb = a.opndB ? a.opndB->expo : sc.eb;
+  int* eb = sc.eb;
   if (!(a.opndA && a.opndA->mode == 2))
     if ((e = digitize<S, IO>(A, a.lda, a.sA, a.opA, 0, a.M, a.K, d, ea, pa, ab ? a.batch : 1, ab ? a.active : nullptr, st))) return e;
-  if (!(a.opndB && a.opndB->mode == 2))
-    if ((e = digitize<S, IO>(B, a.ldb, a.sB, a.opB, 1, a.N, a.K, d, eb, pb, bb_ ? a.batch : 1, bb_ ? a.active : nullptr, st))) return e;
+  if ((e = digitize<S, IO>(B, a.ldb, a.sB, a.opB, 1, a.N, a.K, d, eb, pb, bb_ ? a.batch : 1, bb_ ? a.active : nullptr, st))) return e;
   p.pa = pa;
   p.pb = pb;
   p.eA = ea;
@@ -799,25 +798,19 @@ size_t gemm_tc_scratch_bytes(int M, int N, int K, int batch, int digits) {
 }
 
 static size_t al1k(size_t x) { return (x + 1023) & ~size_t(1023); }
-// digit-plane bytes of one operand (as carve lays them out)
-static size_t plane_bytes_of(int side, const tc::Dims& d, int batch, int S) {
-  return side == 0 ? (size_t)batch * S * d.M_pad * 2 * d.K_pad * 2
-                   : (size_t)batch * S * (d.N_pad / tc::bnc_of(S)) * (d.K_pad / tc::BKS) * 3 * tc::sub_b_of(S);
-}
-
-size_t gemm_tc_operand_bytes(int side, int R, int K, int batch, int digits) {
+size_t gemm_tc_operand_bytes(int R, int K, int batch, int digits) {
   if (k_chunks(K) > 1) return 0;
   const int S = effective_digits(digits, K);
-  const tc::Dims d = side == 0 ? tc::dims_of(R, 1, K, S) : tc::dims_of(1, R, K, S);
-  return al1k(plane_bytes_of(side, d, batch, S)) + al1k((size_t)batch * (side == 0 ? d.M_pad : d.N_pad) * sizeof(int));
+  const tc::Dims d = tc::dims_of(R, 1, K, S);
+  return al1k((size_t)batch * S * d.M_pad * 2 * d.K_pad * 2) + al1k((size_t)batch * d.M_pad * sizeof(int));
 }
 
-TcOperand tc_operand_at(void* base, int side, int R, int K, int batch, int digits) {
+TcOperand tc_operand_at(void* base, int R, int K, int batch, int digits) {
   const int S = effective_digits(digits, K);
-  const tc::Dims d = side == 0 ? tc::dims_of(R, 1, K, S) : tc::dims_of(1, R, K, S);
+  const tc::Dims d = tc::dims_of(R, 1, K, S);
   TcOperand o;
   o.planes = reinterpret_cast<unsigned char*>(base);
-  o.expo = reinterpret_cast<int*>(o.planes + al1k(plane_bytes_of(side, d, batch, S)));
+  o.expo = reinterpret_cast<int*>(o.planes + al1k((size_t)batch * S * d.M_pad * 2 * d.K_pad * 2));
   return o;
 }
 
@@ -887,7 +880,7 @@ cudaError_t gemm_tc(const TcArgs& a, int digits, void* scratch, size_t scratch_b
     for (int c = 0; c < nc; ++c) {
       const int k0 = c * Kc, k1 = a.K < k0 + Kc ? a.K : k0 + Kc;
       TcArgs t = a;
-      t.opndA = t.opndB = nullptr;  // kept operands cover whole contractions only
+      t.opndA = nullptr;  // kept operands cover whole contractions only
       t.K = k1 - k0;
       t.A = a.A + (a.opA == OP_N ? (long)k0 : (long)k0 * a.lda);
       t.B = a.B + (a.opB == OP_N ? (long)k0 * a.ldb : (long)k0);
