@@ -191,6 +191,7 @@ struct GemmArgs {
   double alpha, beta;
   int batch;
   const int* active;
+  bool b64 = false;  // T = df: B holds complex128 values (digitised from them directly)
 };
 
 // Up to four products of one shape and batch in a launch.
@@ -210,7 +211,11 @@ struct TcOperand {
   int mode = 0;
 };
 
-// Arguments of the tensor-core engine (complex df32 operands and result).
+// Element types of the tensor-core engine's operands and results.
+enum Elt : int { EL_DF = 0, EL_F32 = 1, EL_F64 = 2 };
+
+// Arguments of the tensor-core engine.  Operand and result pointers are typed as complex df32; ta, tb and tc
+// say what they hold (complex128 values enter and leave as the df32 pairs they round to).
 struct TcArgs {
   int M, N, K;
   const cx<df>* A; long lda, sA; int opA;
@@ -221,7 +226,8 @@ struct TcArgs {
   int batch;
   const int* active;
   TcOperand* opndA = nullptr;  // optional kept / reused digit planes of op(A)
-  bool f32 = false;            // A, B, C0, C point to cx<float> arrays (four digit planes only)
+  Elt ta = EL_DF, tb = EL_DF;  // elements of A, B
+  Elt tc = EL_DF;              // elements of C0 and C (EL_F32: all three, with four digit planes only)
   int stages = 0;              // schedule: pipeline stages of the product kernel (0 = the variant's
                                // default; only sizes its shared memory allows are taken)
   int ctas = 0;                // schedule: persistent CTAs per launch (0 = one per SM)

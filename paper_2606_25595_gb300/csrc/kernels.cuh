@@ -11,6 +11,8 @@ namespace qtx {
 extern std::atomic<long long> g_launches;
 inline void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
+unsigned long long current_ctx_id();  // id of the current CUDA context, 0 if unknown (noalloc.cu)
+
 // Raise a kernel's dynamic shared-memory limit once per device (`done`: the kernel's bit per device).
 template <typename F>
 inline cudaError_t allow_smem(F* kernel, int bytes, std::atomic<unsigned long long>& done) {
@@ -70,6 +72,8 @@ cudaError_t convert_strided(const cx<Tin>* in, long ldi, long si, cx<Tout>* out,
 cudaError_t pivoted_inverse(cx<double>* A, long sA, int n, int batch, const int* active, int* status, int* perm,
                             cudaStream_t st);
 
+// the b x b identity in complex128 and in df32
+cudaError_t set_identity(cx<double>* I, cx<df>* Idf, int b, cudaStream_t st);
 // X[e] += I
 template <typename T>
 cudaError_t add_identity(cx<T>* X, long sX, int n, int batch, const int* active, cudaStream_t st);

@@ -38,15 +38,19 @@ std::mutex g_mu;
 void* g_addr[kMaxDevices] = {};
 unsigned long long g_ctx[kMaxDevices] = {};  // id of the context g_addr[dev] was resolved in
 
+}  // namespace
+
 // Id of the current context (0 if none is current or the driver cannot say).  The two driver
 // functions are looked up through the runtime, so the library has no link-time dependency on the
 // driver library (it still loads on a machine without a GPU driver).
-unsigned long long current_ctx_id() {
+unsigned long long qtx::current_ctx_id() {
   typedef CUresult (*get_current_t)(CUcontext*);
   typedef CUresult (*get_id_t)(CUcontext, unsigned long long*);
   static get_current_t get_current = nullptr;
   static get_id_t get_id = nullptr;
+  static std::mutex lookup;
   static bool looked_up = false;
+  std::lock_guard<std::mutex> lk(lookup);
   if (!looked_up) {
     void* f1 = nullptr;
     void* f2 = nullptr;
@@ -67,6 +71,8 @@ unsigned long long current_ctx_id() {
   if (get_id(c, &id) != CUDA_SUCCESS) return 0;
   return id;
 }
+
+namespace {
 
 size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 

@@ -104,7 +104,8 @@ struct qtx_rgf_plan_s {
 
 namespace {
 
-Layout make_layout(const qtx_rgf_desc& d) {
+// inverse_only: the areas a batched inverse on its own uses (block g, and the refinement's)
+Layout make_layout(const qtx_rgf_desc& d, bool inverse_only = false) {
   Layout L{};
   const long b = d.block_size, nb = d.n_blocks, Ec = d.max_energies_in_flight;
   const size_t bb = (size_t)b * b;
@@ -113,7 +114,7 @@ Layout make_layout(const qtx_rgf_desc& d) {
   const size_t es = (d.precision == QTX_FP32 && !(d.escalate_tol > 0)) ? sizeof(cx<float>) : sizeof(cx<double>);
   Arena a;
   // 12, 13: Sigma^<_{i,i+1} in the sweep's type and g_i Sigma^<_{i,i+1}; 14: g_i B2_{i,i+1} (second_rhs)
-  L.n_tmp = d.offdiag_sigma ? (d.second_rhs ? 15 : 14) : 12;
+  L.n_tmp = inverse_only ? 0 : (d.offdiag_sigma ? (d.second_rhs ? 15 : 14) : 12);
   if (d.storage_bits) {
     // two working blocks per kind in the sweep's type (slices i and i-1 / i+1), every slice's
     // left-connected blocks in FPX: a slot of fx_slot bytes per slice and kind
@@ -124,7 +125,7 @@ Layout make_layout(const qtx_rgf_desc& d) {
     L.glfx = a.take(nb * L.fx_slot);
   } else {
     L.g = a.take(nb * Ec * bb * es);
-    L.gl = a.take(nb * Ec * bb * es);
+    L.gl = a.take(inverse_only ? 0 : nb * Ec * bb * es);
   }
   L.gl2 = a.take(d.second_rhs ? nb * Ec * bb * es : 0);  // left-connected blocks of the second right-hand side
   // Z_i = V_i g_i of every slice but the last, formed in the forward sweep and kept for the
@@ -151,7 +152,7 @@ Layout make_layout(const qtx_rgf_desc& d) {
   L.perm = a.take(L.refine64 && b <= kPivotedMax ? (size_t)Ec * b * sizeof(int) : 0);
   L.n_dec = 10;
   L.dec = a.take(d.leads ? (size_t)L.n_dec * Ec * bb * sizeof(cx<double>) : 0);
-  L.lead = a.take(d.leads ? 8 * Ec * bb * sizeof(cx<double>) : 0);
+  L.lead = a.take(d.leads && !inverse_only ? 8 * Ec * bb * sizeof(cx<double>) : 0);
   // per-energy observables: current, density, contact(2), transmission, scratch(2)
   L.obs = a.take((size_t)Ec * (2 * nb + 8) * sizeof(double));
   L.flags = a.take((size_t)Ec * 3 * sizeof(int) + 64);
@@ -285,7 +286,7 @@ qtx_status gemm<float>(qtx_rgf_plan_s* P, const GemmArgs<float>& g, cudaStream_t
   if (f32_on_tc(P->d) && g.M >= kTcF32Min && g.N >= kTcF32Min && g.K >= kTcF32Min && g.K <= 1024 &&
       gemm_tc_scratch_bytes(g.M, g.N, g.K, g.batch, 4) <= P->L.tc_bytes) {
     TcArgs a;
-    a.f32 = true;
+    a.ta = a.tb = a.tc = EL_F32;
     a.M = g.M; a.N = g.N; a.K = g.K;
     a.A = reinterpret_cast<const cx<df>*>(g.A); a.lda = g.lda; a.sA = g.sA; a.opA = g.opA;
     a.B = reinterpret_cast<const cx<df>*>(g.B); a.ldb = g.ldb; a.sB = g.sB; a.opB = g.opB;
@@ -338,6 +339,7 @@ qtx_status gemm<df>(qtx_rgf_plan_s* P, const GemmArgs<df>& g, cudaStream_t st, b
     oa.mode = hint.a_mode;
     a.opndA = &oa;
   }
+  if (g.b64) a.tb = EL_F64;
   a.M = g.M; a.N = g.N; a.K = g.K;
   a.A = g.A; a.lda = g.lda; a.sA = g.sA; a.opA = g.opA;
   a.B = g.B; a.ldb = g.ldb; a.sB = g.sB; a.opB = g.opB;
@@ -1185,7 +1187,7 @@ qtx_status validate(const qtx_rgf_desc* d, std::string& err) {
 // block products of the BT factors.  Row i of V P is (V P)_ij = sum_k V_ik P_kj over k = i-1..i+1
 // with |k - j| <= 1 (j = i-1..i+1 for M; i-2..i+2 for B, whose blocks B_ij = sum_l (V P)_il
 // (V_jl)^H need l up to j+1).  Each block product is one batched launch over the chunk's energies,
-// V shared (batch stride 0).  Temporaries: 0-4 V blocks, 5 one P block, 6-10 row i of V P, 11 B.
+// V shared (batch stride 0).  Temporaries: 0-4 V blocks, 5 one P block, 6-9 row i of V P, 11 B.
 template <typename T>
 qtx_status w_assemble_chunk(qtx_rgf_plan_s* P, const qtx_w_inputs* in, const qtx_w_outputs* out, int nb,
                             int e0, int ne, cudaStream_t st) {
@@ -1201,7 +1203,7 @@ qtx_status w_assemble_chunk(qtx_rgf_plan_s* P, const qtx_w_inputs* in, const qtx
   // V slots: 0 V_ii, 1 V_{i+1,i+1}, 2 V_{i-1,i}, 3 V_{i,i+1}, 4 V_{i+1,i+2}
   cx<T>* Vt[5] = {c.tmp(0), c.tmp(1), c.tmp(2), c.tmp(3), c.tmp(4)};
   cx<T>* Pt = c.tmp(5);
-  cx<T>* acc[5] = {c.tmp(6), c.tmp(7), c.tmp(8), c.tmp(9), c.tmp(10)};  // (V P)_{i,i-2} .. (V P)_{i,i+2}
+  cx<T>* acc[4] = {c.tmp(6), c.tmp(7), c.tmp(8), c.tmp(9)};  // (V P)_{i,i-1} .. (V P)_{i,i+2}
   cx<T>* Bt = c.tmp(11);
   auto toT = [&](cx<T>* dst, const cx<double>* src, long sSrc, int batch) {
     return axpby_from64<T>(dst, bb, src, sSrc, 1.0, nullptr, 0, 0.0, b, batch, st);
@@ -1210,6 +1212,18 @@ qtx_status w_assemble_chunk(qtx_rgf_plan_s* P, const qtx_w_inputs* in, const qtx
                 bool first) {
     return gemm<T>(P, gargs<T>(b, b, b, A, b, sA, opA, B, b, sB, opB, first ? nullptr : C, b, bb, C, b, bb, al,
                                first ? 0.0 : 1.0, ne, nullptr), st);
+  };
+  // V_k op(P), P complex128 with batch stride sP: digitised as it is (df32 plans), or through Pt
+  auto mmP = [&](const cx<T>* A, int opA, const cx<double>* Pb, long sP, int opB, cx<T>* C, double al, bool first) -> qtx_status {
+    if constexpr (std::is_same<T, float>::value) {
+      QTX_CK(toT(Pt, Pb, sP, ne));
+      return mm(A, 0, opA, Pt, bb, opB, C, al, first);
+    } else {
+      GemmArgs<T> g = gargs<T>(b, b, b, A, b, 0, opA, reinterpret_cast<const cx<T>*>(Pb), b, sP, opB, first ? nullptr : C, b, bb, C,
+                               b, bb, al, first ? 0.0 : 1.0, ne, nullptr);
+      g.b64 = true;
+      return gemm<T>(P, g, st);
+    }
   };
   // out[e][j] = alpha X (+ I), complex128, n blocks per energy
   auto emit64 = [&](void* dst, long n, long j, const cx<T>* X, double alpha, bool ident) -> qtx_status {
@@ -1227,51 +1241,43 @@ qtx_status w_assemble_chunk(qtx_rgf_plan_s* P, const qtx_w_inputs* in, const qtx
     if (i >= 1) QTX_CK(toT(Vt[2], Vu + (long)(i - 1) * bb, 0, 1));
     if (i + 1 < nb) QTX_CK(toT(Vt[3], Vu + (long)i * bb, 0, 1));
     if (i + 2 < nb) QTX_CK(toT(Vt[4], Vu + (long)(i + 1) * bb, 0, 1));
-    // row i of V P for j = i-W .. i+W.  V_ik: k = i-1 -> V_{i-1,i}^H, k = i -> V_ii, k = i+1 -> V_{i,i+1}.
+    // row i of V P for j = i+j0 .. i+j1.  V_ik: k = i-1 -> V_{i-1,i}^H, k = i -> V_ii, k = i+1 -> V_{i,i+1}.
     // P_kj: diagonal, upper (j = k+1), lower (j = k-1): given, or -(P_{j,j+1})^H for anti-Hermitian P.
-    auto row = [&](const void* Pd, const void* Pu, const void* Pl, int W) -> qtx_status {
-      for (int dj = -W; dj <= W; ++dj) {
-        const int j = i + dj;
-        if (j < 0 || j >= nb) continue;
+    auto row = [&](const void* Pd, const void* Pu, const void* Pl, int j0, int j1) -> qtx_status {
+      for (int j = std::max(i + j0, 0); j <= std::min(i + j1, nb - 1); ++j) {
         bool first = true;
         for (int k = i - 1; k <= i + 1; ++k) {
           if (k < 0 || k >= nb || k - j > 1 || j - k > 1) continue;
           const cx<T>* Vk = k == i ? Vt[0] : (k == i + 1 ? Vt[3] : Vt[2]);
           const int opV = k == i - 1 ? OP_C : OP_N;
-          int opP = OP_N;
-          double al = 1.0;
-          if (k == j) QTX_CK(toT(Pt, pe(Pd, nb, k), (long)nb * bb, ne));
-          else if (j == k + 1) QTX_CK(toT(Pt, pe(Pu, nu, k), nu * bb, ne));
-          else if (Pl) QTX_CK(toT(Pt, pe(Pl, nu, j), nu * bb, ne));
-          else {
-            QTX_CK(toT(Pt, pe(Pu, nu, j), nu * bb, ne));
-            opP = OP_C;
-            al = -1.0;
-          }
-          if ((s = mm(Vk, 0, opV, Pt, bb, opP, acc[dj + 2], al, first))) return s;
+          if (k == j) s = mmP(Vk, opV, pe(Pd, nb, k), (long)nb * bb, OP_N, acc[j - i + 1], 1.0, first);
+          else if (j == k + 1) s = mmP(Vk, opV, pe(Pu, nu, k), nu * bb, OP_N, acc[j - i + 1], 1.0, first);
+          else if (Pl) s = mmP(Vk, opV, pe(Pl, nu, j), nu * bb, OP_N, acc[j - i + 1], 1.0, first);
+          else s = mmP(Vk, opV, pe(Pu, nu, j), nu * bb, OP_C, acc[j - i + 1], -1.0, first);
+          if (s) return s;
           first = false;
         }
       }
       return QTX_OK;
     };
     // M_ii = I - (V P^R)_ii, M_{i,i+1} = -(V P^R)_{i,i+1}, M_{i,i-1} = -(V P^R)_{i,i-1}
-    if ((s = row(in->PR_diag, in->PR_upper, in->PR_lower, 1))) return s;
-    if ((s = emit64(out->M_diag, nb, i, acc[2], -1.0, true))) return s;
-    if (i + 1 < nb && (s = emit64(out->M_upper, nu, i, acc[3], -1.0, false))) return s;
-    if (i >= 1 && (s = emit64(out->M_lower, nu, i - 1, acc[1], -1.0, false))) return s;
+    if ((s = row(in->PR_diag, in->PR_upper, in->PR_lower, -1, 1))) return s;
+    if ((s = emit64(out->M_diag, nb, i, acc[1], -1.0, true))) return s;
+    if (i + 1 < nb && (s = emit64(out->M_upper, nu, i, acc[2], -1.0, false))) return s;
+    if (i >= 1 && (s = emit64(out->M_lower, nu, i - 1, acc[0], -1.0, false))) return s;
     for (int kind = 0; kind < 2; ++kind) {
       const void* Pd = kind ? in->PG_diag : in->PL_diag;
       const void* Pu = kind ? in->PG_upper : in->PL_upper;
       void* Od = kind ? out->BG_diag : out->BL_diag;
       void* Ou = kind ? out->BG_upper : out->BL_upper;
       if (!Pd) continue;
-      if ((s = row(Pd, Pu, nullptr, 2))) return s;
+      if ((s = row(Pd, Pu, nullptr, -1, 2))) return s;  // B's blocks need (V P)_il for l = i-1 .. i+2
       // B_ii = sum_l (V P)_il (V_il)^H, l = i-1..i+1:  (V_{i,i-1})^H = V_{i-1,i}, V_ii^H, V_{i,i+1}^H
       bool first = true;
       for (int l = i - 1; l <= i + 1; ++l) {
         if (l < 0 || l >= nb) continue;
         const cx<T>* Vl = l == i ? Vt[0] : (l == i + 1 ? Vt[3] : Vt[2]);
-        if ((s = mm(acc[l - i + 2], bb, OP_N, Vl, 0, l == i - 1 ? OP_N : OP_C, Bt, 1.0, first))) return s;
+        if ((s = mm(acc[l - i + 1], bb, OP_N, Vl, 0, l == i - 1 ? OP_N : OP_C, Bt, 1.0, first))) return s;
         first = false;
       }
       if ((s = emit64(Od, nb, i, Bt, 1.0, false))) return s;
@@ -1280,7 +1286,7 @@ qtx_status w_assemble_chunk(qtx_rgf_plan_s* P, const qtx_w_inputs* in, const qtx
         first = true;
         for (int l = i; l <= i + 2 && l < nb; ++l) {
           const cx<T>* Vl = l == i ? Vt[3] : (l == i + 1 ? Vt[1] : Vt[4]);
-          if ((s = mm(acc[l - i + 2], bb, OP_N, Vl, 0, l == i ? OP_N : OP_C, Bt, 1.0, first))) return s;
+          if ((s = mm(acc[l - i + 1], bb, OP_N, Vl, 0, l == i ? OP_N : OP_C, Bt, 1.0, first))) return s;
           first = false;
         }
         if ((s = emit64(Ou, nu, i, Bt, 1.0, false))) return s;
@@ -1318,16 +1324,9 @@ qtx_status qtx_rgf_plan_create(const qtx_rgf_desc* desc, qtx_rgf_plan* out) {
   if (e == cudaSuccess) e = cudaMallocHost(&P->h_status, sizeof(int) * P->Ec);
   if (e == cudaSuccess && desc->escalate_tol > 0) e = cudaMallocHost(&P->h_flag, sizeof(int) * P->Ec);
   // identity block for the refinement residual
-  if (e == cudaSuccess) {
-    std::vector<cx<double>> I((size_t)P->bb, mk<double>(0, 0));
-    for (int i = 0; i < P->b; ++i) I[(size_t)i * P->b + i] = mk<double>(1, 0);
-    e = cudaMemcpy(P->ws + P->L.ident, I.data(), I.size() * sizeof(cx<double>), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) {
-      std::vector<float> Idf((size_t)P->bb * 4, 0.f);  // (re.hi, re.lo, im.hi, im.lo)
-      for (int i = 0; i < P->b; ++i) Idf[((size_t)i * P->b + i) * 4] = 1.f;
-      e = cudaMemcpy(P->ws + P->L.ident_df, Idf.data(), Idf.size() * sizeof(float), cudaMemcpyHostToDevice);
-    }
-  }
+  if (e == cudaSuccess)
+    e = set_identity(reinterpret_cast<cx<double>*>(P->ws + P->L.ident), reinterpret_cast<cx<df>*>(P->ws + P->L.ident_df), P->b, nullptr);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
   if (e != cudaSuccess) {
     g_create_error = std::string("plan setup: ") + cudaGetErrorString(e);
     cudaFree(P->ws);
@@ -1490,33 +1489,117 @@ const char* qtx_rgf_version(void) { return "qtx-rgf 0.1 (sm_103a)"; }
 // ============================================================================ component ABI
 namespace {
 
-// FP64 products of at least kTcF64Min in every dimension: straight from the caller's arrays into C on
-// the tensor cores (only digit planes are allocated), unless C overlaps an operand.
-bool overlaps(const void* X, int rows, int cols, long ld, long sX, int nX, const void* Y, int rowsY, int colsY, long ldY,
-              long sY, int nY) {
-  auto span = [](const void* p, int r, int c, long ld, long s, int n, uintptr_t& lo, uintptr_t& hi) {
-    const long row = (long)(r - 1) * ld, ent = (long)(n - 1) * s;
-    const long a = std::min(0L, row) + std::min(0L, ent), b = std::max(0L, row) + std::max(0L, ent) + c;
-    lo = (uintptr_t)((const cx<double>*)p + a);
-    hi = (uintptr_t)((const cx<double>*)p + b);
-  };
-  uintptr_t a0, a1, b0, b1;
-  span(X, rows, cols, ld, sX, nX, a0, a1);
-  span(Y, rowsY, colsY, ldY, sY, nY, b0, b1);
-  return a0 < b1 && b0 < a1;
+// Temporaries of the component calls come from a memory pool of the library's own (one per device): the
+// default pool returns everything to the driver at each synchronisation, and these calls synchronise, so
+// every call paid for mapping its memory again (0.9 ms of a 1.2 ms product).  The pool keeps at most kPoolKeep
+// between calls and gives the rest back; allocation and reuse are stream-ordered, so calls on several
+// streams and threads share it.
+constexpr unsigned long long kPoolKeep = 512ull << 20;
+cudaError_t component_pool(cudaMemPool_t* out) {
+  constexpr int kMaxDev = 64;
+  static std::mutex mu;
+  static cudaMemPool_t pool[kMaxDev] = {};
+  static unsigned long long ctx[kMaxDev] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev >= kMaxDev) return cudaDeviceGetDefaultMemPool(out, dev);
+  std::lock_guard<std::mutex> lk(mu);
+  if (!pool[dev] || current_ctx_id() != ctx[dev]) {  // first call, or a new context after cudaDeviceReset
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p;
+    if ((e = cudaMemPoolCreate(&p, &props)) != cudaSuccess) return e;
+    unsigned long long keep = kPoolKeep;
+    if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+      cudaMemPoolDestroy(p);
+      return e;
+    }
+    pool[dev] = p;
+    ctx[dev] = current_ctx_id();
+  }
+  *out = pool[dev];
+  return cudaSuccess;
 }
-qtx_status zgemm_fp64_direct(const GemmArgs<double>& g, cudaStream_t st, std::string& err) {
-  const size_t bytes = gemm_fp64_tc_scratch_bytes(g.M, g.N, g.K, g.batch);
-  void* scr = nullptr;
-  int* flag = nullptr;
-  int hflag = 0;
-  cudaError_t e = cudaMallocAsync(&scr, bytes, st);
-  if (e == cudaSuccess) e = cudaMallocAsync((void**)&flag, sizeof(int), st);
+// Stream-ordered temporaries of one call, freed when it returns.
+struct Temps {
+  cudaStream_t st;
+  cudaMemPool_t pool = nullptr;
+  cudaError_t e;
+  std::vector<void*> held;
+  explicit Temps(cudaStream_t s) : st(s), e(component_pool(&pool)) {}
+  template <typename T>
+  T* get(size_t count) {
+    void* p = nullptr;
+    if (e == cudaSuccess && count) e = cudaMallocFromPoolAsync(&p, count * sizeof(T), pool, st);
+    if (p) held.push_back(p);
+    return static_cast<T*>(p);
+  }
+  ~Temps() {
+    for (void* p : held) cudaFreeAsync(p, st);
+  }
+};
+
+// whether two batched arrays of complex128 matrices share addresses
+struct Span {
+  uintptr_t lo, hi;
+  Span(const void* p, int rows, int cols, long ld, long s, int n) {
+    const long row = (long)(rows - 1) * ld, ent = (long)(n - 1) * s;
+    lo = (uintptr_t)((const cx<double>*)p + std::min(0L, row) + std::min(0L, ent));
+    hi = (uintptr_t)((const cx<double>*)p + std::max(0L, row) + std::max(0L, ent) + cols);
+  }
+  bool meets(const Span& o) const { return lo < o.hi && o.lo < hi; }
+};
+
+// FP64, EMU64 and BF16X3 products: straight from the caller's complex128 arrays, straight into C unless C
+// shares addresses with an operand (or with C0 in another layout), which then goes through a copy.
+qtx_status zgemm_direct(int precision, GemmArgs<double> g, cudaStream_t st, std::string& err) {
+  const bool emu = precision != QTX_FP64;
+  const bool tc = emu || (g.M >= kTcF64Min && g.N >= kTcF64Min && g.K >= kTcF64Min && tc_available());
+  const int rA = g.opA == OP_N ? g.M : g.K, cA = g.opA == OP_N ? g.K : g.M;
+  const int rB = g.opB == OP_N ? g.K : g.N, cB = g.opB == OP_N ? g.N : g.K;
+  const Span sc(g.C, g.M, g.N, g.ldc, g.sC, g.batch);
+  bool clash = g.K > 0 && (sc.meets(Span(g.A, rA, cA, g.lda, g.sA, g.sA ? g.batch : 1)) ||
+                           sc.meets(Span(g.B, rB, cB, g.ldb, g.sB, g.sB ? g.batch : 1)));
+  if (g.C0 && !(g.C0 == g.C && g.ldc0 == g.ldc && g.sC0 == g.sC))
+    clash |= sc.meets(Span(g.C0, g.M, g.N, g.ldc0, g.sC0, g.sC0 ? g.batch : 1));
+  const int digits = precision == QTX_EMU64 ? 6 : 2;
+  const size_t bytes = !tc ? 0 : (emu ? gemm_tc_scratch_bytes(g.M, g.N, g.K, g.batch, digits)
+                                      : gemm_fp64_tc_scratch_bytes(g.M, g.N, g.K, g.batch));
+  Temps t(st);
+  unsigned char* scr = t.get<unsigned char>(bytes);
+  int* flag = t.get<int>(1);
+  cx<double>* C = clash ? t.get<cx<double>>((size_t)g.batch * g.M * g.N) : g.C;
+  cudaError_t e = t.e;
+  GemmArgs<double> w = g;
+  if (clash) {
+    w.C = C;
+    w.ldc = g.N;
+    w.sC = (long)g.M * g.N;
+  }
   if (e == cudaSuccess) e = cudaMemsetAsync(flag, 0, sizeof(int), st);
-  if (e == cudaSuccess) e = gemm_fp64_tc(g, scr, bytes, flag, st);
+  if (e == cudaSuccess) {
+    if (emu) {
+      TcArgs a;
+      a.M = w.M; a.N = w.N; a.K = w.K;
+      a.ta = a.tb = a.tc = EL_F64;
+      a.A = reinterpret_cast<const cx<df>*>(w.A); a.lda = w.lda; a.sA = w.sA; a.opA = w.opA;
+      a.B = reinterpret_cast<const cx<df>*>(w.B); a.ldb = w.ldb; a.sB = w.sB; a.opB = w.opB;
+      a.C0 = reinterpret_cast<const cx<df>*>(w.C0); a.ldc0 = w.ldc0; a.sC0 = w.sC0;
+      a.C = reinterpret_cast<cx<df>*>(w.C); a.ldc = w.ldc; a.sC = w.sC;
+      a.alpha = w.alpha; a.beta = w.beta;
+      a.batch = w.batch; a.active = nullptr;
+      e = gemm_tc(a, digits, scr, bytes, flag, st);
+    } else {
+      e = tc ? gemm_fp64_tc(w, scr, bytes, flag, st) : gemm_simt<double>(w, st);
+    }
+  }
+  if (e == cudaSuccess && clash)
+    e = convert_strided<double, double>(C, g.N, (long)g.M * g.N, g.C, g.ldc, g.sC, g.M, g.N, g.batch, st);
+  int hflag = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
-  if (scr) cudaFreeAsync(scr, st);
-  if (flag) cudaFreeAsync(flag, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
     err = cudaGetErrorString(e);
@@ -1527,82 +1610,32 @@ qtx_status zgemm_fp64_direct(const GemmArgs<double>& g, cudaStream_t st, std::st
   return QTX_OK;
 }
 
-template <typename T>
-qtx_status zgemm_via(int precision, int M, int N, int K, int opA, const void* A, long lda, long sA, int opB,
-                     const void* B, long ldb, long sB, double alpha, double beta, const void* C0, long ldc0,
-                     long sC0, void* C, long ldc, long sC, int batch, cudaStream_t st, std::string& err) {
-  const int rA = opA == OP_N ? M : K, cA = opA == OP_N ? K : M;
-  const int rB = opB == OP_N ? K : N, cB = opB == OP_N ? N : K;
-  const int nA = sA ? batch : 1, nB = sB ? batch : 1, nC0 = (C0 && beta != 0.0) ? (sC0 ? batch : 1) : 0;
-  if constexpr (std::is_same<T, double>::value) {
-    // C may be C0 itself (same layout); any other overlap takes the copies below
-    const bool c0_ok = !nC0 || (C0 == C && ldc0 == ldc && sC0 == sC) || !overlaps(C, M, N, ldc, sC, batch, C0, M, N, ldc0, sC0, nC0);
-    if (M >= kTcF64Min && N >= kTcF64Min && K >= kTcF64Min && tc_available() && c0_ok &&
-        !overlaps(C, M, N, ldc, sC, batch, A, rA, cA, lda, sA, nA) && !overlaps(C, M, N, ldc, sC, batch, B, rB, cB, ldb, sB, nB)) {
-      return zgemm_fp64_direct(gargs<double>(M, N, K, (const cx<double>*)A, lda, sA, opA, (const cx<double>*)B, ldb, sB, opB,
-                                             nC0 ? (const cx<double>*)C0 : nullptr, ldc0, nC0 > 1 ? sC0 : 0, (cx<double>*)C, ldc, sC,
-                                             alpha, nC0 ? beta : 0.0, batch, nullptr), st, err);
-    }
-  }
-  const size_t es = sizeof(cx<T>);
-  void *a = nullptr, *b = nullptr, *c0 = nullptr, *c = nullptr, *scr = nullptr;
-  int* flag = nullptr;
-  const int digits = precision == QTX_EMU64 ? 6 : 2;
-  const size_t scr_bytes = std::is_same<T, df>::value ? gemm_tc_scratch_bytes(M, N, K, batch, digits) : 0;
-  cudaError_t e = cudaSuccess;
-  qtx_status s = QTX_OK;
-  auto CK = [&](cudaError_t x) {
-    if (x != cudaSuccess && e == cudaSuccess) e = x;
-    return x == cudaSuccess;
-  };
-  CK(cudaMallocAsync(&a, es * (size_t)nA * rA * cA, st));
-  CK(cudaMallocAsync(&b, es * (size_t)nB * rB * cB, st));
-  if (nC0) CK(cudaMallocAsync(&c0, es * (size_t)nC0 * M * N, st));
-  CK(cudaMallocAsync(&c, es * (size_t)batch * M * N, st));
-  if (scr_bytes) CK(cudaMallocAsync(&scr, scr_bytes, st));
-  CK(cudaMallocAsync((void**)&flag, sizeof(int), st));
-  if (e == cudaSuccess) {
-    CK(cudaMemsetAsync(flag, 0, sizeof(int), st));
-    CK(convert_strided<double, T>((const cx<double>*)A, lda, sA, (cx<T>*)a, cA, (long)rA * cA, rA, cA, nA, st));
-    CK(convert_strided<double, T>((const cx<double>*)B, ldb, sB, (cx<T>*)b, cB, (long)rB * cB, rB, cB, nB, st));
-    if (nC0) CK(convert_strided<double, T>((const cx<double>*)C0, ldc0, sC0, (cx<T>*)c0, N, (long)M * N, M, N, nC0, st));
-  }
-  if (e == cudaSuccess) {
-    if constexpr (std::is_same<T, df>::value) {
-      TcArgs t;
-      t.M = M; t.N = N; t.K = K;
-      t.A = (const cx<df>*)a; t.lda = cA; t.sA = nA > 1 ? (long)rA * cA : 0; t.opA = opA;
-      t.B = (const cx<df>*)b; t.ldb = cB; t.sB = nB > 1 ? (long)rB * cB : 0; t.opB = opB;
-      t.C0 = nC0 ? (const cx<df>*)c0 : nullptr; t.ldc0 = N; t.sC0 = nC0 > 1 ? (long)M * N : 0;
-      t.C = (cx<df>*)c; t.ldc = N; t.sC = (long)M * N;
-      t.alpha = alpha; t.beta = nC0 ? beta : 0.0;
-      t.batch = batch; t.active = nullptr;
-      CK(gemm_tc(t, digits, scr, scr_bytes, flag, st));
-    } else {
-      GemmArgs<T> g;
-      g.M = M; g.N = N; g.K = K;
-      g.A = (const cx<T>*)a; g.lda = cA; g.sA = nA > 1 ? (long)rA * cA : 0; g.opA = opA;
-      g.B = (const cx<T>*)b; g.ldb = cB; g.sB = nB > 1 ? (long)rB * cB : 0; g.opB = opB;
-      g.C0 = nC0 ? (const cx<T>*)c0 : nullptr; g.ldc0 = N; g.sC0 = nC0 > 1 ? (long)M * N : 0;
-      g.C = (cx<T>*)c; g.ldc = N; g.sC = (long)M * N;
-      g.alpha = alpha; g.beta = nC0 ? beta : 0.0;
-      g.batch = batch; g.active = nullptr;
-      CK(gemm_simt<T>(g, st));
-    }
-    CK(convert_strided<T, double>((const cx<T>*)c, N, (long)M * N, (cx<double>*)C, ldc, sC, M, N, batch, st));
-  }
-  int hflag = 0;
-  if (e == cudaSuccess) CK(cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, st));
-  for (void* p : {a, b, c0, c, scr, (void*)flag})
-    if (p) cudaFreeAsync(p, st);
-  if (e == cudaSuccess) CK(cudaStreamSynchronize(st));
+// FP32 products: operands rounded to complex64 copies, the result widened into C.
+qtx_status zgemm_f32(const GemmArgs<double>& g, cudaStream_t st, std::string& err) {
+  const int rA = g.opA == OP_N ? g.M : g.K, cA = g.opA == OP_N ? g.K : g.M;
+  const int rB = g.opB == OP_N ? g.K : g.N, cB = g.opB == OP_N ? g.N : g.K;
+  const int nA = g.sA ? g.batch : 1, nB = g.sB ? g.batch : 1, nC0 = g.C0 ? (g.sC0 ? g.batch : 1) : 0;
+  Temps t(st);
+  cx<float>* a = t.get<cx<float>>((size_t)nA * rA * cA);
+  cx<float>* b = t.get<cx<float>>((size_t)nB * rB * cB);
+  cx<float>* c0 = t.get<cx<float>>((size_t)nC0 * g.M * g.N);
+  cx<float>* c = t.get<cx<float>>((size_t)g.batch * g.M * g.N);
+  cudaError_t e = t.e;
+  if (e == cudaSuccess) e = convert_strided<double, float>(g.A, g.lda, g.sA, a, cA, (long)rA * cA, rA, cA, nA, st);
+  if (e == cudaSuccess) e = convert_strided<double, float>(g.B, g.ldb, g.sB, b, cB, (long)rB * cB, rB, cB, nB, st);
+  if (e == cudaSuccess && nC0) e = convert_strided<double, float>(g.C0, g.ldc0, g.sC0, c0, g.N, (long)g.M * g.N, g.M, g.N, nC0, st);
+  if (e == cudaSuccess)
+    e = gemm_simt<float>(gargs<float>(g.M, g.N, g.K, a, cA, nA > 1 ? (long)rA * cA : 0, g.opA, b, cB, nB > 1 ? (long)rB * cB : 0,
+                                      g.opB, nC0 ? c0 : nullptr, g.N, nC0 > 1 ? (long)g.M * g.N : 0, c, g.N, (long)g.M * g.N,
+                                      g.alpha, g.beta, g.batch, nullptr), st);
+  if (e == cudaSuccess) e = convert_strided<float, double>(c, g.N, (long)g.M * g.N, g.C, g.ldc, g.sC, g.M, g.N, g.batch, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
     err = cudaGetErrorString(e);
     cudaGetLastError();
     return QTX_ERR_CUDA;
   }
-  if (hflag) { err = "tensor-core engine: bounded wait expired"; s = QTX_ERR_TIMEOUT; }
-  return s;
+  return QTX_OK;
 }
 
 template <typename T>
@@ -1644,13 +1677,17 @@ qtx_status qtx_zgemm_batched(int precision, int M, int N, int K, int opA, const 
   }
   if (M == 0 || N == 0) return QTX_OK;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  const bool c0 = C0 && beta != 0.0;
+  const GemmArgs<double> g = gargs<double>(M, N, K, (const cx<double>*)A, lda, sA, opA, (const cx<double>*)B, ldb, sB, opB,
+                                           c0 ? (const cx<double>*)C0 : nullptr, ldc0, sC0, (cx<double>*)C, ldc, sC, alpha,
+                                           c0 ? beta : 0.0, batch, nullptr);
   switch (precision) {
-    case QTX_FP64: return zgemm_via<double>(precision, M, N, K, opA, A, lda, sA, opB, B, ldb, sB, alpha, beta, C0, ldc0, sC0, C, ldc, sC, batch, st, g_kernel_error);
-    case QTX_FP32: return zgemm_via<float>(precision, M, N, K, opA, A, lda, sA, opB, B, ldb, sB, alpha, beta, C0, ldc0, sC0, C, ldc, sC, batch, st, g_kernel_error);
+    case QTX_FP32: return zgemm_f32(g, st, g_kernel_error);
     case QTX_EMU64:
     case QTX_BF16X3:
       if (!tc_available()) { g_kernel_error = "tensor-core engine needs an sm_103 GPU"; return QTX_ERR_UNSUPPORTED; }
-      return zgemm_via<df>(precision, M, N, K, opA, A, lda, sA, opB, B, ldb, sB, alpha, beta, C0, ldc0, sC0, C, ldc, sC, batch, st, g_kernel_error);
+      return zgemm_direct(precision, g, st, g_kernel_error);
+    case QTX_FP64: return zgemm_direct(precision, g, st, g_kernel_error);
     default:
       g_kernel_error = "unknown precision";
       return QTX_ERR_INVALID_ARG;
@@ -1665,18 +1702,39 @@ qtx_status qtx_zinv_batched(int precision, int n, void* A, long sA, int batch, i
   d.max_energies_in_flight = batch;
   d.precision = (qtx_precision)precision;
   d.refine_max_iter = refine_iter;
-  qtx_rgf_plan P = nullptr;
-  qtx_status s = qtx_rgf_plan_create(&d, &P);
-  if (s) return s;
+  std::string err;
+  qtx_status s = validate(&d, err);
+  if (s) { g_create_error = err; return s; }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  // a plan of the inverse's areas alone, in stream-ordered memory
+  qtx_rgf_plan_s plan;
+  qtx_rgf_plan_s* P = &plan;
+  P->d = d;
+  P->b = n;
+  P->nb = 1;
+  P->Ec = batch;
+  P->bb = (long)n * n;
+  P->esz = precision == QTX_FP32 ? sizeof(cx<float>) : sizeof(cx<double>);
+  P->L = make_layout(d, true);
+  Temps t(st);
+  P->ws = t.get<unsigned char>(P->L.total);
+  P->d_err_flag = t.get<int>(1);
+  if (t.e != cudaSuccess) {
+    g_create_error = std::string("workspace of ") + std::to_string(P->L.total) + " bytes: " + cudaGetErrorString(t.e);
+    cudaGetLastError();
+    return QTX_ERR_OOM;
+  }
+  cudaError_t e = cudaMemsetAsync(P->d_err_flag, 0, sizeof(int), st);
+  if (e == cudaSuccess)
+    e = set_identity(reinterpret_cast<cx<double>*>(P->ws + P->L.ident), reinterpret_cast<cx<df>*>(P->ws + P->L.ident_df), n, st);
   int* stat = status;
   if (!stat) stat = reinterpret_cast<int*>(P->ws + P->L.flags);
-  if (!status) cudaMemsetAsync(stat, 0, sizeof(int) * batch, st);
+  if (e == cudaSuccess && !status) e = cudaMemsetAsync(stat, 0, sizeof(int) * batch, st);
+  if (e != cudaSuccess) { cudaGetLastError(); return QTX_ERR_CUDA; }
   if (precision == QTX_FP32) s = zinv_via<float>(P, n, A, sA, batch, stat, st);
   else if (precision == QTX_FP64) s = zinv_via<double>(P, n, A, sA, batch, stat, st);
   else s = zinv_via<df>(P, n, A, sA, batch, stat, st);
-  cudaError_t e = cudaStreamSynchronize(st);
-  qtx_rgf_destroy(P);
+  e = cudaStreamSynchronize(st);
   if (s == QTX_OK && e != cudaSuccess) s = QTX_ERR_CUDA;
   return s;
 }
@@ -1693,16 +1751,32 @@ qtx_status qtx_lead_self_energy(int n, const void* H00, const void* H01, const d
   d.leads = 1;
   d.decim_tol = tol;
   d.decim_max_iter = max_iter;
-  qtx_rgf_plan P = nullptr;
-  qtx_status s = qtx_rgf_plan_create(&d, &P);
-  if (s) return s;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  std::string err;
+  qtx_status s = validate(&d, err);
+  if (s) { g_create_error = err; return s; }
+  qtx_rgf_plan_s plan;  // the contact's and the inverse's areas alone, in stream-ordered memory
+  qtx_rgf_plan_s* P = &plan;
+  P->d = d;
+  P->b = n;
+  P->nb = 1;
+  P->Ec = n_energies;
+  P->bb = (long)n * n;
+  P->esz = sizeof(cx<double>);
+  P->L = make_layout(d, true);
+  Temps t(st);
+  P->ws = t.get<unsigned char>(P->L.total);
+  P->d_err_flag = t.get<int>(1);
+  if (t.e != cudaSuccess) {
+    g_create_error = std::string("workspace of ") + std::to_string(P->L.total) + " bytes: " + cudaGetErrorString(t.e);
+    cudaGetLastError();
+    return QTX_ERR_OOM;
+  }
   int* stat = status ? status : reinterpret_cast<int*>(P->ws + P->L.flags) + 2 * P->Ec;
   cudaMemsetAsync(stat, 0, sizeof(int) * n_energies, st);
   Ctx<double> c{P, st, n_energies, energies, stat, (long)n * n, n};
   s = contact<double>(c, (const cx<double>*)H00, (const cx<double>*)H01, eta, (cx<double>*)SigR);
   cudaError_t e = cudaStreamSynchronize(st);
-  qtx_rgf_destroy(P);
   if (s == QTX_OK && e != cudaSuccess) s = QTX_ERR_CUDA;
   return s;
 }

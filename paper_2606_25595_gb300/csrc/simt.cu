@@ -937,6 +937,24 @@ cudaError_t pivoted_inverse(cx<double>* A, long sA, int n, int batch, const int*
   return cudaGetLastError();
 }
 
+__global__ void k_set_identity(cx<double>* I, cx<df>* Idf, int b) {
+  const int bb = b * b;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < bb; i += gridDim.x * blockDim.x) {
+    const float v = i % (b + 1) == 0 ? 1.f : 0.f;
+    I[i] = mk<double>(v, 0.0);
+    cx<df> w;
+    w.re = mkdf(v, 0.f);
+    w.im = mkdf(0.f, 0.f);
+    Idf[i] = w;
+  }
+}
+cudaError_t set_identity(cx<double>* I, cx<df>* Idf, int b, cudaStream_t st) {
+  const long n = ((long)b * b + 255) / 256;
+  k_set_identity<<<(unsigned)(n < 1024 ? n : 1024), 256, 0, st>>>(I, Idf, b);
+  count_launch();
+  return cudaGetLastError();
+}
+
 template <typename T>
 __global__ void k_add_identity(cx<T>* X, long sX, int n, const int* active) {
   const int e = blockIdx.y;

@@ -141,15 +141,18 @@ __device__ __forceinline__ df sum_acc(const uint32_t (&v)[NACC][8], int c) {
 // loads) is paid once per SM rather than once per tile.  The staging area is separate from the
 // stage ring (NST = 3 stages fit beside it for 6 and 4 digit planes, 6 for 2).
 
-// IO: element type of C and C0 -- df (the emulated-FP64 products) or float (the products of the
-// FP32 starting inverse, four digit planes: ~27-bit products, all digit groups exact).
+// IO: element type of C and C0 -- df (the emulated-FP64 products), double (the same with complex128 results:
+// what a separate pass would convert is converted in the store) or float (the products of the FP32 mode and
+// of the FP32 starting inverse, four digit planes: ~27-bit products, all digit groups exact).
 template <typename IO> __device__ __forceinline__ cx<IO> c_from_df(cx<df> v);
 template <> __device__ __forceinline__ cx<df> c_from_df<df>(cx<df> v) { return v; }
 template <> __device__ __forceinline__ cx<float> c_from_df<float>(cx<df> v) {
   return mk<float>(v.re.hi + v.re.lo, v.im.hi + v.im.lo);
 }
+template <> __device__ __forceinline__ cx<double> c_from_df<double>(cx<df> v) { return mk<double>(to_d(v.re), to_d(v.im)); }
 __device__ __forceinline__ df df_of(df x) { return x; }
 __device__ __forceinline__ df df_of(float x) { return mkdf(x, 0.f); }
+__device__ __forceinline__ df df_of(double x) { return from_d<df>(x); }
 
 // GROUP = false: a single product (problem 0; its parameters at fixed offsets); true: a grouped launch.
 template <int S, int NST, typename IO, bool GROUP>
@@ -630,7 +633,7 @@ inline Scratch carve(void* base, const Dims& d, int batch, int S) {
 }
 
 template <int S, typename TI>
-cudaError_t digitize(const cx<TI>* X, long ldx, long sX, int opX, int side, int R, int K, const Dims& d,
+cudaError_t digitize_as(const cx<TI>* X, long ldx, long sX, int opX, int side, int R, int K, const Dims& d,
                      int* eout, unsigned char* planes, int batch, const int* active, cudaStream_t st) {
   // logical row r of the operand: left A = op(X): row r of op(X); right B = op(X): column r of op(X)
   //   left  N: X[r][k] direct      left  H: conj(X[k][r]) transposed
@@ -664,16 +667,25 @@ cudaError_t digitize(const cx<TI>* X, long ldx, long sX, int opX, int side, int 
   }
 }
 
+// ... by the operand's element type (FP32 operands: four digit planes only)
+template <int S>
+cudaError_t digitize(const cx<df>* X, Elt type, long ldx, long sX, int opX, int side, int R, int K, const Dims& d, int* eout,
+                     unsigned char* planes, int batch, const int* active, cudaStream_t st) {
+  if (type == EL_F64)
+    return digitize_as<S, double>(reinterpret_cast<const cx<double>*>(X), ldx, sX, opX, side, R, K, d, eout, planes, batch, active, st);
+  if constexpr (S == 4)
+    if (type == EL_F32)
+      return digitize_as<S, float>(reinterpret_cast<const cx<float>*>(X), ldx, sX, opX, side, R, K, d, eout, planes, batch, active, st);
+  if (type != EL_DF) return cudaErrorInvalidValue;
+  return digitize_as<S, df>(X, ldx, sX, opX, side, R, K, d, eout, planes, batch, active, st);
+}
+
 // Digitise one product's operands (into the scratch, or a kept operand) and fill its kernel
 // parameters and tile counts.
-template <int S, typename IO>
+template <int S>
 cudaError_t prepare(const TcArgs& a, void* scratch, size_t scratch_bytes, int* err_flag, cudaStream_t st,
                     TcPrepared& out) {
   TcParams& p = out.p;
-  // operand and result pointers in the IO type (TcArgs carries the df32 ones; f32 products pass
-  // FP32 arrays through the same fields)
-  const cx<IO>* A = reinterpret_cast<const cx<IO>*>(a.A);
-  const cx<IO>* B = reinterpret_cast<const cx<IO>*>(a.B);
   const Dims d = dims_of(a.M, a.N, a.K, S);
   Scratch sc = carve(scratch, d, a.batch, S);
   if (sc.bytes > scratch_bytes) return cudaErrorInvalidValue;
@@ -686,8 +698,8 @@ cudaError_t prepare(const TcArgs& a, void* scratch, size_t scratch_bytes, int* e
   int* ea = a.opndA ? a.opndA->expo : sc.ea;
   int* eb = sc.eb;
   if (!(a.opndA && a.opndA->mode == 2))
-    if ((e = digitize<S, IO>(A, a.lda, a.sA, a.opA, 0, a.M, a.K, d, ea, pa, ab ? a.batch : 1, ab ? a.active : nullptr, st))) return e;
-  if ((e = digitize<S, IO>(B, a.ldb, a.sB, a.opB, 1, a.N, a.K, d, eb, pb, bb_ ? a.batch : 1, bb_ ? a.active : nullptr, st))) return e;
+    if ((e = digitize<S>(a.A, a.ta, a.lda, a.sA, a.opA, 0, a.M, a.K, d, ea, pa, ab ? a.batch : 1, ab ? a.active : nullptr, st))) return e;
+  if ((e = digitize<S>(a.B, a.tb, a.ldb, a.sB, a.opB, 1, a.N, a.K, d, eb, pb, bb_ ? a.batch : 1, bb_ ? a.active : nullptr, st))) return e;
   p.pa = pa;
   p.pb = pb;
   p.eA = ea;
@@ -817,20 +829,20 @@ TcOperand tc_operand_at(void* base, int R, int K, int batch, int digits) {
 // Pipeline stages of a kernel variant: the requested count if shared memory allows it, else the
 // default.  Beside the 96 KB epilogue staging of 48-column tiles, 6 digit planes take 42 KB a stage
 // and 7 take 49 KB; beside the 128 KB staging of 64-column tiles, 4 planes take 32 KB and 2 take 16 KB.
-static int resolve_stages(int S, bool f32, int want) {
-  if (f32 || S == 4) return (want == 2) ? 2 : 3;  // S = 4 (complex64 or df32 in and out): 2 or 3
+static int resolve_stages(int S, int want) {
+  if (S == 4) return (want == 2) ? 2 : 3;  // 2 or 3
   if (S == 6) return (want == 2) ? 2 : 3;         // 2 or 3
   if (S == 7) return 2;
   return (want == 4) ? 4 : 6;                   // S = 2: 4 or 6
 }
 
-// Kernel variant of a product: digits actually used (effective_digits), the IO type and the stages;
+// Kernel variant of a product: digits actually used (effective_digits), the result type and the stages;
 // -1 when the product is split along K (it then runs as consecutive chunks and cannot be prepared on
 // its own).
 int gemm_tc_variant(const TcArgs& a, int digits) {
   if (k_chunks(a.K) > 1) return -1;
   const int S = effective_digits(digits, a.K);
-  return S * 2 + (a.f32 ? 1 : 0) + 100 * resolve_stages(S, a.f32, a.stages);
+  return S * 3 + (int)a.tc + 100 * resolve_stages(S, a.stages);
 }
 
 cudaError_t gemm_tc_prepare(const TcArgs& a, int digits, void* scratch, size_t scratch_bytes, int* err_flag,
@@ -839,12 +851,11 @@ cudaError_t gemm_tc_prepare(const TcArgs& a, int digits, void* scratch, size_t s
   out->ctas = a.ctas;
   out->tiles = 0;
   if (a.M <= 0 || a.N <= 0 || a.batch <= 0) return cudaSuccess;
-  switch (out->variant % 100) {
-    case 4 * 2 + 1: return tc::prepare<4, float>(a, scratch, scratch_bytes, err_flag, st, *out);
-    case 4 * 2: return tc::prepare<4, df>(a, scratch, scratch_bytes, err_flag, st, *out);
-    case 7 * 2: return tc::prepare<7, df>(a, scratch, scratch_bytes, err_flag, st, *out);
-    case 6 * 2: return tc::prepare<6, df>(a, scratch, scratch_bytes, err_flag, st, *out);
-    case 2 * 2: return tc::prepare<2, df>(a, scratch, scratch_bytes, err_flag, st, *out);
+  switch (out->variant % 100 / 3) {
+    case 4: return tc::prepare<4>(a, scratch, scratch_bytes, err_flag, st, *out);
+    case 7: return tc::prepare<7>(a, scratch, scratch_bytes, err_flag, st, *out);
+    case 6: return tc::prepare<6>(a, scratch, scratch_bytes, err_flag, st, *out);
+    case 2: return tc::prepare<2>(a, scratch, scratch_bytes, err_flag, st, *out);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -854,15 +865,18 @@ cudaError_t gemm_tc_launch(const TcPrepared* const* p, int n, cudaStream_t st, c
   for (int q = 1; q < n; ++q)
     if (p[q]->variant != p[0]->variant) return cudaErrorInvalidValue;
   switch (p[0]->variant) {
-    case 300 + 4 * 2 + 1: return tc::launch<4, 3, float>(p, n, st, ev);
-    case 200 + 4 * 2 + 1: return tc::launch<4, 2, float>(p, n, st, ev);
-    case 300 + 4 * 2: return tc::launch<4, 3, df>(p, n, st, ev);
-    case 200 + 4 * 2: return tc::launch<4, 2, df>(p, n, st, ev);
-    case 200 + 7 * 2: return tc::launch<7, 2, df>(p, n, st, ev);
-    case 300 + 6 * 2: return tc::launch<6, 3, df>(p, n, st, ev);
-    case 200 + 6 * 2: return tc::launch<6, 2, df>(p, n, st, ev);
-    case 600 + 2 * 2: return tc::launch<2, 6, df>(p, n, st, ev);
-    case 400 + 2 * 2: return tc::launch<2, 4, df>(p, n, st, ev);
+    case 300 + 4 * 3 + EL_F32: return tc::launch<4, 3, float>(p, n, st, ev);
+    case 200 + 4 * 3 + EL_F32: return tc::launch<4, 2, float>(p, n, st, ev);
+    case 300 + 4 * 3 + EL_DF: return tc::launch<4, 3, df>(p, n, st, ev);
+    case 200 + 4 * 3 + EL_DF: return tc::launch<4, 2, df>(p, n, st, ev);
+    case 200 + 7 * 3 + EL_DF: return tc::launch<7, 2, df>(p, n, st, ev);
+    case 200 + 7 * 3 + EL_F64: return tc::launch<7, 2, double>(p, n, st, ev);
+    case 300 + 6 * 3 + EL_DF: return tc::launch<6, 3, df>(p, n, st, ev);
+    case 200 + 6 * 3 + EL_DF: return tc::launch<6, 2, df>(p, n, st, ev);
+    case 300 + 6 * 3 + EL_F64: return tc::launch<6, 3, double>(p, n, st, ev);
+    case 600 + 2 * 3 + EL_DF: return tc::launch<2, 6, df>(p, n, st, ev);
+    case 400 + 2 * 3 + EL_DF: return tc::launch<2, 4, df>(p, n, st, ev);
+    case 600 + 2 * 3 + EL_F64: return tc::launch<2, 6, double>(p, n, st, ev);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -871,7 +885,7 @@ cudaError_t gemm_tc(const TcArgs& a, int digits, void* scratch, size_t scratch_b
                     cudaStream_t st, cudaEvent_t* ev) {
   if (a.M <= 0 || a.N <= 0 || a.batch <= 0) return cudaSuccess;
   const int nc = k_chunks(a.K);
-  if (nc > 1 && a.f32) return cudaErrorInvalidValue;  // the FP32 products are short contractions
+  if (nc > 1 && a.tc == EL_F32) return cudaErrorInvalidValue;  // the FP32 products are short contractions
   if (nc > 1) {
     // split K: chunk c covers k in [k0, k1); op N operands advance along their columns (A) or rows
     // (B), op C ones the other way round

@@ -90,8 +90,10 @@ def test_fp64_product_error_not_above_dfma(q):
         assert ec <= ed, (n, ec, ed)
 
 
-def test_fp64_product_strides_and_overlap(q):
-    """Padded rows and gapped batches; C0 = C; C on top of an operand still gives the product."""
+@pytest.mark.parametrize("prec", ["fp64", "emu64"])
+def test_product_strides_and_overlap(q, prec):
+    """Padded rows and gapped batches; C0 = C; C on top of an operand still gives the product (emulated
+    FP64: to its 2^-36 of the operands' magnitudes)."""
     import ctypes
     import torch
     rng = np.random.default_rng(8)
@@ -100,18 +102,19 @@ def test_fp64_product_strides_and_overlap(q):
     C = torch.tensor(_cx(rng, bt, M, N + 2)).cuda()
     C0 = C.clone()
     L = q.load()
-    st = L.qtx_zgemm_batched(0, M, N, K, 0, A.data_ptr(), K + 5, M * (K + 5), 1, B.data_ptr(), K + 3, 0, 1.0, 1.0,
+    p, atol = q.PRECISION[prec], 1e-13 if prec == "fp64" else 1e-8
+    st = L.qtx_zgemm_batched(p, M, N, K, 0, A.data_ptr(), K + 5, M * (K + 5), 1, B.data_ptr(), K + 3, 0, 1.0, 1.0,
                              C.data_ptr(), N + 2, M * (N + 2), C.data_ptr(), N + 2, M * (N + 2), bt,
                              ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
     assert st == 0
     ref = C0.clone()
     ref[:, :, :N] += A[:bt, :, :K] @ B[0, :, :K].conj().T
-    assert torch.allclose(C, ref, rtol=1e-14, atol=1e-13)
+    assert torch.allclose(C, ref, rtol=1e-14, atol=atol)
     X, Y = torch.tensor(_cx(rng, 2, 64, 64)).cuda(), torch.tensor(_cx(rng, 2, 64, 64)).cuda()
     ref = X @ Y
-    st = L.qtx_zgemm_batched(0, 64, 64, 64, 0, X.data_ptr(), 64, 4096, 0, Y.data_ptr(), 64, 4096, 1.0, 0.0, None, 64, 0,
+    st = L.qtx_zgemm_batched(p, 64, 64, 64, 0, X.data_ptr(), 64, 4096, 0, Y.data_ptr(), 64, 4096, 1.0, 0.0, None, 64, 0,
                              X.data_ptr(), 64, 4096, 2, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
-    assert st == 0 and torch.allclose(X, ref, rtol=1e-14, atol=1e-13)
+    assert st == 0 and torch.allclose(X, ref, rtol=1e-14, atol=atol)
 
 
 # refined from an FP32 start (33, 64, 200), beyond its reach (kappa 1e9: elimination), a block whose
