@@ -194,7 +194,7 @@ struct GemmArgs {
   bool b64 = false;  // T = df: B holds complex128 values (digitised from them directly)
 };
 
-// Up to four products of one shape and batch in a launch.
+// Up to four products of one batch in a launch.
 template <typename T>
 struct GemmMulti {
   static constexpr int kMax = 4;

@@ -39,6 +39,9 @@ template <typename T>
 cudaError_t leaf_inverse(cx<T>* A, long lda, long sA, int n, int batch, const int* active,
                          int* status, cudaStream_t st);
 template <>
+cudaError_t leaf_inverse<float>(cx<float>* A, long lda, long sA, int n, int batch, const int* active, int* status,
+                                cudaStream_t st);
+template <>
 cudaError_t leaf_inverse<double>(cx<double>* A, long lda, long sA, int n, int batch, const int* active, int* status,
                                  cudaStream_t st);
 

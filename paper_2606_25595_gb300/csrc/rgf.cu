@@ -281,10 +281,13 @@ qtx_status gemm_simt_prof(qtx_rgf_plan_s* P, const GemmArgs<T>& g, cudaStream_t 
 // products, at least FP32's precision; every digit group exact), the smaller ones on the SIMT GEMM.
 constexpr int kTcF32Min = 96;
 inline bool f32_on_tc(const qtx_rgf_desc& d) { return d.precision != QTX_BF16X3; }
+bool f32_takes_tc(qtx_rgf_plan_s* P, const GemmArgs<float>& g) {
+  return f32_on_tc(P->d) && g.M >= kTcF32Min && g.N >= kTcF32Min && g.K >= kTcF32Min && g.K <= 1024 &&
+         gemm_tc_scratch_bytes(g.M, g.N, g.K, g.batch, 4) <= P->L.tc_bytes;
+}
 template <>
 qtx_status gemm<float>(qtx_rgf_plan_s* P, const GemmArgs<float>& g, cudaStream_t st, bool, DigitHint) {
-  if (f32_on_tc(P->d) && g.M >= kTcF32Min && g.N >= kTcF32Min && g.K >= kTcF32Min && g.K <= 1024 &&
-      gemm_tc_scratch_bytes(g.M, g.N, g.K, g.batch, 4) <= P->L.tc_bytes) {
+  if (f32_takes_tc(P, g)) {
     TcArgs a;
     a.ta = a.tb = a.tc = EL_F32;
     a.M = g.M; a.N = g.N; a.K = g.K;
@@ -363,6 +366,23 @@ qtx_status gemm<df>(qtx_rgf_plan_s* P, const GemmArgs<df>& g, cudaStream_t st, b
   return QTX_OK;
 }
 
+// Two products that do not depend on each other: one SIMT launch where both take the SIMT kernel.
+template <typename T>
+qtx_status gemm_pair(qtx_rgf_plan_s* P, const GemmArgs<T>& g1, const GemmArgs<T>& g2, cudaStream_t st) {
+  if constexpr (std::is_same<T, float>::value) {
+    if (!f32_takes_tc(P, g1) && !f32_takes_tc(P, g2) && !P->prof) {
+      GemmMulti<T> m;
+      m.n = 2;
+      m.g[0] = g1;
+      m.g[1] = g2;
+      QTX_CK(gemm_simt_multi<T>(m, st));
+      return QTX_OK;
+    }
+  }
+  const qtx_status s = gemm<T>(P, g1, st, true);
+  return s ? s : gemm<T>(P, g2, st, true);
+}
+
 // Plain (non-refined) recursive inverse of n x n blocks stored with leading dimension lda.
 // T12/T21 scratch for each recursion level is carved from `scratch` (>= 0.7 n^2 per batch entry).
 template <typename T>
@@ -384,14 +404,14 @@ qtx_status inverse_rec(qtx_rgf_plan_s* P, cx<T>* A, long lda, long sA, int n, in
   qtx_status s;
   if ((s = inverse_rec<T>(P, A11, lda, sA, h, batch, active, status, next, sScr, st, force_simt))) return s;
   // T12 = X11 A12 ; T21 = A21 X11
-  if ((s = gemm<T>(P, gargs<T>(h, r, h, A11, lda, sA, OP_N, A12, lda, sA, OP_N, nullptr, 0, 0, T12, r, sScr, 1.0, 0.0, batch, active), st, force_simt))) return s;
-  if ((s = gemm<T>(P, gargs<T>(r, h, h, A21, lda, sA, OP_N, A11, lda, sA, OP_N, nullptr, 0, 0, T21, h, sScr, 1.0, 0.0, batch, active), st, force_simt))) return s;
+  if ((s = gemm_pair<T>(P, gargs<T>(h, r, h, A11, lda, sA, OP_N, A12, lda, sA, OP_N, nullptr, 0, 0, T12, r, sScr, 1.0, 0.0, batch, active),
+                        gargs<T>(r, h, h, A21, lda, sA, OP_N, A11, lda, sA, OP_N, nullptr, 0, 0, T21, h, sScr, 1.0, 0.0, batch, active), st))) return s;
   // A22 <- A22 - A21 T12 (Schur complement), then invert it in place
   if ((s = gemm<T>(P, gargs<T>(r, r, h, A21, lda, sA, OP_N, T12, r, sScr, OP_N, A22, lda, sA, A22, lda, sA, -1.0, 1.0, batch, active), st, force_simt))) return s;
   if ((s = inverse_rec<T>(P, A22, lda, sA, r, batch, active, status, next, sScr, st, force_simt))) return s;
   // A12 <- -T12 Y ; A21 <- -Y T21 ; A11 <- X11 - T12 A21
-  if ((s = gemm<T>(P, gargs<T>(h, r, r, T12, r, sScr, OP_N, A22, lda, sA, OP_N, nullptr, 0, 0, A12, lda, sA, -1.0, 0.0, batch, active), st, force_simt))) return s;
-  if ((s = gemm<T>(P, gargs<T>(r, h, r, A22, lda, sA, OP_N, T21, h, sScr, OP_N, nullptr, 0, 0, A21, lda, sA, -1.0, 0.0, batch, active), st, force_simt))) return s;
+  if ((s = gemm_pair<T>(P, gargs<T>(h, r, r, T12, r, sScr, OP_N, A22, lda, sA, OP_N, nullptr, 0, 0, A12, lda, sA, -1.0, 0.0, batch, active),
+                        gargs<T>(r, h, r, A22, lda, sA, OP_N, T21, h, sScr, OP_N, nullptr, 0, 0, A21, lda, sA, -1.0, 0.0, batch, active), st))) return s;
   if ((s = gemm<T>(P, gargs<T>(h, h, r, T12, r, sScr, OP_N, A21, lda, sA, OP_N, A11, lda, sA, A11, lda, sA, -1.0, 1.0, batch, active), st, force_simt))) return s;
   return QTX_OK;
 }

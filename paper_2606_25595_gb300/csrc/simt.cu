@@ -147,7 +147,12 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_gemm_multi(const __gr
 template <typename T, int BM, int BN, int BK, int TM, int TN>
 static cudaError_t launch_gemm(const GemmMulti<T>& m, cudaStream_t st) {
   const GemmArgs<T>& g = m.g[0];
-  dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.batch * m.n);
+  int M = 0, N = 0;  // the products may differ in shape: a tile beyond one's M or N stores nothing
+  for (int q = 0; q < m.n; ++q) {
+    M = M > m.g[q].M ? M : m.g[q].M;
+    N = N > m.g[q].N ? N : m.g[q].N;
+  }
+  dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, g.batch * m.n);
   if (m.n == 1) k_gemm<T, BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, st>>>(g);
   else k_gemm_multi<T, BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, st>>>(m);
   count_launch();
@@ -188,12 +193,16 @@ cudaError_t gemm_simt_multi(const GemmMulti<T>& m, cudaStream_t st) {
       default: return launch_gemm<T, 64, 64, 16, 4, 4>(m, st);
     }
   } else {
-    if (g.M <= 32 && g.N <= 32) return launch_gemm<T, 32, 32, 16, 2, 2>(m, st);
-    if (g.M >= 128 && g.N >= 128) return launch_gemm<T, 128, 128, 8, 8, 8>(m, st);
-    return launch_gemm<T, 64, 64, 16, 4, 4>(m, st);
+    // smaller tiles while the larger ones would leave SMs idle (64 x 64 products of 32 entries: 10.9 us in
+    // 64 x 64 tiles; every tile sums in the same order)
+    auto ctas = [&](int t) { return (long)((g.M + t - 1) / t) * ((g.N + t - 1) / t) * g.batch * m.n; };
+    if (g.M >= 128 && g.N >= 128 && ctas(128) >= 152) return launch_gemm<T, 128, 128, 8, 8, 8>(m, st);
+    if ((g.M > 32 || g.N > 32) && ctas(64) >= 152) return launch_gemm<T, 64, 64, 16, 4, 4>(m, st);
+    return launch_gemm<T, 32, 32, 16, 2, 2>(m, st);
   }
 }
 template cudaError_t gemm_simt_multi<double>(const GemmMulti<double>&, cudaStream_t);
+template cudaError_t gemm_simt_multi<float>(const GemmMulti<float>&, cudaStream_t);
 
 template <typename T>
 cudaError_t gemm_simt(const GemmArgs<T>& g, cudaStream_t st) {
@@ -206,7 +215,7 @@ template cudaError_t gemm_simt<double>(const GemmArgs<double>&, cudaStream_t);
 template cudaError_t gemm_simt<float>(const GemmArgs<float>&, cudaStream_t);
 
 // ============================================================================ leaf inverse
-// In-place Gauss-Jordan inverse with partial pivoting (pivot = first row of largest |Re|+|Im| among
+// In-place FP32 Gauss-Jordan inverse with partial pivoting (pivot = first row of largest |Re|+|Im| among
 // the rows not yet used, in the current column), one CTA per block, the block held in registers.
 //
 // Rows are not moved: step k pivots on (p_k, k) wherever row p_k sits.  With P the permutation
@@ -214,140 +223,102 @@ template cudaError_t gemm_simt<float>(const GemmArgs<float>&, cudaStream_t);
 //     A^-1[k][p_j] = B[p_k][j],
 // so each thread scatters its values to (step of its row, pivot row of its column's step).
 //
-// Layout: NMAX/8 warps; warp w owns rows w + (NMAX/8) m, m = 0..7; lane l owns columns l + 32 c,
-// c < NMAX/32.  Entries outside the n x n block are zero and stay zero.  Each step needs one CTA
-// barrier: at the end of step k every warp publishes, for column k+1, its best unused row already
-// scaled by the inverse of its pivot entry (double-buffered in shared memory); after the barrier
-// every thread picks the same winner (largest value, smallest row on ties) and reads the pivot row
-// straight from the winner's slot.
-template <typename T, int NMAX>
-__global__ void __launch_bounds__(NMAX * 4) k_leaf_inverse(cx<T>* Ag, long lda, long sA, int n,
-                                                          const int* active, int* status) {
-  constexpr int WARPS = NMAX / 8, C = NMAX / 32;
+// Bound by the latency of a step's chain, not by its n^2 FMAs.  Layout: 16 x 16 threads, thread (ty, tx)
+// owns rows ty + 16 i and columns tx + 16 j (NMAX = 64: 4 x 4 values, 32: 2 x 2).  Column k of the block
+// lies in shared memory (double-buffered, written by its owners in the last step's update): every warp
+// searches it for the pivot with one integer reduction, the half-warp that owns the pivot row scales it
+// by the reciprocal and publishes it, and after a barrier every thread updates its values from 4 factors
+// and 4 row values.  About 500 cycles a step; with a warp per row group publishing its own candidate,
+// eight reciprocals and 16 shuffles a step, it took 2,000 (62 us for 64 x 64, batch 32).
+template <int NMAX>
+__global__ void __launch_bounds__(256) k_leaf_inverse(cx<float>* Ag, long lda, long sA, int n, const int* active, int* status) {
+  constexpr int R = NMAX / 16;
   const int e = blockIdx.x;
   if (active && !active[e]) return;
-  __shared__ T s_val[2][WARPS];
-  __shared__ int s_row[2][WARPS];
-  __shared__ cx<T> s_prow[2][WARPS][NMAX];
-  cx<T>* A = Ag + (long)e * sA;
-  const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
-  cx<T> a[8][C];
-  int rowstep[8], colpiv[C];
-  unsigned used = 0;
+  __shared__ cx<float> s_col[2][NMAX], s_row[NMAX];
+  __shared__ int s_step[NMAX], s_piv[NMAX];
+  cx<float>* A = Ag + (long)e * sA;
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16, lane = threadIdx.x % 32;
+  cx<float> a[R][R];
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
-    const int i = w + WARPS * m;
-    rowstep[m] = 0;
+  for (int i = 0; i < R; ++i)
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
-      const int j = lane + 32 * c;
-      a[m][c] = (i < n && j < n) ? A[(long)i * lda + j] : mk<T>(T(0), T(0));
+    for (int j = 0; j < R; ++j) {
+      const int r = ty + 16 * i, c = tx + 16 * j;
+      a[i][j] = (r < n && c < n) ? A[(long)r * lda + c] : mk<float>(0.f, 0.f);
     }
-  }
+  if (tx == 0)
 #pragma unroll
-  for (int c = 0; c < C; ++c) colpiv[c] = 0;
-
-  // publish this warp's pivot candidate for column kk into buffer b
-  auto publish = [&](int kk, int b) {
-    const int cc = kk / 32, owner = kk % 32;
-    T best = T(-1);
-    int bm = -1;
-    if (lane == owner) {
-#pragma unroll
-      for (int m = 0; m < 8; ++m) {
-        const int i = w + WARPS * m;
-        const cx<T> v = cc == 0 ? a[m][0] : a[m][C - 1];
-        const T av = cabs1(v);
-        if (i < n && !((used >> m) & 1u) && av > best) {
-          best = av;
-          bm = m;
-        }
-      }
-    }
-    best = __shfl_sync(0xffffffffu, best, owner);
-    bm = __shfl_sync(0xffffffffu, bm, owner);
-    if (bm >= 0) {
-      cx<T> row[C];
-#pragma unroll
-      for (int c = 0; c < C; ++c) row[c] = mk<T>(T(0), T(0));
-#pragma unroll
-      for (int m = 0; m < 8; ++m)
-        if (m == bm)
-#pragma unroll
-          for (int c = 0; c < C; ++c) row[c] = a[m][c];
-      cx<T> pv = cc == 0 ? row[0] : row[C - 1];
-      pv.re = __shfl_sync(0xffffffffu, pv.re, owner);
-      pv.im = __shfl_sync(0xffffffffu, pv.im, owner);
-      const cx<T> r = crecip(pv);
-#pragma unroll
-      for (int c = 0; c < C; ++c) {
-        const int j = lane + 32 * c;
-        s_prow[b][w][j] = (j == kk) ? r : row[c] * r;
-      }
-    }
-    if (lane == 0) {
-      s_val[b][w] = best;
-      s_row[b][w] = bm >= 0 ? w + WARPS * bm : -1;
-    }
-  };
-
-  bool bad = false;
-  if (n > 0) publish(0, 0);
+    for (int i = 0; i < R; ++i) s_col[0][ty + 16 * i] = a[i][0];
   __syncthreads();
+  unsigned used0 = 0, used1 = 0;
+  bool bad = false;
   for (int k = 0; k < n; ++k) {
-    const int b = k & 1;
-    T best = T(-1);
-    int p = -1, ww = 0;
-#pragma unroll
-    for (int q = 0; q < WARPS; ++q) {
-      const T v = s_val[b][q];
-      const int ri = s_row[b][q];
-      if (ri >= 0 && (v > best || (v == best && ri < p))) {
-        best = v;
-        p = ri;
-        ww = q;
-      }
-    }
-    if (!(best > T(0)) || !isfinite(best)) {
+    const cx<float>* col = s_col[k & 1];
+    // |Re| + |Im| >= 0 orders like its bits; NaN never wins
+    auto key = [&](int r, unsigned used) -> unsigned {
+      if (r >= n || ((used >> lane) & 1u)) return 0u;
+      const unsigned v = __float_as_uint(cabs1(col[r]));
+      return v <= 0x7f800000u ? v : 0u;
+    };
+    const unsigned k0 = key(lane, used0), k1 = NMAX > 32 ? key(lane + 32, used1) : 0u;
+    const unsigned best = __reduce_max_sync(0xffffffffu, k0 > k1 ? k0 : k1);
+    if (best == 0 || best >= 0x7f800000u) {
       bad = true;
       break;
     }
-    const cx<T> r = s_prow[b][ww][k];
-    cx<T> prow[C];
+    const unsigned b0 = __ballot_sync(0xffffffffu, k0 == best), b1 = __ballot_sync(0xffffffffu, k1 == best);
+    const int p = b0 ? __ffs((int)b0) - 1 : 31 + __ffs((int)b1);
+    if (p < 32) used0 |= 1u << p;
+    else used1 |= 1u << (p - 32);
+    if (ty == p % 16) {  // the pivot row's owners scale it
+      const cx<float> r = crecip(col[p]);
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
-      prow[c] = s_prow[b][ww][lane + 32 * c];
-      if (lane + 32 * c == k) colpiv[c] = p;
-    }
-    const int cc = k / 32, owner = k % 32;
+      for (int i = 0; i < R; ++i)
+        if (i == p / 16)
 #pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const int i = w + WARPS * m;
-      cx<T> f = cc == 0 ? a[m][0] : a[m][C - 1];
-      f.re = __shfl_sync(0xffffffffu, f.re, owner);
-      f.im = __shfl_sync(0xffffffffu, f.im, owner);
-      if (i == p) {
-#pragma unroll
-        for (int c = 0; c < C; ++c) a[m][c] = prow[c];
-        used |= 1u << m;
-        rowstep[m] = k;
-      } else {
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-          if (lane + 32 * c == k) {
-            a[m][c] = mk<T>(-(f.re * r.re - f.im * r.im), -(f.re * r.im + f.im * r.re));
-          } else {
-            cx<T> v = a[m][c];
-            v.re = fma(-f.re, prow[c].re, v.re);
-            v.re = fma(f.im, prow[c].im, v.re);
-            v.im = fma(-f.re, prow[c].im, v.im);
-            v.im = fma(-f.im, prow[c].re, v.im);
-            a[m][c] = v;
+          for (int j = 0; j < R; ++j) {
+            const int c = tx + 16 * j;
+            const cx<float> x = a[i][j];
+            // the order of the roundings, by padded size
+            const float im = NMAX > 32 ? __fmaf_rn(x.re, r.im, __fmul_rn(x.im, r.re)) : __fmaf_rn(x.im, r.re, __fmul_rn(x.re, r.im));
+            a[i][j] = c == k ? r : mk<float>(__fmaf_rn(x.re, r.re, -__fmul_rn(x.im, r.im)), im);
+            s_row[c] = a[i][j];
           }
-        }
+      if (tx == 0) {
+        s_step[p] = k;
+        s_piv[k] = p;
       }
     }
-    if (k + 1 < n) publish(k + 1, b ^ 1);
+    __syncthreads();
+    cx<float> w[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) w[j] = s_row[tx + 16 * j];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int r = ty + 16 * i;
+      const cx<float> f = col[r];
+      if (r == p) continue;
+#pragma unroll
+      for (int j = 0; j < R; ++j) {
+        cx<float> v = a[i][j];
+        v.re = __fmaf_rn(-f.re, w[j].re, v.re);
+        v.re = __fmaf_rn(f.im, w[j].im, v.re);
+        v.im = __fmaf_rn(-f.re, w[j].im, v.im);
+        v.im = __fmaf_rn(-f.im, w[j].re, v.im);
+        if (tx + 16 * j == k)  // the pivot column: -(f r)
+          v = mk<float>(-__fmaf_rn(f.re, w[j].re, -__fmul_rn(f.im, w[j].im)), -__fmaf_rn(f.re, w[j].im, __fmul_rn(f.im, w[j].re)));
+        a[i][j] = v;
+      }
+    }
+    if (tx == (k + 1) % 16) {
+      cx<float>* next = s_col[(k + 1) & 1];
+#pragma unroll
+      for (int j = 0; j < R; ++j)
+        if (j == (k + 1) / 16)
+#pragma unroll
+          for (int i = 0; i < R; ++i) next[ty + 16 * i] = a[i][j];
+    }
     __syncthreads();
   }
   if (bad) {
@@ -355,28 +326,25 @@ __global__ void __launch_bounds__(NMAX * 4) k_leaf_inverse(cx<T>* Ag, long lda, 
     return;
   }
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
-    const int i = w + WARPS * m;
+  for (int i = 0; i < R; ++i)
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
-      const int j = lane + 32 * c;
-      if (i < n && j < n) A[(long)rowstep[m] * lda + colpiv[c]] = a[m][c];
+    for (int j = 0; j < R; ++j) {
+      const int r = ty + 16 * i, c = tx + 16 * j;
+      if (r < n && c < n) A[(long)s_step[r] * lda + s_piv[c]] = a[i][j];
     }
-  }
 }
 
-template <typename T>
-cudaError_t leaf_inverse(cx<T>* A, long lda, long sA, int n, int batch, const int* active, int* status,
-                         cudaStream_t st) {  // T = double: leaf64.cu
+template <>
+cudaError_t leaf_inverse<float>(cx<float>* A, long lda, long sA, int n, int batch, const int* active, int* status,
+                                cudaStream_t st) {
   if (n <= 0 || n > kLeafMax) return cudaErrorInvalidValue;
   if (n <= 32)
-    k_leaf_inverse<T, 32><<<batch, 128, 0, st>>>(A, lda, sA, n, active, status);
+    k_leaf_inverse<32><<<batch, 256, 0, st>>>(A, lda, sA, n, active, status);
   else
-    k_leaf_inverse<T, 64><<<batch, 256, 0, st>>>(A, lda, sA, n, active, status);
+    k_leaf_inverse<64><<<batch, 256, 0, st>>>(A, lda, sA, n, active, status);
   count_launch();
   return cudaGetLastError();
 }
-template cudaError_t leaf_inverse<float>(cx<float>*, long, long, int, int, const int*, int*, cudaStream_t);
 
 // ============================================================================ elementwise
 // Accumulator of a combination: FP64 when FP64 data is involved, df32 (error-free FP32 steps) when
