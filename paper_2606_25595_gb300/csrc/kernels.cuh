@@ -241,9 +241,13 @@ int gemm_tc_variant(const TcArgs& a, int digits);
 // Digitise a product's operands on `st` (not one split along K) and fill *out.
 cudaError_t gemm_tc_prepare(const TcArgs& a, int digits, void* scratch, size_t scratch_bytes, int* err_flag,
                             cudaStream_t st, TcPrepared* out);
+// The same for n products of one digit count that do not depend on each other, product q in scratch[q]
+// (scratch_bytes each): their operands are digitised in one launch per element type.
+constexpr int kTcMaxGroup = 8;
+cudaError_t gemm_tc_prepare_many(const TcArgs* a, const int* digits, int n, void* const* scratch, size_t scratch_bytes, int* err_flag,
+                                 cudaStream_t st, TcPrepared* out);
 // One persistent launch over the tiles of 1..kTcMaxGroup prepared products of one variant (each
 // product's tiles computed exactly as in a launch of its own: the results are bit-identical).
-constexpr int kTcMaxGroup = 8;
 cudaError_t gemm_tc_launch(const TcPrepared* const* p, int n, cudaStream_t st, cudaEvent_t* ev = nullptr);
 // digit products (pairs i + j <= digits + 1) the engine issues per real product
 inline int tc_pairs(int digits) { return digits * (digits + 1) / 2; }

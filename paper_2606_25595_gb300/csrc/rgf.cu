@@ -48,6 +48,9 @@ constexpr int kTcF64Min = 33;
 // one CTA up to this size, by the recursion above it
 constexpr int kPivotedMax = 256;
 
+// products launched together at most (those of a slice's stage)
+constexpr int kMany = 4;
+
 // U_i, V_i differ per energy when z multiplies an overlap block or Sigma^R_{i,i+1} depends on E.
 inline bool uv_per_energy(const qtx_rgf_desc& d) {
   return d.has_S || d.system_input || (d.offdiag_sigma && d.energy_dependent_sigma);
@@ -58,6 +61,8 @@ struct Layout {
       tc_scratch, total;
   int n_tmp, n_dec;
   size_t tc_bytes;
+  size_t tc_more;  // scratch of further products launched together with one in tc_scratch (n_more of them)
+  int n_more;
   bool refine64;  // FP64 block inverses by refinement (inverse_f64) have their areas
   size_t perm;
 };
@@ -174,6 +179,14 @@ Layout make_layout(const qtx_rgf_desc& d, bool inverse_only = false) {
   if (d.precision == QTX_FP32 && b >= 96 && b <= 1024) L.tc_bytes = gemm_tc_scratch_bytes((int)b, (int)b, (int)b, (int)Ec, 4);
   if (tc64) L.tc_bytes = gemm_fp64_tc_scratch_bytes((int)b, (int)b, (int)b, (int)Ec);
   L.tc_scratch = a.take(L.tc_bytes);
+  // products of a slice that do not depend on each other share launches while one alone fills less than
+  // four waves of the GPU (608 tiles): their further scratch is then a few hundred MB at most, and the
+  // launch's tail, its fixed costs and idle SMs are paid once (b = 120, 24 energies: 72 tiles a product
+  // on 152 SMs).  Larger products fill their waves alone.
+  const long col = d.precision == QTX_EMU64 ? 48 : 64;
+  const long tiles = ((b + 127) / 128) * ((b + col - 1) / col) * Ec;
+  L.n_more = !inverse_only && L.tc_bytes && d.precision != QTX_FP64 && tiles <= 4 * 152 ? kMany - 1 : 0;
+  L.tc_more = a.take((size_t)L.n_more * align_up(L.tc_bytes, 1024));
   // kept digitised operands (emulated modes): two left operands, b x b, E_c energies (none when the
   // products are split along K)
   for (int k = 0; k < 2; ++k) {
@@ -285,20 +298,27 @@ bool f32_takes_tc(qtx_rgf_plan_s* P, const GemmArgs<float>& g) {
   return f32_on_tc(P->d) && g.M >= kTcF32Min && g.N >= kTcF32Min && g.K >= kTcF32Min && g.K <= 1024 &&
          gemm_tc_scratch_bytes(g.M, g.N, g.K, g.batch, 4) <= P->L.tc_bytes;
 }
+inline int tc_digits(const qtx_rgf_desc& d) { return d.precision == QTX_EMU64 ? 6 : 2; }
+template <typename T>
+TcArgs tc_args(qtx_rgf_plan_s* P, const GemmArgs<T>& g) {
+  TcArgs a;
+  if (std::is_same<T, float>::value) a.ta = a.tb = a.tc = EL_F32;
+  if (g.b64) a.tb = EL_F64;
+  a.M = g.M; a.N = g.N; a.K = g.K;
+  a.A = reinterpret_cast<const cx<df>*>(g.A); a.lda = g.lda; a.sA = g.sA; a.opA = g.opA;
+  a.B = reinterpret_cast<const cx<df>*>(g.B); a.ldb = g.ldb; a.sB = g.sB; a.opB = g.opB;
+  a.C0 = reinterpret_cast<const cx<df>*>(g.C0); a.ldc0 = g.ldc0; a.sC0 = g.sC0;
+  a.C = reinterpret_cast<cx<df>*>(g.C); a.ldc = g.ldc; a.sC = g.sC;
+  a.alpha = g.alpha; a.beta = g.beta;
+  a.batch = g.batch; a.active = g.active;
+  a.stages = P->d.tc_stages; a.ctas = P->d.tc_ctas;
+  return a;
+}
 template <>
 qtx_status gemm<float>(qtx_rgf_plan_s* P, const GemmArgs<float>& g, cudaStream_t st, bool, DigitHint) {
   if (f32_takes_tc(P, g)) {
-    TcArgs a;
-    a.ta = a.tb = a.tc = EL_F32;
-    a.M = g.M; a.N = g.N; a.K = g.K;
-    a.A = reinterpret_cast<const cx<df>*>(g.A); a.lda = g.lda; a.sA = g.sA; a.opA = g.opA;
-    a.B = reinterpret_cast<const cx<df>*>(g.B); a.ldb = g.ldb; a.sB = g.sB; a.opB = g.opB;
-    a.C0 = reinterpret_cast<const cx<df>*>(g.C0); a.ldc0 = g.ldc0; a.sC0 = g.sC0;
-    a.C = reinterpret_cast<cx<df>*>(g.C); a.ldc = g.ldc; a.sC = g.sC;
-    a.alpha = g.alpha; a.beta = g.beta;
-    a.batch = g.batch; a.active = g.active;
-    a.stages = P->d.tc_stages; a.ctas = P->d.tc_ctas;
-    // in the FP32 mode these are the plan's own products (profiled); in the emulated mode they
+    const TcArgs a = tc_args<float>(P, g);
+    // in the FP32 mode these are the plan's own products (profiled); in the other modes they
     // belong to the starting inverse (not counted)
     if (P->group && gemm_tc_variant(a, 4) >= 0) {
       QTX_CK(group_gemm(P, a, 4, st));
@@ -329,28 +349,20 @@ qtx_status gemm<double>(qtx_rgf_plan_s* P, const GemmArgs<double>& g, cudaStream
   }
   return gemm_simt_prof<double>(P, g, st);
 }
-inline int tc_digits(const qtx_rgf_desc& d) { return d.precision == QTX_EMU64 ? 6 : 2; }
+// kept left operand: only for the plan's b x b x b products at the plan's digit count, when slots exist
+bool kept_operand(qtx_rgf_plan_s* P, const GemmArgs<df>& g, const DigitHint& hint, int digits, TcOperand& oa) {
+  const bool square = g.M == P->b && g.N == P->b && g.K == P->b && g.batch <= P->Ec && digits == tc_digits(P->d);
+  if (!square || hint.a_mode == DG_NONE || !P->L.opnd_bytes[hint.a_slot]) return false;
+  oa = tc_operand_at(P->ws + P->L.opnd[hint.a_slot], P->b, P->b, P->Ec, tc_digits(P->d));
+  oa.mode = hint.a_mode;
+  return true;
+}
 template <>
 qtx_status gemm<df>(qtx_rgf_plan_s* P, const GemmArgs<df>& g, cudaStream_t st, bool, DigitHint hint) {
-  TcArgs a;
+  TcArgs a = tc_args<df>(P, g);
   const int digits = hint.digits > 0 ? hint.digits : tc_digits(P->d);
-  // kept operands: only for the plan's b x b x b products at the plan's digit count, when slots exist
   TcOperand oa;
-  const bool square = g.M == P->b && g.N == P->b && g.K == P->b && g.batch <= P->Ec && digits == tc_digits(P->d);
-  if (square && hint.a_mode != DG_NONE && P->L.opnd_bytes[hint.a_slot]) {
-    oa = tc_operand_at(P->ws + P->L.opnd[hint.a_slot], P->b, P->b, P->Ec, tc_digits(P->d));
-    oa.mode = hint.a_mode;
-    a.opndA = &oa;
-  }
-  if (g.b64) a.tb = EL_F64;
-  a.M = g.M; a.N = g.N; a.K = g.K;
-  a.A = g.A; a.lda = g.lda; a.sA = g.sA; a.opA = g.opA;
-  a.B = g.B; a.ldb = g.ldb; a.sB = g.sB; a.opB = g.opB;
-  a.C0 = g.C0; a.ldc0 = g.ldc0; a.sC0 = g.sC0;
-  a.C = g.C; a.ldc = g.ldc; a.sC = g.sC;
-  a.alpha = g.alpha; a.beta = g.beta;
-  a.batch = g.batch; a.active = g.active;
-  a.stages = P->d.tc_stages; a.ctas = P->d.tc_ctas;
+  if (kept_operand(P, g, hint, digits, oa)) a.opndA = &oa;
   if (P->group && gemm_tc_variant(a, digits) >= 0) {
     QTX_CK(group_gemm(P, a, digits, st));
     return QTX_OK;
@@ -363,6 +375,58 @@ qtx_status gemm<df>(qtx_rgf_plan_s* P, const GemmArgs<df>& g, cudaStream_t st, b
     P->pipe_flops += f * tc_pairs(digits);
     P->useful_flops += f;
   }
+  return QTX_OK;
+}
+
+// Products that do not depend on each other, issued in order.  Where the plan has scratch for several
+// (Layout::n_more), up to kMany of them share one digitisation and one persistent launch; every tile is
+// computed as in a launch of its own, so the results are the same bits.
+bool group_pools(qtx_rgf_plan_s* P);  // the plan solves in a group that pools products
+template <typename T>
+struct Prods {
+  GemmArgs<T> g[kTcMaxGroup];
+  DigitHint h[kTcMaxGroup];
+  int n = 0;
+  void add(const GemmArgs<T>& x, DigitHint hint = DigitHint{}) {
+    g[n] = x;
+    h[n++] = hint;
+  }
+};
+template <typename T>
+qtx_status run(qtx_rgf_plan_s* P, Prods<T>& q, cudaStream_t st) {
+  int i = 0;
+  if constexpr (!std::is_same<T, double>::value) {
+    bool many = P->L.n_more > 0 && !P->prof && !group_pools(P);
+    if constexpr (std::is_same<T, float>::value)
+      for (int k = 0; k < q.n; ++k) many = many && f32_takes_tc(P, q.g[k]);
+    if (std::is_same<T, df>::value && P->b > 1024) many = false;  // split along K
+    while (many && q.n - i > 1) {
+      const int m = std::min(q.n - i, P->L.n_more + 1);
+      TcArgs a[kMany];
+      int digits[kMany];
+      TcOperand oa[kMany];
+      void* scr[kMany];
+      TcPrepared p[kMany];
+      const TcPrepared* pp[kMany];
+      for (int k = 0; k < m; ++k) {
+        a[k] = tc_args<T>(P, q.g[i + k]);
+        if constexpr (std::is_same<T, float>::value) {
+          digits[k] = 4;
+        } else {
+          digits[k] = tc_digits(P->d);
+          if (kept_operand(P, q.g[i + k], q.h[i + k], digits[k], oa[k])) a[k].opndA = &oa[k];
+        }
+        scr[k] = k ? P->ws + P->L.tc_more + (size_t)(k - 1) * align_up(P->L.tc_bytes, 1024) : P->ws + P->L.tc_scratch;
+        pp[k] = &p[k];
+      }
+      QTX_CK(gemm_tc_prepare_many(a, digits, m, scr, P->L.tc_bytes, P->d_err_flag, st, p));
+      QTX_CK(gemm_tc_launch(pp, m, st));
+      i += m;
+    }
+  }
+  for (; i < q.n; ++i)
+    if (const qtx_status s = gemm<T>(P, q.g[i], st, false, q.h[i])) return s;
+  q.n = 0;
   return QTX_OK;
 }
 
@@ -759,12 +823,12 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
   const cx<double>* SRl = odg && !d.system_input ? reinterpret_cast<const cx<double>*>(in->SigR_lower) + sigUE0 : nullptr;
   const cx<double>* SLu = odg ? reinterpret_cast<const cx<double>*>(in->SigL_upper) + sigUE0 : nullptr;
   const cx<double>* SGu = odg && d.second_rhs ? reinterpret_cast<const cx<double>*>(in->SigG_upper) + sigUE0 : nullptr;
-  // Sigma^<_{i,i+1} in the sweep's type (tmp 12): one block shared by the chunk, or one per energy
+  // Sigma^<_{i,i+1} in the sweep's type (tmp 12; the second right-hand side's: tmp 10): one block shared by the chunk, or one per energy
   const int nLt = d.energy_dependent_sigma ? ne : 1;
   const long sLt = d.energy_dependent_sigma ? bb : 0;
   // right-hand side k's upper block of slice i (k = 1: B2_{i,i+1})
   auto load_L = [&](int k, int i) -> cx<T>* {
-    cx<T>* Lt = c.tmp(12);
+    cx<T>* Lt = c.tmp(k ? 10 : 12);
     if (axpby_from64<T>(Lt, bb, (k ? SGu : SLu) + (long)i * bb, sSigU, 1.0, nullptr, 0, 0.0, b, nLt, st) != cudaSuccess) return nullptr;
     return Lt;
   };
@@ -851,6 +915,12 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
     else QTX_CK(assemble_offdiag<T>(U(i), V(i), Hu + (long)i * bb, nullptr, nullptr, 0.0, b, 1, st, sru, srl, 0));
   }
 
+  // products of a stage, launched together by run(); b x b blocks with batch strides sA_, sB_
+  Prods<T> pr;
+  auto pd = [&](const cx<T>* A, long sA_, int opA, const cx<T>* B, long sB_, int opB, const cx<T>* C0, cx<T>* C, double al, double be) {
+    return gargs<T>(b, b, b, A, b, sA_, opA, B, b, sB_, opB, C0, b, bb, C, b, bb, al, be, ne, nullptr);
+  };
+
   // ---- 2. forward sweep
   for (int i = 0; i < nb; ++i) {
     cx<T>* gi = c.g(i);
@@ -894,29 +964,10 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
       Term<T> t1; t1.p = c.tmp(1); t1.s = bb; t1.alpha = 1.0;
       QTX_CK((combine<T, T>(gi, bb, t0, t1, none, b, ne, nullptr, 0, 0, nullptr, st)));
     }
-    if (i > 0 && c.keep_z()) {
-      // V g U as (V g) U: Z_{i-1} = V_{i-1} g_{i-1} is kept for the backward sweep
-      // (G_{i,i-1} = -G_ii Z_{i-1}), which then needs one product less per slice
-      cx<T>* Zp = c.zk(i - 1);
-      if ((s = gemm<T>(P, gargs<T>(b, b, b, V(i - 1), b, sUV, OP_N, c.g(i - 1), b, bb, OP_N, nullptr, 0, 0, Zp, b, bb, 1.0, 0.0, ne, nullptr), st)))
-        return s;
-      if ((s = gemm<T>(P, gargs<T>(b, b, b, Zp, b, bb, OP_N, U(i - 1), b, sUV, OP_N, gi, b, bb, gi, b, bb, -1.0, 1.0, ne, nullptr), st))) return s;
-    } else if (i > 0) {
-      cx<T>* Tm = c.tmp(0);
-      // g_{i-1} was the left operand of the previous slice's g_{i-1} Sigma^<: its digit planes are kept
-      if ((s = gemm<T>(P, gargs<T>(b, b, b, c.g(i - 1), b, bb, OP_N, U(i - 1), b, sUV, OP_N, nullptr, 0, 0, Tm, b, bb, 1.0, 0.0, ne, nullptr), st,
-                       false, reuseA(1)))) return s;
-      if ((s = gemm<T>(P, gargs<T>(b, b, b, V(i - 1), b, sUV, OP_N, Tm, b, bb, OP_N, gi, b, bb, gi, b, bb, -1.0, 1.0, ne, nullptr), st))) return s;
-    }
-    if ((s = block_inverse<T>(P, gi, b, ne, nullptr, status, st))) return s;
-    // block-tridiagonal right-hand sides: V_{i-1} g_{i-1} of the cross term, shared by both
-    cx<T>* Zf = i > 0 && c.keep_z() ? c.zk(i - 1) : c.tmp(2);
-    if (i > 0 && odg && !c.keep_z() &&
-        (s = gemm<T>(P, gargs<T>(b, b, b, V(i - 1), b, sUV, OP_N, c.g(i - 1), b, bb, OP_N, nullptr, 0, 0, Zf, b, bb, 1.0, 0.0, ne, nullptr), st)))
-      return s;
+    // Sigma^<_ii (+ contacts; or B2_ii) of each right-hand side
+    auto SLk = [&](int k) { return c.tmp(k ? 5 : 1); };
     for (int k = 0; k < nrhs; ++k) {
-      // Sigma^<_ii (+ contacts; or B2_ii), then the left-connected lesser function of right-hand side k
-      cx<T>* SLi = c.tmp(1);
+      cx<T>* SLi = SLk(k);
       const cx<double>* sl = k ? sigG(i) : sLi;
       const cx<double>* lsl = nullptr;
       if (k == 0 && d.leads && i == 0) lsl = SL_L;
@@ -933,26 +984,45 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
         Term<T> t1; t1.p = c.tmp(2); t1.s = bb; t1.alpha = 1.0;
         QTX_CK((combine<T, T>(SLi, bb, t0, t1, none, b, ne, nullptr, 0, 0, nullptr, st)));
       }
-      if (i > 0) {
-        cx<T>* X = c.keep_z() ? c.xk(k, i - 1) : c.tmp(0);  // V_{i-1} g^<_{i-1}
-        if ((s = gemm<T>(P, gargs<T>(b, b, b, V(i - 1), b, sUV, OP_N, c.glk(k, i - 1), b, bb, OP_N, nullptr, 0, 0, X, b, bb, 1.0, 0.0, ne, nullptr), st))) return s;
-        if ((s = gemm<T>(P, gargs<T>(b, b, b, X, b, bb, OP_N, V(i - 1), b, sUV, OP_C, SLi, b, bb, SLi, b, bb, 1.0, 1.0, ne, nullptr), st))) return s;
-        if (odg) {  // block-tridiagonal Sigma^<: bracket += -Y + Y^H, Y = V_{i-1} g_{i-1} Sigma^<_{i-1,i}
-          cx<T>* Yf = c.tmp(3);
+    }
+    if (i > 0) {
+      const bool kz = c.keep_z();
+      // Z = V g and X = V g^<, kept for the backward sweep (G_{i,i-1} = -G_ii Z and Q = X); V g U is then
+      // Z U.  Without them V (g U), where g_{i-1} was the left operand of the previous slice's g Sigma^< and
+      // its digit planes are kept
+      cx<T>* Zf = kz ? c.zk(i - 1) : c.tmp(2);
+      cx<T>* gU = c.tmp(0);
+      auto Xk = [&](int k) { return kz ? c.xk(k, i - 1) : c.tmp(4); };
+      if (kz || odg) pr.add(pd(V(i - 1), sUV, OP_N, c.g(i - 1), bb, OP_N, nullptr, Zf, 1.0, 0.0));
+      if (!kz) pr.add(pd(c.g(i - 1), bb, OP_N, U(i - 1), sUV, OP_N, nullptr, gU, 1.0, 0.0), reuseA(1));
+      for (int k = 0; k < nrhs; ++k) pr.add(pd(V(i - 1), sUV, OP_N, c.glk(k, i - 1), bb, OP_N, nullptr, Xk(k), 1.0, 0.0));
+      if ((s = run<T>(P, pr, st))) return s;
+      if (kz) pr.add(pd(Zf, bb, OP_N, U(i - 1), sUV, OP_N, gi, gi, -1.0, 1.0));
+      else pr.add(pd(V(i - 1), sUV, OP_N, gU, bb, OP_N, gi, gi, -1.0, 1.0));
+      for (int k = 0; k < nrhs; ++k) pr.add(pd(Xk(k), bb, OP_N, V(i - 1), sUV, OP_C, SLk(k), SLk(k), 1.0, 1.0));
+      auto Yf = [&](int k) { return c.tmp(k ? 6 : 3); };
+      if (odg)  // block-tridiagonal Sigma^<: bracket += -Y + Y^H, Y = V_{i-1} g_{i-1} Sigma^<_{i-1,i}
+        for (int k = 0; k < nrhs; ++k) {
           cx<T>* Lt = load_L(k, i - 1);
           if (!Lt) return QTX_ERR_CUDA;
-          if ((s = gemm<T>(P, gargs<T>(b, b, b, Zf, b, bb, OP_N, Lt, b, sLt, OP_N, nullptr, 0, 0, Yf, b, bb, 1.0, 0.0, ne, nullptr), st))) return s;
-          Term<T> t0; t0.p = SLi; t0.s = bb; t0.alpha = 1.0;
-          Term<T> t1; t1.p = Yf; t1.s = bb; t1.alpha = -1.0;
-          Term<T> t2; t2.p = Yf; t2.s = bb; t2.alpha = 1.0; t2.op = OP_C;
-          QTX_CK((combine<T, T>(SLi, bb, t0, t1, t2, b, ne, nullptr, 0, 0, nullptr, st)));
+          pr.add(pd(Zf, bb, OP_N, Lt, sLt, OP_N, nullptr, Yf(k), 1.0, 0.0));
         }
-      }
-      cx<T>* Y = c.tmp(0);
-      if ((s = gemm<T>(P, gargs<T>(b, b, b, gi, b, bb, OP_N, SLi, b, bb, OP_N, nullptr, 0, 0, Y, b, bb, 1.0, 0.0, ne, nullptr), st,
-                       false, k ? reuseA(1) : keepA(1)))) return s;
-      if ((s = gemm<T>(P, gargs<T>(b, b, b, Y, b, bb, OP_N, gi, b, bb, OP_C, nullptr, 0, 0, c.glk(k, i), b, bb, 1.0, 0.0, ne, nullptr), st))) return s;
-    }  // right-hand sides
+      if ((s = run<T>(P, pr, st))) return s;
+      if (odg)
+        for (int k = 0; k < nrhs; ++k) {
+          Term<T> t0; t0.p = SLk(k); t0.s = bb; t0.alpha = 1.0;
+          Term<T> t1; t1.p = Yf(k); t1.s = bb; t1.alpha = -1.0;
+          Term<T> t2; t2.p = Yf(k); t2.s = bb; t2.alpha = 1.0; t2.op = OP_C;
+          QTX_CK((combine<T, T>(SLk(k), bb, t0, t1, t2, b, ne, nullptr, 0, 0, nullptr, st)));
+        }
+    }
+    if ((s = block_inverse<T>(P, gi, b, ne, nullptr, status, st))) return s;
+    // left-connected lesser functions g Sigma g^H
+    auto Yk = [&](int k) { return c.tmp(k ? 6 : 0); };
+    for (int k = 0; k < nrhs; ++k) pr.add(pd(gi, bb, OP_N, SLk(k), bb, OP_N, nullptr, Yk(k), 1.0, 0.0), k ? reuseA(1) : keepA(1));
+    if ((s = run<T>(P, pr, st))) return s;
+    for (int k = 0; k < nrhs; ++k) pr.add(pd(Yk(k), bb, OP_N, gi, bb, OP_C, nullptr, c.glk(k, i), 1.0, 0.0));
+    if ((s = run<T>(P, pr, st))) return s;
     // FPX storage: slices the backward sweep reads back from memory (the last two stay in the
     // working blocks) are kept compressed
     if (d.storage_bits && i < nb - 2) {
@@ -998,89 +1068,90 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
     }
   }
   for (int i = nb - 2; i >= 0; --i) {
+    const bool kz = c.keep_z();
     cx<T>* GRn = c.g(i + 1);
     cx<T>* Pm = c.tmp(2);
-    cx<T>* Z = c.keep_z() ? c.zk(i) : c.tmp(3);  // V_i g_i
+    cx<T>* Z = kz ? c.zk(i) : c.tmp(3);  // V_i g_i
     cx<T>* GRl = c.tmp(4);
     cx<T>* GRu = c.tmp(5);
-    cx<T>* Qw = c.tmp(6);
-    cx<T>* Tm = c.tmp(7);
-    cx<T>* PGL = c.tmp(8);
-    cx<T>* X2 = c.tmp(9);
     cx<T>* GLu = c.tmp(10);
     cx<T>* gi = c.g(i);
+    // per right-hand side (the second one comes with kept Z and X only)
+    auto Qk = [&](int k) { return kz ? c.xk(k, i) : c.tmp(6); };  // V_i g^<_i: the forward sweep's X when kept
+    auto X2k = [&](int k) { return c.tmp(k ? 3 : 9); };
+    auto PGLk = [&](int k) { return c.tmp(k ? 11 : 8); };
+    auto Tk = [&](int k) { return c.tmp(k ? 6 : 7); };
+    auto Rl = [&](int k) { return c.tmp(13 + k); };               // g_i L_k with L_k its upper block
     if (d.storage_bits && i < nb - 2) {  // g_i, g^<_i back from FPX into the working blocks
       QTX_CK(fpx_load<T>(d.storage_bits, c.gfx(i), (long)ne * bb, gi, st));
       QTX_CK(fpx_load<T>(d.storage_bits, c.glfx(i), (long)ne * bb, c.gl(i), st));
     }
-    auto MM = [&](const cx<T>* A, long sA_, int opA, const cx<T>* B, long sB_, int opB, const cx<T>* C0, cx<T>* C, double al, double be,
-                  DigitHint h = DigitHint{}) {
-      return gemm<T>(P, gargs<T>(b, b, b, A, b, sA_, opA, B, b, sB_, opB, C0, b, bb, C, b, bb, al, be, ne, nullptr), st, false, h);
-    };
     // kept digit planes (tensor-core modes): slot 0 = P (left operand of three or four products), slot 1 =
     // G_{i+1,i+1} (left operand of two)
-    if ((s = MM(gi, bb, OP_N, U(i), sUV, OP_N, nullptr, Pm, 1.0, 0.0))) return s;
-    if (!c.keep_z() && (s = MM(V(i), sUV, OP_N, gi, bb, OP_N, nullptr, Z, 1.0, 0.0))) return s;
-    // block-tridiagonal right-hand side k: g_i L_k with L_k its upper block (g_i still left-connected)
-    auto Rl = [&](int k) { return odg ? c.tmp(13 + k) : nullptr; };
-    if (odg) {
-      for (int k = 0; k < nrhs; ++k) {
+    pr.add(pd(gi, bb, OP_N, U(i), sUV, OP_N, nullptr, Pm, 1.0, 0.0));
+    if (!kz) {
+      pr.add(pd(V(i), sUV, OP_N, gi, bb, OP_N, nullptr, Z, 1.0, 0.0));
+      pr.add(pd(V(i), sUV, OP_N, c.gl(i), bb, OP_N, nullptr, Qk(0), 1.0, 0.0));
+    }
+    if (odg)
+      for (int k = 0; k < nrhs; ++k) {  // g_i still left-connected
         cx<T>* Lt = load_L(k, i);
         if (!Lt) return QTX_ERR_CUDA;
-        if ((s = MM(gi, bb, OP_N, Lt, sLt, OP_N, nullptr, Rl(k), 1.0, 0.0))) return s;
+        pr.add(pd(gi, bb, OP_N, Lt, sLt, OP_N, nullptr, Rl(k), 1.0, 0.0));
       }
-    }
-    if ((s = MM(GRn, bb, OP_N, Z, bb, OP_N, nullptr, GRl, -1.0, 0.0, keepA(1)))) return s;
+    if ((s = run<T>(P, pr, st))) return s;
+    if (odg)
+      for (int k = 0; k < nrhs; ++k) {  // Q = V_i g^<_i + (g_i Sigma^<_{i,i+1})^H
+        Term<T> t0; t0.p = Qk(k); t0.s = bb; t0.alpha = 1.0;
+        Term<T> t1; t1.p = Rl(k); t1.s = bb; t1.alpha = 1.0; t1.op = OP_C;
+        QTX_CK((combine<T, T>(Qk(k), bb, t0, t1, none, b, ne, nullptr, 0, 0, nullptr, st)));
+      }
     // G_{i,i+1} only where it is an output (itself, or in G^>_{i,i+1}) or the balance check's K needs it
     const bool want_u = want(QTX_OUT_GR_UPPER, out->GR_upper) || (!d.second_rhs && want(QTX_OUT_GG_UPPER, out->GG_upper)) || cont;
-    if (want_u && (s = MM(Pm, bb, OP_N, GRn, bb, OP_N, nullptr, GRu, -1.0, 0.0, keepA(0)))) return s;
-    if ((s = MM(Pm, bb, OP_N, GRl, bb, OP_N, gi, gi, -1.0, 1.0, want_u ? reuseA(0) : keepA(0)))) return s;   // g_i <- G_ii
-    if (want(QTX_OUT_GR_DIAG, out->GR_diag) && (s = emit<T>(P, out->GR_diag, nb, i, e0, gi, b, ne, st))) return s;
+    pr.add(pd(GRn, bb, OP_N, Z, bb, OP_N, nullptr, GRl, -1.0, 0.0), keepA(1));
+    for (int k = 0; k < nrhs; ++k) pr.add(pd(GRn, bb, OP_N, Qk(k), bb, OP_N, nullptr, X2k(k), 1.0, 0.0), reuseA(1));
+    for (int k = 0; k < nrhs; ++k) pr.add(pd(Pm, bb, OP_N, c.glk(k, i + 1), bb, OP_N, nullptr, PGLk(k), 1.0, 0.0), k ? reuseA(0) : keepA(0));
+    if (want_u) pr.add(pd(Pm, bb, OP_N, GRn, bb, OP_N, nullptr, GRu, -1.0, 0.0), reuseA(0));
+    if ((s = run<T>(P, pr, st))) return s;
     if (want(QTX_OUT_GR_UPPER, out->GR_upper) && (s = emit<T>(P, out->GR_upper, nb - 1, i, e0, GRu, b, ne, st))) return s;
     if (want(QTX_OUT_GR_LOWER, out->GR_lower) && (s = emit<T>(P, out->GR_lower, nb - 1, i, e0, GRl, b, ne, st))) return s;
-    // lesser-type blocks of each right-hand side on the shared retarded ones
+    // G^<_{i,i+1}, written where an output or the balance reads it, with its current trace; X2 becomes the
+    // right operand of T
+    void* traces = c.tmp(0);  // (tmp 0 and 1: lesser_scratch_bytes exceeds one block for b = 1)
+    const bool cur_out = !d.system_input;
     for (int k = 0; k < nrhs; ++k) {
-      cx<T>* gli = c.glk(k, i);
-      cx<T>* GLn = c.glk(k, i + 1);
-      // Q = V_i g^<_i: the forward sweep's X of slice i + 1 when kept
-      cx<T>* Q = c.keep_z() ? c.xk(k, i) : Qw;
-      if (!c.keep_z() && (s = MM(V(i), sUV, OP_N, gli, bb, OP_N, nullptr, Q, 1.0, 0.0))) return s;
-      if (odg) {  // Q = V_i g^<_i + (g_i Sigma^<_{i,i+1})^H
-        Term<T> t0; t0.p = Q; t0.s = bb; t0.alpha = 1.0;
-        Term<T> t1; t1.p = Rl(k); t1.s = bb; t1.alpha = 1.0; t1.op = OP_C;
-        QTX_CK((combine<T, T>(Q, bb, t0, t1, none, b, ne, nullptr, 0, 0, nullptr, st)));
-      }
-      if ((s = MM(GRn, bb, OP_N, Q, bb, OP_N, nullptr, X2, 1.0, 0.0, reuseA(1)))) return s;
-      if ((s = MM(Pm, bb, OP_N, GLn, bb, OP_N, nullptr, PGL, 1.0, 0.0, reuseA(0)))) return s;
-      // G^<_{i,i+1} is written where an output or the balance reads it; its current trace comes with it
-      const bool up_k = k ? want(QTX_OUT_GG_UPPER, out->GG_upper)
-                          : want(QTX_OUT_GL_UPPER, out->GL_upper) || (!d.second_rhs && want(QTX_OUT_GG_UPPER, out->GG_upper)) || cont;
-      const bool cur_k = k == 0 && !d.system_input;
-      void* traces = c.tmp(0);  // (tmp 0 and 1: lesser_scratch_bytes exceeds one block for b = 1)
-      QTX_CK(lesser_offdiag<T>(PGL, X2, up_k ? GLu : nullptr, cur_k ? Hu + (long)i * bb : nullptr,
-                               cur_k && Su ? Su + (long)i * bb : nullptr, c.E, b, ne, traces, st));
-      if (cont) {
-        // plans that check the current balance form K and the congruence apart: T - T^H is anti-Hermitian
-        // whatever the rounding, so the balance would no longer see the part of it that the check measures
-        if ((s = MM(GRu, bb, OP_N, Q, bb, OP_N, nullptr, Tm, -1.0, 0.0))) return s;
-        if ((s = MM(PGL, bb, OP_N, Pm, bb, OP_C, gli, gli, 1.0, 1.0))) return s;
-      } else if ((s = MM(Pm, bb, OP_N, X2, bb, OP_N, nullptr, Tm, 1.0, 0.0, reuseA(0)))) {
-        return s;
-      }
-      const long o64 = ((long)e0 * nb + i) * bb;
-      void* gd = k ? (want(QTX_OUT_GG_DIAG, out->GG_diag) ? out->GG_diag : nullptr)
-                   : (want(QTX_OUT_GL_DIAG, out->GL_diag) ? out->GL_diag : nullptr);
-      QTX_CK(lesser_diag<T>(gli, Tm, gd ? reinterpret_cast<cx<double>*>(gd) + o64 : nullptr, (long)nb * bb,
-                            cur_k ? cur + i : nullptr, ncur, k ? spare : den + i, k ? 1 : nb, b, ne, traces, st));   // G^<_ii
+      const bool gg = !d.second_rhs && want(QTX_OUT_GG_UPPER, out->GG_upper);
+      const bool up = k ? want(QTX_OUT_GG_UPPER, out->GG_upper) : want(QTX_OUT_GL_UPPER, out->GL_upper) || gg || cont;
+      const bool ck = k == 0 && cur_out;
+      QTX_CK(lesser_offdiag<T>(PGLk(k), X2k(k), up ? GLu : nullptr, ck ? Hu + (long)i * bb : nullptr,
+                               ck && Su ? Su + (long)i * bb : nullptr, c.E, b, ne, traces, st));
       if (k == 1) {  // the second right-hand side's blocks are the GG outputs
-        if (up_k && (s = emit<T>(P, out->GG_upper, nb - 1, i, e0, GLu, b, ne, st))) return s;
+        if (up && (s = emit<T>(P, out->GG_upper, nb - 1, i, e0, GLu, b, ne, st))) return s;
         continue;
       }
       if (want(QTX_OUT_GL_UPPER, out->GL_upper) && (s = emit<T>(P, out->GL_upper, nb - 1, i, e0, GLu, b, ne, st))) return s;
-      if (!d.second_rhs) {
-        if (want(QTX_OUT_GG_DIAG, out->GG_diag) && (s = emit<T>(P, out->GG_diag, nb, i, e0, gli, b, ne, st, gi, gi))) return s;
-        if (want(QTX_OUT_GG_UPPER, out->GG_upper) && (s = emit<T>(P, out->GG_upper, nb - 1, i, e0, GLu, b, ne, st, GRu, GRl))) return s;
-      }
+      if (gg && (s = emit<T>(P, out->GG_upper, nb - 1, i, e0, GLu, b, ne, st, GRu, GRl))) return s;
+    }
+    pr.add(pd(Pm, bb, OP_N, GRl, bb, OP_N, gi, gi, -1.0, 1.0), reuseA(0));   // g_i <- G_ii
+    if (cont) {
+      // plans that check the current balance form K and the congruence apart: T - T^H is anti-Hermitian
+      // whatever the rounding, so the balance would no longer see the part of it that the check measures
+      pr.add(pd(GRu, bb, OP_N, Qk(0), bb, OP_N, nullptr, Tk(0), -1.0, 0.0));
+      pr.add(pd(PGLk(0), bb, OP_N, Pm, bb, OP_C, c.gl(i), c.gl(i), 1.0, 1.0));
+    } else {
+      for (int k = 0; k < nrhs; ++k) pr.add(pd(Pm, bb, OP_N, X2k(k), bb, OP_N, nullptr, Tk(k), 1.0, 0.0), reuseA(0));
+    }
+    if ((s = run<T>(P, pr, st))) return s;
+    if (want(QTX_OUT_GR_DIAG, out->GR_diag) && (s = emit<T>(P, out->GR_diag, nb, i, e0, gi, b, ne, st))) return s;
+    for (int k = 0; k < nrhs; ++k) {
+      cx<T>* gli = c.glk(k, i);
+      const long o64 = ((long)e0 * nb + i) * bb;
+      void* gd = k ? (want(QTX_OUT_GG_DIAG, out->GG_diag) ? out->GG_diag : nullptr)
+                   : (want(QTX_OUT_GL_DIAG, out->GL_diag) ? out->GL_diag : nullptr);
+      QTX_CK(lesser_diag<T>(gli, Tk(k), gd ? reinterpret_cast<cx<double>*>(gd) + o64 : nullptr, (long)nb * bb,
+                            k == 0 && cur_out ? cur + i : nullptr, ncur, k ? spare : den + i, k ? 1 : nb, b, ne, traces, st));   // G^<_ii
+      if (k == 1) continue;
+      if (!d.second_rhs && want(QTX_OUT_GG_DIAG, out->GG_diag) && (s = emit<T>(P, out->GG_diag, nb, i, e0, gli, b, ne, st, gi, gi))) return s;
       if (cont)
         QTX_CK(obs_balance<T>(bal + i, bscale + i, bgn + i, bhn + i, nb, sigL(i), sigR(i), sSig, gi, gli, bb, eta, b,
                               ne, st, Hd + (long)i * bb, Hu + (long)i * bb, Su ? Su + (long)i * bb : nullptr, c.E, GLu));
@@ -1880,6 +1951,8 @@ struct qtx_rgf_group_s {
 };
 
 namespace {
+
+bool group_pools(qtx_rgf_plan_s* P) { return P->group && P->group->pool_tiles > 0; }
 
 cudaError_t group_gemm(qtx_rgf_plan_s* P, const TcArgs& a, int digits, cudaStream_t st) {
   qtx_rgf_group_s* G = P->group;

@@ -444,19 +444,36 @@ __device__ __forceinline__ uint32_t bf16x2_bits(float lo_half, float hi_half) {
 // flip, exact).  Rows r >= R and k >= K are written as zero digits, with exponent -1000.
 __host__ __device__ constexpr int strip_skew(int k) { return k + (k >> 3); }
 
+// One operand to digitise; a launch takes up to kTcMaxJobs of one element type (blockIdx.z), e.g. both
+// operands of a product, or those of several products launched together.
+struct DigitJob {
+  const void* X;
+  long ldx, sX;
+  int R, K, R_pad, K_pad, transposed, conj, side, P, batch;
+  int* eout;
+  unsigned char* planes;
+  const int* active;
+};
+constexpr int kTcMaxJobs = 2 * kTcMaxGroup;
+struct DigitJobs {
+  DigitJob j[kTcMaxJobs];
+};
+
 template <int S, int RPC, typename TI>
-__global__ void __launch_bounds__(32 * RPC) k_digitize_rows(const cx<TI>* X, long ldx, long sX, int R, int K, int R_pad,
-                                                       int K_pad, int transposed, int conj_, int side, int* eout,
-                                                       int P, unsigned char* planes, long rows_plane,
-                                                       const int* active) {
+__global__ void __launch_bounds__(32 * RPC) k_digitize_rows(const __grid_constant__ DigitJobs jobs) {
+  const DigitJob& job = jobs.j[blockIdx.z];
   const int e = blockIdx.y;
-  if (active && !active[e]) return;
+  const int R = job.R, K = job.K, R_pad = job.R_pad, K_pad = job.K_pad, side = job.side, P = job.P;
+  const int transposed = job.transposed, conj_ = job.conj;
+  const long ldx = job.ldx;
+  int* eout = job.eout;
+  if (e >= job.batch || (int)blockIdx.x * RPC >= R_pad || (job.active && !job.active[e])) return;
   extern __shared__ __align__(16) unsigned char dsm[];
   const int ldS = strip_skew(K_pad) + 1;  // complex elements per strip row
   cx<df>* strip = reinterpret_cast<cx<df>*>(dsm);
   __shared__ int s_ex[RPC];
   constexpr int NT = 32 * RPC;  // threads: one warp per strip row
-  const cx<TI>* Xe = X + (long)e * sX;
+  const cx<TI>* Xe = static_cast<const cx<TI>*>(job.X) + (long)e * job.sX;
   // an element as df32 (FP32 inputs: lo = 0)
   auto ld = [&](long off) -> cx<df> {
     const cx<TI> x = Xe[off];
@@ -522,8 +539,8 @@ __global__ void __launch_bounds__(32 * RPC) k_digitize_rows(const cx<TI>* X, lon
   // sub-tiles holding Re, Im and -Im (the producer pairs them into the (Re, Im) and (-Im, Re) rows).
   const long nks = 2L * K_pad / BKS, nkb = K_pad / BKS;
   constexpr int BNC = bnc_of(S), SUB_B = sub_b_of(S);
-  const long plane_bytes = side == 0 ? (rows_plane / BM) * nks * (long)TILE_A : (long)(R_pad / BNC) * nkb * 3 * SUB_B;
-  unsigned char* pe = planes + (long)e * S * plane_bytes;
+  const long plane_bytes = side == 0 ? (long)(R_pad / BM) * nks * TILE_A : (long)(R_pad / BNC) * nkb * 3 * SUB_B;
+  unsigned char* pe = job.planes + (long)e * S * plane_bytes;
   const int nkc = K_pad / 8;
   // rows whose planes are written: right-operand columns past N rounded up to 8 are never read (the
   // last column tile's MMA takes only its first bn_last rows), so they stay unwritten
@@ -632,64 +649,88 @@ inline Scratch carve(void* base, const Dims& d, int batch, int S) {
   return s;
 }
 
+// Launch the digitisation of n operands of element type TI.
 template <int S, typename TI>
-cudaError_t digitize_as(const cx<TI>* X, long ldx, long sX, int opX, int side, int R, int K, const Dims& d,
-                     int* eout, unsigned char* planes, int batch, const int* active, cudaStream_t st) {
-  // logical row r of the operand: left A = op(X): row r of op(X); right B = op(X): column r of op(X)
-  //   left  N: X[r][k] direct      left  H: conj(X[k][r]) transposed
-  //   right N: X[k][r] transposed  right H: conj(X[r][k]) direct
-  const int transposed = (side == 0) ? (opX == OP_C) : (opX == OP_N);
-  const int cj = opX == OP_C;
-  const int R_pad = side == 0 ? d.M_pad : d.N_pad;
-  const long rows_plane = side == 0 ? d.M_pad : 2L * d.N_pad;
+cudaError_t digitize_as(const DigitJob* const* jobs, int n, cudaStream_t st) {
+  if (n < 1) return cudaSuccess;
+  DigitJobs all;
+  int R_pad = 0, K_pad = 0, batch = 0;
+  for (int q = 0; q < n; ++q) {
+    all.j[q] = *jobs[q];
+    R_pad = R_pad > all.j[q].R_pad ? R_pad : all.j[q].R_pad;
+    K_pad = K_pad > all.j[q].K_pad ? K_pad : all.j[q].K_pad;
+    batch = batch > all.j[q].batch ? batch : all.j[q].batch;
+  }
   // fused pass: RPC rows per CTA with one warp per row -- two rows while the strip stays within
   // 48 KB of shared memory (many small CTAs per SM, so loads, digit arithmetic and stores of
   // different CTAs overlap), else a single row up to the 200 KB the kernel is allowed
-  const size_t row_bytes = (size_t)(strip_skew(d.K_pad) + 1) * sizeof(cx<df>);
+  const size_t row_bytes = (size_t)(strip_skew(K_pad) + 1) * sizeof(cx<df>);
   const int rpc = 2 * row_bytes <= 48 * 1024 ? 2 : 1;
   if (rpc * row_bytes > 200 * 1024) return cudaErrorInvalidValue;  // K-chunks of <= 1024 always fit
-  {
-    static bool attr = false;
-    if (!attr) {
-      cudaError_t ea = cudaFuncSetAttribute(k_digitize_rows<S, 2, TI>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      if (ea == cudaSuccess) ea = cudaFuncSetAttribute(k_digitize_rows<S, 1, TI>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-      if (ea != cudaSuccess) return ea;
-      attr = true;
-    }
-    const size_t smem = rpc * row_bytes;
-    dim3 g(R_pad / rpc, batch);
-    if (rpc == 2)
-      k_digitize_rows<S, 2, TI><<<g, 64, smem, st>>>(X, ldx, sX, R, K, R_pad, d.K_pad, transposed, cj, side, eout, d.P, planes, rows_plane, active);
-    else
-      k_digitize_rows<S, 1, TI><<<g, 32, smem, st>>>(X, ldx, sX, R, K, R_pad, d.K_pad, transposed, cj, side, eout, d.P, planes, rows_plane, active);
-    count_launch();
-    return cudaGetLastError();
+  static std::atomic<unsigned long long> done2{0}, done1{0};
+  cudaError_t e = rpc == 2 ? allow_smem(k_digitize_rows<S, 2, TI>, 200 * 1024, done2) : allow_smem(k_digitize_rows<S, 1, TI>, 200 * 1024, done1);
+  if (e != cudaSuccess) return e;
+  const size_t smem = rpc * row_bytes;
+  const dim3 g((R_pad + rpc - 1) / rpc, batch, n);
+  if (rpc == 2) k_digitize_rows<S, 2, TI><<<g, 64, smem, st>>>(all);
+  else k_digitize_rows<S, 1, TI><<<g, 32, smem, st>>>(all);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// Operands waiting to be digitised, by element type; flush launches each type's at once.
+struct DigitQueue {
+  DigitJob job[kTcMaxJobs];
+  Elt type[kTcMaxJobs];
+  int n = 0;
+};
+template <int S>
+cudaError_t flush(DigitQueue& q, cudaStream_t st) {
+  for (Elt t : {EL_DF, EL_F32, EL_F64}) {
+    const DigitJob* sel[kTcMaxJobs];
+    int n = 0;
+    for (int k = 0; k < q.n; ++k)
+      if (q.type[k] == t) sel[n++] = &q.job[k];
+    if (!n) continue;
+    cudaError_t e = cudaErrorInvalidValue;
+    if (t == EL_DF) e = digitize_as<S, df>(sel, n, st);
+    if (t == EL_F64) e = digitize_as<S, double>(sel, n, st);
+    if constexpr (S == 4)  // FP32 operands: four digit planes only
+      if (t == EL_F32) e = digitize_as<S, float>(sel, n, st);
+    if (e != cudaSuccess) return e;
   }
+  q.n = 0;
+  return cudaSuccess;
+}
+inline void queue_operand(DigitQueue& q, const void* X, Elt type, long ldx, long sX, int opX, int side, int R, int K, const Dims& d,
+                          int* eout, unsigned char* planes, int batch, const int* active) {
+  // logical row r of the operand: left A = op(X): row r of op(X); right B = op(X): column r of op(X)
+  //   left  N: X[r][k] direct      left  H: conj(X[k][r]) transposed
+  //   right N: X[k][r] transposed  right H: conj(X[r][k]) direct
+  DigitJob& j = q.job[q.n];
+  j.X = X; j.ldx = ldx; j.sX = sX;
+  j.R = R; j.K = K;
+  j.R_pad = side == 0 ? d.M_pad : d.N_pad;
+  j.K_pad = d.K_pad;
+  j.transposed = (side == 0) ? (opX == OP_C) : (opX == OP_N);
+  j.conj = opX == OP_C;
+  j.side = side;
+  j.P = d.P;
+  j.batch = batch;
+  j.eout = eout;
+  j.planes = planes;
+  j.active = active;
+  q.type[q.n++] = type;
 }
 
-// ... by the operand's element type (FP32 operands: four digit planes only)
+// Queue the digitisation of one product's operands (into the scratch, or a kept operand) and fill its
+// kernel parameters and tile counts.
 template <int S>
-cudaError_t digitize(const cx<df>* X, Elt type, long ldx, long sX, int opX, int side, int R, int K, const Dims& d, int* eout,
-                     unsigned char* planes, int batch, const int* active, cudaStream_t st) {
-  if (type == EL_F64)
-    return digitize_as<S, double>(reinterpret_cast<const cx<double>*>(X), ldx, sX, opX, side, R, K, d, eout, planes, batch, active, st);
-  if constexpr (S == 4)
-    if (type == EL_F32)
-      return digitize_as<S, float>(reinterpret_cast<const cx<float>*>(X), ldx, sX, opX, side, R, K, d, eout, planes, batch, active, st);
-  if (type != EL_DF) return cudaErrorInvalidValue;
-  return digitize_as<S, df>(X, ldx, sX, opX, side, R, K, d, eout, planes, batch, active, st);
-}
-
-// Digitise one product's operands (into the scratch, or a kept operand) and fill its kernel
-// parameters and tile counts.
-template <int S>
-cudaError_t prepare(const TcArgs& a, void* scratch, size_t scratch_bytes, int* err_flag, cudaStream_t st,
-                    TcPrepared& out) {
+cudaError_t prepare(const TcArgs& a, void* scratch, size_t scratch_bytes, int* err_flag, DigitQueue& queue, TcPrepared& out) {
   TcParams& p = out.p;
   const Dims d = dims_of(a.M, a.N, a.K, S);
   Scratch sc = carve(scratch, d, a.batch, S);
   if (sc.bytes > scratch_bytes) return cudaErrorInvalidValue;
-  cudaError_t e;
   const int ab = a.sA != 0, bb_ = a.sB != 0;
   // digit planes and exponents of each operand: in the scratch, or (left operand) in a kept operand,
   // digitised there now or reused as they are
@@ -698,8 +739,8 @@ cudaError_t prepare(const TcArgs& a, void* scratch, size_t scratch_bytes, int* e
   int* ea = a.opndA ? a.opndA->expo : sc.ea;
   int* eb = sc.eb;
   if (!(a.opndA && a.opndA->mode == 2))
-    if ((e = digitize<S>(a.A, a.ta, a.lda, a.sA, a.opA, 0, a.M, a.K, d, ea, pa, ab ? a.batch : 1, ab ? a.active : nullptr, st))) return e;
-  if ((e = digitize<S>(a.B, a.tb, a.ldb, a.sB, a.opB, 1, a.N, a.K, d, eb, pb, bb_ ? a.batch : 1, bb_ ? a.active : nullptr, st))) return e;
+    queue_operand(queue, a.A, a.ta, a.lda, a.sA, a.opA, 0, a.M, a.K, d, ea, pa, ab ? a.batch : 1, ab ? a.active : nullptr);
+  queue_operand(queue, a.B, a.tb, a.ldb, a.sB, a.opB, 1, a.N, a.K, d, eb, pb, bb_ ? a.batch : 1, bb_ ? a.active : nullptr);
   p.pa = pa;
   p.pb = pb;
   p.eA = ea;
@@ -845,19 +886,39 @@ int gemm_tc_variant(const TcArgs& a, int digits) {
   return S * 3 + (int)a.tc + 100 * resolve_stages(S, a.stages);
 }
 
+cudaError_t gemm_tc_prepare_many(const TcArgs* a, const int* digits, int n, void* const* scratch, size_t scratch_bytes, int* err_flag,
+                                 cudaStream_t st, TcPrepared* out) {
+  if (n < 1 || n > kTcMaxGroup) return cudaErrorInvalidValue;
+  tc::DigitQueue queue;
+  int S = 0;
+  for (int q = 0; q < n; ++q) {
+    out[q].variant = gemm_tc_variant(a[q], digits[q]);
+    out[q].ctas = a[q].ctas;
+    out[q].tiles = 0;
+    if (out[q].variant < 0 || (q && out[q].variant % 100 / 3 != S)) return cudaErrorInvalidValue;
+    S = out[q].variant % 100 / 3;
+    if (a[q].M <= 0 || a[q].N <= 0 || a[q].batch <= 0) continue;
+    cudaError_t e = cudaErrorInvalidValue;
+    switch (S) {
+      case 4: e = tc::prepare<4>(a[q], scratch[q], scratch_bytes, err_flag, queue, out[q]); break;
+      case 7: e = tc::prepare<7>(a[q], scratch[q], scratch_bytes, err_flag, queue, out[q]); break;
+      case 6: e = tc::prepare<6>(a[q], scratch[q], scratch_bytes, err_flag, queue, out[q]); break;
+      case 2: e = tc::prepare<2>(a[q], scratch[q], scratch_bytes, err_flag, queue, out[q]); break;
+    }
+    if (e != cudaSuccess) return e;
+  }
+  switch (S) {
+    case 4: return tc::flush<4>(queue, st);
+    case 7: return tc::flush<7>(queue, st);
+    case 6: return tc::flush<6>(queue, st);
+    case 2: return tc::flush<2>(queue, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
 cudaError_t gemm_tc_prepare(const TcArgs& a, int digits, void* scratch, size_t scratch_bytes, int* err_flag,
                             cudaStream_t st, TcPrepared* out) {
-  out->variant = gemm_tc_variant(a, digits);
-  out->ctas = a.ctas;
-  out->tiles = 0;
-  if (a.M <= 0 || a.N <= 0 || a.batch <= 0) return cudaSuccess;
-  switch (out->variant % 100 / 3) {
-    case 4: return tc::prepare<4>(a, scratch, scratch_bytes, err_flag, st, *out);
-    case 7: return tc::prepare<7>(a, scratch, scratch_bytes, err_flag, st, *out);
-    case 6: return tc::prepare<6>(a, scratch, scratch_bytes, err_flag, st, *out);
-    case 2: return tc::prepare<2>(a, scratch, scratch_bytes, err_flag, st, *out);
-    default: return cudaErrorInvalidValue;
-  }
+  return gemm_tc_prepare_many(&a, &digits, 1, &scratch, scratch_bytes, err_flag, st, out);
 }
 
 cudaError_t gemm_tc_launch(const TcPrepared* const* p, int n, cudaStream_t st, cudaEvent_t* ev) {

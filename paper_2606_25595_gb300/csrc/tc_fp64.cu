@@ -277,18 +277,32 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__
 // and writes 36 (left) or 54 B (right operand: Re, Im, -Im) per complex value.
 __host__ __device__ constexpr int skew9(int k) { return k + (k >> 3); }
 
+// Both operands of a product share the launch (blockIdx.z).
+struct Operand {
+  const cx<double>* X;
+  long ldx, sX;
+  int R, R_pad, transposed, conj, batch;
+  int* eout;
+  unsigned char* planes;
+  const int* active;
+};
+struct Operands {
+  Operand o[2];  // left, right
+};
 template <int RPC>
-__global__ void __launch_bounds__(32 * RPC) k_digitize_fp64(const cx<double>* X, long ldx, long sX, int R, int K, int R_pad,
-                                                            int K_pad, int transposed, int conj_, int side, int* eout, int P,
-                                                            unsigned char* planes, const int* active) {
-  const int e = blockIdx.y;
-  if (active && !active[e]) return;
+__global__ void __launch_bounds__(32 * RPC) k_digitize_fp64(const __grid_constant__ Operands ops, int K, int K_pad, int P) {
+  const int side = blockIdx.z, e = blockIdx.y;
+  const Operand& op = ops.o[side];
+  const int R = op.R, R_pad = op.R_pad, transposed = op.transposed, conj_ = op.conj;
+  const long ldx = op.ldx;
+  if (e >= op.batch || (int)blockIdx.x * RPC >= R_pad || (op.active && !op.active[e])) return;
   extern __shared__ __align__(16) unsigned char dsm[];
   constexpr int NT = 32 * RPC;
   const int ldS = skew9(K_pad) + 1;
   cx<double>* strip = reinterpret_cast<cx<double>*>(dsm);
   __shared__ int s_ex[RPC];
-  const cx<double>* Xe = X + (long)e * sX;
+  const cx<double>* Xe = op.X + (long)e * op.sX;
+  int* eout = op.eout;
   const int r0 = blockIdx.x * RPC, t = threadIdx.x;
   if (t < RPC) s_ex[t] = kExpoZero;
   __syncthreads();
@@ -321,7 +335,7 @@ __global__ void __launch_bounds__(32 * RPC) k_digitize_fp64(const cx<double>* X,
   if (t < RPC && r0 + t < R_pad) eout[(long)e * R_pad + r0 + t] = s_ex[t];
   const long nks = 2L * K_pad / BKS, nkb = K_pad / BKS;
   const long plane_bytes = side == 0 ? (long)(R_pad / BM) * nks * TILE_A : (long)(R_pad / BNC9) * nkb * 3 * SUB_B9;
-  unsigned char* pe = planes + (long)e * S9 * plane_bytes;
+  unsigned char* pe = op.planes + (long)e * S9 * plane_bytes;
   const int nkc = K_pad / 8;
   const int R_wr = side == 1 ? min(R_pad, (R + 7) / 8 * 8) : R_pad;  // columns past bn_last are never read
 #pragma unroll 1
@@ -403,14 +417,15 @@ int chunk_k(int K) {
   return nc <= 1 ? K : (K + nc - 1) / nc;
 }
 
-cudaError_t digitize9(const cx<double>* X, long ldx, long sX, int opX, int side, int R, int K, const Dims9& d, int* eout,
-                      unsigned char* planes, int batch, const int* active, cudaStream_t st) {
-  const int transposed = (side == 0) ? (opX == OP_C) : (opX == OP_N);
-  const int R_pad = side == 0 ? d.M_pad : d.N_pad;
+cudaError_t digitize9(const GemmArgs<double>& g, const Dims9& d, int* eA, unsigned char* pa, int na, int* eB, unsigned char* pb,
+                      int nb, cudaStream_t st) {
   constexpr int RPC = 4;  // transposed strips read four values of 16 bytes in a row: whole 32-byte sectors
   const size_t smem = (size_t)RPC * (skew9(d.K_pad) + 1) * sizeof(cx<double>);  // at most 37 KB
-  k_digitize_fp64<RPC><<<dim3(R_pad / RPC, batch), 32 * RPC, smem, st>>>(X, ldx, sX, R, K, R_pad, d.K_pad, transposed,
-                                                                        opX == OP_C, side, eout, d.P, planes, active);
+  Operands o;
+  o.o[0] = Operand{g.A, g.lda, g.sA, g.M, d.M_pad, g.opA == OP_C, g.opA == OP_C, na, eA, pa, g.sA ? g.active : nullptr};
+  o.o[1] = Operand{g.B, g.ldb, g.sB, g.N, d.N_pad, g.opB == OP_N, g.opB == OP_C, nb, eB, pb, g.sB ? g.active : nullptr};
+  const int R = d.M_pad > d.N_pad ? d.M_pad : d.N_pad;
+  k_digitize_fp64<RPC><<<dim3(R / RPC, na > nb ? na : nb, 2), 32 * RPC, smem, st>>>(o, g.K, d.K_pad, d.P);
   count_launch();
   return cudaGetLastError();
 }
@@ -434,8 +449,7 @@ cudaError_t product9(const GemmArgs<double>& g, unsigned char* scratch, int* err
   unsigned char* pb = pa + na * d.a;
   int* eA = reinterpret_cast<int*>(pb + nb * d.b);
   int* eB = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(eA) + na * d.ea);
-  if ((e = digitize9(g.A, g.lda, g.sA, g.opA, 0, g.M, g.K, d, eA, pa, (int)na, ab ? g.active : nullptr, st))) return e;
-  if ((e = digitize9(g.B, g.ldb, g.sB, g.opB, 1, g.N, g.K, d, eB, pb, (int)nb, bb ? g.active : nullptr, st))) return e;
+  if ((e = digitize9(g, d, eA, pa, (int)na, eB, pb, (int)nb, st))) return e;
   p.pa = pa;
   p.pb = pb;
   p.eA = eA;
