@@ -9,10 +9,8 @@
 // rounds to zero keeps its sign, and the cutoff gives +0.  A stream of n values is the
 // concatenation of their X/8-byte little-endian codes.
 //
-// Kernels: one thread per group of 8 values -- it reads 8 consecutive reals (64 bytes of FP64)
-// and writes the group's X bytes as X/8 aligned 64-bit words (the codes of the group laid end to
-// end), so both sides are contiguous across a warp.  The plan uses the same kernels on its own
-// sweep types (FP64, FP32 and df32 values, converted exactly to FP64 first) to keep the
+// Kernels: one thread per group of 8 values, whose X bytes are X/8 aligned 64-bit words (the codes of
+// the group laid end to end).  The plan uses the same kernels on its own sweep types (FP64, FP32 and df32 values, converted exactly to FP64 first) to keep the
 // left-connected blocks compressed between the forward and the backward sweeps.
 #include <type_traits>
 
@@ -23,8 +21,9 @@
 namespace qtx {
 namespace {
 
+// the general case: specials, zeros, subnormal results and magnitudes below the cutoff
 template <int BITS>
-__device__ __forceinline__ uint64_t fpx_encode(double x, double cutoff) {
+__device__ __noinline__ uint64_t fpx_encode_rare(double x, double cutoff) {
   constexpr int m = BITS - 9;
   const uint64_t u = (uint64_t)__double_as_longlong(x);
   const uint64_t s = u >> 63;
@@ -34,7 +33,8 @@ __device__ __forceinline__ uint64_t fpx_encode(double x, double cutoff) {
     if (f) return (0xFFull << m) | (1ull << (m - 1));
     return (s << (BITS - 1)) | (0xFFull << m);
   }
-  if (fabs(x) < cutoff) return 0;
+  // magnitudes order like their bits
+  if ((u & 0x7fffffffffffffffull) < (uint64_t)__double_as_longlong(cutoff)) return 0;
   if (e == 0) return s << (BITS - 1);  // FP64 zero or subnormal: far below the smallest FPX value
   const int E = e - 1023 + 127;       // FPX biased exponent of the value
   const uint64_t F = (1ull << 52) | f;
@@ -56,6 +56,19 @@ __device__ __forceinline__ uint64_t fpx_encode(double x, double cutoff) {
 }
 
 template <int BITS>
+__device__ __forceinline__ uint64_t fpx_encode(double x, double cutoff) {
+  constexpr int m = BITS - 9, sh = 52 - m;
+  const uint64_t u = (uint64_t)__double_as_longlong(x), v = u & 0x7fffffffffffffffull;
+  const uint32_t e = (uint32_t)(v >> 52);
+  // normal results: exponent and significand rounded as one integer (ties to even; a carry moves on into
+  // the exponent), rebiased; magnitudes order like their bits
+  if (e < 1023 - 126 || e == 0x7ff || v < (uint64_t)__double_as_longlong(cutoff)) return fpx_encode_rare<BITS>(x, cutoff);
+  const uint64_t r = (v + (((uint64_t)1 << (sh - 1)) - 1) + ((v >> sh) & 1)) >> sh;
+  const uint64_t field = r - ((uint64_t)(1023 - 127) << m), inf = (uint64_t)0xFF << m;
+  return ((u >> 63) << (BITS - 1)) | (field < inf ? field : inf);
+}
+
+template <int BITS>
 __device__ __forceinline__ double fpx_decode(uint64_t c) {
   constexpr int m = BITS - 9;
   const uint64_t s = (c >> (BITS - 1)) & 1ull;
@@ -65,109 +78,121 @@ __device__ __forceinline__ double fpx_decode(uint64_t c) {
   if (ef == 0xFF) {
     u = (s << 63) | (0x7FFull << 52) | (q ? (1ull << 51) : 0ull);
   } else if (ef == 0) {
-    // q 2^(-126 - m): exact in FP64 (q < 2^47, no FP64 underflow)
-    const double v = (double)q * __longlong_as_double((long long)((uint64_t)(1023 - 126 - m) << 52));
-    u = (uint64_t)__double_as_longlong(v) | (s << 63);
+    // q 2^(-126 - m): an FP64 normal number (q < 2^47), its leading bit at position p
+    const int p = 63 - __clzll((long long)(q | 1));
+    u = (s << 63) | (q ? ((uint64_t)(p - 126 - m + 1023) << 52) | ((q << (52 - p)) & ((1ull << 52) - 1)) : 0ull);
   } else {
     u = (s << 63) | ((uint64_t)(ef - 127 + 1023) << 52) | (q << (52 - m));
   }
   return __longlong_as_double((long long)u);
 }
 
-// real value k of an FP64 array, or of an array of T-typed complex numbers viewed as 2n reals
-__device__ __forceinline__ double real_at(const double* x, long k) { return x[k]; }
-__device__ __forceinline__ void set_real(double* x, long k, double v) { x[k] = v; }
-template <typename T>
-__device__ __forceinline__ double real_at(const cx<T>* x, long k) {
-  const T v = (k & 1) ? x[k >> 1].im : x[k >> 1].re;
-  if constexpr (std::is_same<T, df>::value) return (double)v.hi + (double)v.lo;  // exact: |lo| <= ulp(hi)/2
-  else return (double)v;
-}
-template <typename T>
-__device__ __forceinline__ void set_real(cx<T>* x, long k, double v) {
-  T t;
-  if constexpr (std::is_same<T, df>::value) {
-    const float hi = __double2float_rn(v);
-    t = mkdf(hi, __double2float_rn(v - (double)hi));
-  } else {
-    t = (T)v;
+// One block codes 2048 reals (256 groups of 8).  A thread's group is 64 consecutive bytes of FP64 and X
+// bytes of codes, so reading and writing it directly touches 32 separate lines a warp and instruction;
+// both sides pass through shared memory instead (skewed: thread-wise and warp-wise accesses fall in
+// distinct banks), and global accesses are whole lines.  PLACEHOLDER
+// -> see kTile below; the conversions of df32 values and the cutoff are integer operations (FP64 pipe).
+constexpr int kT = 256, kTile = 8 * kT;
+__host__ __device__ constexpr int skew(int k) { return k + (k >> 3); }
+
+template <int BITS, typename T>
+__global__ void __launch_bounds__(kT) k_fpx_compress(const T* x, long n, double cutoff, uint64_t* out) {
+  constexpr int W = BITS / 8, LD = W | 1;  // 64-bit words per group of 8 codes
+  __shared__ T s_x[skew(kTile)];
+  __shared__ uint64_t s_w[kT * LD];
+  const long k0 = (long)blockIdx.x * kTile;
+  const int t = threadIdx.x, m = (int)(n - k0 < kTile ? n - k0 : kTile);
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    if (t + kT * j < m) s_x[skew(t + kT * j)] = x[k0 + t + kT * j];
+  __syncthreads();
+  const int groups = (m + 7) / 8;
+  if (t < groups) {
+    uint64_t w[W];
+#pragma unroll
+    for (int i = 0; i < W; ++i) w[i] = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const uint64_t c = 8 * t + j < m ? fpx_encode<BITS>(to_d(s_x[skew(8 * t + j)]), cutoff) : 0ull;
+      const int bit = j * BITS, wi = bit / 64, off = bit % 64;
+      w[wi] |= c << off;
+      if (off + BITS > 64) w[wi + 1] |= c >> (64 - off);
+    }
+#pragma unroll
+    for (int i = 0; i < W; ++i) s_w[t * LD + i] = w[i];
   }
-  if (k & 1) x[k >> 1].im = t;
-  else x[k >> 1].re = t;
+  __syncthreads();
+  uint64_t* o = out + (long)blockIdx.x * kT * W;
+#pragma unroll
+  for (int i = 0; i < W; ++i) {
+    const int q = t + kT * i;
+    if (q < groups * W) o[q] = s_w[q / W * LD + q % W];
+  }
 }
 
-template <int BITS, typename P>
-__global__ void __launch_bounds__(256) k_fpx_compress(const P* x, long n, double cutoff, uint64_t* out) {
-  constexpr int W = BITS / 8;  // 64-bit words per group of 8 codes
-  const long g = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g * 8 >= n) return;
-  uint64_t w[W];
-#pragma unroll
-  for (int i = 0; i < W; ++i) w[i] = 0;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const long k = g * 8 + j;
-    const uint64_t c = k < n ? fpx_encode<BITS>(real_at(x, k), cutoff) : 0ull;
-    const int bit = j * BITS, wi = bit / 64, off = bit % 64;
-    w[wi] |= c << off;
-    if (off + BITS > 64) w[wi + 1] |= c >> (64 - off);
-  }
-#pragma unroll
-  for (int i = 0; i < W; ++i) out[g * W + i] = w[i];
-}
-
-template <int BITS, typename P>
-__global__ void __launch_bounds__(256) k_fpx_decompress(const uint64_t* in, long n, P* x) {
-  constexpr int W = BITS / 8;
+template <int BITS, typename T>
+__global__ void __launch_bounds__(kT) k_fpx_decompress(const uint64_t* in, long n, T* x) {
+  constexpr int W = BITS / 8, LD = W | 1;
   constexpr uint64_t MASK = (1ull << BITS) - 1;
-  const long g = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g * 8 >= n) return;
-  uint64_t w[W];
+  __shared__ T s_x[skew(kTile)];
+  __shared__ uint64_t s_w[kT * LD];
+  const long k0 = (long)blockIdx.x * kTile;
+  const int t = threadIdx.x, m = (int)(n - k0 < kTile ? n - k0 : kTile), groups = (m + 7) / 8;
+  const uint64_t* src = in + (long)blockIdx.x * kT * W;
 #pragma unroll
-  for (int i = 0; i < W; ++i) w[i] = in[g * W + i];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const long k = g * 8 + j;
-    if (k >= n) break;
-    const int bit = j * BITS, wi = bit / 64, off = bit % 64;
-    uint64_t c = w[wi] >> off;
-    if (off + BITS > 64) c |= w[wi + 1] << (64 - off);
-    set_real(x, k, fpx_decode<BITS>(c & MASK));
+  for (int i = 0; i < W; ++i) {
+    const int q = t + kT * i;
+    if (q < groups * W) s_w[q / W * LD + q % W] = src[q];
   }
+  __syncthreads();
+  if (t < groups) {
+    uint64_t w[W];
+#pragma unroll
+    for (int i = 0; i < W; ++i) w[i] = s_w[t * LD + i];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int bit = j * BITS, wi = bit / 64, off = bit % 64;
+      uint64_t c = w[wi] >> off;
+      if (off + BITS > 64) c |= w[wi + 1] << (64 - off);
+      s_x[skew(8 * t + j)] = from_d<T>(fpx_decode<BITS>(c & MASK));
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    if (t + kT * j < m) x[k0 + t + kT * j] = s_x[skew(t + kT * j)];
 }
 
-template <typename P>
-cudaError_t launch_compress(int bits, const P* x, long n, double cutoff, void* out, cudaStream_t st) {
+template <typename T>
+cudaError_t launch_compress(int bits, const T* x, long n, double cutoff, void* out, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  const long groups = (n + 7) / 8;
-  const unsigned blocks = (unsigned)((groups + 255) / 256);
+  const unsigned blocks = (unsigned)((n + kTile - 1) / kTile);
   uint64_t* o = reinterpret_cast<uint64_t*>(out);
   switch (bits) {
-    case 56: k_fpx_compress<56, P><<<blocks, 256, 0, st>>>(x, n, cutoff, o); break;
-    case 48: k_fpx_compress<48, P><<<blocks, 256, 0, st>>>(x, n, cutoff, o); break;
-    case 40: k_fpx_compress<40, P><<<blocks, 256, 0, st>>>(x, n, cutoff, o); break;
-    case 32: k_fpx_compress<32, P><<<blocks, 256, 0, st>>>(x, n, cutoff, o); break;
-    case 24: k_fpx_compress<24, P><<<blocks, 256, 0, st>>>(x, n, cutoff, o); break;
-    case 16: k_fpx_compress<16, P><<<blocks, 256, 0, st>>>(x, n, cutoff, o); break;
+    case 56: k_fpx_compress<56, T><<<blocks, 256, 0, st>>>(x, n, cutoff, o); break;
+    case 48: k_fpx_compress<48, T><<<blocks, 256, 0, st>>>(x, n, cutoff, o); break;
+    case 40: k_fpx_compress<40, T><<<blocks, 256, 0, st>>>(x, n, cutoff, o); break;
+    case 32: k_fpx_compress<32, T><<<blocks, 256, 0, st>>>(x, n, cutoff, o); break;
+    case 24: k_fpx_compress<24, T><<<blocks, 256, 0, st>>>(x, n, cutoff, o); break;
+    case 16: k_fpx_compress<16, T><<<blocks, 256, 0, st>>>(x, n, cutoff, o); break;
     default: return cudaErrorInvalidValue;
   }
   count_launch();
   return cudaGetLastError();
 }
 
-template <typename P>
-cudaError_t launch_decompress(int bits, const void* in, long n, P* x, cudaStream_t st) {
+template <typename T>
+cudaError_t launch_decompress(int bits, const void* in, long n, T* x, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  const long groups = (n + 7) / 8;
-  const unsigned blocks = (unsigned)((groups + 255) / 256);
+  const unsigned blocks = (unsigned)((n + kTile - 1) / kTile);
   const uint64_t* i = reinterpret_cast<const uint64_t*>(in);
   switch (bits) {
-    case 56: k_fpx_decompress<56, P><<<blocks, 256, 0, st>>>(i, n, x); break;
-    case 48: k_fpx_decompress<48, P><<<blocks, 256, 0, st>>>(i, n, x); break;
-    case 40: k_fpx_decompress<40, P><<<blocks, 256, 0, st>>>(i, n, x); break;
-    case 32: k_fpx_decompress<32, P><<<blocks, 256, 0, st>>>(i, n, x); break;
-    case 24: k_fpx_decompress<24, P><<<blocks, 256, 0, st>>>(i, n, x); break;
-    case 16: k_fpx_decompress<16, P><<<blocks, 256, 0, st>>>(i, n, x); break;
+    case 56: k_fpx_decompress<56, T><<<blocks, 256, 0, st>>>(i, n, x); break;
+    case 48: k_fpx_decompress<48, T><<<blocks, 256, 0, st>>>(i, n, x); break;
+    case 40: k_fpx_decompress<40, T><<<blocks, 256, 0, st>>>(i, n, x); break;
+    case 32: k_fpx_decompress<32, T><<<blocks, 256, 0, st>>>(i, n, x); break;
+    case 24: k_fpx_decompress<24, T><<<blocks, 256, 0, st>>>(i, n, x); break;
+    case 16: k_fpx_decompress<16, T><<<blocks, 256, 0, st>>>(i, n, x); break;
     default: return cudaErrorInvalidValue;
   }
   count_launch();
@@ -183,11 +208,11 @@ size_t fpx_bytes(int bits, long n_reals) { return n_reals <= 0 ? 0 : (size_t)((n
 
 template <typename T>
 cudaError_t fpx_store(int bits, const cx<T>* x, long n_complex, void* out, cudaStream_t st) {
-  return launch_compress<cx<T>>(bits, x, 2 * n_complex, 0.0, out, st);
+  return launch_compress<T>(bits, reinterpret_cast<const T*>(x), 2 * n_complex, 0.0, out, st);
 }
 template <typename T>
 cudaError_t fpx_load(int bits, const void* in, long n_complex, cx<T>* x, cudaStream_t st) {
-  return launch_decompress<cx<T>>(bits, in, 2 * n_complex, x, st);
+  return launch_decompress<T>(bits, in, 2 * n_complex, reinterpret_cast<T*>(x), st);
 }
 template cudaError_t fpx_store<double>(int, const cx<double>*, long, void*, cudaStream_t);
 template cudaError_t fpx_store<float>(int, const cx<float>*, long, void*, cudaStream_t);

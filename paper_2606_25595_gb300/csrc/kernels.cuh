@@ -268,6 +268,11 @@ bool gemm_fp64_tc_fits(int M, int N, int K, size_t scratch_bytes);
 cudaError_t gemm_fp64_tc(const GemmArgs<double>& g, void* scratch, size_t scratch_bytes, int* err_flag, cudaStream_t st,
                          cudaEvent_t* ev = nullptr);
 constexpr int tc_pairs_fp64() { return 45; }
+// How many of the first n products (independent of each other) one launch can take with this scratch (at
+// least 1, at most 4), and that launch (for a count of 2 and more).
+int gemm_fp64_tc_many(const GemmArgs<double>* g, int n, size_t scratch_bytes);
+cudaError_t gemm_fp64_tc_launch(const GemmArgs<double>* g, int n, void* scratch, size_t scratch_bytes, int* err_flag,
+                                cudaStream_t st);
 
 // ---- FPX storage codec (fpx.cu): n_complex T-typed complex values <-> their FPX codes
 bool fpx_width_ok(int bits);

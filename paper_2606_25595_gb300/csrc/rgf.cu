@@ -12,6 +12,7 @@
 // safe here for the same reason it is safe between slices: the anti-Hermitian part of M,
 // eta S + Gamma/2, is positive definite, so every leading principal block and every Schur
 // complement is nonsingular.
+#include <algorithm>
 #include <chrono>
 #include <condition_variable>
 #include <cstdio>
@@ -144,13 +145,13 @@ Layout make_layout(const qtx_rgf_desc& d, bool inverse_only = false) {
   const size_t ou = uv_per_energy(d) ? (size_t)(nb > 1 ? nb - 1 : 0) * Ec * bb * es : (size_t)(nb > 1 ? nb - 1 : 0) * bb * es;
   L.U = a.take(ou);
   L.V = a.take(ou);
-  L.ident = a.take(bb * sizeof(cx<double>));
-  L.ident_df = a.take(bb * sizeof(cx<double>));
   // one block shared by every energy (the slice's -(H + Sigma^R) or Sigma^<, converted once)
   L.shared_blk = a.take(d.precision == QTX_FP64 ? 0 : bb * sizeof(cx<double>));
   const bool mixed = d.precision == QTX_EMU64 || d.precision == QTX_BF16X3;
   const bool tc64 = d.precision == QTX_FP64 && b >= kTcF64Min;
   L.refine64 = mixed || tc64;
+  L.ident = a.take(L.refine64 ? bb * sizeof(cx<double>) : 0);
+  L.ident_df = a.take(L.refine64 ? bb * sizeof(cx<double>) : 0);
   L.ref = a.take((L.refine64 || b > kLeafMax) ? 3 * Ec * bb * sizeof(cx<double>) : 0);
   L.f32a = a.take(L.refine64 ? Ec * bb * sizeof(cx<float>) : 0);
   L.f32tmp = a.take(L.refine64 ? Ec * bb * sizeof(cx<float>) + 4096 : 0);
@@ -177,7 +178,8 @@ Layout make_layout(const qtx_rgf_desc& d, bool inverse_only = false) {
     L.tc_bytes = std::max(L.tc_bytes, gemm_tc_scratch_bytes((int)b, (int)b, (int)b, (int)Ec, 4));
   // the FP32 mode's products of 96 and more (four digit planes; the recursive inverse's halves too)
   if (d.precision == QTX_FP32 && b >= 96 && b <= 1024) L.tc_bytes = gemm_tc_scratch_bytes((int)b, (int)b, (int)b, (int)Ec, 4);
-  if (tc64) L.tc_bytes = gemm_fp64_tc_scratch_bytes((int)b, (int)b, (int)b, (int)Ec);
+  // (FP64: digit planes of up to kMany products while they are small, see gemm_fp64_tc_scratch_bytes)
+  if (tc64) L.tc_bytes = gemm_fp64_tc_scratch_bytes((int)b, (int)b, (int)b, (int)(inverse_only ? Ec : kMany * Ec));
   L.tc_scratch = a.take(L.tc_bytes);
   // products of a slice that do not depend on each other share launches while one alone fills less than
   // four waves of the GPU (608 tiles): their further scratch is then a few hundred MB at most, and the
@@ -421,6 +423,16 @@ qtx_status run(qtx_rgf_plan_s* P, Prods<T>& q, cudaStream_t st) {
       }
       QTX_CK(gemm_tc_prepare_many(a, digits, m, scr, P->L.tc_bytes, P->d_err_flag, st, p));
       QTX_CK(gemm_tc_launch(pp, m, st));
+      i += m;
+    }
+  }
+  if constexpr (std::is_same<T, double>::value) {
+    while (!P->prof && q.n - i > 1) {
+      int m = 0;  // leading products that take the tensor cores
+      while (i + m < q.n && q.g[i + m].M >= kTcF64Min && q.g[i + m].N >= kTcF64Min && q.g[i + m].K >= kTcF64Min) ++m;
+      m = m > 1 ? gemm_fp64_tc_many(q.g + i, m, P->L.tc_bytes) : m;
+      if (m < 2) break;
+      QTX_CK(gemm_fp64_tc_launch(q.g + i, m, P->ws + P->L.tc_scratch, P->L.tc_bytes, P->d_err_flag, st));
       i += m;
     }
   }
@@ -1278,7 +1290,7 @@ qtx_status validate(const qtx_rgf_desc* d, std::string& err) {
 // block products of the BT factors.  Row i of V P is (V P)_ij = sum_k V_ik P_kj over k = i-1..i+1
 // with |k - j| <= 1 (j = i-1..i+1 for M; i-2..i+2 for B, whose blocks B_ij = sum_l (V P)_il
 // (V_jl)^H need l up to j+1).  Each block product is one batched launch over the chunk's energies,
-// V shared (batch stride 0).  Temporaries: 0-4 V blocks, 5 one P block, 6-9 row i of V P, 11 B.
+// V shared (batch stride 0).  Temporaries: 0-4 V blocks, 5 one P block, 6-9 row i of V P, 10-11 B.
 template <typename T>
 qtx_status w_assemble_chunk(qtx_rgf_plan_s* P, const qtx_w_inputs* in, const qtx_w_outputs* out, int nb,
                             int e0, int ne, cudaStream_t st) {
@@ -1296,6 +1308,7 @@ qtx_status w_assemble_chunk(qtx_rgf_plan_s* P, const qtx_w_inputs* in, const qtx
   cx<T>* Pt = c.tmp(5);
   cx<T>* acc[4] = {c.tmp(6), c.tmp(7), c.tmp(8), c.tmp(9)};  // (V P)_{i,i-1} .. (V P)_{i,i+2}
   cx<T>* Bt = c.tmp(11);
+  cx<T>* Bu = c.tmp(10);
   auto toT = [&](cx<T>* dst, const cx<double>* src, long sSrc, int batch) {
     return axpby_from64<T>(dst, bb, src, sSrc, 1.0, nullptr, 0, 0.0, b, batch, st);
   };
@@ -1304,8 +1317,9 @@ qtx_status w_assemble_chunk(qtx_rgf_plan_s* P, const qtx_w_inputs* in, const qtx
     return gemm<T>(P, gargs<T>(b, b, b, A, b, sA, opA, B, b, sB, opB, first ? nullptr : C, b, bb, C, b, bb, al,
                                first ? 0.0 : 1.0, ne, nullptr), st);
   };
-  // V_k op(P), P complex128 with batch stride sP: digitised as it is (df32 plans), or through Pt
-  auto mmP = [&](const cx<T>* A, int opA, const cx<double>* Pb, long sP, int opB, cx<T>* C, double al, bool first) -> qtx_status {
+  // C (+)= al V_k op(P), P complex128 with batch stride sP: digitised as it is (df32 plans), or through Pt
+  Prods<T> pr;
+  auto addP = [&](const cx<T>* A, int opA, const cx<double>* Pb, long sP, int opB, cx<T>* C, double al, bool first) -> qtx_status {
     if constexpr (std::is_same<T, float>::value) {
       QTX_CK(toT(Pt, Pb, sP, ne));
       return mm(A, 0, opA, Pt, bb, opB, C, al, first);
@@ -1313,7 +1327,8 @@ qtx_status w_assemble_chunk(qtx_rgf_plan_s* P, const qtx_w_inputs* in, const qtx
       GemmArgs<T> g = gargs<T>(b, b, b, A, b, 0, opA, reinterpret_cast<const cx<T>*>(Pb), b, sP, opB, first ? nullptr : C, b, bb, C,
                                b, bb, al, first ? 0.0 : 1.0, ne, nullptr);
       g.b64 = true;
-      return gemm<T>(P, g, st);
+      pr.add(g);
+      return QTX_OK;
     }
   };
   // out[e][j] = alpha X (+ I), complex128, n blocks per energy
@@ -1334,20 +1349,22 @@ qtx_status w_assemble_chunk(qtx_rgf_plan_s* P, const qtx_w_inputs* in, const qtx
     if (i + 2 < nb) QTX_CK(toT(Vt[4], Vu + (long)(i + 1) * bb, 0, 1));
     // row i of V P for j = i+j0 .. i+j1.  V_ik: k = i-1 -> V_{i-1,i}^H, k = i -> V_ii, k = i+1 -> V_{i,i+1}.
     // P_kj: diagonal, upper (j = k+1), lower (j = k-1): given, or -(P_{j,j+1})^H for anti-Hermitian P.
+    // The sums over k of different j are independent: their n-th terms are launched together.
     auto row = [&](const void* Pd, const void* Pu, const void* Pl, int j0, int j1) -> qtx_status {
-      for (int j = std::max(i + j0, 0); j <= std::min(i + j1, nb - 1); ++j) {
-        bool first = true;
-        for (int k = i - 1; k <= i + 1; ++k) {
-          if (k < 0 || k >= nb || k - j > 1 || j - k > 1) continue;
+      for (int term = 0; term < 3; ++term) {
+        for (int j = std::max(i + j0, 0); j <= std::min(i + j1, nb - 1); ++j) {
+          const int k = std::max({i - 1, j - 1, 0}) + term;  // k in [i-1, i+1] and [j-1, j+1]
+          if (k > std::min({i + 1, j + 1, nb - 1})) continue;
           const cx<T>* Vk = k == i ? Vt[0] : (k == i + 1 ? Vt[3] : Vt[2]);
           const int opV = k == i - 1 ? OP_C : OP_N;
-          if (k == j) s = mmP(Vk, opV, pe(Pd, nb, k), (long)nb * bb, OP_N, acc[j - i + 1], 1.0, first);
-          else if (j == k + 1) s = mmP(Vk, opV, pe(Pu, nu, k), nu * bb, OP_N, acc[j - i + 1], 1.0, first);
-          else if (Pl) s = mmP(Vk, opV, pe(Pl, nu, j), nu * bb, OP_N, acc[j - i + 1], 1.0, first);
-          else s = mmP(Vk, opV, pe(Pu, nu, j), nu * bb, OP_C, acc[j - i + 1], -1.0, first);
+          cx<T>* C = acc[j - i + 1];
+          if (k == j) s = addP(Vk, opV, pe(Pd, nb, k), (long)nb * bb, OP_N, C, 1.0, term == 0);
+          else if (j == k + 1) s = addP(Vk, opV, pe(Pu, nu, k), nu * bb, OP_N, C, 1.0, term == 0);
+          else if (Pl) s = addP(Vk, opV, pe(Pl, nu, j), nu * bb, OP_N, C, 1.0, term == 0);
+          else s = addP(Vk, opV, pe(Pu, nu, j), nu * bb, OP_C, C, -1.0, term == 0);
           if (s) return s;
-          first = false;
         }
+        if ((s = run<T>(P, pr, st))) return s;
       }
       return QTX_OK;
     };
@@ -1364,24 +1381,23 @@ qtx_status w_assemble_chunk(qtx_rgf_plan_s* P, const qtx_w_inputs* in, const qtx
       if (!Pd) continue;
       if ((s = row(Pd, Pu, nullptr, -1, 2))) return s;  // B's blocks need (V P)_il for l = i-1 .. i+2
       // B_ii = sum_l (V P)_il (V_il)^H, l = i-1..i+1:  (V_{i,i-1})^H = V_{i-1,i}, V_ii^H, V_{i,i+1}^H
-      bool first = true;
-      for (int l = i - 1; l <= i + 1; ++l) {
-        if (l < 0 || l >= nb) continue;
-        const cx<T>* Vl = l == i ? Vt[0] : (l == i + 1 ? Vt[3] : Vt[2]);
-        if ((s = mm(acc[l - i + 1], bb, OP_N, Vl, 0, l == i - 1 ? OP_N : OP_C, Bt, 1.0, first))) return s;
-        first = false;
+      // B_{i,i+1} = sum_l (V P)_il (V_{i+1,l})^H, l = i..i+2:  V_{i,i+1}, V_{i+1,i+1}^H, V_{i+1,i+2}^H
+      // (the two sums' n-th terms together)
+      auto close = [&](int l, const cx<T>* Vl, int op, cx<T>* C, bool first) {
+        pr.add(gargs<T>(b, b, b, acc[l - i + 1], b, bb, OP_N, Vl, b, 0, op, first ? nullptr : C, b, bb, C, b, bb, 1.0,
+                        first ? 0.0 : 1.0, ne, nullptr));
+      };
+      const int d0 = std::max(i - 1, 0);
+      for (int term = 0; term < 3; ++term) {
+        const int ld = d0 + term, lu = i + term;
+        if (ld <= std::min(i + 1, nb - 1))
+          close(ld, ld == i ? Vt[0] : (ld == i + 1 ? Vt[3] : Vt[2]), ld == i - 1 ? OP_N : OP_C, Bt, term == 0);
+        if (i + 1 < nb && lu <= std::min(i + 2, nb - 1))
+          close(lu, lu == i ? Vt[3] : (lu == i + 1 ? Vt[1] : Vt[4]), lu == i ? OP_N : OP_C, Bu, term == 0);
+        if ((s = run<T>(P, pr, st))) return s;
       }
       if ((s = emit64(Od, nb, i, Bt, 1.0, false))) return s;
-      if (i + 1 < nb) {
-        // B_{i,i+1} = sum_l (V P)_il (V_{i+1,l})^H, l = i..i+2:  V_{i,i+1}, V_{i+1,i+1}^H, V_{i+1,i+2}^H
-        first = true;
-        for (int l = i; l <= i + 2 && l < nb; ++l) {
-          const cx<T>* Vl = l == i ? Vt[3] : (l == i + 1 ? Vt[1] : Vt[4]);
-          if ((s = mm(acc[l - i + 1], bb, OP_N, Vl, 0, l == i ? OP_N : OP_C, Bt, 1.0, first))) return s;
-          first = false;
-        }
-        if ((s = emit64(Ou, nu, i, Bt, 1.0, false))) return s;
-      }
+      if (i + 1 < nb && (s = emit64(Ou, nu, i, Bu, 1.0, false))) return s;
     }
   }
   return QTX_OK;
@@ -1414,10 +1430,10 @@ qtx_status qtx_rgf_plan_create(const qtx_rgf_desc* desc, qtx_rgf_plan* out) {
   if (e == cudaSuccess) e = cudaMemset(P->d_err_flag, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMallocHost(&P->h_status, sizeof(int) * P->Ec);
   if (e == cudaSuccess && desc->escalate_tol > 0) e = cudaMallocHost(&P->h_flag, sizeof(int) * P->Ec);
-  // identity block for the refinement residual
-  if (e == cudaSuccess)
+  // identity block for the refinement residual (plans whose inverses are refined)
+  if (e == cudaSuccess && P->L.refine64)
     e = set_identity(reinterpret_cast<cx<double>*>(P->ws + P->L.ident), reinterpret_cast<cx<df>*>(P->ws + P->L.ident_df), P->b, nullptr);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+  if (e == cudaSuccess && P->L.refine64) e = cudaStreamSynchronize(nullptr);
   if (e != cudaSuccess) {
     g_create_error = std::string("plan setup: ") + cudaGetErrorString(e);
     cudaFree(P->ws);
@@ -1816,7 +1832,7 @@ qtx_status qtx_zinv_batched(int precision, int n, void* A, long sA, int batch, i
     return QTX_ERR_OOM;
   }
   cudaError_t e = cudaMemsetAsync(P->d_err_flag, 0, sizeof(int), st);
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && P->L.refine64)
     e = set_identity(reinterpret_cast<cx<double>*>(P->ws + P->L.ident), reinterpret_cast<cx<df>*>(P->ws + P->L.ident_df), n, st);
   int* stat = status;
   if (!stat) stat = reinterpret_cast<int*>(P->ws + P->L.flags);

@@ -230,6 +230,11 @@ template cudaError_t gemm_simt<float>(const GemmArgs<float>&, cudaStream_t);
 // by the reciprocal and publishes it, and after a barrier every thread updates its values from 4 factors
 // and 4 row values.  About 500 cycles a step; with a warp per row group publishing its own candidate,
 // eight reciprocals and 16 shuffles a step, it took 2,000 (62 us for 64 x 64, batch 32).
+// c ? x : y by selects (register arrays indexed by a step's row or column would go to local memory)
+__device__ __forceinline__ cx<float> pick(bool c, cx<float> x, cx<float> y) {
+  return mk<float>(c ? x.re : y.re, c ? x.im : y.im);
+}
+
 template <int NMAX>
 __global__ void __launch_bounds__(256) k_leaf_inverse(cx<float>* Ag, long lda, long sA, int n, const int* active, int* status) {
   constexpr int R = NMAX / 16;
@@ -273,18 +278,20 @@ __global__ void __launch_bounds__(256) k_leaf_inverse(cx<float>* Ag, long lda, l
     else used1 |= 1u << (p - 32);
     if (ty == p % 16) {  // the pivot row's owners scale it
       const cx<float> r = crecip(col[p]);
+      const int pi = p / 16;
 #pragma unroll
-      for (int i = 0; i < R; ++i)
-        if (i == p / 16)
+      for (int j = 0; j < R; ++j) {
+        const int c = tx + 16 * j;
+        cx<float> x = a[0][j];
 #pragma unroll
-          for (int j = 0; j < R; ++j) {
-            const int c = tx + 16 * j;
-            const cx<float> x = a[i][j];
-            // the order of the roundings, by padded size
-            const float im = NMAX > 32 ? __fmaf_rn(x.re, r.im, __fmul_rn(x.im, r.re)) : __fmaf_rn(x.im, r.re, __fmul_rn(x.re, r.im));
-            a[i][j] = c == k ? r : mk<float>(__fmaf_rn(x.re, r.re, -__fmul_rn(x.im, r.im)), im);
-            s_row[c] = a[i][j];
-          }
+        for (int i = 1; i < R; ++i) x = pick(pi == i, a[i][j], x);
+        // the order of the roundings, by padded size
+        const float im = NMAX > 32 ? __fmaf_rn(x.re, r.im, __fmul_rn(x.im, r.re)) : __fmaf_rn(x.im, r.re, __fmul_rn(x.re, r.im));
+        x = pick(c == k, r, mk<float>(__fmaf_rn(x.re, r.re, -__fmul_rn(x.im, r.im)), im));
+#pragma unroll
+        for (int i = 0; i < R; ++i) a[i][j] = pick(pi == i, x, a[i][j]);
+        s_row[c] = x;
+      }
       if (tx == 0) {
         s_step[p] = k;
         s_piv[k] = p;
@@ -313,11 +320,14 @@ __global__ void __launch_bounds__(256) k_leaf_inverse(cx<float>* Ag, long lda, l
     }
     if (tx == (k + 1) % 16) {
       cx<float>* next = s_col[(k + 1) & 1];
+      const int jn = (k + 1) / 16;
 #pragma unroll
-      for (int j = 0; j < R; ++j)
-        if (j == (k + 1) / 16)
+      for (int i = 0; i < R; ++i) {
+        cx<float> x = a[i][0];
 #pragma unroll
-          for (int i = 0; i < R; ++i) next[ty + 16 * i] = a[i][j];
+        for (int j = 1; j < R; ++j) x = pick(jn == j, a[i][j], x);
+        next[ty + 16 * i] = x;
+      }
     }
     __syncthreads();
   }

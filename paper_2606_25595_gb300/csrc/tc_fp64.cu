@@ -60,10 +60,27 @@ struct Params {
   double alpha, beta;
   int akind, bkind;         // alpha: 0 = +1, 1 = -1, 2 = general; beta the same, 3 = no C0 term
   const int* active;
-  int* err;
-  int NBt, MBt, n_tiles, hold;
-  uint64_t limit_ns;
+  int NBt, MBt;
 };
+// A launch covers the tiles of 1..kMany9 products: product q owns tiles [tile0[q], tile0[q+1]), column tile
+// fastest, then row tile, then batch entry.
+constexpr int kMany9 = 4;
+struct Launch {
+  int n, hold;
+  int* err;
+  uint64_t limit_ns;
+  int tile0[kMany9 + 1];
+  Params p[kMany9];
+};
+// product of global tile t, and t's index within it
+template <bool MANY>
+__device__ __forceinline__ int product_of(const Launch& L, long t, int& lt) {
+  int q = 0;
+  if (MANY)
+    while (q + 1 < L.n && t >= L.tile0[q + 1]) ++q;
+  lt = (int)t - (MANY ? L.tile0[q] : 0);
+  return q;
+}
 
 __device__ __forceinline__ int at9(int r, int c) { return r * BNC9 + (c ^ (r & 7)); }
 
@@ -91,7 +108,9 @@ __device__ __noinline__ cx<double> dot_dfma(const Params& p, int e, int m, int n
   return acc;
 }
 
-__global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__ Params p) {
+template <bool MANY>
+__global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__ Launch L) {
+  const int n_tiles = L.tile0[L.n];
   extern __shared__ __align__(1024) unsigned char base[];
   cx<double>* out = reinterpret_cast<cx<double>*>(base + NST9 * STAGE9);
   int* s_eA = reinterpret_cast<int*>(base + NST9 * STAGE9 + OUT9);
@@ -125,23 +144,24 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tslot;
-  const int per_e = p.NBt * p.MBt;
 
   if (warp == 0) {
     if (lane == 0) {
       long g = 0;
       bool ok = true;
-      const long MB = p.M_pad / BM, NB = p.N_pad / BNC9, nkb = p.nks / 2;
       for (int k = 0; ok; ++k) {
         const long t = tile_at(k);
-        if (t >= p.n_tiles) break;
-        const int e = (int)(t / per_e), mblk = (int)((t / p.NBt) % p.MBt), nblk = (int)(t % p.NBt);
+        if (t >= n_tiles) break;
+        int lt;
+        const Params& p = L.p[product_of<MANY>(L, t, lt)];
+        const long MB = p.M_pad / BM, NB = p.N_pad / BNC9, nkb = p.nks / 2;
+        const int e = lt / (p.NBt * p.MBt), mblk = (lt / p.NBt) % p.MBt, nblk = lt % p.NBt;
         if (p.active && !p.active[e]) continue;
         const long ea = p.a_batched ? e : 0, eb = p.b_batched ? e : 0;
         const uint32_t sub = (uint32_t)(nblk == p.NBt - 1 ? p.bn_last : BNC9) * BKS * 2;
         for (int ks = 0; ks < p.nks; ++ks, ++g) {
           const int s = (int)(g % NST9);
-          if (!mbar_wait(&empty[s], ((uint32_t)(g / NST9) & 1u) ^ 1u, p.err, p.limit_ns)) { ok = false; break; }
+          if (!mbar_wait(&empty[s], ((uint32_t)(g / NST9) & 1u) ^ 1u, L.err, L.limit_ns)) { ok = false; break; }
           mbar_expect_tx(&full[s], S9 * (TILE_A + 2 * sub));
           unsigned char* st = base + s * STAGE9;
           // K-stages [0, nkb): A's real parts against (Re, Im); [nkb, 2 nkb): imaginary against (-Im, Re)
@@ -165,18 +185,20 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__
       long g = 0;
       int j = 0;
       bool ok = true;
-      if (p.hold && !mbar_wait(holdbar, 0u, p.err, p.limit_ns)) ok = false;
+      if (L.hold && !mbar_wait(holdbar, 0u, L.err, L.limit_ns)) ok = false;
       for (int k = 0; ok; ++k) {
         const long t = tile_at(k);
-        if (t >= p.n_tiles) break;
-        if (p.active && !p.active[(int)(t / per_e)]) continue;
-        const uint32_t idesc = idesc_n(2 * ((int)(t % p.NBt) == p.NBt - 1 ? p.bn_last : BNC9));
-        if (!mbar_wait(acce, ((uint32_t)j & 1u) ^ 1u, p.err, p.limit_ns)) break;
+        if (t >= n_tiles) break;
+        int lt;
+        const Params& p = L.p[product_of<MANY>(L, t, lt)];
+        if (p.active && !p.active[lt / (p.NBt * p.MBt)]) continue;
+        const uint32_t idesc = idesc_n(2 * (lt % p.NBt == p.NBt - 1 ? p.bn_last : BNC9));
+        if (!mbar_wait(acce, ((uint32_t)j & 1u) ^ 1u, L.err, L.limit_ns)) break;
         fence_after();
         uint32_t started = 0;
         for (int ks = 0; ks < p.nks; ++ks, ++g) {
           const int s = (int)(g % NST9);
-          if (!mbar_wait(&full[s], (uint32_t)(g / NST9) & 1u, p.err, p.limit_ns)) { ok = false; break; }
+          if (!mbar_wait(&full[s], (uint32_t)(g / NST9) & 1u, L.err, L.limit_ns)) { ok = false; break; }
           fence_after();
           const uint32_t sa = su32(base + s * STAGE9);
 #pragma unroll
@@ -208,15 +230,17 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__
     int j = 0;
     for (int k = 0;; ++k) {
       const long t = tile_at(k);
-      if (t >= p.n_tiles) break;
-      const int e = (int)(t / per_e), mblk = (int)((t / p.NBt) % p.MBt), nblk = (int)(t % p.NBt);
+      if (t >= n_tiles) break;
+      int lt;
+      const Params& p = L.p[product_of<MANY>(L, t, lt)];
+      const int e = lt / (p.NBt * p.MBt), mblk = (lt / p.NBt) % p.MBt, nblk = lt % p.NBt;
       if (p.active && !p.active[e]) continue;
       const int bn = nblk == p.NBt - 1 ? p.bn_last : BNC9;
       __syncwarp();
       asm volatile("bar.sync 1, 256;" ::: "memory");  // the previous tile's staging area is free
       if (et < BNC9) s_eB[et] = p.eB[(long)(p.b_batched ? e : 0) * p.N_pad + nblk * BNC9 + et];
       if (et >= 64 && et < 64 + BM) s_eA[et - 64] = p.eA[(long)(p.a_batched ? e : 0) * p.M_pad + mblk * BM + et - 64];
-      if (et == 0) *s_got = mbar_wait(accf, (uint32_t)j & 1u, p.err, p.limit_ns) ? 1 : 0;
+      if (et == 0) *s_got = mbar_wait(accf, (uint32_t)j & 1u, L.err, L.limit_ns) ? 1 : 0;
       __syncwarp();
       asm volatile("bar.sync 2, 256;" ::: "memory");
       if (!*s_got) break;
@@ -277,22 +301,23 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__
 // and writes 36 (left) or 54 B (right operand: Re, Im, -Im) per complex value.
 __host__ __device__ constexpr int skew9(int k) { return k + (k >> 3); }
 
-// Both operands of a product share the launch (blockIdx.z).
+// Both operands of every product of a launch share one digitisation (blockIdx.z).
 struct Operand {
   const cx<double>* X;
   long ldx, sX;
-  int R, R_pad, transposed, conj, batch;
+  int R, R_pad, K, K_pad, P, transposed, conj, batch;
   int* eout;
   unsigned char* planes;
   const int* active;
 };
 struct Operands {
-  Operand o[2];  // left, right
+  Operand o[2 * kMany9];  // left, right of each product
 };
 template <int RPC>
-__global__ void __launch_bounds__(32 * RPC) k_digitize_fp64(const __grid_constant__ Operands ops, int K, int K_pad, int P) {
-  const int side = blockIdx.z, e = blockIdx.y;
-  const Operand& op = ops.o[side];
+__global__ void __launch_bounds__(32 * RPC) k_digitize_fp64(const __grid_constant__ Operands ops) {
+  const int side = blockIdx.z & 1, e = blockIdx.y;
+  const Operand& op = ops.o[blockIdx.z];
+  const int K = op.K, K_pad = op.K_pad, P = op.P;
   const int R = op.R, R_pad = op.R_pad, transposed = op.transposed, conj_ = op.conj;
   const long ldx = op.ldx;
   if (e >= op.batch || (int)blockIdx.x * RPC >= R_pad || (op.active && !op.active[e])) return;
@@ -417,19 +442,6 @@ int chunk_k(int K) {
   return nc <= 1 ? K : (K + nc - 1) / nc;
 }
 
-cudaError_t digitize9(const GemmArgs<double>& g, const Dims9& d, int* eA, unsigned char* pa, int na, int* eB, unsigned char* pb,
-                      int nb, cudaStream_t st) {
-  constexpr int RPC = 4;  // transposed strips read four values of 16 bytes in a row: whole 32-byte sectors
-  const size_t smem = (size_t)RPC * (skew9(d.K_pad) + 1) * sizeof(cx<double>);  // at most 37 KB
-  Operands o;
-  o.o[0] = Operand{g.A, g.lda, g.sA, g.M, d.M_pad, g.opA == OP_C, g.opA == OP_C, na, eA, pa, g.sA ? g.active : nullptr};
-  o.o[1] = Operand{g.B, g.ldb, g.sB, g.N, d.N_pad, g.opB == OP_N, g.opB == OP_C, nb, eB, pb, g.sB ? g.active : nullptr};
-  const int R = d.M_pad > d.N_pad ? d.M_pad : d.N_pad;
-  k_digitize_fp64<RPC><<<dim3(R / RPC, na > nb ? na : nb, 2), 32 * RPC, smem, st>>>(o, g.K, d.K_pad, d.P);
-  count_launch();
-  return cudaGetLastError();
-}
-
 // SM count of the current device
 cudaError_t sm_count(int& sms) {
   int dev = 0;
@@ -437,50 +449,73 @@ cudaError_t sm_count(int& sms) {
   return e != cudaSuccess ? e : cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
 }
 
-cudaError_t product9(const GemmArgs<double>& g, unsigned char* scratch, int* err_flag, cudaStream_t st, cudaEvent_t* ev) {
+// n products, each with `bytes` of scratch behind the last one's
+cudaError_t products9(const GemmArgs<double>* g, int n, unsigned char* scratch, size_t bytes, int* err_flag, cudaStream_t st,
+                      cudaEvent_t* ev) {
   cudaError_t e;
-  const Dims9 d = dims9(g.M, g.N, g.K);
-  const int ab = g.sA != 0, bb = g.sB != 0;
-  const size_t na = ab ? g.batch : 1, nb = bb ? g.batch : 1;
-  Params p;
-  p.M_pad = d.M_pad;
-  p.N_pad = d.N_pad;
-  unsigned char* pa = scratch;
-  unsigned char* pb = pa + na * d.a;
-  int* eA = reinterpret_cast<int*>(pb + nb * d.b);
-  int* eB = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(eA) + na * d.ea);
-  if ((e = digitize9(g, d, eA, pa, (int)na, eB, pb, (int)nb, st))) return e;
-  p.pa = pa;
-  p.pb = pb;
-  p.eA = eA;
-  p.eB = eB;
-  p.nks = 2 * d.K_pad / BKS;
-  p.M = g.M; p.N = g.N; p.K = g.K;
-  p.escale = 2 * d.l1 - 2;
-  p.a_batched = ab; p.b_batched = bb;
-  p.A = g.A; p.B = g.B; p.lda = g.lda; p.sA = g.sA; p.ldb = g.ldb; p.sB = g.sB;
-  p.opA = g.opA; p.opB = g.opB;
-  p.C = g.C; p.ldc = g.ldc; p.sC = g.sC;
-  p.C0 = g.C0; p.ldc0 = g.ldc0; p.sC0 = g.sC0;
-  p.alpha = g.alpha; p.beta = g.beta;
-  auto kind = [](double x) { return x == 1.0 ? 0 : (x == -1.0 ? 1 : 2); };
-  p.akind = kind(g.alpha);
-  p.bkind = (g.C0 && g.beta != 0.0) ? kind(g.beta) : 3;
-  p.active = g.active;
-  p.err = err_flag;
-  p.NBt = d.N_pad / BNC9;
-  p.MBt = d.M_pad / BM;
-  p.bn_last = (g.N - (p.NBt - 1) * BNC9 + 7) / 8 * 8;
-  const long tiles = (long)p.NBt * p.MBt * g.batch;
-  if (tiles > 0x7fffffffL) return cudaErrorInvalidValue;
-  p.n_tiles = (int)tiles;
-  p.hold = wait_test();
-  p.limit_ns = p.hold ? kWaitTestLimitNs : kWaitLimitNs;
+  Launch L;
+  Operands o;
+  L.n = n;
+  L.hold = wait_test();
+  L.limit_ns = L.hold ? kWaitTestLimitNs : kWaitLimitNs;
+  L.err = err_flag;
+  long tiles = 0;
+  int R = 0, K_pad = 0, batch = 0;
+  for (int q = 0; q < n; ++q) {
+    const GemmArgs<double>& x = g[q];
+    Params& p = L.p[q];
+    const Dims9 d = dims9(x.M, x.N, x.K);
+    const int ab = x.sA != 0, bb = x.sB != 0;
+    const size_t na = ab ? x.batch : 1, nb = bb ? x.batch : 1;
+    p.M_pad = d.M_pad;
+    p.N_pad = d.N_pad;
+    unsigned char* pa = scratch + (size_t)q * bytes;
+    unsigned char* pb = pa + na * d.a;
+    int* eA = reinterpret_cast<int*>(pb + nb * d.b);
+    int* eB = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(eA) + na * d.ea);
+    o.o[2 * q] = Operand{x.A, x.lda, x.sA, x.M, d.M_pad, x.K, d.K_pad, d.P, x.opA == OP_C, x.opA == OP_C, (int)na, eA, pa, ab ? x.active : nullptr};
+    o.o[2 * q + 1] = Operand{x.B, x.ldb, x.sB, x.N, d.N_pad, x.K, d.K_pad, d.P, x.opB == OP_N, x.opB == OP_C, (int)nb, eB, pb, bb ? x.active : nullptr};
+    R = R > d.M_pad ? R : d.M_pad;
+    R = R > d.N_pad ? R : d.N_pad;
+    K_pad = K_pad > d.K_pad ? K_pad : d.K_pad;
+    batch = batch > x.batch ? batch : x.batch;
+    p.pa = pa;
+    p.pb = pb;
+    p.eA = eA;
+    p.eB = eB;
+    p.nks = 2 * d.K_pad / BKS;
+    p.M = x.M; p.N = x.N; p.K = x.K;
+    p.escale = 2 * d.l1 - 2;
+    p.a_batched = ab; p.b_batched = bb;
+    p.A = x.A; p.B = x.B; p.lda = x.lda; p.sA = x.sA; p.ldb = x.ldb; p.sB = x.sB;
+    p.opA = x.opA; p.opB = x.opB;
+    p.C = x.C; p.ldc = x.ldc; p.sC = x.sC;
+    p.C0 = x.C0; p.ldc0 = x.ldc0; p.sC0 = x.sC0;
+    p.alpha = x.alpha; p.beta = x.beta;
+    auto kind = [](double v) { return v == 1.0 ? 0 : (v == -1.0 ? 1 : 2); };
+    p.akind = kind(x.alpha);
+    p.bkind = (x.C0 && x.beta != 0.0) ? kind(x.beta) : 3;
+    p.active = x.active;
+    p.NBt = d.N_pad / BNC9;
+    p.MBt = d.M_pad / BM;
+    p.bn_last = (x.N - (p.NBt - 1) * BNC9 + 7) / 8 * 8;
+    L.tile0[q] = (int)tiles;
+    tiles += (long)p.NBt * p.MBt * x.batch;
+    if (tiles > 0x7fffffffL) return cudaErrorInvalidValue;
+  }
+  L.tile0[n] = (int)tiles;
+  constexpr int RPC = 4;  // transposed strips read four values of 16 bytes in a row: whole 32-byte sectors
+  const size_t smem = (size_t)RPC * (skew9(K_pad) + 1) * sizeof(cx<double>);  // at most 37 KB
+  k_digitize_fp64<RPC><<<dim3(R / RPC, batch, 2 * n), 32 * RPC, smem, st>>>(o);
+  count_launch();
+  if ((e = cudaGetLastError())) return e;
   int sms = 0;
-  static std::atomic<unsigned long long> done{0};
-  if ((e = allow_smem(k_tc_gemm_fp64, SMEM9, done)) || (e = sm_count(sms))) return e;
+  static std::atomic<unsigned long long> done1{0}, done2{0};
+  if ((e = n == 1 ? allow_smem(k_tc_gemm_fp64<false>, SMEM9, done1) : allow_smem(k_tc_gemm_fp64<true>, SMEM9, done2)) || (e = sm_count(sms))) return e;
+  const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);
   if (ev) cudaEventRecord(ev[0], st);
-  k_tc_gemm_fp64<<<(unsigned)(tiles < sms ? tiles : sms), 320, SMEM9, st>>>(p);
+  if (n == 1) k_tc_gemm_fp64<false><<<grid, 320, SMEM9, st>>>(L);
+  else k_tc_gemm_fp64<true><<<grid, 320, SMEM9, st>>>(L);
   count_launch();
   if (ev) cudaEventRecord(ev[1], st);
   return cudaGetLastError();
@@ -538,12 +573,28 @@ cudaError_t gemm_fp64_tc(const GemmArgs<double>& g0, void* scratch, size_t scrat
         t.sC0 = g.sC;
         t.beta = 1.0;
       }
-      const cudaError_t e = tc::product9(t, reinterpret_cast<unsigned char*>(scratch), err_flag, st, one ? ev : nullptr);
+      const cudaError_t e = tc::products9(&t, 1, reinterpret_cast<unsigned char*>(scratch), 0, err_flag, st, one ? ev : nullptr);
       if (e != cudaSuccess) return e;
     }
   }
   if (ev && !one) cudaEventRecord(ev[1], st);
   return cudaSuccess;
+}
+
+int gemm_fp64_tc_many(const GemmArgs<double>* g, int n, size_t scratch_bytes) {
+  size_t most = 0;
+  for (int q = 0; q < n; ++q) {
+    if (g[q].M <= 0 || g[q].N <= 0 || g[q].K < 1 || g[q].batch <= 0 || tc::chunk_k(g[q].K) != g[q].K) return 1;
+    const size_t need = entry_bytes(g[q].M, g[q].N, g[q].K) * g[q].batch;
+    most = most > need ? most : need;
+  }
+  const size_t fit = most ? scratch_bytes / most : 1;
+  const int k = fit < (size_t)tc::kMany9 ? (int)fit : tc::kMany9;
+  return k < 1 ? 1 : (k < n ? k : n);
+}
+
+cudaError_t gemm_fp64_tc_launch(const GemmArgs<double>* g, int n, void* scratch, size_t scratch_bytes, int* err_flag, cudaStream_t st) {
+  return tc::products9(g, n, reinterpret_cast<unsigned char*>(scratch), (scratch_bytes / n) & ~size_t(1023), err_flag, st, nullptr);
 }
 
 }  // namespace qtx
