@@ -26,28 +26,38 @@
 // so one MMA chain with N = 2 BNC real columns produces BNC complex columns (BNC = 48 for 6 and 7
 // digit planes, 64 for 4 and 2: bnc_of; the last column tile of a product takes only its
 // N - BNC (tiles - 1) columns rounded up to 8, with a narrower MMA N).  The right operand's digit
-// planes are stored transposed (N x K, K-major) as three BNC-row sub-tiles per block of BNC columns
-// and 16 complex k -- Re B, Im B and -Im B -- which the producer pairs into the 2 BNC rows the MMA
-// reads: (Re, Im) against A's real parts, (-Im, Re) against its imaginary parts.
+// planes are stored transposed (N x K, K-major) as three parts of BNC rows per block of BNC columns and
+// 16 complex k -- -Im B, Re B and Im B -- of which the MMA reads two neighbours as its 2 BNC rows:
+// (Re, Im) against A's real parts, (-Im, Re) against its imaginary parts.
 //
-// Kernel structure (persistent: one CTA per SM walking 128 x BNC complex output tiles, 10 warps):
-//   warp 0   producer: one bulk asynchronous copy (cp.async.bulk, mbarrier complete-tx) per plane
-//            tile of one K-stage (16 K-elements; the digitiser stores every tile contiguously, already
-//            in the 32-byte-swizzled K-major layout the MMA descriptors expect), a ring of 2-6 stages
-//            that runs on across tiles;
-//   warp 1   allocates 512 TMEM columns once; one thread issues the tcgen05.mma's (2 K16 steps x
-//            pairs), tcgen05.commit's each stage back to the producer and each finished tile to the
-//            epilogue, and waits for the epilogue to release TMEM before the next tile;
+// Kernel structure (persistent: one CTA per SM walking 128 x BNC complex output tiles, 11 warps):
+//   warp 0   producer: two rings of bulk asynchronous copies (cp.async.bulk, mbarrier complete-tx) that run
+//            on across tiles: all planes of a left tile's K-step (16 real or imaginary k), and all planes
+//            and parts of a right tile's K-block (16 complex k, two steps).  The digitiser stores both
+//            contiguously, in the 32-byte-swizzled K-major layout the MMA descriptors expect, so a
+//            K-block takes three copies of 24 to 28 KB (6 planes).  An SM's copies cost about 50 cycles
+//            each beside 64 B per cycle (2 KB copies: 22 B per cycle; 24 KB: 61): with a copy per plane
+//            and part, 36 a K-block, the copies bounded the kernel (64 products of 256^3, 6 planes:
+//            188 -> 173 us; an FP32 solve of b = 384: 33.1 -> 30.6 ms);
+//   warps 1, 10  warp 1 allocates 512 TMEM columns once; one thread of each issues the tcgen05.mma's of half
+//            the digit groups (an accumulator belongs to one thread), tcgen05.commit's each slot back to
+//            the producer and each finished tile to the epilogue, and waits for the epilogue to release
+//            TMEM before the next tile.  Two streams of MMAs leave fewer gaps behind a digit group's
+//            dependent accumulations than one (a solve of 6 planes at b = 256: 91.7 -> 87.6 ms);
 //   warps 2-9 epilogue (two warps per TMEM lane quarter, one per column half): tcgen05.ld of the
 //            accumulators and their recombination into df32 in a staging area, release of TMEM, then
 //            the row/column scaling, the alpha and beta * C0 terms and coalesced stores --
 //            overlapping the next tile's mainloop.
+// What bounds it (64 products of 256^3, 6 planes): the MMAs, 58 cycles each with their operands read from
+// shared memory (7 KB at 128 B per cycle: 56; the tensor core alone 48), 78% of an SM's time; waits for
+// copies 11% and for the epilogue 7%.
 // Every mbarrier wait is bounded (2 s of %globaltimer); on expiry the kernel sets *err and unwinds.
 #include <cuda_bf16.h>
 
 #include <atomic>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 
 #include "df32.cuh"
@@ -62,9 +72,14 @@ namespace tc {
 // columns; 64 for 4 and 2 planes, whose digit groups all stay exact in at most four accumulators
 // (4 x 128 columns), so a tile covers a third more columns at N = 128.
 __host__ __device__ constexpr int bnc_of(int S) { return S >= 6 ? 48 : 64; }
-// bytes of one B-plane tile in shared memory (2 BNC rows x 32 B) and of one BNC-row sub-tile
-__host__ __device__ constexpr int tile_b_of(int S) { return 2 * bnc_of(S) * BKS * 2; }
+// bytes of one BNC-row part of a right operand's plane, and of the shared-memory slots: all planes of a left
+// tile's K-step, all planes and parts of a right tile's K-block
 __host__ __device__ constexpr int sub_b_of(int S) { return bnc_of(S) * BKS * 2; }
+__host__ __device__ constexpr int slot_a_of(int S) { return S * TILE_A; }
+__host__ __device__ constexpr int slot_b_of(int S) { return S * 3 * sub_b_of(S); }
+// slots of the two rings of a kernel with NST left slots
+__host__ __device__ constexpr int nsb_of(int NST) { return NST >= 4 ? NST / 2 : 2; }
+__host__ __device__ constexpr int ring_bytes_of(int S, int NST) { return NST * slot_a_of(S) + nsb_of(NST) * slot_b_of(S); }
 // the epilogue's staging area: BM x BNC df32 complex values (16 bytes), the 16-byte column index
 // XOR-swizzled by the row's low three bits, so rows written by consecutive lanes and columns read by
 // consecutive threads both fall in distinct bank groups
@@ -74,6 +89,10 @@ __host__ __device__ constexpr int out_at(int r, int c, int S) { return r * bnc_o
 // accumulator of digit pair (i, j): exact groups i + j = 2..5, then one rounded group
 __host__ __device__ constexpr int acc_of(int i, int j) { return (i + j <= 5) ? (i + j - 2) : 4; }
 __host__ __device__ constexpr int n_acc(int S) { return S + 1 >= 6 ? 5 : S; }
+
+// which of the two MMA threads issues the digit products of group i + j: half of them each, as far as the
+// groups allow (those of one accumulator stay together)
+__host__ __device__ constexpr int mma_half(int S, int g) { return S >= 6 ? g >= 6 : (S == 4 ? (g == 3 || g == 4) : g == 3); }
 
 // ------------------------------------------------------------------------------ GEMM kernel
 // TcParams (per-product kernel parameters) is declared in kernels.cuh.
@@ -139,7 +158,7 @@ __device__ __forceinline__ df sum_acc(const uint32_t (&v)[NACC][8], int c) {
 // registers and the staging area).  So the producer's loads and the MMAs of tile j+1 overlap the
 // epilogue's global stores of tile j, and the prologue (TMEM allocation, barrier set-up, first
 // loads) is paid once per SM rather than once per tile.  The staging area is separate from the
-// stage ring (NST = 3 stages fit beside it for 6 and 4 digit planes, 6 for 2).
+// rings (NST left slots: 3 fit beside it for 6 and 4 digit planes, 6 for 2, 2 for 7; nsb_of right slots).
 
 // IO: element type of C and C0 -- df (the emulated-FP64 products), double (the same with complex128 results:
 // what a separate pass would convert is converted in the store) or float (the products of the FP32 mode and
@@ -156,18 +175,21 @@ __device__ __forceinline__ df df_of(double x) { return from_d<df>(x); }
 
 // GROUP = false: a single product (problem 0; its parameters at fixed offsets); true: a grouped launch.
 template <int S, int NST, typename IO, bool GROUP>
-__global__ void __launch_bounds__(320, 1) k_tc_gemm(const __grid_constant__ TcGroup G) {
+__global__ void __launch_bounds__(352, 1) k_tc_gemm(const __grid_constant__ TcGroup G) {
   const int n_tiles = G.tile0[G.n];
-  constexpr int BNC = bnc_of(S), TILE_B = tile_b_of(S), SUB_B = sub_b_of(S), ACC_COLS = 2 * BNC;
-  constexpr int OUT_BYTES = out_bytes_of(S);
-  constexpr int STAGE = S * (TILE_A + TILE_B);
+  constexpr int BNC = bnc_of(S), ACC_COLS = 2 * BNC;
+  constexpr int OUT_BYTES = out_bytes_of(S), RING = ring_bytes_of(S, NST);
+  constexpr int SLOT_A = slot_a_of(S), SLOT_B = slot_b_of(S), NSB = nsb_of(NST);
   constexpr int NACC = n_acc(S);
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  cx<df>* out = reinterpret_cast<cx<df>*>(base + NST * STAGE);  // [BM][BNC] staging (out_at)
-  uint64_t* full = reinterpret_cast<uint64_t*>(base + NST * STAGE + OUT_BYTES);
-  uint64_t* empty = full + NST;
-  uint64_t* accf = empty + NST;
+  unsigned char* ringB = base + NST * SLOT_A;
+  cx<df>* out = reinterpret_cast<cx<df>*>(base + RING);  // [BM][BNC] staging (out_at)
+  uint64_t* fullA = reinterpret_cast<uint64_t*>(base + RING + OUT_BYTES);
+  uint64_t* emptyA = fullA + NST;
+  uint64_t* fullB = emptyA + NST;
+  uint64_t* emptyB = fullB + NSB;
+  uint64_t* accf = emptyB + NSB;
   uint64_t* acce = accf + 1;
   uint64_t* holdbar = acce + 1;   // never arrived at (the wait test)
   uint64_t* drainbar = acce + 2;  // the MMA thread's final commit
@@ -179,13 +201,17 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm(const __grid_constant__ TcGr
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NST; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
+      mbar_init(&fullA[s], 1);
+      mbar_init(&emptyA[s], 2);  // both MMA threads' commits
     }
-    mbar_init(accf, 1);
+    for (int s = 0; s < NSB; ++s) {
+      mbar_init(&fullB[s], 1);
+      mbar_init(&emptyB[s], 2);
+    }
+    mbar_init(accf, 2);
     mbar_init(acce, 1);
     mbar_init(holdbar, 1);
-    mbar_init(drainbar, 1);
+    mbar_init(drainbar, 2);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -199,7 +225,7 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm(const __grid_constant__ TcGr
 
   if (warp == 0) {
     if (lane == 0) {
-      long g = 0;  // stage counter across tiles
+      long ga = 0, gb = 0;  // copies into the left and the right ring so far
       bool ok = true;
       for (int k = 0; ok; ++k) {
         const long t = tile_at(k);
@@ -212,37 +238,37 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm(const __grid_constant__ TcGr
         if (p.active && !p.active[e]) continue;
         const long MB = p.M_pad / BM, NB = p.N_pad / BNC, nkb = p.nks / 2;
         const long ea = p.a_batched ? e : 0, eb = p.b_batched ? e : 0;
-        // rows taken from each BNC-row sub-tile: all of them, or the last tile's first bn_last (a
-        // multiple of 8 rows = whole 256-byte swizzle groups, so the pair stays in the MMA layout)
-        const uint32_t sub = (uint32_t)(nblk == NBt - 1 ? p.bn_last : BNC) * BKS * 2;
-        for (int ks = 0; ks < p.nks; ++ks, ++g) {
-          const int s = (int)(g % NST);
-          const uint32_t ph = (uint32_t)(g / NST) & 1u;
-          if (!mbar_wait(&empty[s], ph ^ 1u, G.p[0].err, G.limit_ns)) { ok = false; break; }
-          mbar_expect_tx(&full[s], S * (TILE_A + 2 * sub));
-          unsigned char* st = base + s * STAGE;
-          // K-stages [0, nkb) meet A's real parts: B rows (Re, Im); stages [nkb, 2 nkb) meet A's
-          // imaginary parts: B rows (-Im, Re)
-          const int part = ks >= nkb, kb = (int)(ks - part * nkb);
-          const int s0 = part ? 2 : 0, s1 = part ? 0 : 1;
-          for (int d = 0; d < S; ++d) {
-            bulk_load(st + d * TILE_A, p.pa + (((ea * S + d) * MB + mblk) * p.nks + ks) * (long)TILE_A, TILE_A, &full[s]);
-            const unsigned char* sb = p.pb + (((eb * S + d) * NB + nblk) * nkb + kb) * 3L * SUB_B;
-            unsigned char* db = st + S * TILE_A + d * TILE_B;
-            bulk_load(db, sb + s0 * SUB_B, sub, &full[s]);
-            bulk_load(db + sub, sb + s1 * SUB_B, sub, &full[s]);
+        // rows of a right part: BNC, or the last tile's first bn_last (a multiple of 8 rows = whole
+        // 256-byte swizzle groups, so the parts stay in the MMA layout)
+        const uint32_t bytesB = S * 3u * (uint32_t)(nblk == NBt - 1 ? p.bn_last : BNC) * BKS * 2;
+        const unsigned char* srcA = p.pa + (ea * MB + mblk) * p.nks * (long)SLOT_A;
+        const unsigned char* srcB = p.pb + (eb * NB + nblk) * nkb * (long)SLOT_B;
+        for (int ks = 0; ks < p.nks; ++ks, ++ga) {
+          if (!(ks & 1)) {
+            const int s = (int)(gb % NSB);
+            if (!mbar_wait(&emptyB[s], ((uint32_t)(gb / NSB) & 1u) ^ 1u, G.p[0].err, G.limit_ns)) { ok = false; break; }
+            mbar_expect_tx(&fullB[s], bytesB);
+            bulk_load(ringB + s * SLOT_B, srcB + (ks / 2) * (long)bytesB, bytesB, &fullB[s]);
+            ++gb;
           }
+          const int s = (int)(ga % NST);
+          if (!mbar_wait(&emptyA[s], ((uint32_t)(ga / NST) & 1u) ^ 1u, G.p[0].err, G.limit_ns)) { ok = false; break; }
+          mbar_expect_tx(&fullA[s], SLOT_A);
+          bulk_load(base + s * SLOT_A, srcA + ks * (long)SLOT_A, SLOT_A, &fullA[s]);
         }
       }
-      // the copies of the last stages issued (at most NST of them, one per slot) land before the
-      // CTA goes on to exit, also when a wait gave up and the MMA thread no longer consumes them
-      for (long gi = g > NST ? g - NST : 0; gi < g; ++gi)
-        mbar_wait_drain(&full[gi % NST], (uint32_t)(gi / NST) & 1u, kWaitLimitNs);
+      // the last copies issued (at most one per slot) land before the CTA goes on to exit, also when a
+      // wait gave up and the MMA threads no longer consume them
+      for (long g = ga > NST ? ga - NST : 0; g < ga; ++g)
+        mbar_wait_drain(&fullA[g % NST], (uint32_t)(g / NST) & 1u, kWaitLimitNs);
+      for (long g = gb > NSB ? gb - NSB : 0; g < gb; ++g)
+        mbar_wait_drain(&fullB[g % NSB], (uint32_t)(g / NSB) & 1u, kWaitLimitNs);
     }
     __syncwarp();
-  } else if (warp == 1) {
+  } else if (warp == 1 || warp == 10) {
+    const int half = warp == 10;
     if (lane == 0) {
-      long g = 0;
+      long ga = 0, gb = 0;
       int j = 0;  // tiles processed by this CTA
       bool ok = true;
       // wait test: a barrier nothing arrives at, so the wait gives up before any MMA is issued
@@ -256,29 +282,42 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm(const __grid_constant__ TcGr
         const int NBt = G.NBt[q], MBt = G.MBt[q];
         const int e = (int)(lt / (NBt * MBt));
         if (p.active && !p.active[e]) continue;
-        const uint32_t idesc = idesc_n(2 * (lt % NBt == NBt - 1 ? p.bn_last : BNC));
+        const uint32_t rows = lt % NBt == NBt - 1 ? p.bn_last : BNC;
+        const uint32_t idesc = idesc_n(2 * rows);
+        const uint32_t part = rows * BKS * 2 / 16;  // a descriptor's address counts 16-byte units
         // TMEM is free once the epilogue has read the previous tile's accumulators
         if (!mbar_wait(acce, ((uint32_t)j & 1u) ^ 1u, G.p[0].err, G.limit_ns)) break;
         fence_after();
-        uint32_t started = 0;
-        for (int ks = 0; ks < p.nks; ++ks, ++g) {
-          const int s = (int)(g % NST);
-          const uint32_t ph = (uint32_t)(g / NST) & 1u;
-          if (!mbar_wait(&full[s], ph, G.p[0].err, G.limit_ns)) { ok = false; break; }
+        for (int ks = 0; ks < p.nks; ++ks, ++ga) {
+          const int sb = (int)(gb % NSB), sa = (int)(ga % NST);
+          if (!(ks & 1) && !mbar_wait(&fullB[sb], (uint32_t)(gb / NSB) & 1u, G.p[0].err, G.limit_ns)) { ok = false; break; }
+          if (!mbar_wait(&fullA[sa], (uint32_t)(ga / NST) & 1u, G.p[0].err, G.limit_ns)) { ok = false; break; }
           fence_after();
-          const uint32_t sa = su32(base + s * STAGE);
+          // A's real parts (even steps) meet the B rows (Re, Im), its imaginary parts (-Im, Re)
+          const uint64_t ad = sdesc(su32(base + sa * SLOT_A));
+          const uint64_t bd = sdesc(su32(ringB + sb * SLOT_B)) + ((ks & 1) ? 0 : part);
+          auto issue = [&](auto H) {
+            constexpr int HALF = decltype(H)::value;
 #pragma unroll
-          for (int i = 1; i <= S; ++i) {
+            for (int i = 1; i <= S; ++i) {
 #pragma unroll
-            for (int jj = 1; jj <= S + 1 - i; ++jj) {
-              const int gacc = acc_of(i, jj);
-              const uint64_t ad = sdesc(sa + (i - 1) * TILE_A);
-              const uint64_t bd = sdesc(sa + S * TILE_A + (jj - 1) * TILE_B);
-              mma(tmem + gacc * ACC_COLS, ad, bd, idesc, (started >> gacc) & 1u);
-              started |= 1u << gacc;
+              for (int jj = 1; jj <= S + 1 - i; ++jj) {
+                if (mma_half(S, i + jj) != HALF) continue;
+                const int gacc = acc_of(i, jj);
+                // the first product of an accumulator's first step overwrites it
+                const bool first = i == 1 && jj == gacc + 1;
+                mma(tmem + gacc * ACC_COLS, ad + (i - 1) * TILE_A / 16, bd + (jj - 1) * 3 * part, idesc,
+                    first ? (uint32_t)(ks > 0) : 1u);
+              }
             }
+          };
+          if (half) issue(std::integral_constant<int, 1>());
+          else issue(std::integral_constant<int, 0>());
+          mma_commit(&emptyA[sa]);
+          if (ks & 1) {
+            mma_commit(&emptyB[sb]);
+            ++gb;
           }
-          mma_commit(&empty[s]);
         }
         if (!ok) break;
         mma_commit(accf);
@@ -534,27 +573,16 @@ __global__ void __launch_bounds__(32 * RPC) k_digitize_rows(const __grid_constan
   __syncthreads();
   if (t < RPC && r0 + t < R_pad) eout[(long)e * R_pad + r0 + t] = s_ex[t];
   // ---- digits: item = (row rr, complex k = 8 kc .. 8 kc + 7)
-  // left operand: [row_block of 128][k_stage of 16 embedded k][128 x 32 B] tiles, embedded k' = k for
-  // Re, K_pad + k for Im.  right operand: [col_block of BNC][k_block of 16 complex k][3][BNC x 32 B]
-  // sub-tiles holding Re, Im and -Im (the producer pairs them into the (Re, Im) and (-Im, Re) rows).
-  const long nks = 2L * K_pad / BKS, nkb = K_pad / BKS;
-  constexpr int BNC = bnc_of(S), SUB_B = sub_b_of(S);
-  const long plane_bytes = side == 0 ? (long)(R_pad / BM) * nks * TILE_A : (long)(R_pad / BNC) * nkb * 3 * SUB_B;
-  unsigned char* pe = job.planes + (long)e * S * plane_bytes;
+  // left operand: [row block of 128][k block of 16][part: Re, Im][plane][128 x 32 B].  right operand:
+  // [column block of BNC][k block of 16][plane][part: -Im, Re, Im][rows x 32 B], rows = BNC, or those of
+  // the last block rounded up to 8: each is what one copy of the product kernel takes.
+  const int nkb = K_pad / BKS;
+  constexpr int BNC = bnc_of(S), SLOT_A = slot_a_of(S), SLOT_B = slot_b_of(S);
+  unsigned char* pe = job.planes + (long)e * (side == 0 ? (long)(R_pad / BM) * 2 * nkb * SLOT_A : (long)(R_pad / BNC) * nkb * SLOT_B);
   const int nkc = K_pad / 8;
   // rows whose planes are written: right-operand columns past N rounded up to 8 are never read (the
   // last column tile's MMA takes only its first bn_last rows), so they stay unwritten
   const int R_wr = side == 1 ? min(R_pad, (R + 7) / 8 * 8) : R_pad;
-  // byte offset of the 16-byte chunk holding embedded k' .. k' + 7 (k' a multiple of 8) of row r (left)
-  auto chunk_off = [&](long row, int kp) -> long {
-    const long blk = row / BM, rr_ = row % BM, ks = kp / BKS, kk = kp % BKS;
-    return (blk * nks + ks) * TILE_A + sw32_offset((uint32_t)rr_, (uint32_t)kk);
-  };
-  // ... of complex k .. k + 7 of column r (right), in sub-tile `sub`
-  auto sub_off = [&](long col, int k, int sub) -> long {
-    const long cb = col / BNC, rr_ = col % BNC, kb = k / BKS, kk = k % BKS;
-    return ((cb * nkb + kb) * 3 + sub) * (long)SUB_B + sw32_offset((uint32_t)rr_, (uint32_t)kk);
-  };
 #pragma unroll 1
   for (int item = t; item < RPC * nkc; item += NT) {
     const int rr = item / nkc, kc = item % nkc, r = r0 + rr;
@@ -585,23 +613,23 @@ __global__ void __launch_bounds__(32 * RPC) k_digitize_rows(const __grid_constan
     }
     const int k8 = 8 * kc;
     if (side == 0) {
-      const long o_re = chunk_off(r, k8), o_im = chunk_off(r, K_pad + k8);
+      const int blk = r / BM, rw = r % BM;
+      unsigned char* pl = pe + ((long)blk * nkb + k8 / BKS) * 2 * SLOT_A + sw32_offset((uint32_t)rw, (uint32_t)(k8 % BKS));
 #pragma unroll
       for (int i = 0; i < S; ++i) {
-        unsigned char* pl = pe + (long)i * plane_bytes;
-        *reinterpret_cast<uint4*>(pl + o_re) = make_uint4(wre[i][0], wre[i][1], wre[i][2], wre[i][3]);
-        *reinterpret_cast<uint4*>(pl + o_im) = make_uint4(wim[i][0], wim[i][1], wim[i][2], wim[i][3]);
+        *reinterpret_cast<uint4*>(pl + i * TILE_A) = make_uint4(wre[i][0], wre[i][1], wre[i][2], wre[i][3]);
+        *reinterpret_cast<uint4*>(pl + SLOT_A + i * TILE_A) = make_uint4(wim[i][0], wim[i][1], wim[i][2], wim[i][3]);
       }
     } else {
-      const long o0 = sub_off(r, k8, 0), o1 = sub_off(r, k8, 1), o2 = sub_off(r, k8, 2);
+      const int cb = r / BNC, rw = r % BNC;
+      const int rows = cb == R_pad / BNC - 1 ? (R - cb * BNC + 7) / 8 * 8 : BNC, part = rows * BKS * 2;
+      unsigned char* pl = pe + (long)cb * nkb * SLOT_B + (long)(k8 / BKS) * (S * 3 * part) + sw32_offset((uint32_t)rw, (uint32_t)(k8 % BKS));
       const uint32_t SGN = 0x80008000u;  // bf16 sign bits of both halves
 #pragma unroll
-      for (int i = 0; i < S; ++i) {
-        unsigned char* pl = pe + (long)i * plane_bytes;
-        *reinterpret_cast<uint4*>(pl + o0) = make_uint4(wre[i][0], wre[i][1], wre[i][2], wre[i][3]);
-        *reinterpret_cast<uint4*>(pl + o1) = make_uint4(wim[i][0], wim[i][1], wim[i][2], wim[i][3]);
-        *reinterpret_cast<uint4*>(pl + o2) =
-            make_uint4(wim[i][0] ^ SGN, wim[i][1] ^ SGN, wim[i][2] ^ SGN, wim[i][3] ^ SGN);
+      for (int i = 0; i < S; ++i, pl += 3 * part) {
+        *reinterpret_cast<uint4*>(pl) = make_uint4(wim[i][0] ^ SGN, wim[i][1] ^ SGN, wim[i][2] ^ SGN, wim[i][3] ^ SGN);
+        *reinterpret_cast<uint4*>(pl + part) = make_uint4(wre[i][0], wre[i][1], wre[i][2], wre[i][3]);
+        *reinterpret_cast<uint4*>(pl + 2 * part) = make_uint4(wim[i][0], wim[i][1], wim[i][2], wim[i][3]);
       }
     }
   }
@@ -638,7 +666,7 @@ inline Scratch carve(void* base, const Dims& d, int batch, int S) {
   Scratch s;
   unsigned char* p = reinterpret_cast<unsigned char*>(base);
   const size_t a = al((size_t)batch * S * d.M_pad * 2 * d.K_pad * sizeof(__nv_bfloat16));
-  const size_t b = al((size_t)batch * S * (d.N_pad / bnc_of(S)) * (d.K_pad / BKS) * 3 * sub_b_of(S));  // Re, Im, -Im sub-tiles
+  const size_t b = al((size_t)batch * (d.N_pad / bnc_of(S)) * (d.K_pad / BKS) * slot_b_of(S));
   const size_t ea = al((size_t)batch * d.M_pad * sizeof(int));
   const size_t eb = al((size_t)batch * d.N_pad * sizeof(int));
   s.pa = p;
@@ -782,7 +810,7 @@ template <int S, int NST, typename IO>
 cudaError_t launch(const TcPrepared* const* pp, int n, cudaStream_t st, cudaEvent_t* ev) {
   if (n < 1 || n > kMaxGroup) return cudaErrorInvalidValue;
   cudaError_t e;
-  const size_t smem = (size_t)NST * S * (TILE_A + tile_b_of(S)) + out_bytes_of(S) + 1024 + 256;
+  const size_t smem = (size_t)ring_bytes_of(S, NST) + out_bytes_of(S) + 1024 + 256;
   static bool attr = false;
   static int sms = 0;
   if (!attr) {
@@ -814,8 +842,8 @@ cudaError_t launch(const TcPrepared* const* pp, int n, cudaStream_t st, cudaEven
     if (pp[q]->ctas > 0 && pp[q]->ctas < ctas) ctas = pp[q]->ctas;
   const int grid = (int)(total < ctas ? total : ctas);
   if (ev) cudaEventRecord(ev[0], st);
-  if (n == 1) k_tc_gemm<S, NST, IO, false><<<grid, 320, smem, st>>>(G);
-  else k_tc_gemm<S, NST, IO, true><<<grid, 320, smem, st>>>(G);
+  if (n == 1) k_tc_gemm<S, NST, IO, false><<<grid, 352, smem, st>>>(G);
+  else k_tc_gemm<S, NST, IO, true><<<grid, 352, smem, st>>>(G);
   count_launch();
   if (ev) cudaEventRecord(ev[1], st);
   return cudaGetLastError();
@@ -867,9 +895,9 @@ TcOperand tc_operand_at(void* base, int R, int K, int batch, int digits) {
   return o;
 }
 
-// Pipeline stages of a kernel variant: the requested count if shared memory allows it, else the
-// default.  Beside the 96 KB epilogue staging of 48-column tiles, 6 digit planes take 42 KB a stage
-// and 7 take 49 KB; beside the 128 KB staging of 64-column tiles, 4 planes take 32 KB and 2 take 16 KB.
+// Left slots of a kernel variant: the requested count if shared memory allows it, else the default.
+// Beside the 96 KB epilogue staging of 48-column tiles and two right slots, 6 digit planes have room for
+// three and 7 for two; beside the 128 KB of 64-column tiles, 4 planes for three and 2 for six.
 static int resolve_stages(int S, int want) {
   if (S == 4) return (want == 2) ? 2 : 3;  // 2 or 3
   if (S == 6) return (want == 2) ? 2 : 3;         // 2 or 3

@@ -22,10 +22,15 @@
 // DFMA from the operands themselves, so they propagate as in an FP64 product.
 //
 // Kernel structure: as the product kernel of tc_engine.cu (persistent, one CTA per SM, a producer
-// warp of bulk copies, one MMA-issuing thread, eight epilogue warps, every wait bounded).
+// warp of bulk copies, two MMA-issuing threads, eight epilogue warps, every wait bounded).
+//
+// What bounds it (products of 256^3): the MMAs, 46 cycles each with their operands read from shared
+// memory (6 KB at 128 B per cycle: 48; the tensor core alone 32), 78% of an SM's time, and the
+// recombination while it holds TMEM, 14%.
 #include <cuda_bf16.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "fix64.cuh"
 #include "kernels.cuh"
@@ -39,16 +44,17 @@ constexpr int S9 = kDig64;
 constexpr int BNC9 = 32;                    // complex output columns per tile (MMA N = 64)
 constexpr int NACC9 = 8;
 constexpr int ACC9 = 2 * BNC9;              // TMEM columns of one accumulator
-constexpr int TILE_B9 = 2 * BNC9 * BKS * 2;  // bytes of one B-plane tile (Re and Im rows)
 constexpr int SUB_B9 = BNC9 * BKS * 2;
-constexpr int STAGE9 = S9 * (TILE_A + TILE_B9);  // 54 KB
-constexpr int NST9 = 3;
+constexpr int SLOT_A9 = S9 * TILE_A;       // the planes of a left tile's K-step (36 KB)
+constexpr int SLOT_B9 = S9 * 3 * SUB_B9;   // the planes and parts of a right tile's K-block (27 KB)
+constexpr int NSA9 = 3, NSB9 = 2;          // slots of the two rings
+constexpr int RING9 = NSA9 * SLOT_A9 + NSB9 * SLOT_B9;
 constexpr int OUT9 = BM * BNC9 * 16;        // staging: [BM][BNC9] complex128, XOR-swizzled
-constexpr int SMEM9 = NST9 * STAGE9 + OUT9 + (BM + BNC9) * 4 + 128;
+constexpr int SMEM9 = RING9 + OUT9 + (BM + BNC9) * 4 + 128;
 
 struct Params {
-  const unsigned char* pa;  // A plane tiles [batch'][9][M_pad/128][nks][128 x 32 B]
-  const unsigned char* pb;  // B sub-tiles [batch'][9][N_pad/32][K_pad/16][3][32 x 32 B]: Re, Im, -Im
+  const unsigned char* pa;  // A [batch'][M_pad/128][K_pad/16][Re, Im][9][128 x 32 B]
+  const unsigned char* pb;  // B [batch'][N_pad/32][K_pad/16][9][-Im, Re, Im][rows x 32 B], rows = 32 or bn_last
   const int *eA, *eB;
   int M_pad, N_pad, nks, M, N, K, bn_last, escale;
   int a_batched, b_batched;
@@ -82,6 +88,9 @@ __device__ __forceinline__ int product_of(const Launch& L, long t, int& lt) {
   return q;
 }
 
+// the MMA thread that issues accumulator ga's digit products: 22 of the 45 one, 23 the other
+__host__ __device__ constexpr int mma_half9(int ga) { return ga == 5 || ga == 7; }
+
 __device__ __forceinline__ int at9(int r, int c) { return r * BNC9 + (c ^ (r & 7)); }
 
 // one output value from the eight accumulators (pre-scaled digit products), times 2^Es
@@ -109,15 +118,18 @@ __device__ __noinline__ cx<double> dot_dfma(const Params& p, int e, int m, int n
 }
 
 template <bool MANY>
-__global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__ Launch L) {
+__global__ void __launch_bounds__(352, 1) k_tc_gemm_fp64(const __grid_constant__ Launch L) {
   const int n_tiles = L.tile0[L.n];
   extern __shared__ __align__(1024) unsigned char base[];
-  cx<double>* out = reinterpret_cast<cx<double>*>(base + NST9 * STAGE9);
-  int* s_eA = reinterpret_cast<int*>(base + NST9 * STAGE9 + OUT9);
+  unsigned char* ringB = base + NSA9 * SLOT_A9;
+  cx<double>* out = reinterpret_cast<cx<double>*>(base + RING9);
+  int* s_eA = reinterpret_cast<int*>(base + RING9 + OUT9);
   int* s_eB = s_eA + BM;
-  uint64_t* full = reinterpret_cast<uint64_t*>(s_eB + BNC9);
-  uint64_t* empty = full + NST9;
-  uint64_t* accf = empty + NST9;
+  uint64_t* fullA = reinterpret_cast<uint64_t*>(s_eB + BNC9);
+  uint64_t* emptyA = fullA + NSA9;
+  uint64_t* fullB = emptyA + NSA9;
+  uint64_t* emptyB = fullB + NSB9;
+  uint64_t* accf = emptyB + NSB9;
   uint64_t* acce = accf + 1;
   uint64_t* holdbar = acce + 1;   // never arrived at (the wait test)
   uint64_t* drainbar = acce + 2;  // the MMA thread's final commit
@@ -126,14 +138,18 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < NST9; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
+    for (int s = 0; s < NSA9; ++s) {
+      mbar_init(&fullA[s], 1);
+      mbar_init(&emptyA[s], 2);  // both MMA threads' commits
     }
-    mbar_init(accf, 1);
+    for (int s = 0; s < NSB9; ++s) {
+      mbar_init(&fullB[s], 1);
+      mbar_init(&emptyB[s], 2);
+    }
+    mbar_init(accf, 2);
     mbar_init(acce, 1);
     mbar_init(holdbar, 1);
-    mbar_init(drainbar, 1);
+    mbar_init(drainbar, 2);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -147,7 +163,7 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__
 
   if (warp == 0) {
     if (lane == 0) {
-      long g = 0;
+      long ga = 0, gb = 0;  // copies into the left and the right ring so far
       bool ok = true;
       for (int k = 0; ok; ++k) {
         const long t = tile_at(k);
@@ -158,31 +174,34 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__
         const int e = lt / (p.NBt * p.MBt), mblk = (lt / p.NBt) % p.MBt, nblk = lt % p.NBt;
         if (p.active && !p.active[e]) continue;
         const long ea = p.a_batched ? e : 0, eb = p.b_batched ? e : 0;
-        const uint32_t sub = (uint32_t)(nblk == p.NBt - 1 ? p.bn_last : BNC9) * BKS * 2;
-        for (int ks = 0; ks < p.nks; ++ks, ++g) {
-          const int s = (int)(g % NST9);
-          if (!mbar_wait(&empty[s], ((uint32_t)(g / NST9) & 1u) ^ 1u, L.err, L.limit_ns)) { ok = false; break; }
-          mbar_expect_tx(&full[s], S9 * (TILE_A + 2 * sub));
-          unsigned char* st = base + s * STAGE9;
-          // K-stages [0, nkb): A's real parts against (Re, Im); [nkb, 2 nkb): imaginary against (-Im, Re)
-          const int part = ks >= nkb, kb = (int)(ks - part * nkb), s0 = part ? 2 : 0, s1 = part ? 0 : 1;
-          for (int d = 0; d < S9; ++d) {
-            bulk_load(st + d * TILE_A, p.pa + (((ea * S9 + d) * MB + mblk) * p.nks + ks) * (long)TILE_A, TILE_A, &full[s]);
-            const unsigned char* sb = p.pb + (((eb * S9 + d) * NB + nblk) * nkb + kb) * 3L * SUB_B9;
-            unsigned char* db = st + S9 * TILE_A + d * TILE_B9;
-            bulk_load(db, sb + s0 * SUB_B9, sub, &full[s]);
-            bulk_load(db + sub, sb + s1 * SUB_B9, sub, &full[s]);
+        const uint32_t bytesB = S9 * 3u * (uint32_t)(nblk == p.NBt - 1 ? p.bn_last : BNC9) * BKS * 2;
+        const unsigned char* srcA = p.pa + (ea * MB + mblk) * p.nks * (long)SLOT_A9;
+        const unsigned char* srcB = p.pb + (eb * NB + nblk) * nkb * (long)SLOT_B9;
+        for (int ks = 0; ks < p.nks; ++ks, ++ga) {
+          if (!(ks & 1)) {
+            const int s = (int)(gb % NSB9);
+            if (!mbar_wait(&emptyB[s], ((uint32_t)(gb / NSB9) & 1u) ^ 1u, L.err, L.limit_ns)) { ok = false; break; }
+            mbar_expect_tx(&fullB[s], bytesB);
+            bulk_load(ringB + s * SLOT_B9, srcB + (ks / 2) * (long)bytesB, bytesB, &fullB[s]);
+            ++gb;
           }
+          const int s = (int)(ga % NSA9);
+          if (!mbar_wait(&emptyA[s], ((uint32_t)(ga / NSA9) & 1u) ^ 1u, L.err, L.limit_ns)) { ok = false; break; }
+          mbar_expect_tx(&fullA[s], SLOT_A9);
+          bulk_load(base + s * SLOT_A9, srcA + ks * (long)SLOT_A9, SLOT_A9, &fullA[s]);
         }
       }
-      // the copies of the last stages issued land before the CTA goes on to exit
-      for (long gi = g > NST9 ? g - NST9 : 0; gi < g; ++gi)
-        mbar_wait_drain(&full[gi % NST9], (uint32_t)(gi / NST9) & 1u, kWaitLimitNs);
+      // the last copies issued land before the CTA goes on to exit
+      for (long g = ga > NSA9 ? ga - NSA9 : 0; g < ga; ++g)
+        mbar_wait_drain(&fullA[g % NSA9], (uint32_t)(g / NSA9) & 1u, kWaitLimitNs);
+      for (long g = gb > NSB9 ? gb - NSB9 : 0; g < gb; ++g)
+        mbar_wait_drain(&fullB[g % NSB9], (uint32_t)(g / NSB9) & 1u, kWaitLimitNs);
     }
     __syncwarp();
-  } else if (warp == 1) {
+  } else if (warp == 1 || warp == 10) {
+    const int half = warp == 10;
     if (lane == 0) {
-      long g = 0;
+      long ga = 0, gb = 0;
       int j = 0;
       bool ok = true;
       if (L.hold && !mbar_wait(holdbar, 0u, L.err, L.limit_ns)) ok = false;
@@ -192,26 +211,39 @@ __global__ void __launch_bounds__(320, 1) k_tc_gemm_fp64(const __grid_constant__
         int lt;
         const Params& p = L.p[product_of<MANY>(L, t, lt)];
         if (p.active && !p.active[lt / (p.NBt * p.MBt)]) continue;
-        const uint32_t idesc = idesc_n(2 * (lt % p.NBt == p.NBt - 1 ? p.bn_last : BNC9));
+        const uint32_t rows = lt % p.NBt == p.NBt - 1 ? p.bn_last : BNC9;
+        const uint32_t idesc = idesc_n(2 * rows);
+        const uint32_t part = rows * BKS * 2 / 16;  // a descriptor's address counts 16-byte units
         if (!mbar_wait(acce, ((uint32_t)j & 1u) ^ 1u, L.err, L.limit_ns)) break;
         fence_after();
-        uint32_t started = 0;
-        for (int ks = 0; ks < p.nks; ++ks, ++g) {
-          const int s = (int)(g % NST9);
-          if (!mbar_wait(&full[s], (uint32_t)(g / NST9) & 1u, L.err, L.limit_ns)) { ok = false; break; }
+        for (int ks = 0; ks < p.nks; ++ks, ++ga) {
+          const int sb = (int)(gb % NSB9), sa = (int)(ga % NSA9);
+          if (!(ks & 1) && !mbar_wait(&fullB[sb], (uint32_t)(gb / NSB9) & 1u, L.err, L.limit_ns)) { ok = false; break; }
+          if (!mbar_wait(&fullA[sa], (uint32_t)(ga / NSA9) & 1u, L.err, L.limit_ns)) { ok = false; break; }
           fence_after();
-          const uint32_t sa = su32(base + s * STAGE9);
+          // A's real parts (even steps) meet the B rows (Re, Im), its imaginary parts (-Im, Re)
+          const uint64_t ad = sdesc(su32(base + sa * SLOT_A9));
+          const uint64_t bd = sdesc(su32(ringB + sb * SLOT_B9)) + ((ks & 1) ? 0 : part);
+          auto issue = [&](auto H) {
 #pragma unroll
-          for (int i = 1; i <= S9; ++i) {
+            for (int i = 1; i <= S9; ++i) {
 #pragma unroll
-            for (int jj = 1; jj <= S9 + 1 - i; ++jj) {
-              const int ga = i + jj - 2 < NACC9 - 1 ? i + jj - 2 : NACC9 - 1;
-              mma(tmem + ga * ACC9, sdesc(sa + (i - 1) * TILE_A), sdesc(sa + S9 * TILE_A + (jj - 1) * TILE_B9), idesc,
-                  (started >> ga) & 1u);
-              started |= 1u << ga;
+              for (int jj = 1; jj <= S9 + 1 - i; ++jj) {
+                const int ga9 = i + jj - 2 < NACC9 - 1 ? i + jj - 2 : NACC9 - 1;
+                if (mma_half9(ga9) != decltype(H)::value) continue;
+                // the first product of an accumulator's first step overwrites it
+                const bool first = i == 1 && jj == ga9 + 1;
+                mma(tmem + ga9 * ACC9, ad + (i - 1) * TILE_A / 16, bd + (jj - 1) * 3 * part, idesc, first ? (uint32_t)(ks > 0) : 1u);
+              }
             }
+          };
+          if (half) issue(std::integral_constant<int, 1>());
+          else issue(std::integral_constant<int, 0>());
+          mma_commit(&emptyA[sa]);
+          if (ks & 1) {
+            mma_commit(&emptyB[sb]);
+            ++gb;
           }
-          mma_commit(&empty[s]);
         }
         if (!ok) break;
         mma_commit(accf);
@@ -358,9 +390,9 @@ __global__ void __launch_bounds__(32 * RPC) k_digitize_fp64(const __grid_constan
   }
   __syncthreads();
   if (t < RPC && r0 + t < R_pad) eout[(long)e * R_pad + r0 + t] = s_ex[t];
-  const long nks = 2L * K_pad / BKS, nkb = K_pad / BKS;
-  const long plane_bytes = side == 0 ? (long)(R_pad / BM) * nks * TILE_A : (long)(R_pad / BNC9) * nkb * 3 * SUB_B9;
-  unsigned char* pe = op.planes + (long)e * S9 * plane_bytes;
+  // the layouts of Params::pa and Params::pb: each block is what one copy of the product kernel takes
+  const int nkb = K_pad / BKS;
+  unsigned char* pe = op.planes + (long)e * (side == 0 ? (long)(R_pad / BM) * 2 * nkb * SLOT_A9 : (long)(R_pad / BNC9) * nkb * SLOT_B9);
   const int nkc = K_pad / 8;
   const int R_wr = side == 1 ? min(R_pad, (R + 7) / 8 * 8) : R_pad;  // columns past bn_last are never read
 #pragma unroll 1
@@ -377,18 +409,18 @@ __global__ void __launch_bounds__(32 * RPC) k_digitize_fp64(const __grid_constan
       vr[j] = dead ? kDigBias : fix_biased(v.re, P - ex);
       vi[j] = dead ? kDigBias : fix_biased(v.im, P - ex);
     }
-    long o0, o1, o2 = 0;
+    unsigned char *pr, *pi, *pn = nullptr;  // the chunk of Re, Im and -Im in the first plane; bytes from plane to plane
+    long step;
     if (side == 0) {
-      const long blk = r / BM, rw = r % BM;
-      auto off = [&](int kp) { return (blk * nks + kp / BKS) * TILE_A + sw32_offset((uint32_t)rw, (uint32_t)(kp % BKS)); };
-      o0 = off(k8);
-      o1 = off(K_pad + k8);
+      pr = pe + ((long)(r / BM) * nkb + k8 / BKS) * 2 * SLOT_A9 + sw32_offset((uint32_t)(r % BM), (uint32_t)(k8 % BKS));
+      pi = pr + SLOT_A9;
+      step = TILE_A;
     } else {
-      const long cb = r / BNC9, rw = r % BNC9;
-      const long o = (cb * nkb + k8 / BKS) * 3 * (long)SUB_B9 + sw32_offset((uint32_t)rw, (uint32_t)(k8 % BKS));
-      o0 = o;
-      o1 = o + SUB_B9;
-      o2 = o + 2 * SUB_B9;
+      const int cb = r / BNC9, rows = cb == R_pad / BNC9 - 1 ? (R - cb * BNC9 + 7) / 8 * 8 : BNC9, part = rows * BKS * 2;
+      pn = pe + (long)cb * nkb * SLOT_B9 + (long)(k8 / BKS) * (S9 * 3 * part) + sw32_offset((uint32_t)(r % BNC9), (uint32_t)(k8 % BKS));
+      pr = pn + part;
+      pi = pr + part;
+      step = 3 * part;
     }
 #pragma unroll
     for (int i = 0; i < S9; ++i) {
@@ -399,14 +431,13 @@ __global__ void __launch_bounds__(32 * RPC) k_digitize_fp64(const __grid_constan
                                          *reinterpret_cast<const __nv_bfloat162*>(&sh));
         return *reinterpret_cast<const uint32_t*>(&d);
       };
-      unsigned char* pl = pe + (long)i * plane_bytes;
       const uint4 re = make_uint4(word(vr[0], vr[1]), word(vr[2], vr[3]), word(vr[4], vr[5]), word(vr[6], vr[7]));
       const uint4 im = make_uint4(word(vi[0], vi[1]), word(vi[2], vi[3]), word(vi[4], vi[5]), word(vi[6], vi[7]));
-      *reinterpret_cast<uint4*>(pl + o0) = re;
-      *reinterpret_cast<uint4*>(pl + o1) = im;
+      *reinterpret_cast<uint4*>(pr + i * step) = re;
+      *reinterpret_cast<uint4*>(pi + i * step) = im;
       if (side == 1) {
         const uint32_t g = 0x80008000u;  // the bf16 sign bits
-        *reinterpret_cast<uint4*>(pl + o2) = make_uint4(im.x ^ g, im.y ^ g, im.z ^ g, im.w ^ g);
+        *reinterpret_cast<uint4*>(pn + i * step) = make_uint4(im.x ^ g, im.y ^ g, im.z ^ g, im.w ^ g);
       }
     }
   }
@@ -432,7 +463,7 @@ Dims9 dims9(int M, int N, int K) {
   d.l1 = 2 * d.K_pad <= 512 ? 7 : 6;
   d.P = DW * (S9 - 1) + d.l1 - 1;
   d.a = al1k((size_t)S9 * d.M_pad * 2 * d.K_pad * 2);
-  d.b = al1k((size_t)S9 * (d.N_pad / BNC9) * (d.K_pad / BKS) * 3 * SUB_B9);
+  d.b = al1k((size_t)(d.N_pad / BNC9) * (d.K_pad / BKS) * SLOT_B9);
   d.ea = al1k((size_t)d.M_pad * sizeof(int));
   d.eb = al1k((size_t)d.N_pad * sizeof(int));
   return d;
@@ -514,8 +545,8 @@ cudaError_t products9(const GemmArgs<double>* g, int n, unsigned char* scratch, 
   if ((e = n == 1 ? allow_smem(k_tc_gemm_fp64<false>, SMEM9, done1) : allow_smem(k_tc_gemm_fp64<true>, SMEM9, done2)) || (e = sm_count(sms))) return e;
   const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);
   if (ev) cudaEventRecord(ev[0], st);
-  if (n == 1) k_tc_gemm_fp64<false><<<grid, 320, SMEM9, st>>>(L);
-  else k_tc_gemm_fp64<true><<<grid, 320, SMEM9, st>>>(L);
+  if (n == 1) k_tc_gemm_fp64<false><<<grid, 352, SMEM9, st>>>(L);
+  else k_tc_gemm_fp64<true><<<grid, 352, SMEM9, st>>>(L);
   count_launch();
   if (ev) cudaEventRecord(ev[1], st);
   return cudaGetLastError();
