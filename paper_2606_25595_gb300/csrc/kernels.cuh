@@ -154,12 +154,15 @@ cudaError_t continuity(const double* cur, long ldc, const double* J, const doubl
 // ---- lead post-processing: from Sigma^R (complex128) build Gamma, Sigma^<, Sigma^>
 cudaError_t lead_sigmas(const cx<double>* SR, cx<double>* Gam, cx<double>* SL, cx<double>* SG,
                         const double* E, double mu, double kT, int b, int batch, cudaStream_t st);
-// one sweep's sums of the launched decimation (es += x, ep = (ep + x) + y) and, per active batch entry, its
-// convergence: active[e] = 0 once the largest modulus over al and be is < tol_rel * (*scale, or 1 if 0)
-// (scale is a device scalar, e.g. from max_modulus)
+// one sweep's sums of the launched decimation (es += x, ep = (ep + x) + y), the next sweep's g = E + i eta - ep
+// and, per active batch entry, its convergence: active[e] = 0 once the largest modulus over al and be is
+// < tol_rel * (scale, or 1 if 0).  Entry e is energy e % ne of contact e / ne (scale: one device scalar per
+// contact, e.g. from max_modulus)
 cudaError_t decim_update(cx<double>* es, cx<double>* ep, const cx<double>* x, const cx<double>* y, const cx<double>* al,
-                         const cx<double>* be, int b, double tol_rel, const double* scale, int* active, int batch,
-                         cudaStream_t st);
+                         const cx<double>* be, cx<double>* g, const double* E, double eta, int ne, int leads, int b,
+                         double tol_rel, const double* scale, int* active, cudaStream_t st);
+// status[e] <- the first nonzero of the codes st[k ne + e] of `leads` contacts, if it is still 0
+cudaError_t merge_status(const int* st, int leads, int ne, int* status, cudaStream_t stream);
 // out[0] = largest modulus of the n complex values X[0..n) (device scalar)
 cudaError_t max_modulus(const cx<double>* X, long n, double* out, cudaStream_t st);
 // p[0..n) = v

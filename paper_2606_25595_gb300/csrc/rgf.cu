@@ -58,7 +58,7 @@ inline bool uv_per_energy(const qtx_rgf_desc& d) {
 }
 
 struct Layout {
-  size_t g, gl, gl2, zk, xk, gfx, glfx, fx_slot, sig_stage, opnd[2], opnd_bytes[2], refine_act, tmp, inv_tmp, U, V, ident, ident_df, shared_blk, ref, f32a, f32tmp, dec, lead, obs, flags, dscale, bal, bscale, bgn, bhn, cres, cflag,
+  size_t g, gl, gl2, zk, xk, gfx, glfx, fx_slot, sig_stage, opnd[2], opnd_bytes[2], refine_act, tmp, inv_tmp, U, V, ident, ident_df, shared_blk, ref, f32a, f32tmp, dec, dec_flags, lead, obs, flags, dscale, bal, bscale, bgn, bhn, cres, cflag,
       tc_scratch, total;
   int n_tmp, n_dec;
   size_t tc_bytes;
@@ -110,6 +110,14 @@ struct qtx_rgf_plan_s {
 
 namespace {
 
+// Whether a device's two contacts are iterated in the same launches: their elimination is then a leaf, one CTA
+// (or cluster) a block that leaves SMs idle and lasts as long for two contacts as for one (b = 48, 12 energies:
+// 20.6 -> 13.9 ms a solve).  Larger blocks run one contact after the other through one contact's buffers.
+// (2 x 32767 entries: a grid's y and z extents.)
+bool contacts_together(const qtx_rgf_desc& d, bool single) {
+  return d.leads && !single && d.block_size <= kLeafMax && d.max_energies_in_flight <= 32767;
+}
+
 // inverse_only: the areas a batched inverse on its own uses (block g, and the refinement's)
 Layout make_layout(const qtx_rgf_desc& d, bool inverse_only = false) {
   Layout L{};
@@ -157,7 +165,9 @@ Layout make_layout(const qtx_rgf_desc& d, bool inverse_only = false) {
   L.f32tmp = a.take(L.refine64 ? Ec * bb * sizeof(cx<float>) + 4096 : 0);
   L.perm = a.take(L.refine64 && b <= kPivotedMax ? (size_t)Ec * b * sizeof(int) : 0);
   L.n_dec = 10;
-  L.dec = a.take(d.leads ? (size_t)L.n_dec * Ec * bb * sizeof(cx<double>) : 0);
+  const long nl = contacts_together(d, inverse_only) ? 2 : 1;  // contacts iterated in the same launches
+  L.dec = a.take(d.leads ? (size_t)L.n_dec * nl * Ec * bb * sizeof(cx<double>) : 0);
+  L.dec_flags = a.take(d.leads ? 2 * nl * Ec * sizeof(int) : 0);
   L.lead = a.take(d.leads && !inverse_only ? 8 * Ec * bb * sizeof(cx<double>) : 0);
   // per-energy observables: current, density, contact(2), transmission, scratch(2)
   L.obs = a.take((size_t)Ec * (2 * nb + 8) * sizeof(double));
@@ -658,49 +668,56 @@ qtx_status block_inverse<df>(qtx_rgf_plan_s* P, cx<df>* A, int n, int batch, con
 }
 
 // ----------------------------------------------------------------------------- contacts
-// Batched Sancho-Rubio decimation for one contact (FP64); result Sigma^R = H01 g_s H01^H in SR.
+// Batched Sancho-Rubio decimation (FP64) of one or both contacts; result Sigma^R = H01 g_s H01^H in SR.
 // Nothing here reads back to the host: for lead blocks of at most kDecimSmallMax the whole iteration
-// of an energy runs in one CTA (decimate_small); larger blocks run decim_max_iter sweeps of batched
-// launches in which converged energies are masked off on the device (their launches return at once),
+// of an energy and contact runs in one cluster (decimate_small); larger blocks run decim_max_iter sweeps of
+// batched launches in which converged energies are masked off on the device (their launches return at once),
 // with the tolerance scale max|H01| computed on the device too.  A solve with contacts therefore
-// makes no host synchronisation and can be captured in a CUDA graph.
+// makes no host synchronisation and can be captured in a CUDA graph.  Two contacts share the launches
+// (energies of the first, then of the second) where contacts_together.
 template <typename T>
-qtx_status contact(const Ctx<T>& c, const cx<double>* H00, const cx<double>* H01, double eta,
-                   cx<double>* SR) {
+qtx_status contacts(const Ctx<T>& c, int nl, const cx<double>* const* H00, const cx<double>* const* H01, double eta,
+                    cx<double>* const* SR) {
   qtx_rgf_plan_s* P = c.P;
   const int b = c.b, ne = c.ne;
   const long bb = c.bb;
   cudaStream_t st = c.st;
   if (b <= kDecimSmallMax) {
-    QTX_CK(decimate_small(1, &H00, &H01, &SR, c.E, eta, P->d.decim_tol, P->d.decim_max_iter, b, ne, c.status, st));
+    QTX_CK(decimate_small(nl, H00, H01, SR, c.E, eta, P->d.decim_tol, P->d.decim_max_iter, b, ne, c.status, st));
     return QTX_OK;
   }
+  const int N = nl * ne;
   cx<double>* D = reinterpret_cast<cx<double>*>(P->ws + P->L.dec);
-  auto buf = [&](int k) { return D + (size_t)k * P->Ec * bb; };
+  auto buf = [&](int k) { return D + (size_t)k * nl * P->Ec * bb; };
   cx<double>*alpha = buf(0), *beta = buf(1), *eps = buf(2), *eps_s = buf(3), *g = buf(4), *ag = buf(5),
   *bg = buf(6), *t1 = buf(7), *t2 = buf(8), *t3 = buf(9);
-  int* active = reinterpret_cast<int*>(P->ws + P->L.flags);
+  int* active = reinterpret_cast<int*>(P->ws + P->L.dec_flags);
+  int* status = nl > 1 ? active + (size_t)nl * P->Ec : c.status;
   double* scale = reinterpret_cast<double*>(P->ws + P->L.dscale);
-  QTX_CK(max_modulus(H01, bb, scale, st));
 
   Term<double> none;
-  Term<double> t01; t01.p = H01; t01.s = 0; t01.alpha = 1.0;
-  Term<double> t01h = t01; t01h.op = OP_C;
-  Term<double> t00; t00.p = H00; t00.s = 0; t00.alpha = 1.0;
-  QTX_CK((combine<double, double>(alpha, bb, t01, none, none, b, ne, nullptr, 0, 0, nullptr, st)));
-  QTX_CK((combine<double, double>(beta, bb, t01h, none, none, b, ne, nullptr, 0, 0, nullptr, st)));
-  QTX_CK((combine<double, double>(eps, bb, t00, none, none, b, ne, nullptr, 0, 0, nullptr, st)));
-  QTX_CK((combine<double, double>(eps_s, bb, t00, none, none, b, ne, nullptr, 0, 0, nullptr, st)));
-  QTX_CK(fill_int(active, 1, ne, st));
+  for (int k = 0; k < nl; ++k) {
+    const size_t o = (size_t)k * ne * bb;
+    QTX_CK(max_modulus(H01[k], bb, scale + k, st));
+    Term<double> t01; t01.p = H01[k]; t01.s = 0; t01.alpha = 1.0;
+    Term<double> t01h = t01; t01h.op = OP_C;
+    Term<double> t00; t00.p = H00[k]; t00.s = 0; t00.alpha = 1.0;
+    QTX_CK((combine<double, double>(alpha + o, bb, t01, none, none, b, ne, nullptr, 0, 0, nullptr, st)));
+    QTX_CK((combine<double, double>(beta + o, bb, t01h, none, none, b, ne, nullptr, 0, 0, nullptr, st)));
+    QTX_CK((combine<double, double>(eps + o, bb, t00, none, none, b, ne, nullptr, 0, 0, nullptr, st)));
+    QTX_CK((combine<double, double>(eps_s + o, bb, t00, none, none, b, ne, nullptr, 0, 0, nullptr, st)));
+    t00.alpha = -1.0;
+    QTX_CK((combine<double, double>(g + o, bb, t00, none, none, b, ne, c.E, eta, 1.0, nullptr, st)));  // z - eps
+  }
+  QTX_CK(fill_int(active, 1, N, st));
+  if (nl > 1) QTX_CK(fill_int(status, 0, N, st));
   qtx_status s;
   auto G = [&](const cx<double>* A, const cx<double>* B, cx<double>* C) {
-    return gargs<double>(b, b, b, A, b, bb, OP_N, B, b, bb, OP_N, nullptr, 0, 0, C, b, bb, 1.0, 0.0, ne, active);
+    return gargs<double>(b, b, b, A, b, bb, OP_N, B, b, bb, OP_N, nullptr, 0, 0, C, b, bb, 1.0, 0.0, N, active);
   };
   for (int it = 1; it <= P->d.decim_max_iter; ++it) {
-    // four launches a sweep beside the inverse's: a converged energy's CTAs return at once
-    Term<double> te; te.p = eps; te.s = bb; te.alpha = -1.0;
-    QTX_CK((combine<double, double>(g, bb, te, none, none, b, ne, c.E, eta, 1.0, active, st)));  // z - eps
-    if ((s = inverse_refined<double>(P, g, b, ne, active, c.status, st))) return s;
+    // three launches a sweep beside the inverse's: a converged energy's CTAs return at once
+    if ((s = inverse_refined<double>(P, g, b, N, active, status, st))) return s;
     GemmMulti<double> m;
     m.n = 2;
     m.g[0] = G(alpha, g, ag);
@@ -715,15 +732,28 @@ qtx_status contact(const Ctx<T>& c, const cx<double>* H00, const cx<double>* H01
     // converged energies leave stale blocks in the exchanged buffers, which nothing reads again
     std::swap(alpha, t3);
     std::swap(beta, g);
-    QTX_CK(decim_update(eps_s, eps, t1, t2, alpha, beta, b, P->d.decim_tol, scale, active, ne, st));
+    // eps_s, eps, the convergence flags and the next sweep's z - eps (in g)
+    QTX_CK(decim_update(eps_s, eps, t1, t2, alpha, beta, g, c.E, eta, ne, nl, b, P->d.decim_tol, scale, active, st));
   }
-  QTX_CK(flag_active(active, c.status, (int)QTX_ERR_NOT_CONVERGED, ne, st));
-  Term<double> tes; tes.p = eps_s; tes.s = bb; tes.alpha = -1.0;
-  QTX_CK((combine<double, double>(g, bb, tes, none, none, b, ne, c.E, eta, 1.0, nullptr, st)));  // z - eps_s
-  if ((s = inverse_refined<double>(P, g, b, ne, nullptr, c.status, st))) return s;
+  QTX_CK(flag_active(active, status, (int)QTX_ERR_NOT_CONVERGED, N, st));
+  for (int k = 0; k < nl; ++k) {
+    const size_t o = (size_t)k * ne * bb;
+    Term<double> tes; tes.p = eps_s + o; tes.s = bb; tes.alpha = -1.0;
+    QTX_CK((combine<double, double>(g + o, bb, tes, none, none, b, ne, c.E, eta, 1.0, nullptr, st)));  // z - eps_s
+  }
+  if ((s = inverse_refined<double>(P, g, b, N, nullptr, status, st))) return s;
   // Sigma^R = H01 g_s H01^H
-  if ((s = gemm<double>(P, gargs<double>(b, b, b, H01, b, 0, OP_N, g, b, bb, OP_N, nullptr, 0, 0, t1, b, bb, 1.0, 0.0, ne, nullptr), st, true))) return s;
-  if ((s = gemm<double>(P, gargs<double>(b, b, b, t1, b, bb, OP_N, H01, b, 0, OP_C, nullptr, 0, 0, SR, b, bb, 1.0, 0.0, ne, nullptr), st, true))) return s;
+  GemmMulti<double> m;
+  m.n = nl;
+  for (int k = 0; k < nl; ++k)
+    m.g[k] = gargs<double>(b, b, b, H01[k], b, 0, OP_N, g + (size_t)k * ne * bb, b, bb, OP_N, nullptr, 0, 0, t1 + (size_t)k * ne * bb, b,
+                           bb, 1.0, 0.0, ne, nullptr);
+  QTX_CK(gemm_simt_multi<double>(m, st));
+  for (int k = 0; k < nl; ++k)
+    m.g[k] = gargs<double>(b, b, b, t1 + (size_t)k * ne * bb, b, bb, OP_N, H01[k], b, 0, OP_C, nullptr, 0, 0, SR[k], b, bb, 1.0, 0.0, ne,
+                           nullptr);
+  QTX_CK(gemm_simt_multi<double>(m, st));
+  if (nl > 1) QTX_CK(merge_status(status, nl, ne, c.status, st));
   return QTX_OK;
 }
 
@@ -856,12 +886,9 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
     const cx<double>* H00[2] = {(const cx<double>*)in->lead_H00_L, (const cx<double>*)in->lead_H00_R};
     const cx<double>* H01[2] = {(const cx<double>*)in->lead_H01_L, (const cx<double>*)in->lead_H01_R};
     cx<double>* SR[2] = {SR_L, SR_R};
-    if (b <= kDecimSmallMax) {  // both contacts of every energy in one launch
-      QTX_CK(decimate_small(2, H00, H01, SR, c.E, eta, d.decim_tol, d.decim_max_iter, b, ne, status, st));
-    } else {
-      for (int k = 0; k < 2; ++k)
-        if ((s = contact<T>(c, H00[k], H01[k], eta, SR[k]))) return s;
-    }
+    const int nl = contacts_together(d, false) ? 2 : 1;
+    for (int k = 0; k < 2; k += nl)
+      if ((s = contacts<T>(c, nl, H00 + k, H01 + k, eta, SR + k))) return s;
     QTX_CK(lead_sigmas(SR_L, Gam_L, SL_L, SG_L, c.E, in->mu_L, in->kT, b, ne, st));
     QTX_CK(lead_sigmas(SR_R, Gam_R, SL_R, SG_R, c.E, in->mu_R, in->kT, b, ne, st));
   }
@@ -1882,7 +1909,9 @@ qtx_status qtx_lead_self_energy(int n, const void* H00, const void* H01, const d
   int* stat = status ? status : reinterpret_cast<int*>(P->ws + P->L.flags) + 2 * P->Ec;
   cudaMemsetAsync(stat, 0, sizeof(int) * n_energies, st);
   Ctx<double> c{P, st, n_energies, energies, stat, (long)n * n, n};
-  s = contact<double>(c, (const cx<double>*)H00, (const cx<double>*)H01, eta, (cx<double>*)SigR);
+  const cx<double>*h00 = (const cx<double>*)H00, *h01 = (const cx<double>*)H01;
+  cx<double>* sr = (cx<double>*)SigR;
+  s = contacts<double>(c, 1, &h00, &h01, eta, &sr);
   cudaError_t e = cudaStreamSynchronize(st);
   if (s == QTX_OK && e != cudaSuccess) s = QTX_ERR_CUDA;
   return s;

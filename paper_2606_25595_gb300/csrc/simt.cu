@@ -1255,17 +1255,22 @@ cudaError_t fill_int(int* p, int v, int n, cudaStream_t st) {
 // One sweep's sums of the launched decimation and its convergence test: es += x, ep = (ep + x) + y, then
 // active[e] = 0 once the largest modulus over alpha and beta is below tol_rel * (*scale, or 1 if 0).
 __global__ void __launch_bounds__(512) k_decim_update(cx<double>* es, cx<double>* ep, const cx<double>* x, const cx<double>* y,
-                                                      const cx<double>* al, const cx<double>* be, int b, double tol_rel,
+                                                      const cx<double>* al, const cx<double>* be, cx<double>* g,
+                                                      const double* E, double eta, int ne, int b, double tol_rel,
                                                       const double* scale, int* active) {
-  const int e = blockIdx.x;
+  const int e = blockIdx.x, lead = e / ne;
   if (!active[e]) return;
-  const double tol = tol_rel * (*scale > 0.0 ? *scale : 1.0);
+  const double tol = tol_rel * (scale[lead] > 0.0 ? scale[lead] : 1.0);
+  const double Er = E[e - lead * ne];
   const long bb = (long)b * b, o = (long)e * bb;
   unsigned h = 0;
   auto hw = [](double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; };
   for (long i = o + threadIdx.x; i < o + bb; i += blockDim.x) {
     es[i] = es[i] + x[i];
-    ep[i] = (ep[i] + x[i]) + y[i];
+    const cx<double> p = (ep[i] + x[i]) + y[i];
+    const bool diag = (int)(i - o) % (b + 1) == 0;
+    ep[i] = p;
+    g[i] = mk<double>((0.0 - p.re) + (diag ? Er : 0.0), (0.0 - p.im) + (diag ? eta : 0.0));
     h = max(h, max(max(hw(al[i].re), hw(al[i].im)), max(hw(be[i].re), hw(be[i].im))));
   }
   // the largest |re|, |im| decides by its high word unless it lies within sqrt(2) of tol or is not a number
@@ -1294,9 +1299,9 @@ __global__ void __launch_bounds__(512) k_decim_update(cx<double>* es, cx<double>
   }
 }
 cudaError_t decim_update(cx<double>* es, cx<double>* ep, const cx<double>* x, const cx<double>* y, const cx<double>* al,
-                         const cx<double>* be, int b, double tol_rel, const double* scale, int* active, int batch,
-                         cudaStream_t st) {
-  k_decim_update<<<batch, 512, 0, st>>>(es, ep, x, y, al, be, b, tol_rel, scale, active);
+                         const cx<double>* be, cx<double>* g, const double* E, double eta, int ne, int leads, int b, double tol_rel,
+                         const double* scale, int* active, cudaStream_t st) {
+  k_decim_update<<<ne * leads, 512, 0, st>>>(es, ep, x, y, al, be, g, E, eta, ne, b, tol_rel, scale, active);
   count_launch();
   return cudaGetLastError();
 }
@@ -1307,6 +1312,22 @@ __global__ void k_flag_active(const int* active, int* status, int code, int batc
 }
 cudaError_t flag_active(const int* active, int* status, int code, int batch, cudaStream_t st) {
   k_flag_active<<<(batch + 127) / 128, 128, 0, st>>>(active, status, code, batch);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// first failure of an energy over its contacts (leads x ne codes) into its status
+__global__ void k_merge_status(const int* st, int leads, int ne, int* status) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= ne) return;
+  for (int k = 0; k < leads; ++k)
+    if (st[k * ne + e]) {
+      atomicCAS(status + e, 0, st[k * ne + e]);
+      return;
+    }
+}
+cudaError_t merge_status(const int* st, int leads, int ne, int* status, cudaStream_t stream) {
+  k_merge_status<<<(ne + 127) / 128, 128, 0, stream>>>(st, leads, ne, status);
   count_launch();
   return cudaGetLastError();
 }
