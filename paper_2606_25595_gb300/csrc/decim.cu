@@ -74,8 +74,12 @@ __device__ __forceinline__ cx<double> upd_col(cx<double> f, cx<double> r) {
 // 520 cycles) -- runs in warp 0 while the other warps make step k - 1's update of the remaining columns.
 template <int NM>
 __device__ cx<double>* eliminate(DSmem<NM>& s, cx<double>* A, cx<double>* B, const gj::FastDiv& fd) {
-  constexpr int LD = DSmem<NM>::LD, kUpd = kThreads - 32;
+  constexpr int LD = DSmem<NM>::LD;
   const int t = threadIdx.x, n = fd.n;
+  // the update's threads: warps 1 to 7, or while the chain decides (n <= 24) those of the other quarters of the SM,
+  // each with an FP64 pipe of its own (warps 0 and 4 share one)
+  const bool apart = n <= 24;
+  const int kUpd = apart ? 192 : 224, u = t < 32 ? -1 : (apart ? (t < 128 ? t - 32 : (t < 160 ? kUpd * 64 : t - 64)) : t - 32);
   // pivot row of column k of block X and the reciprocal of its entry (warp 0)
   auto pivot = [&](const cx<double>* X, int k) {
     const unsigned long long key = (t >= k && t < n) ? gj::pivot_key(X[t * LD + k]) : 0ull;
@@ -111,12 +115,12 @@ __device__ cx<double>* eliminate(DSmem<NM>& s, cx<double>* A, cx<double>* B, con
         pivot(B, c1);
       }
     } else {
-      for (int idx = t - 32; idx < n * n; idx += kUpd) {
+      for (int idx = u; idx < n * n; idx += kUpd) {
         const int i = fd.div(idx), j = idx - i * n;
         if (j != k && j != c1) B[i * LD + j] = i == k ? s.rowk[j] : upd(A[src(i) * LD + j], A[src(i) * LD + k], s.rowk[j]);
       }
-      if (t >= kUpd) {
-        const int i = t - kUpd;
+      if (t >= kThreads - 32) {
+        const int i = t - (kThreads - 32);
         if (i < n) B[i * LD + k] = i == k ? s.rowk[k] : upd_col(A[src(i) * LD + k], s.rowk[k]);
       }
     }

@@ -96,3 +96,78 @@ def test_decimation_of_ill_conditioned_leads(q):
     zero, st = q.lead_self_energy(torch.tensor(H00).cuda(), torch.zeros_like(torch.tensor(H01)).cuda(),
                                   torch.tensor(E[1:]).cuda(), 1e-6)
     assert (st.cpu().numpy() == 0).all() and (zero == 0).all()
+
+
+# the FP64 elimination in clusters of 8, 4, 2 and 1 CTAs (as the batch grows): columns split unevenly, one or two
+# rows a lane; every split rounds alike, so a block's inverse does not depend on the batch it is in
+@pytest.mark.parametrize("n", [1, 9, 17, 31, 32])
+def test_fp64_leaf_inverse_is_the_same_in_every_cluster_size(q, n):
+    import torch
+    rng = np.random.default_rng(n)
+    A = rng.standard_normal((200, n, n)) + 1j * rng.standard_normal((200, n, n))
+    dev = torch.tensor(A).cuda()
+    full, st = q.zinv_batched(dev.clone(), precision="fp64")
+    assert not st.any()
+    X = full.cpu().numpy()
+    for e in range(0, 200, 40):  # Gauss-Jordan with partial pivoting: a few n eps kappa
+        ref = np.linalg.inv(A[e])
+        assert np.abs(X[e] - ref).max() <= 16 * n * 2.0**-53 * np.linalg.cond(A[e]) * np.abs(ref).max()
+    for batch in (1, 30, 70):
+        part, _ = q.zinv_batched(dev[:batch].clone(), precision="fp64")
+        assert torch.equal(part, full[:batch])
+
+
+# launched contacts (blocks above 32): their eliminations over 8 to 1 CTAs, and a device's two contacts together
+@pytest.mark.parametrize("n", [33, 50, 64])
+def test_launched_contacts_are_the_same_in_every_cluster_size(q, n):
+    import torch
+    rng = np.random.default_rng(n)
+    H00 = rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))
+    H00 = torch.tensor((H00 + H00.conj().T) / 4).cuda()
+    H01 = torch.tensor((rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))) / 8).cuda()
+    E = torch.linspace(-1, 1, 160, dtype=torch.float64).cuda()
+    full, st = q.lead_self_energy(H00, H01, E, 1e-2, max_iter=30)
+    assert not st.any() and torch.isfinite(torch.view_as_real(full)).all()
+    for ne in (1, 12, 40):
+        part, _ = q.lead_self_energy(H00, H01, E[:ne].clone(), 1e-2, max_iter=30)
+        assert torch.equal(part, full[:ne])
+
+
+def test_two_launched_contacts_in_uneven_chunks(q):
+    dev = _device(40, 2, 5, 0, 1, 0, 0)
+    ref = O.solve(dev)
+    res = q.solve_device(dev, "fp64", max_energies_in_flight=2)  # chunks of 2, 2 and 1 energies
+    for k in ("GR_diag", "GL_diag", "current"):  # 2^-53 times the decimation's conditioning (kappa to 1e4, squared)
+        assert np.linalg.norm(res[k] - ref[k]) <= 1e-8 * np.linalg.norm(ref[k]), k
+    bad = np.array(dev["energies"])
+    bad[1] = np.nan
+    r2 = q.solve_device(dev, "fp64", energies=bad, weights=np.ones(5), max_energies_in_flight=2)
+    assert r2["status"].tolist() == [0, 4, 0, 0, 0]
+    for e in (0, 2, 3, 4):
+        assert np.array_equal(r2["GL_diag"][e], res["GL_diag"][e])
+
+
+def test_fp64_elimination_reciprocal(q):
+    """1 x 1 inverses: Smith's quotients, each rounded to nearest, over both orders of the parts, signs, exponents
+    inside and outside the range of the FP32-seeded divisions, tiny parts and zeros."""
+    import torch
+    from fractions import Fraction as F
+    rng = np.random.default_rng(3)
+    m = rng.uniform(1, 2, (4000, 2)) * rng.choice([-1, 1], (4000, 2))
+    ex = np.concatenate([rng.integers(-3, 4, (2000, 2)), rng.integers(-90, 90, (1000, 2)), rng.integers(-480, 480, (1000, 1)) + rng.integers(-70, 70, (1000, 2))])
+    z = np.ldexp(m, ex)
+    z[:6] = [[1, 0], [0, 1], [3, -0.0], [1, 1], [-1.5, 1.5], [1 + 2.0**-52, 1 - 2.0**-53]]
+    got, st = q.zinv_batched(torch.tensor(z[:, 0] + 1j * z[:, 1]).reshape(-1, 1, 1).cuda(), precision="fp64")
+    assert not st.any()
+    got = got.cpu().numpy().ravel()
+    for (re, im), w in zip(z, got):
+        tall = abs(re) >= abs(im)
+        p, d0 = (im, re) if tall else (re, im)
+        r = float(F(p) / F(d0))
+        d = float(F(p) * F(r) + F(d0))  # one rounding, as a fused multiply-add
+        one, other = float(1 / F(d)), float(F(r) / F(d))
+        ref = complex(one, -other) if tall else complex(other, -one)
+        if (re, im) == (z[5, 0], z[5, 1]):  # 1/d within 2^-106 of the middle of two numbers: either may come
+            assert abs(w.real - ref.real) <= 2.0**-53 and abs(w.imag - ref.imag) <= 2.0**-53
+        else:
+            assert w == ref, (re, im, w, ref)
