@@ -99,6 +99,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_lesser_offdiag(const cx<T>* PGL, cx<T>* X2, cx<T>* GLu, const cx<double>* Hup,
                                                         const cx<double>* Sup, const double* E, int b, int nt,
                                                         typename PartialOf<T>::type* part) {
+  after_previous();
   using Acc = typename PartialOf<T>::type;
   extern __shared__ __align__(16) unsigned char dsm[];
   cx<T>(*pij)[TS + 1] = reinterpret_cast<cx<T>(*)[TS + 1]>(dsm);
@@ -160,6 +161,7 @@ __global__ void __launch_bounds__(256) k_lesser_offdiag(const cx<T>* PGL, cx<T>*
 template <typename T>
 __global__ void __launch_bounds__(256) k_lesser_diag(cx<T>* gl, const cx<T>* X, cx<double>* out64, long so, int b, int nt,
                                                      double* part) {
+  after_previous();
   extern __shared__ __align__(16) unsigned char dsm[];
   cx<T>(*tij)[TS + 1] = reinterpret_cast<cx<T>(*)[TS + 1]>(dsm);
   cx<T>(*tji)[TS + 1] = tij + TS;
@@ -206,6 +208,7 @@ __global__ void __launch_bounds__(256) k_lesser_diag(cx<T>* gl, const cx<T>* X, 
 template <typename Acc>
 __global__ void k_trace_sums(double* cur, long ldcur, const Acc* pc, int nc, double* den, long ldden, const double* pd,
                              int nd) {
+  after_previous();
   const int e = blockIdx.x, l = threadIdx.x;
   if (cur) {
     Acc a;
@@ -237,7 +240,7 @@ cudaError_t lesser_offdiag(const cx<T>* PGL, cx<T>* X2, cx<T>* GLu, const cx<dou
   static std::atomic<unsigned long long> done{0};
   const cudaError_t e = allow_smem(k_lesser_offdiag<T>, smem, done);
   if (e != cudaSuccess) return e;
-  k_lesser_offdiag<T><<<dim3(nt * (nt + 1) / 2, batch), 256, smem, st>>>(
+  launch_after(k_lesser_offdiag<T>, dim3(nt * (nt + 1) / 2, batch), 256, smem, st, 
       PGL, X2, GLu, Hup, Sup, E, b, nt, reinterpret_cast<typename PartialOf<T>::type*>(scratch));
   count_launch();
   return cudaGetLastError();
@@ -249,9 +252,9 @@ cudaError_t lesser_diag(cx<T>* gl, const cx<T>* X, cx<double>* out64, long so, d
   using Acc = typename PartialOf<T>::type;
   const int nt = tiles_of(b), np = nt * (nt + 1) / 2;
   double* pd = reinterpret_cast<double*>(scratch) + (size_t)batch * np;
-  k_lesser_diag<T><<<dim3(np, batch), 256, 2 * TS * (TS + 1) * sizeof(cx<T>), st>>>(gl, X, out64, so, b, nt, pd);
+  launch_after(k_lesser_diag<T>, dim3(np, batch), 256, 2 * TS * (TS + 1) * sizeof(cx<T>), st, gl, X, out64, so, b, nt, pd);
   count_launch();
-  k_trace_sums<Acc><<<batch, 32, 0, st>>>(cur, ldcur, reinterpret_cast<const Acc*>(scratch), np, den, ldden, pd, nt);
+  launch_after(k_trace_sums<Acc>, batch, 32, 0, st, cur, ldcur, reinterpret_cast<const Acc*>(scratch), np, den, ldden, pd, nt);
   count_launch();
   return cudaGetLastError();
 }

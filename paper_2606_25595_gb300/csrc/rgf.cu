@@ -64,6 +64,7 @@ struct Layout {
   size_t tc_bytes;
   size_t tc_more;  // scratch of further products launched together with one in tc_scratch (n_more of them)
   int n_more;
+  bool short_launches;  // a product fills less than four waves of the GPU (see launch_after)
   bool refine64;  // FP64 block inverses by refinement (inverse_f64) have their areas
   size_t perm;
 };
@@ -197,6 +198,7 @@ Layout make_layout(const qtx_rgf_desc& d, bool inverse_only = false) {
   // on 152 SMs).  Larger products fill their waves alone.
   const long col = d.precision == QTX_EMU64 ? 48 : 64;
   const long tiles = ((b + 127) / 128) * ((b + col - 1) / col) * Ec;
+  L.short_launches = tiles <= 4 * 152;
   L.n_more = !inverse_only && L.tc_bytes && d.precision != QTX_FP64 && tiles <= 4 * 152 ? kMany - 1 : 0;
   L.tc_more = a.take((size_t)L.n_more * align_up(L.tc_bytes, 1024));
   // kept digitised operands (emulated modes): two left operands, b x b, E_c energies (none when the
@@ -1493,6 +1495,7 @@ qtx_status qtx_rgf_solve(qtx_rgf_plan P, const qtx_rgf_inputs* in, const qtx_rgf
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   P->last = st;
   P->worst = 0;
+  EarlyLaunches early(P->L.short_launches && !P->group ? 2 : 1);
   // the bounded-wait flag of the tensor-core launches starts clear for every solve
   if (cudaMemsetAsync(P->d_err_flag, 0, sizeof(int), st) != cudaSuccess) {
     P->err = "clearing the wait flag failed";
@@ -1532,6 +1535,7 @@ qtx_status qtx_w_assemble(qtx_rgf_plan P, const qtx_w_inputs* in, const qtx_w_ou
   }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   P->last = st;
+  EarlyLaunches early(P->L.short_launches && !P->group ? 2 : 1);
   if (cudaMemsetAsync(P->d_err_flag, 0, sizeof(int), st) != cudaSuccess) {
     P->err = "clearing the wait flag failed";
     cudaGetLastError();
@@ -1966,6 +1970,7 @@ struct qtx_rgf_group_s {
   // with mu held: launch every pending product and release the posting threads
   void launch_pending() {
     cudaError_t e = cudaSuccess;
+    EarlyLaunches none(0);  // behind events of other streams
     for (Req* r : pending)
       if (e == cudaSuccess) e = cudaStreamWaitEvent(gst, ready[r->member], 0);
     std::vector<bool> taken(pending.size(), false);

@@ -135,11 +135,13 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs<T>& g, const int e) {
 
 template <typename T, int BM, int BN, int BK, int TM, int TN>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_gemm(GemmArgs<T> g) {
+  after_previous();
   gemm_tile<T, BM, BN, BK, TM, TN>(g, blockIdx.z);
 }
 // several products of the same M, N and batch in one launch (blockIdx.z: product, then batch entry)
 template <typename T, int BM, int BN, int BK, int TM, int TN>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_gemm_multi(const __grid_constant__ GemmMulti<T> m) {
+  after_previous();
   const int q = blockIdx.z / m.g[0].batch;
   gemm_tile<T, BM, BN, BK, TM, TN>(m.g[q], blockIdx.z - q * m.g[0].batch);
 }
@@ -153,8 +155,8 @@ static cudaError_t launch_gemm(const GemmMulti<T>& m, cudaStream_t st) {
     N = N > m.g[q].N ? N : m.g[q].N;
   }
   dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, g.batch * m.n);
-  if (m.n == 1) k_gemm<T, BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, st>>>(g);
-  else k_gemm_multi<T, BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, st>>>(m);
+  if (m.n == 1) launch_after(k_gemm<T, BM, BN, BK, TM, TN>, grid, (BM / TM) * (BN / TN), 0, st, g);
+  else launch_after(k_gemm_multi<T, BM, BN, BK, TM, TN>, grid, (BM / TM) * (BN / TN), 0, st, m);
   count_launch();
   return cudaGetLastError();
 }
@@ -237,6 +239,7 @@ __device__ __forceinline__ cx<float> pick(bool c, cx<float> x, cx<float> y) {
 
 template <int NMAX>
 __global__ void __launch_bounds__(256) k_leaf_inverse(cx<float>* Ag, long lda, long sA, int n, const int* active, int* status) {
+  after_previous();
   constexpr int R = NMAX / 16;
   const int e = blockIdx.x;
   if (active && !active[e]) return;
@@ -349,9 +352,9 @@ cudaError_t leaf_inverse<float>(cx<float>* A, long lda, long sA, int n, int batc
                                 cudaStream_t st) {
   if (n <= 0 || n > kLeafMax) return cudaErrorInvalidValue;
   if (n <= 32)
-    k_leaf_inverse<32><<<batch, 256, 0, st>>>(A, lda, sA, n, active, status);
+    launch_after(k_leaf_inverse<32>, batch, 256, 0, st, A, lda, sA, n, active, status);
   else
-    k_leaf_inverse<64><<<batch, 256, 0, st>>>(A, lda, sA, n, active, status);
+    launch_after(k_leaf_inverse<64>, batch, 256, 0, st, A, lda, sA, n, active, status);
   count_launch();
   return cudaGetLastError();
 }
@@ -441,6 +444,7 @@ template <typename Tin, typename Tout>
 __global__ void __launch_bounds__(256) k_combine(cx<Tout>* out, long sOut, Term<Tin> t0, Term<Tin> t1,
                                                  Term<Tin> t2, int b, const double* E, double eta,
                                                  double diag_coef, int has_diag, const int* active) {
+  after_previous();
   using Acc = typename AccSel<Tin, Tout>::type;
   const int e = blockIdx.z;
   if (active && !active[e]) return;
@@ -513,6 +517,7 @@ template <typename Tin, typename Tout>
 __global__ void __launch_bounds__(256) k_combine_flat(cx<Tout>* out, long sOut, Term<Tin> t0, Term<Tin> t1,
                                                       Term<Tin> t2, int b, const double* E, double eta,
                                                       double diag_coef, int has_diag, const int* active) {
+  after_previous();
   using Acc = typename AccSel<Tin, Tout>::type;
   const int e = blockIdx.y;
   if (active && !active[e]) return;
@@ -571,13 +576,13 @@ cudaError_t combine(cx<Tout>* out, long sOut, Term<Tin> t0, Term<Tin> t1, Term<T
   auto direct = [](const Term<Tin>& t) { return !t.p || t.op != OP_C; };  // absent terms count as direct
   if (direct(t0) && direct(t1) && direct(t2)) {
     dim3 fgrid(flat_ctas((long)b * b, batch), batch);
-    k_combine_flat<Tin, Tout><<<fgrid, 256, 0, st>>>(out, sOut, t0, t1, t2, b, E, eta, diag_coef, diag_coef != 0.0,
+    launch_after(k_combine_flat<Tin, Tout>, fgrid, 256, 0, st, out, sOut, t0, t1, t2, b, E, eta, diag_coef, diag_coef != 0.0,
                                                      active);
     count_launch();
     return cudaGetLastError();
   }
   dim3 grid((b + 31) / 32, (b + 31) / 32, batch);
-  k_combine<Tin, Tout><<<grid, 256, 0, st>>>(out, sOut, t0, t1, t2, b, E, eta, diag_coef, diag_coef != 0.0, active);
+  launch_after(k_combine<Tin, Tout>, grid, 256, 0, st, out, sOut, t0, t1, t2, b, E, eta, diag_coef, diag_coef != 0.0, active);
   count_launch();
   return cudaGetLastError();
 }
@@ -595,6 +600,7 @@ template <typename T>
 __global__ void k_assemble_diag(cx<T>* out, const cx<double>* H, const cx<double>* S,
                                 const cx<double>* SigR, long sSig, const cx<double>* lead,
                                 long sLead, const double* E, double eta, int b) {
+  after_previous();
   const int e = blockIdx.y;
   const int bb = b * b;  // b <= 4096: 32-bit indices (no 64-bit division per element)
   const double Er = E[e];
@@ -636,7 +642,7 @@ cudaError_t assemble_diag(cx<T>* out, const cx<double>* H, const cx<double>* S,
                           const double* E, double eta, int b, int batch, cudaStream_t st) {
   const long bb = (long)b * b;
   dim3 grid((unsigned)((bb + 255) / 256 < 1024 ? (bb + 255) / 256 : 1024), batch);
-  k_assemble_diag<T><<<grid, 256, 0, st>>>(out, H, S, SigR, sSig, lead, sLead, E, eta, b);
+  launch_after(k_assemble_diag<T>, grid, 256, 0, st, out, H, S, SigR, sSig, lead, sLead, E, eta, b);
   count_launch();
   return cudaGetLastError();
 }
@@ -647,6 +653,7 @@ template cudaError_t assemble_diag<df>(cx<df>*, const cx<double>*, const cx<doub
 template <typename T>
 __global__ void k_axpby_from64(cx<T>* out, long sOut, const cx<double>* X, long sX, double c1,
                                const cx<double>* Y, long sY, double c2, int b, int k1, int k2) {
+  after_previous();
   const int e = blockIdx.y;
   const long bb = (long)b * b;
   for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < bb; idx += (long)gridDim.x * blockDim.x) {
@@ -680,7 +687,7 @@ cudaError_t axpby_from64(cx<T>* out, long sOut, const cx<double>* X, long sX, do
   const long bb = (long)b * b;
   dim3 grid((unsigned)((bb + 255) / 256 < 1024 ? (bb + 255) / 256 : 1024), batch);
   const int k1 = c1 == 1.0 ? 1 : (c1 == -1.0 ? -1 : 0), k2 = c2 == 1.0 ? 1 : (c2 == -1.0 ? -1 : 0);
-  k_axpby_from64<T><<<grid, 256, 0, st>>>(out, sOut, X, sX, c1, Y, sY, c2, b, k1, k2);
+  launch_after(k_axpby_from64<T>, grid, 256, 0, st, out, sOut, X, sX, c1, Y, sY, c2, b, k1, k2);
   count_launch();
   return cudaGetLastError();
 }
@@ -696,6 +703,7 @@ __device__ __forceinline__ float add_t(float a, float c) { return a + c; }
 template <typename T>
 __global__ void __launch_bounds__(256) k_broadcast_diag(cx<T>* out, long sOut, const cx<T>* src, int b,
                                                         const double* E, double eta) {
+  after_previous();
   const int e = blockIdx.y;
   const int bb = b * b;
   cx<T> z;
@@ -717,7 +725,7 @@ template <typename T>
 cudaError_t broadcast_diag(cx<T>* out, long sOut, const cx<T>* src, int b, const double* E, double eta, int batch,
                            cudaStream_t st) {
   dim3 grid(flat_ctas((long)b * b, batch), batch);
-  k_broadcast_diag<T><<<grid, 256, 0, st>>>(out, sOut, src, b, E, eta);
+  launch_after(k_broadcast_diag<T>, grid, 256, 0, st, out, sOut, src, b, E, eta);
   count_launch();
   return cudaGetLastError();
 }
@@ -728,6 +736,7 @@ template <typename T>
 __global__ void k_assemble_offdiag(cx<T>* U, cx<T>* V, const cx<double>* Hup, const cx<double>* Sup,
                                    const double* E, double eta, int b, const cx<double>* SRu,
                                    const cx<double>* SRl, long sSR) {
+  after_previous();
   const int e = blockIdx.z;
   __shared__ cx<double> tile[32][33];
   const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
@@ -773,7 +782,7 @@ cudaError_t assemble_offdiag(cx<T>* U, cx<T>* V, const cx<double>* Hup, const cx
                              const double* E, double eta, int b, int batch, cudaStream_t st,
                              const cx<double>* SRu, const cx<double>* SRl, long sSR) {
   dim3 grid((b + 31) / 32, (b + 31) / 32, batch);
-  k_assemble_offdiag<T><<<grid, 256, 0, st>>>(U, V, Hup, Sup, E, eta, b, SRu, SRl, sSR);
+  launch_after(k_assemble_offdiag<T>, grid, 256, 0, st, U, V, Hup, Sup, E, eta, b, SRu, SRl, sSR);
   count_launch();
   return cudaGetLastError();
 }
@@ -793,6 +802,7 @@ __device__ __forceinline__ float mag32(double x) {
 template <typename T>
 __global__ void __launch_bounds__(512) k_residual_mask(const cx<T>* R, long sR, long nn, float tol2,
                                                        const int* active, int* next, int* status) {
+  after_previous();
   const int e = blockIdx.x;
   if (active && !active[e]) {
     if (threadIdx.x == 0) next[e] = 0;
@@ -820,7 +830,7 @@ __global__ void __launch_bounds__(512) k_residual_mask(const cx<T>* R, long sR, 
 template <typename T>
 cudaError_t residual_mask(const cx<T>* R, long sR, int n, int batch, double tol, const int* active, int* next,
                           int* status, cudaStream_t st) {
-  k_residual_mask<T><<<batch, 512, 0, st>>>(R, sR, (long)n * n, (float)(tol * tol), active, next, status);
+  launch_after(k_residual_mask<T>, batch, 512, 0, st, R, sR, (long)n * n, (float)(tol * tol), active, next, status);
   count_launch();
   return cudaGetLastError();
 }
@@ -935,6 +945,7 @@ cudaError_t set_identity(cx<double>* I, cx<df>* Idf, int b, cudaStream_t st) {
 
 template <typename T>
 __global__ void k_add_identity(cx<T>* X, long sX, int n, const int* active) {
+  after_previous();
   const int e = blockIdx.y;
   if (active && !active[e]) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -943,7 +954,7 @@ __global__ void k_add_identity(cx<T>* X, long sX, int n, const int* active) {
 template <typename T>
 cudaError_t add_identity(cx<T>* X, long sX, int n, int batch, const int* active, cudaStream_t st) {
   dim3 grid((n + 127) / 128, batch);
-  k_add_identity<T><<<grid, 128, 0, st>>>(X, sX, n, active);
+  launch_after(k_add_identity<T>, grid, 128, 0, st, X, sX, n, active);
   count_launch();
   return cudaGetLastError();
 }
@@ -954,6 +965,7 @@ template cudaError_t add_identity<float>(cx<float>*, long, int, int, const int*,
 template <typename Tin, typename Tout>
 __global__ void k_convert(const cx<Tin>* in, long ldi, long si, cx<Tout>* out, long ldo, long so, int rows,
                           int cols) {
+  after_previous();
   const int e = blockIdx.z;
   const int r = blockIdx.y;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < cols; c += gridDim.x * blockDim.x)
@@ -964,7 +976,7 @@ cudaError_t convert_strided(const cx<Tin>* in, long ldi, long si, cx<Tout>* out,
                             int cols, int batch, cudaStream_t st) {
   if (rows <= 0 || cols <= 0 || batch <= 0) return cudaSuccess;
   dim3 grid((cols + 127) / 128 < 8 ? (cols + 127) / 128 : 8, rows, batch);
-  k_convert<Tin, Tout><<<grid, 128, 0, st>>>(in, ldi, si, out, ldo, so, rows, cols);
+  launch_after(k_convert<Tin, Tout>, grid, 128, 0, st, in, ldi, si, out, ldo, so, rows, cols);
   count_launch();
   return cudaGetLastError();
 }
@@ -990,6 +1002,7 @@ __device__ __forceinline__ double block_sum(double v) {
 
 template <typename T>
 __global__ void k_obs_density(double* den, long ldden, const cx<T>* GL, long sG, int b) {
+  after_previous();
   const int e = blockIdx.x;
   const cx<T>* G = GL + (long)e * sG;
   double s = 0.0;
@@ -999,7 +1012,7 @@ __global__ void k_obs_density(double* den, long ldden, const cx<T>* GL, long sG,
 }
 template <typename T>
 cudaError_t obs_density(double* den, long ldden, const cx<T>* GL, long sG, int b, int batch, cudaStream_t st) {
-  k_obs_density<T><<<batch, 128, 0, st>>>(den, ldden, GL, sG, b);
+  launch_after(k_obs_density<T>, batch, 128, 0, st, den, ldden, GL, sG, b);
   count_launch();
   return cudaGetLastError();
 }
@@ -1012,6 +1025,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_obs_trace2(double* out, long ld, const cx<double>* X, long sX,
                                                     const cx<T>* Y, long sY, const cx<double>* Z, long sZ,
                                                     const cx<T>* W, long sW, int b, int part, double scale) {
+  after_previous();
   const int e = blockIdx.x;
   const long bb = (long)b * b;
   double s = 0.0;
@@ -1033,7 +1047,7 @@ template <typename T>
 cudaError_t obs_trace2(double* out, long ld, const cx<double>* X, long sX, const cx<T>* Y, long sY,
                        const cx<double>* Z, long sZ, const cx<T>* Wm, long sW, int b, int batch,
                        cudaStream_t st, int part, double scale) {
-  k_obs_trace2<T><<<batch, 256, 0, st>>>(out, ld, X, sX, Y, sY, Z, sZ, Wm, sW, b, part, scale);
+  launch_after(k_obs_trace2<T>, batch, 256, 0, st, out, ld, X, sX, Y, sY, Z, sZ, Wm, sW, b, part, scale);
   count_launch();
   return cudaGetLastError();
 }
@@ -1258,6 +1272,7 @@ __global__ void __launch_bounds__(512) k_decim_update(cx<double>* es, cx<double>
                                                       const cx<double>* al, const cx<double>* be, cx<double>* g,
                                                       const double* E, double eta, int ne, int b, double tol_rel,
                                                       const double* scale, int* active) {
+  after_previous();
   const int e = blockIdx.x, lead = e / ne;
   if (!active[e]) return;
   const double tol = tol_rel * (scale[lead] > 0.0 ? scale[lead] : 1.0);
@@ -1301,7 +1316,7 @@ __global__ void __launch_bounds__(512) k_decim_update(cx<double>* es, cx<double>
 cudaError_t decim_update(cx<double>* es, cx<double>* ep, const cx<double>* x, const cx<double>* y, const cx<double>* al,
                          const cx<double>* be, cx<double>* g, const double* E, double eta, int ne, int leads, int b, double tol_rel,
                          const double* scale, int* active, cudaStream_t st) {
-  k_decim_update<<<ne * leads, 512, 0, st>>>(es, ep, x, y, al, be, g, E, eta, ne, b, tol_rel, scale, active);
+  launch_after(k_decim_update, ne * leads, 512, 0, st, es, ep, x, y, al, be, g, E, eta, ne, b, tol_rel, scale, active);
   count_launch();
   return cudaGetLastError();
 }

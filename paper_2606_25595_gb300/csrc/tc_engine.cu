@@ -214,6 +214,8 @@ __global__ void __launch_bounds__(352, 1) k_tc_gemm(const __grid_constant__ TcGr
     mbar_init(drainbar, 2);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // (the previous launch's CTAs may still hold TMEM, or wait for it: nothing is allocated before they end)
+  after_previous();
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -500,6 +502,7 @@ struct DigitJobs {
 
 template <int S, int RPC, typename TI>
 __global__ void __launch_bounds__(32 * RPC) k_digitize_rows(const __grid_constant__ DigitJobs jobs) {
+  after_previous();
   const DigitJob& job = jobs.j[blockIdx.z];
   const int e = blockIdx.y;
   const int R = job.R, K = job.K, R_pad = job.R_pad, K_pad = job.K_pad, side = job.side, P = job.P;
@@ -700,8 +703,8 @@ cudaError_t digitize_as(const DigitJob* const* jobs, int n, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   const size_t smem = rpc * row_bytes;
   const dim3 g((R_pad + rpc - 1) / rpc, batch, n);
-  if (rpc == 2) k_digitize_rows<S, 2, TI><<<g, 64, smem, st>>>(all);
-  else k_digitize_rows<S, 1, TI><<<g, 32, smem, st>>>(all);
+  if (rpc == 2) launch_after(k_digitize_rows<S, 2, TI>, g, 64, smem, st, all);
+  else launch_after(k_digitize_rows<S, 1, TI>, g, 32, smem, st, all);
   count_launch();
   return cudaGetLastError();
 }
@@ -842,8 +845,8 @@ cudaError_t launch(const TcPrepared* const* pp, int n, cudaStream_t st, cudaEven
     if (pp[q]->ctas > 0 && pp[q]->ctas < ctas) ctas = pp[q]->ctas;
   const int grid = (int)(total < ctas ? total : ctas);
   if (ev) cudaEventRecord(ev[0], st);
-  if (n == 1) k_tc_gemm<S, NST, IO, false><<<grid, 352, smem, st>>>(G);
-  else k_tc_gemm<S, NST, IO, true><<<grid, 352, smem, st>>>(G);
+  if (n == 1) launch_after<1>(k_tc_gemm<S, NST, IO, false>, grid, 352, smem, st, G);
+  else launch_after<1>(k_tc_gemm<S, NST, IO, true>, grid, 352, smem, st, G);
   count_launch();
   if (ev) cudaEventRecord(ev[1], st);
   return cudaGetLastError();

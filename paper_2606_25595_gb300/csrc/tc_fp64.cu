@@ -152,6 +152,8 @@ __global__ void __launch_bounds__(352, 1) k_tc_gemm_fp64(const __grid_constant__
     mbar_init(drainbar, 2);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // (the previous launch's CTAs may still hold TMEM, or wait for it: nothing is allocated before they end)
+  after_previous();
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tslot)), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -347,6 +349,7 @@ struct Operands {
 };
 template <int RPC>
 __global__ void __launch_bounds__(32 * RPC) k_digitize_fp64(const __grid_constant__ Operands ops) {
+  after_previous();
   const int side = blockIdx.z & 1, e = blockIdx.y;
   const Operand& op = ops.o[blockIdx.z];
   const int K = op.K, K_pad = op.K_pad, P = op.P;
@@ -537,7 +540,7 @@ cudaError_t products9(const GemmArgs<double>* g, int n, unsigned char* scratch, 
   L.tile0[n] = (int)tiles;
   constexpr int RPC = 4;  // transposed strips read four values of 16 bytes in a row: whole 32-byte sectors
   const size_t smem = (size_t)RPC * (skew9(K_pad) + 1) * sizeof(cx<double>);  // at most 37 KB
-  k_digitize_fp64<RPC><<<dim3(R / RPC, batch, 2 * n), 32 * RPC, smem, st>>>(o);
+  launch_after(k_digitize_fp64<RPC>, dim3(R / RPC, batch, 2 * n), 32 * RPC, smem, st, o);
   count_launch();
   if ((e = cudaGetLastError())) return e;
   int sms = 0;
@@ -545,8 +548,8 @@ cudaError_t products9(const GemmArgs<double>* g, int n, unsigned char* scratch, 
   if ((e = n == 1 ? allow_smem(k_tc_gemm_fp64<false>, SMEM9, done1) : allow_smem(k_tc_gemm_fp64<true>, SMEM9, done2)) || (e = sm_count(sms))) return e;
   const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);
   if (ev) cudaEventRecord(ev[0], st);
-  if (n == 1) k_tc_gemm_fp64<false><<<grid, 352, SMEM9, st>>>(L);
-  else k_tc_gemm_fp64<true><<<grid, 352, SMEM9, st>>>(L);
+  if (n == 1) launch_after<1>(k_tc_gemm_fp64<false>, grid, 352, SMEM9, st, L);
+  else launch_after<1>(k_tc_gemm_fp64<true>, grid, 352, SMEM9, st, L);
   count_launch();
   if (ev) cudaEventRecord(ev[1], st);
   return cudaGetLastError();
