@@ -167,7 +167,9 @@ Layout make_layout(const qtx_rgf_desc& d, bool inverse_only = false) {
   L.perm = a.take(L.refine64 && b <= kPivotedMax ? (size_t)Ec * b * sizeof(int) : 0);
   L.n_dec = 10;
   const long nl = contacts_together(d, inverse_only) ? 2 : 1;  // contacts iterated in the same launches
-  L.dec = a.take(d.leads ? (size_t)L.n_dec * nl * Ec * bb * sizeof(cx<double>) : 0);
+  // (smaller lead blocks are iterated in shared memory; the transmission's four blocks remain)
+  const long dec_blocks = !d.leads ? 0 : (b > kDecimSmallMax ? L.n_dec * nl : 4);
+  L.dec = a.take((size_t)dec_blocks * Ec * bb * sizeof(cx<double>));
   L.dec_flags = a.take(d.leads ? 2 * nl * Ec * sizeof(int) : 0);
   L.lead = a.take(d.leads && !inverse_only ? 8 * Ec * bb * sizeof(cx<double>) : 0);
   // per-energy observables: current, density, contact(2), transmission, scratch(2)
