@@ -225,124 +225,173 @@ template cudaError_t gemm_simt<float>(const GemmArgs<float>&, cudaStream_t);
 //     A^-1[k][p_j] = B[p_k][j],
 // so each thread scatters its values to (step of its row, pivot row of its column's step).
 //
-// Bound by the latency of a step's chain, not by its n^2 FMAs.  Layout: 16 x 16 threads, thread (ty, tx)
-// owns rows ty + 16 i and columns tx + 16 j (NMAX = 64: 4 x 4 values, 32: 2 x 2).  Column k of the block
-// lies in shared memory (double-buffered, written by its owners in the last step's update): every warp
-// searches it for the pivot with one integer reduction, the half-warp that owns the pivot row scales it
-// by the reciprocal and publishes it, and after a barrier every thread updates its values from 4 factors
-// and 4 row values.  About 500 cycles a step; with a warp per row group publishing its own candidate,
-// eight reciprocals and 16 shuffles a step, it took 2,000 (62 us for 64 x 64, batch 32).
-// c ? x : y by selects (register arrays indexed by a step's row or column would go to local memory)
+// Bound by the latency of a step's chain, not by its n^2 FMAs, so the chain runs one column ahead in a warp of its
+// own (the last): while the others make step k, it takes step k for column k + 1 alone, from the column as it was
+// after step k - 1, finds the pivot (one integer reduction) and its reciprocal (1/d and r/d as one division in two
+// lanes).  The others hold the block in registers, thread (ty, tx) rows ty + TY i and columns tx + 16 j (NMAX =
+// 64: 32 x 16 threads of 2 x 4 values, 32: 16 x 16 of 2 x 2): the half-warp that owns the pivot row scales and
+// publishes it, every thread updates its values from 2 factors and 4 row values, and column k + 2 goes to shared
+// memory.  64 x 64, batch 24: 51 us with the chain in every warp before the update, 43 with it ahead of 8 warps of
+// 4 x 4 values, 37 of 16 warps (dependent instructions and branches of few warps: a scheduler issues every third
+// cycle).
+// c ? x : y by selects
 __device__ __forceinline__ cx<float> pick(bool c, cx<float> x, cx<float> y) {
   return mk<float>(c ? x.re : y.re, c ? x.im : y.im);
 }
 
+// f(I) with the compile-time index I = i < R (i uniform over the warp): register arrays are indexed by constants
+template <int R, typename F>
+__device__ __forceinline__ void at_index(int i, F&& f) {
+  if (i == 0) f(std::integral_constant<int, 0>());
+  else if (i == 1) f(std::integral_constant<int, 1>());
+  if constexpr (R == 4) {
+    if (i == 2) f(std::integral_constant<int, 2>());
+    else if (i == 3) f(std::integral_constant<int, 3>());
+  }
+}
+
+__host__ __device__ constexpr int leaf_threads(int nmax) { return 8 * nmax + 32; }
+
 template <int NMAX>
-__global__ void __launch_bounds__(256) k_leaf_inverse(cx<float>* Ag, long lda, long sA, int n, const int* active, int* status) {
+__global__ void __launch_bounds__(leaf_threads(NMAX)) k_leaf_inverse(cx<float>* Ag, long lda, long sA, int n, const int* active, int* status) {
   after_previous();
-  constexpr int R = NMAX / 16;
+  constexpr int TY = NMAX / 2, RI = 2, RJ = NMAX / 16, NT = 16 * TY;  // update threads
   const int e = blockIdx.x;
   if (active && !active[e]) return;
-  __shared__ cx<float> s_col[2][NMAX], s_row[NMAX];
-  __shared__ int s_step[NMAX], s_piv[NMAX];
+  // column k before step k (s_f[k & 1]) and column k + 1 before it (s_raw[(k + 1) & 1]); step k's pivot, reciprocal
+  __shared__ cx<float> s_f[2][NMAX], s_raw[2][NMAX], s_row[NMAX], s_rec[2];
+  __shared__ int s_p[2], s_step[NMAX], s_piv[NMAX];
   cx<float>* A = Ag + (long)e * sA;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16, lane = threadIdx.x % 32;
-  cx<float> a[R][R];
+  const int t = threadIdx.x, tx = t % 16, ty = t / 16, lane = t % 32;
+  const bool ahead = t >= NT;
+  // the pivot row's value, by the order of the roundings of the padded size
+  auto scaled = [](cx<float> x, cx<float> r) {
+    const float im = NMAX > 32 ? __fmaf_rn(x.re, r.im, __fmul_rn(x.im, r.re)) : __fmaf_rn(x.im, r.re, __fmul_rn(x.re, r.im));
+    return mk<float>(__fmaf_rn(x.re, r.re, -__fmul_rn(x.im, r.im)), im);
+  };
+  auto update = [](cx<float> v, cx<float> f, cx<float> w) {
+    v.re = __fmaf_rn(-f.re, w.re, v.re);
+    v.re = __fmaf_rn(f.im, w.im, v.re);
+    v.im = __fmaf_rn(-f.re, w.im, v.im);
+    v.im = __fmaf_rn(-f.im, w.re, v.im);
+    return v;
+  };
+  unsigned used[2] = {0, 0};
+  // the last warp: column k after step k - 1 (pivot row p; k = 0: as it is), its pivot and reciprocal
+  auto lead = [&](int k, int p) {
+    const cx<float>* raw = s_raw[k & 1];
+    const cx<float>* f = s_f[(k & 1) ^ 1];
+    cx<float> v[2], w = mk<float>(0.f, 0.f);
+    if (k) w = scaled(raw[p], s_rec[(k & 1) ^ 1]);
+    unsigned key[2];
 #pragma unroll
-  for (int i = 0; i < R; ++i)
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-      const int r = ty + 16 * i, c = tx + 16 * j;
-      a[i][j] = (r < n && c < n) ? A[(long)r * lda + c] : mk<float>(0.f, 0.f);
+    for (int h = 0; h < (NMAX > 32 ? 2 : 1); ++h) {
+      const int i = lane + 32 * h;
+      v[h] = raw[i];
+      if (k) v[h] = pick(i == p, w, update(v[h], f[i], w));
+      s_f[k & 1][i] = v[h];
+      // |Re| + |Im| >= 0 orders like its bits; NaN never wins
+      const unsigned u = __float_as_uint(cabs1(v[h]));
+      key[h] = i >= n || ((used[h] >> lane) & 1u) || u > 0x7f800000u ? 0u : u;
     }
-  if (tx == 0)
+    if (NMAX == 32) {
+      v[1] = v[0];
+      key[1] = 0;
+    }
+    const unsigned best = __reduce_max_sync(0xffffffffu, key[0] > key[1] ? key[0] : key[1]);
+    const unsigned b0 = __ballot_sync(0xffffffffu, key[0] == best), b1 = __ballot_sync(0xffffffffu, key[1] == best);
+    const int q = best == 0 || best >= 0x7f800000u ? -1 : (b0 ? __ffs((int)b0) - 1 : 31 + __ffs((int)b1));
+    if (q >= 0) {
+      const cx<float> x = pick(q < 32, v[0], v[1]);
+      const float re = __shfl_sync(0xffffffffu, x.re, q & 31), im = __shfl_sync(0xffffffffu, x.im, q & 31);
+      // 1 / x as crecip does it
+      const bool tall = fabsf(re) >= fabsf(im);
+      const float c = tall ? im : re, d = tall ? re : im, r = c / d, m = __fmaf_rn(c, r, d);
+      const float z = (tall ? (lane ? -r : 1.f) : (lane ? -1.f : r)) / m;
+      if (lane == 0) s_rec[k & 1].re = z;
+      if (lane == 1) s_rec[k & 1].im = z;
+    }
+    if (lane == 0) s_p[k & 1] = q;
+    __syncwarp();
+  };
+  cx<float> a[RI][RJ];
+  if (!ahead) {
 #pragma unroll
-    for (int i = 0; i < R; ++i) s_col[0][ty + 16 * i] = a[i][0];
+    for (int i = 0; i < RI; ++i)
+#pragma unroll
+      for (int j = 0; j < RJ; ++j) {
+        const int r = ty + TY * i, c = tx + 16 * j;
+        a[i][j] = (r < n && c < n) ? A[(long)r * lda + c] : mk<float>(0.f, 0.f);
+      }
+    if (tx < 2)
+#pragma unroll
+      for (int i = 0; i < RI; ++i) s_raw[tx][ty + TY * i] = a[i][0];
+  }
   __syncthreads();
-  unsigned used0 = 0, used1 = 0;
-  bool bad = false;
+  if (ahead) lead(0, 0);
+  __syncthreads();
   for (int k = 0; k < n; ++k) {
-    const cx<float>* col = s_col[k & 1];
-    // |Re| + |Im| >= 0 orders like its bits; NaN never wins
-    auto key = [&](int r, unsigned used) -> unsigned {
-      if (r >= n || ((used >> lane) & 1u)) return 0u;
-      const unsigned v = __float_as_uint(cabs1(col[r]));
-      return v <= 0x7f800000u ? v : 0u;
-    };
-    const unsigned k0 = key(lane, used0), k1 = NMAX > 32 ? key(lane + 32, used1) : 0u;
-    const unsigned best = __reduce_max_sync(0xffffffffu, k0 > k1 ? k0 : k1);
-    if (best == 0 || best >= 0x7f800000u) {
-      bad = true;
-      break;
+    const int p = s_p[k & 1];
+    if (p < 0) {  // in every thread alike
+      if (t == 0 && status) atomicCAS(status + e, 0, (int)QTX_ERR_SINGULAR);
+      return;
     }
-    const unsigned b0 = __ballot_sync(0xffffffffu, k0 == best), b1 = __ballot_sync(0xffffffffu, k1 == best);
-    const int p = b0 ? __ffs((int)b0) - 1 : 31 + __ffs((int)b1);
-    if (p < 32) used0 |= 1u << p;
-    else used1 |= 1u << (p - 32);
-    if (ty == p % 16) {  // the pivot row's owners scale it
-      const cx<float> r = crecip(col[p]);
-      const int pi = p / 16;
+    if (ahead) {
+      if (p < 32) used[0] |= 1u << p;
+      else used[1] |= 1u << (p - 32);
+      if (k + 1 < n) lead(k + 1, p);
+    } else {
+      const cx<float>* col = s_f[k & 1];
+      if (ty == p % TY) {  // the pivot row's owners scale it
+        const cx<float> r = s_rec[k & 1];
+        at_index<RI>(p / TY, [&](auto I) {
 #pragma unroll
-      for (int j = 0; j < R; ++j) {
-        const int c = tx + 16 * j;
-        cx<float> x = a[0][j];
-#pragma unroll
-        for (int i = 1; i < R; ++i) x = pick(pi == i, a[i][j], x);
-        // the order of the roundings, by padded size
-        const float im = NMAX > 32 ? __fmaf_rn(x.re, r.im, __fmul_rn(x.im, r.re)) : __fmaf_rn(x.im, r.re, __fmul_rn(x.re, r.im));
-        x = pick(c == k, r, mk<float>(__fmaf_rn(x.re, r.re, -__fmul_rn(x.im, r.im)), im));
-#pragma unroll
-        for (int i = 0; i < R; ++i) a[i][j] = pick(pi == i, x, a[i][j]);
-        s_row[c] = x;
+          for (int j = 0; j < RJ; ++j) {
+            const int c = tx + 16 * j;
+            a[I.value][j] = s_row[c] = pick(c == k, r, scaled(a[I.value][j], r));
+          }
+        });
+        if (tx == 0) {
+          s_step[p] = k;
+          s_piv[k] = p;
+        }
       }
-      if (tx == 0) {
-        s_step[p] = k;
-        s_piv[k] = p;
-      }
-    }
-    __syncthreads();
-    cx<float> w[R];
+      asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
+      cx<float> w[RJ];
 #pragma unroll
-    for (int j = 0; j < R; ++j) w[j] = s_row[tx + 16 * j];
+      for (int j = 0; j < RJ; ++j) w[j] = s_row[tx + 16 * j];
+      const bool mine = tx == k % 16;  // one of this thread's columns is the pivot column: -(f r)
+      at_index<RJ>(k / 16, [&](auto J) {
 #pragma unroll
-    for (int i = 0; i < R; ++i) {
-      const int r = ty + 16 * i;
-      const cx<float> f = col[r];
-      if (r == p) continue;
+        for (int i = 0; i < RI; ++i) {
+          const int r = ty + TY * i;
+          const cx<float> f = col[r];
 #pragma unroll
-      for (int j = 0; j < R; ++j) {
-        cx<float> v = a[i][j];
-        v.re = __fmaf_rn(-f.re, w[j].re, v.re);
-        v.re = __fmaf_rn(f.im, w[j].im, v.re);
-        v.im = __fmaf_rn(-f.re, w[j].im, v.im);
-        v.im = __fmaf_rn(-f.im, w[j].re, v.im);
-        if (tx + 16 * j == k)  // the pivot column: -(f r)
-          v = mk<float>(-__fmaf_rn(f.re, w[j].re, -__fmul_rn(f.im, w[j].im)), -__fmaf_rn(f.re, w[j].im, __fmul_rn(f.im, w[j].re)));
-        a[i][j] = v;
-      }
-    }
-    if (tx == (k + 1) % 16) {
-      cx<float>* next = s_col[(k + 1) & 1];
-      const int jn = (k + 1) / 16;
+          for (int j = 0; j < RJ; ++j) {
+            cx<float> v = update(a[i][j], f, w[j]);
+            if (j == J.value)
+              v = pick(mine, mk<float>(-__fmaf_rn(f.re, w[j].re, -__fmul_rn(f.im, w[j].im)),
+                                       -__fmaf_rn(f.re, w[j].im, __fmul_rn(f.im, w[j].re))), v);
+            if (r != p) a[i][j] = v;
+          }
+        }
+      });
+      if (tx == (k + 2) % 16 && k + 2 < NMAX) {
+        cx<float>* next = s_raw[k & 1];
+        at_index<RJ>((k + 2) / 16, [&](auto J) {
 #pragma unroll
-      for (int i = 0; i < R; ++i) {
-        cx<float> x = a[i][0];
-#pragma unroll
-        for (int j = 1; j < R; ++j) x = pick(jn == j, a[i][j], x);
-        next[ty + 16 * i] = x;
+          for (int i = 0; i < RI; ++i) next[ty + TY * i] = a[i][J.value];
+        });
       }
     }
     __syncthreads();
   }
-  if (bad) {
-    if (threadIdx.x == 0 && status) atomicCAS(status + e, 0, (int)QTX_ERR_SINGULAR);
-    return;
-  }
+  if (ahead) return;
 #pragma unroll
-  for (int i = 0; i < R; ++i)
+  for (int i = 0; i < RI; ++i)
 #pragma unroll
-    for (int j = 0; j < R; ++j) {
-      const int r = ty + 16 * i, c = tx + 16 * j;
+    for (int j = 0; j < RJ; ++j) {
+      const int r = ty + TY * i, c = tx + 16 * j;
       if (r < n && c < n) A[(long)s_step[r] * lda + s_piv[c]] = a[i][j];
     }
 }
@@ -352,9 +401,9 @@ cudaError_t leaf_inverse<float>(cx<float>* A, long lda, long sA, int n, int batc
                                 cudaStream_t st) {
   if (n <= 0 || n > kLeafMax) return cudaErrorInvalidValue;
   if (n <= 32)
-    launch_after(k_leaf_inverse<32>, batch, 256, 0, st, A, lda, sA, n, active, status);
+    launch_after(k_leaf_inverse<32>, batch, leaf_threads(32), 0, st, A, lda, sA, n, active, status);
   else
-    launch_after(k_leaf_inverse<64>, batch, 256, 0, st, A, lda, sA, n, active, status);
+    launch_after(k_leaf_inverse<64>, batch, leaf_threads(64), 0, st, A, lda, sA, n, active, status);
   count_launch();
   return cudaGetLastError();
 }
