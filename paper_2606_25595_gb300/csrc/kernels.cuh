@@ -2,6 +2,7 @@
 // host orchestration (rgf.cu).  All launchers are asynchronous on `st` and return the launch status.
 #pragma once
 #include <atomic>
+#include <utility>
 
 #include "common.cuh"
 
@@ -26,19 +27,33 @@ struct EarlyLaunches {
   explicit EarlyLaunches(int level) { t_early = level; }
   ~EarlyLaunches() { t_early = old; }
 };
+// In clusters of `cluster` CTAs (along x).
 template <int LEVEL = 2, typename... P, typename... A>
-inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+inline cudaError_t launch_after_clusters(void (*kernel)(P...), int cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                         A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute at[2];
+  if (cluster > 1) {
+    at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    at[cfg.numAttrs].val.clusterDim.x = cluster;
+    at[cfg.numAttrs].val.clusterDim.y = at[cfg.numAttrs].val.clusterDim.z = 1;
+    ++cfg.numAttrs;
+  }
+  if (t_early >= LEVEL) {
+    at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+    ++cfg.numAttrs;
+  }
   cfg.attrs = at;
-  cfg.numAttrs = t_early >= LEVEL ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+template <int LEVEL = 2, typename... P, typename... A>
+inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  return launch_after_clusters<LEVEL>(kernel, 1, grid, block, smem, st, std::forward<A>(args)...);
 }
 #ifdef __CUDACC__
 // Lets the next launch begin once every CTA of this one is here, and waits until the previous launch has ended
