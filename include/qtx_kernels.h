@@ -3,8 +3,8 @@
  * exposed on their own, on complex128 device arrays, for testing and for callers that assemble their
  * own solvers.  Same conventions as qtx_rgf.h: device pointers owned by the caller, interleaved
  * (re, im) doubles, row-major blocks, asynchronous on `stream` (a cudaStream_t), status codes from
- * qtx_status.  Each call allocates its temporaries with stream-ordered cudaMallocAsync and frees them
- * before returning.  Nothing falls back to the CPU.
+ * qtx_status.  Each call takes its temporaries stream-ordered from a memory pool of the library's own (one
+ * per device, which keeps at most 512 MiB between calls) and returns them before it returns.  Nothing falls back to the CPU.
  */
 #ifndef QTX_KERNELS_H
 #define QTX_KERNELS_H

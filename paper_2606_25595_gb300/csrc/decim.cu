@@ -20,8 +20,8 @@
 // 16 x 16 blocks are 115,000 DFMA a sweep, 57,000 cycles on one SM.  Few energies leave SMs idle, so a cluster
 // splits the products' rows (each CTA writes its rows into every CTA's copy through distributed shared
 // memory; two cluster barriers a sweep) while every CTA eliminates for itself.  In the elimination one
-// warp finds the pivot and forms its reciprocal once -- 1/d and r/d as one division in two lanes -- and
-// scales the pivot row; the rows then update from one copy of the block into another.
+// warp finds the pivot and forms its reciprocal one step ahead, and the rows update from one copy of the block
+// into another.  Contacts of b = 16 with 4 energies: 2 x 2.5 ms with a CTA each, one after the other; 0.88 ms so.
 #include <cooperative_groups.h>
 
 #include "gj64.cuh"
