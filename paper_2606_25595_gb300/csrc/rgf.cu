@@ -150,7 +150,8 @@ Layout make_layout(const qtx_rgf_desc& d, bool inverse_only = false) {
   L.xk = a.take(!d.storage_bits && nb > 1 ? (size_t)(d.second_rhs ? 2 : 1) * (nb - 1) * Ec * bb * es : 0);
   L.tmp = a.take((size_t)L.n_tmp * Ec * bb * es);
   L.sig_stage = a.take(d.sigma_stream ? 2 * Ec * bb * sizeof(cx<double>) : 0);  // Sigma^R_ii, Sigma^<_ii
-  L.inv_tmp = a.take(Ec * bb * es + 4096);
+  // (the contacts' elimination recurses in complex128 whatever the sweep's type)
+  L.inv_tmp = a.take(Ec * bb * (d.leads && b > kLeafMax ? sizeof(cx<double>) : es) + 4096);
   const size_t ou = uv_per_energy(d) ? (size_t)(nb > 1 ? nb - 1 : 0) * Ec * bb * es : (size_t)(nb > 1 ? nb - 1 : 0) * bb * es;
   L.U = a.take(ou);
   L.V = a.take(ou);

@@ -123,3 +123,14 @@ def test_second_rhs_descriptor(libpath):
     two = q.footprint(q.make_desc(nb, b, "fp64", ec, outputs=["GR_diag", "GL_diag", "GG_diag"],
                                   second_rhs=True, **kw))
     assert two - one == (nb + 1) * ec * b * b * 16 + (nb - 1) * ec * b * b * 16
+
+
+@pytest.mark.parametrize("b,nb,ec", [(96, 6, 16), (128, 2, 8), (100, 4, 12)])
+def test_fp32_contacts_have_complex128_inverse_scratch(libpath, b, nb, ec):
+    """Contacts above 64 orbitals are eliminated by a recursion in complex128 in every precision: an FP32 plan's
+    inverse scratch grows from 8 to 16 b^2 bytes per energy, beside the decimation's ten blocks, the contacts'
+    eight, and two convergence flags."""
+    import paper_2606_25595_gb300 as q
+    fp = lambda leads: q.footprint(q.make_desc(nb, b, "fp32", ec, leads=leads, outputs=["GR_diag"]))  # noqa: E731
+    more = ec * b * b * (18 * 16 + 8) + 2 * ec * 4
+    assert more <= fp(True) - fp(False) <= more + 8 * 256
