@@ -235,6 +235,8 @@ qtx_status qtx_fpx_compress(int bits, const double* x, long n, double cutoff, vo
   if (n == 0) return QTX_OK;
   if (!x || !out || (reinterpret_cast<uintptr_t>(x) & 7) || (reinterpret_cast<uintptr_t>(out) & 7))
     return QTX_ERR_INVALID_ARG;
+  // (the kernel compares bit patterns: a cutoff of -0.0 is none, like 0.0)
+  if (cutoff == 0.0) cutoff = 0.0;
   const cudaError_t e = launch_compress<double>(bits, x, n, cutoff, out, reinterpret_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? QTX_OK : QTX_ERR_CUDA;
 }

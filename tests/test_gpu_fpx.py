@@ -84,6 +84,18 @@ def test_cutoff_complex_and_small_sizes(q):
         assert c.cpu().numpy().tobytes()[: 5 * n] == F.compress(x, 40)
 
 
+# no cutoff by either zero; the smallest subnormal and normal numbers; above and at the edge values; infinity
+@pytest.mark.parametrize("cutoff", [-0.0, 0.0, 5e-324, 2.0 ** -1022, 2.0 ** -126, 1.5, math.inf])
+def test_cutoff_compares_like_numbers(q, cutoff):
+    import torch
+    x = np.concatenate([_values(3, 400), [2.0 ** -1022, -2.0 ** -1022, math.nan]])
+    x[x == 0.0] = 0.0  # (the oracle keeps the sign of an exact zero below a cutoff)
+    for bits in (56, 24):
+        got = q.fpx_compress(torch.tensor(x, device="cuda"), bits, cutoff=cutoff).cpu().numpy().tobytes()
+        ref = F.compress(x, bits, cutoff=cutoff)
+        assert got[: len(ref)] == ref
+
+
 def test_invalid_arguments(q):
     import ctypes
     import torch
