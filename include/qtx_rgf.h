@@ -48,8 +48,9 @@ typedef enum {
 } qtx_status;
 
 /* Arithmetic of the block products and inverses (Sec. IV, V-A of the paper: the solve of Eq. 2 is
- * ZGEMM-dominated; lower precision is traded against accuracy).  Observables are always reduced
- * in FP64 and the lead decimation always runs in FP64. */
+ * ZGEMM-dominated; lower precision is traded against accuracy).  Observables are reduced in FP64
+ * (the emulated modes' bond current without an overlap matrix: in df32 pairs, ~48 bits) and the lead
+ * decimation always runs in FP64. */
 typedef enum {
   QTX_FP64 = 0,   /* complex128 throughout -- the plain FP64 path.  Products with all dimensions above 32
                      on the tcgen05 tensor cores from 9 bf16 digit planes per operand (45 digit products,

@@ -163,13 +163,14 @@ cudaError_t assemble_offdiag(cx<T>* U, cx<T>* V, const cx<double>* Hup, const cx
 // The backward sweep's elementwise passes (lesser.cu).  lesser_offdiag: GLu = X2^H - PGL (GLu may be null),
 // X2 <- X2 - PGL^H / 2, and, with Hup given, the partial sums of Re Tr[(Hup - E Sup) GLu^H] into `scratch`.
 // lesser_diag: gl <- gl + X - X^H, out64 (may be null; batch stride so) a complex128 copy, den[e * ldden] = Im Tr gl,
-// and cur[e * ldcur] = -2 times lesser_offdiag's sums (cur may be null).  scratch: lesser_scratch_bytes.
+// and cur[e * ldcur] = -2 times lesser_offdiag's sums (cur may be null; overlap: Sup was given).  scratch:
+// lesser_scratch_bytes.
 size_t lesser_scratch_bytes(int b, int batch);
 template <typename T>
 cudaError_t lesser_offdiag(const cx<T>* PGL, cx<T>* X2, cx<T>* GLu, const cx<double>* Hup, const cx<double>* Sup,
                            const double* E, int b, int batch, void* scratch, cudaStream_t st);
 template <typename T>
-cudaError_t lesser_diag(cx<T>* gl, const cx<T>* X, cx<double>* out64, long so, double* cur, long ldcur, double* den,
+cudaError_t lesser_diag(cx<T>* gl, const cx<T>* X, cx<double>* out64, long so, double* cur, long ldcur, bool overlap, double* den,
                         long ldden, int b, int batch, void* scratch, cudaStream_t st);
 // den[e * ldden] = Im Tr GL[e]
 template <typename T>

@@ -46,14 +46,14 @@ __device__ __forceinline__ void pair_of(int q, int nt, int& I, int& J) {
   J = I + q;
 }
 
-// Trace partials: df32 sums for df32 blocks (error-free FP32 steps: the FP64 pipe runs at 1/64 of the FP32 rate;
-// with an overlap matrix, and for the other types, FP64)
-template <typename T>
+// Trace partials: df32 sums for df32 blocks without an overlap matrix (error-free FP32 steps: the FP64 pipe runs at
+// 1/64 of the FP32 rate); with one, where H - E S is formed in FP64, and for the other types, FP64
+template <typename T, bool OVERLAP>
 struct PartialOf {
   using type = double;
 };
 template <>
-struct PartialOf<df> {
+struct PartialOf<df, false> {
   using type = df;
 };
 __device__ __forceinline__ void acc_add(double& a, double b) { a += b; }
@@ -95,12 +95,13 @@ __device__ __forceinline__ void trace_term(double& a, cx<double> h, cx<T> u) {
   a += h.re * to_d(u.re) + h.im * to_d(u.im);
 }
 
-template <typename T>
+// OVERLAP: Sup is given
+template <typename T, bool OVERLAP>
 __global__ void __launch_bounds__(256) k_lesser_offdiag(const cx<T>* PGL, cx<T>* X2, cx<T>* GLu, const cx<double>* Hup,
                                                         const cx<double>* Sup, const double* E, int b, int nt,
-                                                        typename PartialOf<T>::type* part) {
+                                                        typename PartialOf<T, OVERLAP>::type* part) {
   after_previous();
-  using Acc = typename PartialOf<T>::type;
+  using Acc = typename PartialOf<T, OVERLAP>::type;
   extern __shared__ __align__(16) unsigned char dsm[];
   cx<T>(*pij)[TS + 1] = reinterpret_cast<cx<T>(*)[TS + 1]>(dsm);
   cx<T>(*pji)[TS + 1] = pij + TS;
@@ -122,7 +123,7 @@ __global__ void __launch_bounds__(256) k_lesser_offdiag(const cx<T>* PGL, cx<T>*
   __syncthreads();
   Acc acc;
   zero(acc);
-  const double Ee = (Hup && Sup) ? E[e] : 0.0;
+  const double Ee = OVERLAP ? E[e] : 0.0;
   for (int side = 0; side < (I == J ? 1 : 2); ++side) {
     const int r0 = (side ? J : I) * TS, c0 = (side ? I : J) * TS;
     cx<T>(*p)[TS + 1] = side ? pji : pij;
@@ -141,7 +142,7 @@ __global__ void __launch_bounds__(256) k_lesser_offdiag(const cx<T>* PGL, cx<T>*
       if (GLu) GLu[o + at] = u;
       if (Hup) {
         cx<double> h = Hup[at];
-        if (Sup) h = h - Ee * Sup[at];
+        if (OVERLAP) h = h - Ee * Sup[at];
         trace_term(acc, h, u);
       }
       cx<T> hp;  // PGL^H / 2 before conjugation
@@ -232,29 +233,39 @@ size_t lesser_scratch_bytes(int b, int batch) {
   return (size_t)batch * (nt * (nt + 1) / 2 + nt) * sizeof(double);
 }
 
-template <typename T>
-cudaError_t lesser_offdiag(const cx<T>* PGL, cx<T>* X2, cx<T>* GLu, const cx<double>* Hup, const cx<double>* Sup,
-                           const double* E, int b, int batch, void* scratch, cudaStream_t st) {
+template <typename T, bool OVERLAP>
+static cudaError_t launch_offdiag(const cx<T>* PGL, cx<T>* X2, cx<T>* GLu, const cx<double>* Hup, const cx<double>* Sup,
+                                  const double* E, int b, int batch, void* scratch, cudaStream_t st) {
   const int nt = tiles_of(b);
   const int smem = 4 * TS * (TS + 1) * (int)sizeof(cx<T>);
   static std::atomic<unsigned long long> done{0};
-  const cudaError_t e = allow_smem(k_lesser_offdiag<T>, smem, done);
+  const cudaError_t e = allow_smem(k_lesser_offdiag<T, OVERLAP>, smem, done);
   if (e != cudaSuccess) return e;
-  launch_after(k_lesser_offdiag<T>, dim3(nt * (nt + 1) / 2, batch), 256, smem, st, 
-      PGL, X2, GLu, Hup, Sup, E, b, nt, reinterpret_cast<typename PartialOf<T>::type*>(scratch));
+  launch_after(k_lesser_offdiag<T, OVERLAP>, dim3(nt * (nt + 1) / 2, batch), 256, smem, st, PGL, X2, GLu, Hup, Sup, E, b, nt,
+               reinterpret_cast<typename PartialOf<T, OVERLAP>::type*>(scratch));
   count_launch();
   return cudaGetLastError();
 }
+template <typename T>
+cudaError_t lesser_offdiag(const cx<T>* PGL, cx<T>* X2, cx<T>* GLu, const cx<double>* Hup, const cx<double>* Sup,
+                           const double* E, int b, int batch, void* scratch, cudaStream_t st) {
+  return Hup && Sup ? launch_offdiag<T, true>(PGL, X2, GLu, Hup, Sup, E, b, batch, scratch, st)
+                    : launch_offdiag<T, false>(PGL, X2, GLu, Hup, Sup, E, b, batch, scratch, st);
+}
 
 template <typename T>
-cudaError_t lesser_diag(cx<T>* gl, const cx<T>* X, cx<double>* out64, long so, double* cur, long ldcur, double* den,
+cudaError_t lesser_diag(cx<T>* gl, const cx<T>* X, cx<double>* out64, long so, double* cur, long ldcur, bool overlap, double* den,
                         long ldden, int b, int batch, void* scratch, cudaStream_t st) {
-  using Acc = typename PartialOf<T>::type;
   const int nt = tiles_of(b), np = nt * (nt + 1) / 2;
   double* pd = reinterpret_cast<double*>(scratch) + (size_t)batch * np;
   launch_after(k_lesser_diag<T>, dim3(np, batch), 256, 2 * TS * (TS + 1) * sizeof(cx<T>), st, gl, X, out64, so, b, nt, pd);
   count_launch();
-  launch_after(k_trace_sums<Acc>, batch, 32, 0, st, cur, ldcur, reinterpret_cast<const Acc*>(scratch), np, den, ldden, pd, nt);
+  auto sums = [&](auto A) {
+    using Acc = decltype(A);
+    launch_after(k_trace_sums<Acc>, batch, 32, 0, st, cur, ldcur, reinterpret_cast<const Acc*>(scratch), np, den, ldden, pd, nt);
+  };
+  if (overlap) sums(typename PartialOf<T, true>::type{});
+  else sums(typename PartialOf<T, false>::type{});
   count_launch();
   return cudaGetLastError();
 }
@@ -262,7 +273,7 @@ cudaError_t lesser_diag(cx<T>* gl, const cx<T>* X, cx<double>* out64, long so, d
 #define QTX_LESSER(T)                                                                                                   \
   template cudaError_t lesser_offdiag<T>(const cx<T>*, cx<T>*, cx<T>*, const cx<double>*, const cx<double>*,           \
                                          const double*, int, int, void*, cudaStream_t);                                \
-  template cudaError_t lesser_diag<T>(cx<T>*, const cx<T>*, cx<double>*, long, double*, long, double*, long, int, int, \
+  template cudaError_t lesser_diag<T>(cx<T>*, const cx<T>*, cx<double>*, long, double*, long, bool, double*, long, int, int, \
                                       void*, cudaStream_t);
 QTX_LESSER(double)
 QTX_LESSER(float)

@@ -1194,7 +1194,7 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
       void* gd = k ? (want(QTX_OUT_GG_DIAG, out->GG_diag) ? out->GG_diag : nullptr)
                    : (want(QTX_OUT_GL_DIAG, out->GL_diag) ? out->GL_diag : nullptr);
       QTX_CK(lesser_diag<T>(gli, Tk(k), gd ? reinterpret_cast<cx<double>*>(gd) + o64 : nullptr, (long)nb * bb,
-                            k == 0 && cur_out ? cur + i : nullptr, ncur, k ? spare : den + i, k ? 1 : nb, b, ne, traces, st));   // G^<_ii
+                            k == 0 && cur_out ? cur + i : nullptr, ncur, Su != nullptr, k ? spare : den + i, k ? 1 : nb, b, ne, traces, st));   // G^<_ii
       if (k == 1) continue;
       if (!d.second_rhs && want(QTX_OUT_GG_DIAG, out->GG_diag) && (s = emit<T>(P, out->GG_diag, nb, i, e0, gli, b, ne, st, gi, gi))) return s;
       if (cont)
