@@ -42,7 +42,9 @@ qtx_status qtx_zgemm_batched(int precision, int M, int N, int K, int opA, const 
  * residual is at FP64 level and eliminates in FP64 (pivoted) the blocks where that does not converge;
  * QTX_EMU64 / QTX_BF16X3 start from the FP32 inverse and apply `refine_iter` Newton sweeps with
  * tensor-core products.  status[e] (device, may be NULL) receives
- * QTX_ERR_SINGULAR for a zero pivot. */
+ * QTX_ERR_SINGULAR for a zero pivot.  Synchronises `stream` before returning.  Errors:
+ * QTX_ERR_INVALID_ARG, QTX_ERR_UNSUPPORTED, QTX_ERR_OOM, QTX_ERR_CUDA, QTX_ERR_TIMEOUT (a bounded wait
+ * inside a tensor-core product expired; A is then not valid, the context stays usable). */
 qtx_status qtx_zinv_batched(int precision, int n, void *A, long strideA, int batch, int refine_iter,
                             int *status, void *stream);
 
@@ -76,8 +78,8 @@ qtx_status qtx_fpx_decompress(int bits, const void *in, long n, double *x, void 
  * tensor-core product launch first makes its MMA-issuing thread wait on a barrier that nothing arrives
  * at, with every wait of the launch limited to 100 us: the wait gives up before any MMA is issued,
  * the launch raises its wait flag, drains the bulk copies it has issued, frees its tensor memory and
- * returns, and the call that launched it reports QTX_ERR_TIMEOUT (qtx_zgemm_batched, or
- * qtx_rgf_status after a solve; the products' outputs are then not valid).  The context stays usable
+ * returns, and the call that launched it reports QTX_ERR_TIMEOUT (qtx_zgemm_batched,
+ * qtx_zgemm_emu64_noalloc, qtx_zinv_batched, or qtx_rgf_status after a solve; the products' outputs are then not valid).  The context stays usable
  * and the next call after disabling the switch computes normally.  Process-wide; not for production
  * use.  Always returns QTX_OK. */
 qtx_status qtx_tc_wait_test(int enable);

@@ -227,3 +227,24 @@ def test_bounded_wait_gives_up_and_the_context_stays_usable(q):
     for k in outs:
         assert np.array_equal(again[k], good[k]), k
     P.close()
+
+
+# the block inverse's products on the tensor cores: nine planes (fp64), six and four (emu64), four (fp32)
+@pytest.mark.parametrize("prec,n", [("fp64", 40), ("emu64", 64), ("fp32", 200)])
+def test_block_inverse_reports_an_expired_wait(q, prec, n):
+    import torch
+    L = q.load()
+    rng = np.random.default_rng(n)
+    A = _t(rng.standard_normal((2, n, n)) + 1j * rng.standard_normal((2, n, n)) + 4 * np.sqrt(n) * np.eye(n))
+    ref, st = q.zinv_batched(A.clone(), prec)
+    assert not st.any()
+    L.qtx_tc_wait_test(1)
+    try:
+        with pytest.raises(q.QtxError) as ei:
+            q.zinv_batched(A.clone(), prec)
+        assert ei.value.status == 6  # QTX_ERR_TIMEOUT
+    finally:
+        L.qtx_tc_wait_test(0)
+    torch.cuda.synchronize()
+    again, st = q.zinv_batched(A.clone(), prec)
+    assert torch.equal(again, ref) and not st.any()
