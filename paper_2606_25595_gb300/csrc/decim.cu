@@ -317,7 +317,11 @@ __global__ void __launch_bounds__(kThreads) k_decimate(const DecimArgs a) {
     __syncthreads();
     for (int idx = t; idx < n * n; idx += kThreads) out[idx] = dot<NM>(T, be, idx / n, idx % n, n);  // (H01 g_s) H01^H
   }
-  if (t == 0 && st && a.status) atomicCAS(a.status + e, 0, st);
+  // of two failing contacts the first one's code stands, whichever cluster ends first
+  if (t == 0 && st && a.status) {
+    if (blockIdx.y == 0 && gridDim.y > 1) atomicExch(a.status + e, st);
+    else atomicCAS(a.status + e, 0, st);
+  }
 }
 
 template <int NM>

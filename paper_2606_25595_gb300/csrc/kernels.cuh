@@ -219,9 +219,10 @@ cudaError_t merge_status(const int* st, int leads, int ne, int* status, cudaStre
 cudaError_t max_modulus(const cx<double>* X, long n, double* out, cudaStream_t st);
 // p[0..n) = v
 cudaError_t fill_int(int* p, int v, int n, cudaStream_t st);
-// The whole decimation of lead blocks of size n <= kDecimSmallMax per energy and contact in one CTA
-// (decim.cu), one launch for 1 or 2 contacts: SR[k][e] = H01[k] g_s(E[e] + i eta) H01[k]^H; status[e] =
-// QTX_ERR_NOT_CONVERGED / QTX_ERR_SINGULAR (only raised from 0).  No host synchronisation.
+// The whole decimation of lead blocks of size n <= kDecimSmallMax per energy and contact in one cluster of 1 to 8
+// CTAs (decim.cu), one launch for 1 or 2 contacts: SR[k][e] = H01[k] g_s(E[e] + i eta) H01[k]^H; status[e] =
+// QTX_ERR_NOT_CONVERGED / QTX_ERR_SINGULAR, the first failing contact's (one contact: only raised from 0; two:
+// status is 0 before).  No host synchronisation.
 constexpr int kDecimSmallMax = 32;
 cudaError_t decimate_small(int leads, const cx<double>* const* H00, const cx<double>* const* H01, cx<double>* const* SR,
                            const double* E, double eta, double tol_rel, int max_iter, int n, int batch, int* status,

@@ -171,3 +171,18 @@ def test_fp64_elimination_reciprocal(q):
             assert abs(w.real - ref.real) <= 2.0**-53 and abs(w.imag - ref.imag) <= 2.0**-53
         else:
             assert w == ref, (re, im, w, ref)
+
+
+# both contacts in one launch (8), and in the same launches one kernel at a time (40)
+@pytest.mark.parametrize("b", [8, 40])
+def test_of_two_failing_contacts_the_left_code_stands(q, b):
+    dev = _device(b, 2, 6, 0, 1, 0, 0)
+    dev["energies"] = np.full(6, 0.25)
+    z = 0.25 + 1j * dev["eta"]
+    sing, slow = (z * np.eye(b), 0.5 * np.eye(b) + 0j), (dev["leads"]["H00_R"], dev["leads"]["H01_R"])
+    for left, right, code in ((sing, slow, 4), (slow, sing, 5)):  # z - H00 = 0; one sweep is not enough
+        dev["leads"] = dict(H00_L=left[0], H01_L=left[1], H00_R=right[0], H01_R=right[1])
+        plan = q.Plan(q.make_desc(2, b, "fp64", 6, has_scattering=False, leads=True, decim_max_iter=1, outputs=["density"]))
+        for _ in range(5):
+            assert q.solve_device(dev, "fp64", outputs=["density"], plan=plan)["status"].tolist() == [code] * 6
+        plan.close()
