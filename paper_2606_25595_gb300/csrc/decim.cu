@@ -197,6 +197,14 @@ __device__ __forceinline__ cx<double> dot(const cx<double>* A, const cx<double>*
   return acc;
 }
 
+// A contact's failure into its energy's status: of two failing contacts the first one's code stands, whichever
+// cluster ends first.  Out of line: inlined, it changes the code of the
+// sweeps (4 energies at b = 16: 1394 -> 1403 us a solve).
+__device__ __noinline__ void raise_status(int* status, int st) {
+  if (blockIdx.y == 0 && gridDim.y > 1) atomicExch(status, st);
+  else atomicCAS(status, 0, st);
+}
+
 template <int NM>
 __global__ void __launch_bounds__(kThreads) k_decimate(const DecimArgs a) {
   extern __shared__ __align__(16) unsigned char dsm[];
@@ -317,11 +325,7 @@ __global__ void __launch_bounds__(kThreads) k_decimate(const DecimArgs a) {
     __syncthreads();
     for (int idx = t; idx < n * n; idx += kThreads) out[idx] = dot<NM>(T, be, idx / n, idx % n, n);  // (H01 g_s) H01^H
   }
-  // of two failing contacts the first one's code stands, whichever cluster ends first
-  if (t == 0 && st && a.status) {
-    if (blockIdx.y == 0 && gridDim.y > 1) atomicExch(a.status + e, st);
-    else atomicCAS(a.status + e, 0, st);
-  }
+  if (t == 0 && st && a.status) raise_status(a.status + e, st);
 }
 
 template <int NM>
