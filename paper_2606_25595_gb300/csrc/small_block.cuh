@@ -1,5 +1,5 @@
-// FP64 block arithmetic inside one CTA for blocks of at most 32 (the solve of small blocks and the
-// contacts' decimation): products and inverses of complex128 blocks held in shared memory.
+// FP64 block arithmetic inside one CTA for blocks of at most 32 (the solve of small blocks, small.cu): products
+// and inverses of complex128 blocks held in shared memory.
 //
 // GB300's FP64 pipe issues two DFMA a cycle and SM, so a product of two 16 x 16 complex blocks is
 // 8,600 cycles of it.  Products here run on the tensor cores instead, as in tc_fp64.cu: each row of
@@ -78,7 +78,7 @@ __device__ __forceinline__ void digitize(const cx<double>* X, int trans, int cj,
     const double give = odd ? v.re : v.im;
     const double got = __shfl_xor_sync(0xffffffffu, give, 1);
     const double x0 = odd ? got : v.re, x1 = odd ? v.im : got;
-    const bool dead = e >= kExpoNonFinite;  // zero digits; the product's result is set to NaN
+    const bool dead = e >= kExpoNonFinite;  // zero digits; mm computes these by DFMA
     const uint64_t a = dead ? kDigBias : fix_biased(x0, kFix62 - e), b = dead ? kDigBias : fix_biased(x1, kFix62 - e);
     const int at = r * PK + (odd ? NM + k - 1 : k);
 #pragma unroll
@@ -126,8 +126,25 @@ __device__ __forceinline__ int64_t parts_lo(const float (&acc)[8][4], int v) {
   return unit_int(acc[6][v], 42) * (1 << 14) + unit_int(acc[7][v], 48) * (1 << 8);
 }
 
-// C = sign op(A) op(B) (+ C0) (+ diag I on the first b rows), all blocks in shared memory.  C may be A, B
-// or C0.  da / db: digitise A / B (false: its planes are those of the last product with it on that side).
+// The value of fixed-point parts hi, lo at (r, c) where the fast sum cannot form it: outside the normal range, or in a
+// row or column that holds an infinity or a NaN, where one part of (op(A) op(B))(r, c) is formed by DFMA in ascending
+// k from the operands themselves and propagates them as in the launched path's product.
+template <int NM>
+__device__ __noinline__ double rare_value(const Smem<NM>& s, const cx<double>* A, int opA, const cx<double>* B, int opB, int r, int c,
+                                          int part, int b, int64_t hi, int64_t lo) {
+  constexpr int LD = Smem<NM>::LD;
+  const int ea = s.ea[r], eb = s.eb[c];
+  if (ea < kExpoNonFinite && eb < kExpoNonFinite) return scale64(fix_sum(hi, lo), ea + eb - 12);
+  cx<double> acc = mk<double>(0.0, 0.0);
+  if (r < b && c < b)
+    for (int k = 0; k < b; ++k)
+      cfma(acc, opA == OP_N ? A[r * LD + k] : conj(A[k * LD + r]), opB == OP_N ? B[k * LD + c] : conj(B[c * LD + k]));
+  return part ? acc.im : acc.re;
+}
+
+// C = sign op(A) op(B) (+ C0) (+ diag I on the first b rows), all blocks in shared memory.  C may be C0, and A or
+// B where both are finite.  da / db: digitise A / B (false: its planes are those of the last product with it on
+// that side).
 // Begins on operands that every thread has written before a barrier; ends with one.  Not inlined: the
 // kernels call it from some twenty places, and inlined copies miss the instruction cache on every call.
 //
@@ -161,11 +178,7 @@ __device__ __noinline__ void mm(Smem<NM>& s, int b, cx<double>* C, double sign, 
 #pragma unroll
     for (int q = 0; q < n; ++q) {
       const int v = v0 + q, r = mt * 16 + lane / 4 + (v / 2) * 8, c = nt * 8 + (lane % 4) * 2 + (v & 1);
-      if (bad) {
-        const int ea = s.ea[r], eb = s.eb[c];
-        x[q] = scale64(fix_sum(hi[q], lo[q]), ea + eb - 12);
-        if (ea >= kExpoNonFinite || eb >= kExpoNonFinite) x[q] = __longlong_as_double(0x7ff8000000000000ll);
-      }
+      if (bad) x[q] = rare_value<NM>(s, A, opA, B, opB, r, c, part, b, hi[q], lo[q]);
       if (sign < 0) x[q] = -x[q];
       if (C0) x[q] += (&C0[r * LD + c].re)[part];
       if (diag != 0.0 && part == 0 && r == c && r < b) x[q] += diag;

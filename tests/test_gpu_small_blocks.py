@@ -186,3 +186,21 @@ def test_of_two_failing_contacts_the_left_code_stands(q, b):
         for _ in range(5):
             assert q.solve_device(dev, "fp64", outputs=["density"], plan=plan)["status"].tolist() == [code] * 6
         plan.close()
+
+
+# one value of Sigma^< of one energy infinite: G^< = (g Sigma^<) g^H takes infinities and NaN where the launched path's
+# DFMA products do (same order of the sums), and the padded rows and the other energies nothing
+@pytest.mark.parametrize("b", [3, 16, 21, 32])
+def test_small_blocks_propagate_infinities(q, b):
+    dev = _device(b, 1, 3, 0, 0, 1, 1)
+    names = ["GR_diag", "GL_diag", "GG_diag", "density"]
+    clean = q.solve_device(dev, "fp64", outputs=names)
+    dev["SigL"][1, 0, 1, 2] = np.inf
+    got = q.solve_device(dev, "fp64", outputs=names)
+    ref = q.solve_device(dev, "fp64", outputs=names + ["continuity"])
+    parts = lambda x: np.stack([x.real, x.imag])  # noqa: E731
+    for k in names:
+        x, y = parts(got[k][1]), parts(ref[k][1])
+        assert np.array_equal(np.isnan(x), np.isnan(y)) and np.array_equal(x[np.isinf(x)], y[np.isinf(y)]), k
+        assert np.array_equal(got[k][[0, 2]], clean[k][[0, 2]])
+    assert np.isinf(parts(got["GL_diag"][1])).any()
