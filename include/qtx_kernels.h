@@ -22,8 +22,14 @@ enum { QTX_OP_N = 0, QTX_OP_C = 1 /* conjugate transpose */ };
  *     C[e] = alpha * op(A[e]) * op(B[e]) + beta * C0[e],   e = 0 .. batch-1,
  * op(A) is M x K, op(B) is K x N, C and C0 are M x N.  lda/ldb/ldc0/ldc are row strides and
  * strideA/B/C0/C batch strides in complex elements (0 shares one matrix across the batch).
- * precision: QTX_FP32 on the CUDA cores; QTX_FP64 on the tensor cores with 9 bf16 digit planes (one
- * FP64 rounding of the whole sum) when every dimension is above 32, else on the CUDA cores; QTX_EMU64 / QTX_BF16X3 on the tcgen05 tensor cores
+ * precision: QTX_FP32 on the CUDA cores; QTX_FP64 on the tensor cores with 9 bf16 digit planes when every
+ * dimension is above 32, else on the CUDA cores (DFMA).  With digit planes an operand value is held to 2^-62
+ * of the largest in its row of op(A) or column of op(B) (2^-61 for K > 256) and the sum is rounded to FP64
+ * once per 512 k, so
+ *     |C - exact| <= 2^-53 |C| + K 2^-54 max_k |A(m, k)| max_k |B(k, n)|   (alpha = 1, beta = 0, K <= 512):
+ * below DFMA's error for values of like size, but values below 2^-9 of their row's largest keep fewer bits
+ * than the 53 that DFMA takes (one of 2^-40 of it 22, below 2^-62 none), which shows where large values meet
+ * only small ones.  QTX_EMU64 / QTX_BF16X3 on the tcgen05 tensor cores
  * with 6 (7 when K > 512) / 2 bf16 digit planes per operand (Ozaki-style slicing, Sec. II-D), inputs
  * and outputs rounded to df32 (hi + lo FP32 pairs) on the way in and out; alpha and beta are applied as
  * df32 pairs as well (~48 bits: a scalar such as 0.1 adds no FP32-sized error).  C0 may be NULL when beta == 0; C may
@@ -38,8 +44,8 @@ qtx_status qtx_zgemm_batched(int precision, int M, int N, int K, int opA, const 
 /* Batched inverse of n x n complex blocks, in place (A[e] -> A[e]^-1, batch stride strideA), as used
  * by the forward sweep (g_i = (A_i - V g U)^-1): Gauss-Jordan with partial pivoting on blocks of at
  * most 64, a 2 x 2 Schur-complement recursion above that, plus one Newton step X += X (I - A X) for
- * recursed FP32 blocks; QTX_FP64 above 32 refines the FP32 inverse with FP64 products until its
- * residual is at FP64 level and eliminates in FP64 (pivoted) the blocks where that does not converge;
+ * recursed FP32 blocks; QTX_FP64 above 32 refines the FP32 inverse with FP64 products (qtx_zgemm_batched)
+ * until its residual's norm is at FP64 level and eliminates in FP64 (pivoted) the blocks where that does not converge;
  * QTX_EMU64 / QTX_BF16X3 start from the FP32 inverse and apply `refine_iter` Newton sweeps with
  * tensor-core products.  status[e] (device, may be NULL) receives
  * QTX_ERR_SINGULAR for a zero pivot.  Synchronises `stream` before returning.  Errors:

@@ -69,6 +69,25 @@ def test_fp64_product_scales_and_specials(q):
     assert not np.isfinite(C[5]).any() and np.isnan(C[:, 11]).all() and (C[4][np.isfinite(C[4])] == 0).all()
 
 
+# values of mixed size inside rows and columns: graded over `decades`, in an order of k shared by A and B (large meets
+# large) or opposite (large meets small), and with large values meeting zeros
+@pytest.mark.parametrize("K", [64, 300])
+@pytest.mark.parametrize("decades", [8, 16, 30])
+@pytest.mark.parametrize("meet", ["large", "small", "zeros"])
+def test_fp64_product_of_mixed_sizes_within_the_stated_bound(q, K, decades, meet):
+    import torch
+    rng = np.random.default_rng(K + decades)
+    n = 40
+    grade = 10.0 ** -np.linspace(0, decades, K)
+    A, B = _cx(rng, 1, n, K) * grade, _cx(rng, 1, K, n) * (grade[::-1] if meet == "small" else grade)[:, None]
+    if meet == "zeros":
+        B[0, : K // 2] = 0
+    C = q.zgemm_batched(torch.tensor(A).cuda(), torch.tensor(B).cuda(), "fp64").cpu().numpy()[0]
+    ref = _ld(A[0]) @ _ld(B[0])
+    bound = 2.0 ** -53 * np.abs(ref) + K * 2.0 ** -54 * np.abs(A[0]).max(1)[:, None] * np.abs(B[0]).max(0)[None, :]
+    assert np.all(np.abs(C - ref) <= bound), float((np.abs(C - ref) / bound).max())
+
+
 def test_fp64_product_error_not_above_dfma(q):
     """Error against exact rational sums, beside that of a plain FP64 product (the library's own below
     33 rows is DFMA: the same operands, 32 rows at a time)."""
