@@ -851,42 +851,56 @@ __device__ __forceinline__ float mag32(double x) {
   return e <= 0 ? 0.f : __uint_as_float(((unsigned)e << 23) | ((h & 0xfffffu) << 3) | ((unsigned)__double2loint(x) >> 29));
 }
 // One cluster of 1 to 8 CTAs per block: a single CTA's loads are latency-bound (8 blocks of 128 x 128 complex128,
-// masked sweeps included: 9.9 us in one CTA each, 4.2 us in eight).
-template <typename T>
+// masked sweeps included: 9.9 us in one CTA each, 4.2 us in eight).  The sum is always that of the same eight slices,
+// SL = 8 / C of them to a CTA, so that whether an energy goes on does not depend on the batch it is in.
+template <typename T, int SL>
 __global__ void __launch_bounds__(512) k_residual_mask(const cx<T>* R, long sR, long nn, float tol2,
                                                        const int* active, int* next, int* status) {
   after_previous();
   cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
-  const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank(), e = blockIdx.x / C;
+  constexpr int C = 8 / SL, STEP = 8 * 512;
+  const int rank = (int)cl.block_rank(), e = blockIdx.x / C, t = threadIdx.x;
   if (active && !active[e]) {  // the whole cluster
-    if (rank == 0 && threadIdx.x == 0) next[e] = 0;
+    if (rank == 0 && t == 0) next[e] = 0;
     return;
   }
   const cx<T>* X = R + (long)e * sR;
-  float s = 0.f;
-#pragma unroll 4
-  for (long i = rank * (long)blockDim.x + threadIdx.x; i < nn; i += C * (long)blockDim.x) {
-    const cx<T> x = X[i];
-    const float a = mag32(x.re), c = mag32(x.im);
-    s = fmaf(a, a, fmaf(c, c, s));
+  float s[SL];
+#pragma unroll
+  for (int u = 0; u < SL; ++u) s[u] = 0.f;
+  // slice q: values 512 q .. 512 q + 511 of every 4096
+#pragma unroll (SL == 1 ? 4 : 1)
+  for (long i = (long)rank * SL * 512 + t; i < nn; i += STEP)
+#pragma unroll
+    for (int u = 0; u < SL; ++u)
+      if (i + 512 * u < nn) {
+        const cx<T> x = X[i + 512 * u];
+        const float a = mag32(x.re), c = mag32(x.im);
+        s[u] = fmaf(a, a, fmaf(c, c, s[u]));
+      }
+  __shared__ float red[SL][16], part[8];
+#pragma unroll
+  for (int u = 0; u < SL; ++u) {
+    for (int off = 16; off > 0; off >>= 1) s[u] += __shfl_down_sync(0xffffffffu, s[u], off);
+    if (t % 32 == 0) red[u][t / 32] = s[u];
   }
-  __shared__ float red[16], part[8];
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-  if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = s;
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int w = 1; w < 16; ++w) s += red[w];
-  if (C > 1) {
-    cl.sync();  // the first CTA's shared memory exists
-    if (threadIdx.x == 0) *cl.map_shared_rank(&part[rank], 0) = s;
-    cl.sync();
+  if (C > 1) cl.sync();  // the first CTA's shared memory exists, and red is written
+  else __syncthreads();
+  if (t < SL) {
+    float v = red[t][0];
+    for (int w = 1; w < 16; ++w) v += red[t][w];
+    if (C > 1) *cl.map_shared_rank(&part[rank * SL + t], 0) = v;
+    else part[t] = v;
   }
-  if (rank == 0 && threadIdx.x == 0) {
-    for (int q = 1; q < C; ++q) s += part[q];
+  if (C > 1) cl.sync();
+  else __syncthreads();
+  if (rank == 0 && t == 0) {
+    float v = part[0];
+    for (int q = 1; q < 8; ++q) v += part[q];
     // a NaN or infinite norm compares false against tol2: such an energy keeps refining, and its
     // block inverse has failed, so it is reported singular
-    next[e] = (s <= tol2) ? 0 : 1;
-    if (status && !(s <= 3.0e38f)) atomicCAS(status + e, 0, (int)QTX_ERR_SINGULAR);
+    next[e] = (v <= tol2) ? 0 : 1;
+    if (status && !(v <= 3.0e38f)) atomicCAS(status + e, 0, (int)QTX_ERR_SINGULAR);
   }
 }
 template <typename T>
@@ -895,8 +909,14 @@ cudaError_t residual_mask(const cx<T>* R, long sR, int n, int batch, double tol,
   // CTAs a block: up to two per SM over the batch, at least 2,048 values each
   int C = 1;
   while (C < 8 && (long)batch * C * 2 <= 304 && (long)n * n >= 4096L * C) C *= 2;
-  const cudaError_t le = launch_after_clusters(k_residual_mask<T>, C, batch * C, 512, 0, st, R, sR, (long)n * n, (float)(tol * tol),
-                                               active, next, status);
+  auto go = [&](auto SL) {
+    return launch_after_clusters(k_residual_mask<T, decltype(SL)::value>, C, batch * C, 512, 0, st, R, sR, (long)n * n,
+                                 (float)(tol * tol), active, next, status);
+  };
+  const cudaError_t le = C == 8   ? go(std::integral_constant<int, 1>())
+                         : C == 4 ? go(std::integral_constant<int, 2>())
+                         : C == 2 ? go(std::integral_constant<int, 4>())
+                                  : go(std::integral_constant<int, 8>());
   count_launch();
   return le != cudaSuccess ? le : cudaGetLastError();
 }
