@@ -77,6 +77,18 @@ inline cudaError_t allow_smem(F* kernel, int bytes, std::atomic<unsigned long lo
   return cudaSuccess;
 }
 
+// SM count of the current device
+inline cudaError_t sm_count(int& sms) {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 64 && (sms = known[dev].load(std::memory_order_relaxed)) > 0) return cudaSuccess;
+  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess && dev < 64) known[dev].store(sms, std::memory_order_relaxed);
+  return e;
+}
+
 // ---- batched complex GEMM on the CUDA cores (T = double: DFMA, T = float: FFMA)
 template <typename T>
 cudaError_t gemm_simt(const GemmArgs<T>& g, cudaStream_t st);

@@ -814,16 +814,11 @@ cudaError_t launch(const TcPrepared* const* pp, int n, cudaStream_t st, cudaEven
   if (n < 1 || n > kMaxGroup) return cudaErrorInvalidValue;
   cudaError_t e;
   const size_t smem = (size_t)ring_bytes_of(S, NST) + out_bytes_of(S) + 1024 + 256;
-  static bool attr = false;
-  static int sms = 0;
-  if (!attr) {
-    if ((e = cudaFuncSetAttribute(k_tc_gemm<S, NST, IO, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
-    if ((e = cudaFuncSetAttribute(k_tc_gemm<S, NST, IO, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
-    int dev = 0;
-    if ((e = cudaGetDevice(&dev))) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
-    attr = true;
-  }
+  static std::atomic<unsigned long long> done1{0}, done2{0};
+  int sms = 0;
+  if ((e = allow_smem(k_tc_gemm<S, NST, IO, false>, (int)smem, done1)) || (e = allow_smem(k_tc_gemm<S, NST, IO, true>, (int)smem, done2)) ||
+      (e = sm_count(sms)))
+    return e;
   TcGroup G;
   G.n = n;
   G.hold = g_wait_test.load(std::memory_order_relaxed);

@@ -476,13 +476,6 @@ int chunk_k(int K) {
   return nc <= 1 ? K : (K + nc - 1) / nc;
 }
 
-// SM count of the current device
-cudaError_t sm_count(int& sms) {
-  int dev = 0;
-  const cudaError_t e = cudaGetDevice(&dev);
-  return e != cudaSuccess ? e : cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-}
-
 // n products, each with `bytes` of scratch behind the last one's
 cudaError_t products9(const GemmArgs<double>* g, int n, unsigned char* scratch, size_t bytes, int* err_flag, cudaStream_t st,
                       cudaEvent_t* ev) {
