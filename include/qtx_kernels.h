@@ -4,7 +4,8 @@
  * own solvers.  Same conventions as qtx_rgf.h: device pointers owned by the caller, interleaved
  * (re, im) doubles, row-major blocks, asynchronous on `stream` (a cudaStream_t), status codes from
  * qtx_status.  Each call takes its temporaries stream-ordered from a memory pool of the library's own (one
- * per device, which keeps at most 512 MiB between calls) and returns them before it returns.  Nothing falls back to the CPU.
+ * per device, which keeps at most 512 MiB between calls) and returns them before it returns;
+ * qtx_release_memory empties the pool.  Nothing falls back to the CPU.
  */
 #ifndef QTX_KERNELS_H
 #define QTX_KERNELS_H
@@ -40,6 +41,11 @@ qtx_status qtx_zgemm_batched(int precision, int M, int N, int K, int opA, const 
                              long strideA, int opB, const void *B, long ldb, long strideB, double alpha,
                              double beta, const void *C0, long ldc0, long strideC0, void *C, long ldc,
                              long strideC, int batch, void *stream);
+
+/* Give the device memory that the calls of this header keep between them on the current device back to the
+ * driver.  Synchronises the device; not during a stream capture.  The next call takes its memory anew.
+ * Errors: QTX_ERR_CUDA. */
+qtx_status qtx_release_memory(void);
 
 /* Batched inverse of n x n complex blocks, in place (A[e] -> A[e]^-1, batch stride strideA), as used
  * by the forward sweep (g_i = (A_i - V g U)^-1): Gauss-Jordan with partial pivoting on blocks of at

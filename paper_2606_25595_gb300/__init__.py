@@ -36,7 +36,7 @@ EXPORTED = ("qtx_rgf_plan_create", "qtx_rgf_solve", "qtx_rgf_status", "qtx_rgf_d
             "qtx_fpx_bytes", "qtx_fpx_compress", "qtx_fpx_decompress", "qtx_w_assemble",
             "qtx_rgf_group_create", "qtx_rgf_group_solve", "qtx_rgf_group_destroy",
             "qtx_rgf_group_last_error", "qtx_rgf_group_launches", "qtx_rgf_group_pooled_products",
-            "qtx_tc_wait_test", "qtx_rgf_group_set_pool_waves")
+            "qtx_tc_wait_test", "qtx_rgf_group_set_pool_waves", "qtx_release_memory")
 
 
 class QtxError(RuntimeError):
@@ -150,6 +150,8 @@ def load() -> ctypes.CDLL:
     L.qtx_rgf_group_set_pool_waves.restype = i
     L.qtx_rgf_group_pooled_products.argtypes = [vp]
     L.qtx_rgf_group_pooled_products.restype = ctypes.c_longlong
+    L.qtx_release_memory.argtypes = []
+    L.qtx_release_memory.restype = i
     L.qtx_tc_wait_test.argtypes = [i]
     L.qtx_tc_wait_test.restype = i
     L.qtx_fpx_bytes.argtypes = [i, l]
@@ -189,6 +191,13 @@ def make_desc(n_blocks, block_size, precision="fp64", max_energies_in_flight=64,
 
 def kernel_launches() -> int:
     return int(load().qtx_kernel_launches())
+
+
+def release_memory() -> None:
+    """Give the memory that component calls keep on the current device back to the driver."""
+    s = load().qtx_release_memory()
+    if s != 0:
+        raise QtxError(s, "qtx_release_memory")
 
 
 def footprint(desc: Desc) -> int:

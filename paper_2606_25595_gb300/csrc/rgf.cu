@@ -1635,9 +1635,11 @@ namespace {
 // default pool returns everything to the driver at each synchronisation, and these calls synchronise, so
 // every call paid for mapping its memory again (0.9 ms of a 1.2 ms product).  The pool keeps at most kPoolKeep
 // between calls and gives the rest back; allocation and reuse are stream-ordered, so calls on several
-// streams and threads share it.
+// streams and threads share it.  qtx_release_memory gives the rest back too, and the driver takes it for an allocation
+// of this process that would not fit beside it.
 constexpr unsigned long long kPoolKeep = 512ull << 20;
-cudaError_t component_pool(cudaMemPool_t* out) {
+// make = false: the pool of the current device and context if there is one, else an error
+cudaError_t component_pool(cudaMemPool_t* out, bool make = true) {
   constexpr int kMaxDev = 64;
   static std::mutex mu;
   static cudaMemPool_t pool[kMaxDev] = {};
@@ -1645,8 +1647,9 @@ cudaError_t component_pool(cudaMemPool_t* out) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (dev >= kMaxDev) return cudaDeviceGetDefaultMemPool(out, dev);
+  if (dev >= kMaxDev) return make ? cudaDeviceGetDefaultMemPool(out, dev) : cudaErrorInvalidValue;
   std::lock_guard<std::mutex> lk(mu);
+  if (!make && (!pool[dev] || current_ctx_id() != ctx[dev])) return cudaErrorInvalidValue;
   if (!pool[dev] || current_ctx_id() != ctx[dev]) {  // first call, or a new context after cudaDeviceReset
     cudaMemPoolProps props = {};
     props.allocType = cudaMemAllocationTypePinned;
@@ -1834,6 +1837,15 @@ qtx_status qtx_zgemm_batched(int precision, int M, int N, int K, int opA, const 
       g_kernel_error = "unknown precision";
       return QTX_ERR_INVALID_ARG;
   }
+}
+
+qtx_status qtx_release_memory(void) {
+  cudaMemPool_t p = nullptr;
+  if (component_pool(&p, false) != cudaSuccess) return QTX_OK;  // none yet
+  // (a block counts as free once the host has seen its free complete)
+  if (cudaDeviceSynchronize() == cudaSuccess && cudaMemPoolTrimTo(p, 0) == cudaSuccess) return QTX_OK;
+  cudaGetLastError();
+  return QTX_ERR_CUDA;
 }
 
 qtx_status qtx_zinv_batched(int precision, int n, void* A, long sA, int batch, int refine_iter, int* status, void* stream) {
