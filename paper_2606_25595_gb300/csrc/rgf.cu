@@ -1640,32 +1640,37 @@ namespace {
 constexpr unsigned long long kPoolKeep = 512ull << 20;
 // make = false: the pool of the current device and context if there is one, else an error
 cudaError_t component_pool(cudaMemPool_t* out, bool make = true) {
-  constexpr int kMaxDev = 64;
+  struct Entry {
+    int dev;
+    unsigned long long ctx;  // ids are not used again: one of a context that cudaDeviceReset ended matches no other
+    cudaMemPool_t pool;
+  };
   static std::mutex mu;
-  static cudaMemPool_t pool[kMaxDev] = {};
-  static unsigned long long ctx[kMaxDev] = {};
+  static std::vector<Entry> pools;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (dev >= kMaxDev) return make ? cudaDeviceGetDefaultMemPool(out, dev) : cudaErrorInvalidValue;
   std::lock_guard<std::mutex> lk(mu);
-  if (!make && (!pool[dev] || current_ctx_id() != ctx[dev])) return cudaErrorInvalidValue;
-  if (!pool[dev] || current_ctx_id() != ctx[dev]) {  // first call, or a new context after cudaDeviceReset
-    cudaMemPoolProps props = {};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = dev;
-    cudaMemPool_t p;
-    if ((e = cudaMemPoolCreate(&p, &props)) != cudaSuccess) return e;
-    unsigned long long keep = kPoolKeep;
-    if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
-      cudaMemPoolDestroy(p);
-      return e;
+  const unsigned long long ctx = current_ctx_id();
+  for (const Entry& p : pools)
+    if (p.dev == dev && p.ctx == ctx) {
+      *out = p.pool;
+      return cudaSuccess;
     }
-    pool[dev] = p;
-    ctx[dev] = current_ctx_id();
+  if (!make) return cudaErrorInvalidValue;
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  cudaMemPool_t p;
+  if ((e = cudaMemPoolCreate(&p, &props)) != cudaSuccess) return e;
+  unsigned long long keep = kPoolKeep;
+  if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+    cudaMemPoolDestroy(p);
+    return e;
   }
-  *out = pool[dev];
+  pools.push_back({dev, current_ctx_id(), p});  // (the pool's creation made a context if there was none)
+  *out = p;
   return cudaSuccess;
 }
 // Stream-ordered temporaries of one call, freed when it returns.
