@@ -296,10 +296,11 @@ const char *qtx_rgf_version(void);
 /* Profiling of the block products (the ZGEMM-class kernel that dominates the solve, Sec. IV).
  * When enabled, every later product-kernel launch of this plan is bracketed by a pair of CUDA events
  * recorded on the solve's stream (for the tensor-core modes, around the tcgen05 GEMM kernel itself,
- * not the digit-plane preparation).  qtx_rgf_gemm_profile synchronises on those events and returns,
- * since enabling or the previous query: the number of launches, their summed device time in
- * milliseconds, the tensor-pipe (or FP pipe) flops issued, and the FP64-equivalent useful flops
- * (8 M N K per complex product), then resets the counters.  Any output pointer may be NULL. */
+ * not the digit-plane preparation; for an FP64 plan of b <= 32 whose sweeps run in one CTA per energy,
+ * around that kernel, whose time includes the block inverses).  qtx_rgf_gemm_profile synchronises on
+ * those events and returns, since enabling or the previous query: the number of launches, their summed
+ * device time in milliseconds, the tensor-pipe (or FP pipe) flops issued, and the FP64-equivalent useful
+ * flops (8 M N K per complex product), then resets the counters.  Any output pointer may be NULL. */
 qtx_status qtx_rgf_set_profiling(qtx_rgf_plan plan, int enable);
 qtx_status qtx_rgf_gemm_profile(qtx_rgf_plan plan, long long *launches, double *ms,
                                 double *pipe_flops, double *useful_flops);

@@ -932,7 +932,17 @@ qtx_status solve_chunk(qtx_rgf_plan_s* P, const qtx_rgf_inputs* in, const qtx_rg
       a.cur = ob.cur; a.den = ob.den; a.con = ob.con; a.tra = ob.tra;
       a.ldcur = ob.ncur;
       a.status = status;
+      cudaEvent_t* ev = P->prof ? P->next_events() : nullptr;
+      if (ev) cudaEventRecord(ev[0], st);
       QTX_CK(rgf_small(a, ne, st));
+      if (ev) {
+        cudaEventRecord(ev[1], st);
+        // its products: 6 a slice (2 of the first) and 6 an interface (7 with G_{i,i+1}), 2 of the transmission
+        const int n = 6 * nb - 4 + (nb - 1) * (6 + (a.GR_upper || a.GG_upper)) + (d.leads ? 2 : 0);
+        const double f = 8.0 * b * b * b * n * ne;
+        P->pipe_flops += f * tc_pairs_fp64();
+        P->useful_flops += f;
+      }
       return finish_chunk<T>(P, in, out, e0, ne, st);
     }
   }

@@ -188,6 +188,21 @@ def test_of_two_failing_contacts_the_left_code_stands(q, b):
         plan.close()
 
 
+def test_profile_of_small_blocks(q):
+    """One kernel launch a chunk; 6 products a slice (2 of the first), 6 an interface, 7 with G_{i,i+1}; 2 more with
+    contacts."""
+    b, nb, ne = 7, 4, 5
+    for leads, outs, n in ((0, ["GR_diag"], 20 + 18), (1, ["GR_diag", "GR_upper"], 20 + 21 + 2)):
+        dev = _device(b, nb, ne, 0, leads, 1 - leads, 0)
+        plan = q.Plan(q.make_desc(nb, b, "fp64", 2, has_scattering=not leads, leads=bool(leads), outputs=outs))
+        plan.set_profiling(True)
+        q.solve_device(dev, "fp64", outputs=outs, plan=plan)
+        prof = plan.gemm_profile()
+        assert prof["launches"] == 3 and prof["ms"] > 0  # chunks of 2, 2 and 1 energies
+        assert prof["useful_flops"] == 8 * b ** 3 * n * ne and prof["pipe_flops"] == 45 * prof["useful_flops"]
+        plan.close()
+
+
 # one value of Sigma^< of one energy infinite: G^< = (g Sigma^<) g^H takes infinities and NaN where the launched path's
 # DFMA products do (same order of the sums), and the padded rows and the other energies nothing
 @pytest.mark.parametrize("b", [3, 16, 21, 32])
