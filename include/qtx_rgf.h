@@ -214,7 +214,7 @@ qtx_status qtx_rgf_plan_create(const qtx_rgf_desc *desc, qtx_rgf_plan *out);
 /* Enqueue the solve of all n_energies on `stream` (a cudaStream_t; NULL = legacy default stream).
  * Energies are processed in chunks of max_energies_in_flight.  Returns after enqueueing: the lead
  * decimation tests convergence on the device (lead blocks of at most 32: the whole iteration of an
- * energy in one CTA; larger: decim_max_iter masked sweeps), so with status_per_energy given the
+ * energy and contact in one cluster of 1 to 8 CTAs; larger: decim_max_iter masked sweeps), so with status_per_energy given the
  * solve makes no host synchronisation and can be captured in a CUDA graph.  Without
  * status_per_energy the library synchronises once per chunk to keep the worst status. */
 qtx_status qtx_rgf_solve(qtx_rgf_plan plan, const qtx_rgf_inputs *in, const qtx_rgf_outputs *out,

@@ -8,6 +8,8 @@
 
 namespace qtx {
 
+constexpr int kSms = 152;  // SMs of a GB300: the rules that split work by size count waves of these
+
 template <typename T>
 struct alignas(2 * sizeof(T)) cx {
   T re, im;

@@ -333,9 +333,9 @@ cudaError_t launch(const DecimArgs& a, int batch, int leads, cudaStream_t st) {
   static std::atomic<unsigned long long> done{0};
   cudaError_t e = allow_smem(k_decimate<NM>, (int)sizeof(DSmem<NM>), done);
   if (e != cudaSuccess) return e;
-  // CTAs of a cluster: as many as leave every energy and contact resident at once on 152 SMs
+  // CTAs of a cluster: as many as leave every energy and contact resident at once on the SMs
   int C = 1;
-  while (C < 8 && (long)batch * leads * C * 2 <= 152 && 4 * C <= a.n) C *= 2;
+  while (C < 8 && (long)batch * leads * C * 2 <= kSms && 4 * C <= a.n) C *= 2;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(batch * C, leads);
   cfg.blockDim = dim3(kThreads);

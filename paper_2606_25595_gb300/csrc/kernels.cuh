@@ -96,7 +96,7 @@ template <typename T>
 cudaError_t gemm_simt_multi(const GemmMulti<T>& m, cudaStream_t st);
 
 // ---- in-place inverse of n x n blocks (n <= kLeafMax) by Gauss-Jordan elimination with partial
-// (row) pivoting, one CTA per block.  A zero pivot stores QTX_ERR_SINGULAR into status[e].
+// (row) pivoting, one CTA per block (FP32) or one cluster of 1 to 8 CTAs (FP64).  A zero pivot stores QTX_ERR_SINGULAR into status[e].
 constexpr int kLeafMax = 64;
 template <typename T>
 cudaError_t leaf_inverse(cx<T>* A, long lda, long sA, int n, int batch, const int* active,
@@ -271,20 +271,20 @@ cudaError_t integrate_add(double* acc, const double* val, long ld, int n, const 
 
 // ---- tensor-core engine (tc_engine.cu): emulated-precision batched complex GEMM on sm_103a.
 // `digits` bf16 digit planes per operand (6: ~41-bit products from 21 digit products, 7 of them
-// taken for K > 512; 2: ~13-bit products from 3; 4 with a.f32: ~27-bit products from 10 for FP32
-// operands and results).  `scratch` holds the digit planes and scale exponents.
+// taken for K > 512; 2: ~13-bit products from 3; 4: ~27-bit products from 10, for FP32
+// operands and results and for the emulated modes' Newton corrections).  `scratch` holds the digit planes and scale exponents.
 // `ev` (optional, two events) brackets the tensor-core GEMM kernel itself (not the digitiser).
 cudaError_t gemm_tc(const TcArgs& a, int digits, void* scratch, size_t scratch_bytes, int* err_flag,
                     cudaStream_t st, cudaEvent_t* ev = nullptr);
 // Kernel parameters of one tensor-core product (filled by gemm_tc_prepare).
 struct TcParams {
-  const unsigned char* pa;  // A plane tiles [batch'][S][M_pad/128][nks][128 x 32 B]
-  const unsigned char* pb;  // B plane sub-tiles [batch'][S][N_pad/48][K_pad/16][3][48 x 32 B]: Re, Im, -Im
+  const unsigned char* pa;  // A digit planes [batch'][M_pad/128][K_pad/16][Re, Im][S][128 x 32 B]
+  const unsigned char* pb;  // B's [batch'][N_pad/BNC][K_pad/16][S][-Im, Re, Im][rows x 32 B], rows = BNC or bn_last
   const int* eA;   // [batch][M_pad] row exponents of op(A)
   const int* eB;   // [batch][N_pad] column exponents of op(B)
   int M_pad, N_pad, nks;  // nks: K-stages of 16 over the embedded K (2 * K_pad)
   int M, N;
-  int bn_last;     // complex columns the last column tile computes: N - 48 (NBt - 1), rounded up to 8
+  int bn_last;     // complex columns the last column tile computes: N - BNC (NBt - 1), rounded up to 8
   void* C; long ldc, sC;         // cx<df>, or cx<float> for the FP32 products
   const void* C0; long ldc0, sC0;
   df alpha, beta;  // as df32 pairs; the kinds say how they enter the epilogue:

@@ -161,9 +161,9 @@ cudaError_t launch(cx<double>* A, long lda, long sA, int n, int batch, const int
   static std::atomic<unsigned long long> done{0};
   const cudaError_t e = allow_smem(k_leaf_fp64<LARGE>, kLeafMax * kLeafMax * (int)sizeof(cx<double>), done);
   if (e != cudaSuccess) return e;
-  // CTAs of a cluster: as many as leave every block resident at once on 152 SMs, with columns for each
+  // CTAs of a cluster: as many as leave every block resident at once on the SMs, with columns for each
   int C = 1;
-  while (C < 8 && (long)batch * C * 2 <= 152 && 8 * C < n) C *= 2;
+  while (C < 8 && (long)batch * C * 2 <= kSms && 8 * C < n) C *= 2;
   const size_t smem = (size_t)n * ((n + C - 1) / C) * sizeof(cx<double>);
   EarlyLaunches none(0);  // (clusters that wait on SMs early: contacts of b = 48 in 12.0 instead of 9.5 ms)
   const cudaError_t le = launch_after_clusters(k_leaf_fp64<LARGE>, C, batch * C, kT, smem, st, A, lda, sA, n, active, status);

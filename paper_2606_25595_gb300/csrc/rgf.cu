@@ -64,7 +64,7 @@ struct Layout {
   size_t tc_bytes;
   size_t tc_more;  // scratch of further products launched together with one in tc_scratch (n_more of them)
   int n_more;
-  bool short_launches;  // a product fills less than four waves of the GPU (see launch_after)
+  bool short_launches;  // a product has at most four tiles per SM (make_layout, launch_after)
   bool refine64;  // FP64 block inverses by refinement (inverse_f64) have their areas
   size_t perm;
 };
@@ -195,14 +195,17 @@ Layout make_layout(const qtx_rgf_desc& d, bool inverse_only = false) {
   // (FP64: digit planes of up to kMany products while they are small, see gemm_fp64_tc_scratch_bytes)
   if (tc64) L.tc_bytes = gemm_fp64_tc_scratch_bytes((int)b, (int)b, (int)b, (int)(inverse_only ? Ec : kMany * Ec));
   L.tc_scratch = a.take(L.tc_bytes);
-  // products of a slice that do not depend on each other share launches while one alone fills less than
-  // four waves of the GPU (608 tiles): their further scratch is then a few hundred MB at most, and the
+  // products of a slice that do not depend on each other share launches while one alone has at most
+  // four tiles per SM (608): their further scratch is then a few hundred MB at most, and the
   // launch's tail, its fixed costs and idle SMs are paid once (b = 120, 24 energies: 72 tiles a product
-  // on 152 SMs).  Larger products fill their waves alone.
+  // on 152 SMs).  Larger products fill their waves alone.  Early launches of everything (launch_after) follow the same
+  // count.  FP64 is counted in 64 columns too, though its tiles have 32: between four and eight waves of those, early
+  // launches take 16.5 against 17.0 ms at b = 64, 23.2 against 23.7 at 100, 14.9 against 15.0 at 128 and 22.4 against 21.7
+  // at 256 (310, 200, 160 and 40 energies).
   const long col = d.precision == QTX_EMU64 ? 48 : 64;
   const long tiles = ((b + 127) / 128) * ((b + col - 1) / col) * Ec;
-  L.short_launches = tiles <= 4 * 152;
-  L.n_more = !inverse_only && L.tc_bytes && d.precision != QTX_FP64 && tiles <= 4 * 152 ? kMany - 1 : 0;
+  L.short_launches = tiles <= 4 * kSms;
+  L.n_more = !inverse_only && L.tc_bytes && d.precision != QTX_FP64 && tiles <= 4 * kSms ? kMany - 1 : 0;
   L.tc_more = a.take((size_t)L.n_more * align_up(L.tc_bytes, 1024));
   // kept digitised operands (emulated modes): two left operands, b x b, E_c energies (none when the
   // products are split along K)
@@ -1988,7 +1991,7 @@ struct qtx_rgf_group_s {
   std::vector<cudaEvent_t> join;
   cudaEvent_t gjoin = nullptr;
   long pool_tiles = 304;             // pooling threshold in tiles: waves x SMs
-  int sms = 152;
+  int sms = kSms;
   std::mutex mu;
   std::condition_variable cv;
   struct Req {
@@ -2083,7 +2086,7 @@ qtx_status qtx_rgf_group_create(int n_plans, const qtx_rgf_plan* plans, qtx_rgf_
     if (!plans[m] || plans[m]->group) return QTX_ERR_INVALID_ARG;
   auto* G = new qtx_rgf_group_s();
   G->plans.assign(plans, plans + n_plans);
-  int dev = 0, sms = 152;
+  int dev = 0, sms = kSms;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   G->pool_tiles = (long)kPoolWaves * sms;

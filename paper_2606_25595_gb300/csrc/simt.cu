@@ -164,14 +164,14 @@ static cudaError_t launch_gemm(const GemmMulti<T>& m, cudaStream_t st) {
 }
 
 // FP64 tile by the FP64 pipe's work: tiles beyond M and N multiply zeros, and few tiles leave SMs idle, so
-// the tile with the least tile area times rounds of 152 SMs is taken (the sums' order is the same in all).
+// the tile with the least tile area times rounds of the SMs is taken (the sums' order is the same in all).
 // 48 x 48 products of 12 entries: 216 us in 64 x 64 tiles (12 CTAs), 13 us in 16 x 16 (108 CTAs).
 static int fp64_tile(int M, int N, long batch) {
   int best = 64;
   long least = 0;
   for (int t : {64, 32, 16}) {
     const long ctas = (long)((M + t - 1) / t) * ((N + t - 1) / t) * batch;
-    const long cost = (ctas + 151) / 152 * t * t;
+    const long cost = (ctas + kSms - 1) / kSms * t * t;
     if (t == 64 || cost < least) {
       best = t;
       least = cost;
@@ -200,8 +200,8 @@ cudaError_t gemm_simt_multi(const GemmMulti<T>& m, cudaStream_t st) {
     // smaller tiles while the larger ones would leave SMs idle (64 x 64 products of 32 entries: 10.9 us in
     // 64 x 64 tiles; every tile sums in the same order)
     auto ctas = [&](int t) { return (long)((g.M + t - 1) / t) * ((g.N + t - 1) / t) * g.batch * m.n; };
-    if (g.M >= 128 && g.N >= 128 && ctas(128) >= 152) return launch_gemm<T, 128, 128, 8, 8, 8>(m, st);
-    if ((g.M > 32 || g.N > 32) && ctas(64) >= 152) return launch_gemm<T, 64, 64, 16, 4, 4>(m, st);
+    if (g.M >= 128 && g.N >= 128 && ctas(128) >= kSms) return launch_gemm<T, 128, 128, 8, 8, 8>(m, st);
+    if ((g.M > 32 || g.N > 32) && ctas(64) >= kSms) return launch_gemm<T, 64, 64, 16, 4, 4>(m, st);
     return launch_gemm<T, 32, 32, 16, 2, 2>(m, st);
   }
 }
@@ -448,17 +448,7 @@ __device__ __forceinline__ void acc_zero(df& a) { a = mkdf(0.f, 0.f); }
 __device__ __forceinline__ df as_df(float x) { return mkdf(x, 0.f); }
 __device__ __forceinline__ df as_df(df x) { return x; }
 __device__ __forceinline__ df as_df(double x) { return from_d<df>(x); }
-template <typename X>
-__device__ __forceinline__ void acc_axpy(double& a, double alpha, X x) { a += alpha * to_d(x); }
-template <typename X>
-__device__ __forceinline__ void acc_axpy(float& a, double alpha, X x) { a = fmaf((float)alpha, (float)to_d(x), a); }
-__device__ __forceinline__ void acc_axpy(float& a, double alpha, float x) { a = fmaf((float)alpha, x, a); }
-template <typename X>
-__device__ __forceinline__ void acc_axpy(df& a, double alpha, X x) {
-  const df v = as_df(x);
-  a = df_add(a, alpha == 1.0 ? v : (alpha == -1.0 ? df_neg(v) : df_mulf(v, (float)alpha)));
-}
-// the same with the coefficient classified on the host (kind +1 / -1 / 0 = general, alpha in FP32)
+// a += alpha x, the coefficient classified on the host (kind +1 / -1 / 0 = general, alpha in FP32)
 template <typename X>
 __device__ __forceinline__ void acc_axpy_k(df& a, int kind, float alpha_f, double, X x) {
   const df v = as_df(x);
@@ -609,7 +599,7 @@ __global__ void __launch_bounds__(256) k_combine_flat(cx<Tout>* out, long sOut, 
 }
 // CTAs along one energy's elements: about eight per SM over the whole batch, at least one per energy
 static unsigned flat_ctas(long bb, int batch) {
-  const long want = (8L * 152 + batch - 1) / batch, most = (bb + 255) / 256;
+  const long want = (8L * kSms + batch - 1) / batch, most = (bb + 255) / 256;
   return (unsigned)(want < 1 ? 1 : (want > most ? most : want));
 }
 
@@ -908,7 +898,7 @@ cudaError_t residual_mask(const cx<T>* R, long sR, int n, int batch, double tol,
                           int* status, cudaStream_t st) {
   // CTAs a block: up to two per SM over the batch, at least 2,048 values each
   int C = 1;
-  while (C < 8 && (long)batch * C * 2 <= 304 && (long)n * n >= 4096L * C) C *= 2;
+  while (C < 8 && (long)batch * C * 2 <= 2 * kSms && (long)n * n >= 4096L * C) C *= 2;
   auto go = [&](auto SL) {
     return launch_after_clusters(k_residual_mask<T, decltype(SL)::value>, C, batch * C, 512, 0, st, R, sR, (long)n * n,
                                  (float)(tol * tol), active, next, status);

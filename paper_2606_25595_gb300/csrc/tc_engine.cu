@@ -481,8 +481,8 @@ __device__ __forceinline__ uint32_t bf16x2_bits(float lo_half, float hi_half) {
 // are reduced on the way in, and every thread then turns one (row, 8 complex k) item into the S
 // digit planes with 16-byte stores -- one swizzled half-row chunk per plane and part.  The strip is
 // skewed by one element per 8 so that the threads' 128-byte item reads fall in distinct banks.
-// Item layout as k_digitize: A rows [Re | Im]; B re row [Re | -Im], im row [Im | Re] (a bf16 sign
-// flip, exact).  Rows r >= R and k >= K are written as zero digits, with exponent -1000.
+// A's planes are written as real and imaginary parts, B's as -Im, Re and Im (a bf16 sign flip, exact; the
+// layouts stand at the store).  Rows r >= R and k >= K are written as zero digits, with exponent -1000.
 __host__ __device__ constexpr int strip_skew(int k) { return k + (k >> 3); }
 
 // One operand to digitise; a launch takes up to kTcMaxJobs of one element type (blockIdx.z), e.g. both

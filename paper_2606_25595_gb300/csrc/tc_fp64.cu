@@ -562,7 +562,7 @@ size_t gemm_fp64_tc_scratch_bytes(int M, int N, int K, int batch) {
   // taken in portions of what fits
   const size_t one = entry_bytes(M, N, K);
   const long tiles = (long)((M + tc::BM - 1) / tc::BM) * ((N + tc::BNC9 - 1) / tc::BNC9);
-  size_t n = (size_t)((4 * 152 + tiles - 1) / tiles);
+  size_t n = (size_t)((4 * kSms + tiles - 1) / tiles);
   const size_t cap = ((size_t)384 << 20) / one;
   if (n > cap) n = cap;
   if (n > (size_t)batch) n = (size_t)batch;
