@@ -649,7 +649,7 @@ inline Dims dims_of(int M, int N, int K, int S) {
   Dims d;
   d.M_pad = (M + BM - 1) / BM * BM;
   d.N_pad = (N + bnc_of(S) - 1) / bnc_of(S) * bnc_of(S);
-  d.K_pad = (K + 31) / 32 * 32;
+  d.K_pad = K > 0 ? (K + 31) / 32 * 32 : 32;  // (an empty contraction multiplies zeros: it must write the accumulators)
   // Leading digit bound L = 2^(l1-1), others 64: per K term the exact groups are bounded by
   //   i+j=2: L^2,  3: 2 L 64,  4: 2 L 64 + 64^2,  5: 2 L 64 + 2 * 64^2
   // units, so with Keff = 2 K_pad terms they stay below 2^24 for l1 = 7 up to Keff = 512 and

@@ -229,6 +229,23 @@ def test_bounded_wait_gives_up_and_the_context_stays_usable(q):
     P.close()
 
 
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "emu64", "bf16x3"])
+def test_empty_contraction_gives_beta_c0(q, prec):
+    import ctypes
+    import torch
+    L, rng = q.load(), np.random.default_rng(3)
+    M, N, bt = 70, 50, 3
+    x = _t(rng.standard_normal((bt, 512, 512)) + 1j * rng.standard_normal((bt, 512, 512)))
+    C0 = _t((rng.integers(-9, 10, (bt, M, N)) + 1j * rng.integers(-9, 10, (bt, M, N))).astype(complex))
+    C = torch.empty_like(C0)
+    for c0, want in ((C0, 2 * C0), (None, 0 * C0)):
+        q.zgemm_batched(1e30 * x, x, prec)  # large values in the accumulators
+        st = L.qtx_zgemm_batched(q.PRECISION[prec], M, N, 0, 0, x.data_ptr(), 1, M, 0, x.data_ptr(), N, 1, 1.0, 2.0 if c0 is not None else 0.0,
+                                 c0.data_ptr() if c0 is not None else None, N, M * N, C.data_ptr(), N, M * N, bt,
+                                 ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert st == 0 and torch.equal(C, want)
+
+
 # the block inverse's products on the tensor cores: nine planes (fp64), six and four (emu64), four (fp32)
 @pytest.mark.parametrize("prec,n", [("fp64", 40), ("emu64", 64), ("fp32", 200)])
 def test_block_inverse_reports_an_expired_wait(q, prec, n):
