@@ -670,13 +670,17 @@ def main():
 
     # ---------------------------------------------------------------- roofline of the product kernel
     peaks, peak_src = measured_peaks()
+    peak, bound = peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops")), "tensor"
     if args.precision in ("emu64", "bf16x3"):
-        peak = peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops"))
-        bound, kernel = "tensor", "k_tc_gemm (tcgen05 bf16 digit products)"
+        kernel = "k_tc_gemm (tcgen05 bf16 digit products)"
+    elif args.precision == "fp32" and 96 <= b <= 1024:
+        kernel = "k_tc_gemm (tcgen05 bf16 digit products, 4 planes)"
     elif args.precision == "fp32":
         peak, bound, kernel = 69.7, "alu", "k_gemm<float> (SIMT FFMA)"
+    elif b > 32:
+        kernel = "k_tc_gemm_fp64 (tcgen05 bf16 digit products, 9 planes)"
     else:
-        peak, bound, kernel = 1.1, "alu", "k_gemm<double> (SIMT DFMA)"
+        kernel = "k_rgf_small (mma.sync bf16 digit products, with the block inverses in its time)"
     # achieved: the method's own flops (8 M N K per complex product, 136 b^3 per slice) over the
     # kernel's live launch time; the tensor pipe's flops (every digit product) are reported beside
     avg_ms = prof["ms"] / max(prof["launches"], 1)
