@@ -119,7 +119,8 @@ bool contacts_together(const qtx_rgf_desc& d, bool single) {
   return d.leads && !single && d.block_size <= kLeafMax && d.max_energies_in_flight <= 32767;
 }
 
-// inverse_only: the areas a batched inverse on its own uses (block g, and the refinement's)
+// inverse_only: the areas a batched inverse on its own uses (block g, and the refinement's), or with leads a contact
+// on its own
 Layout make_layout(const qtx_rgf_desc& d, bool inverse_only = false) {
   Layout L{};
   const long b = d.block_size, nb = d.n_blocks, Ec = d.max_energies_in_flight;
@@ -158,7 +159,8 @@ Layout make_layout(const qtx_rgf_desc& d, bool inverse_only = false) {
   // one block shared by every energy (the slice's -(H + Sigma^R) or Sigma^<, converted once)
   L.shared_blk = a.take(d.precision == QTX_FP64 ? 0 : bb * sizeof(cx<double>));
   const bool mixed = d.precision == QTX_EMU64 || d.precision == QTX_BF16X3;
-  const bool tc64 = d.precision == QTX_FP64 && b >= kTcF64Min;
+  // (a contact on its own takes neither: its products and inverses stay with DFMA in a fixed order)
+  const bool tc64 = d.precision == QTX_FP64 && b >= kTcF64Min && !(inverse_only && d.leads);
   L.refine64 = mixed || tc64;
   L.ident = a.take(L.refine64 ? bb * sizeof(cx<double>) : 0);
   L.ident_df = a.take(L.refine64 ? bb * sizeof(cx<double>) : 0);
