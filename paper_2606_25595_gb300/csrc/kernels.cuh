@@ -132,11 +132,10 @@ template <typename Tin, typename Tout>
 cudaError_t convert_strided(const cx<Tin>* in, long ldi, long si, cx<Tout>* out, long ldo, long so, int rows,
                             int cols, int batch, cudaStream_t st);
 
-// ---- in-place inverse of n x n blocks by Gauss-Jordan elimination with partial pivoting over the whole
-// block, in global memory, one CTA per active entry: the few energies whose refined inverse did not
-// converge.  perm: n ints per batch entry.  A zero or non-finite pivot stores QTX_ERR_SINGULAR.
-cudaError_t pivoted_inverse(cx<double>* A, long sA, int n, int batch, const int* active, int* status, int* perm,
-                            cudaStream_t st);
+// ---- in-place inverse of n x n blocks (n <= 256) by Gauss-Jordan elimination with partial pivoting over the whole
+// block, in global memory, one cluster per active entry: the few energies whose refined inverse did not
+// converge.  A zero or non-finite pivot stores QTX_ERR_SINGULAR.
+cudaError_t pivoted_inverse(cx<double>* A, long sA, int n, int batch, const int* active, int* status, cudaStream_t st);
 
 // the b x b identity in complex128 and in df32
 cudaError_t set_identity(cx<double>* I, cx<df>* Idf, int b, cudaStream_t st);

@@ -45,8 +45,8 @@ struct Arena {
 
 // FP64 products of at least kTcF64Min in every dimension run on the tensor cores (tc_fp64.cu)
 constexpr int kTcF64Min = 33;
-// FP64 block inverses that do not converge by refinement are eliminated with full column pivoting in
-// one CTA up to this size, by the recursion above it
+// FP64 block inverses that do not converge by refinement are eliminated with pivots over the whole column
+// up to this size (as leaves, or in global memory), by the recursion above it
 constexpr int kPivotedMax = 256;
 
 // products launched together at most (those of a slice's stage)
@@ -66,7 +66,6 @@ struct Layout {
   int n_more;
   bool short_launches;  // a product has at most four tiles per SM (make_layout, launch_after)
   bool refine64;  // FP64 block inverses by refinement (inverse_f64) have their areas
-  size_t perm;
 };
 }  // namespace
 
@@ -167,7 +166,6 @@ Layout make_layout(const qtx_rgf_desc& d, bool inverse_only = false) {
   L.ref = a.take((L.refine64 || b > kLeafMax) ? 3 * Ec * bb * sizeof(cx<double>) : 0);
   L.f32a = a.take(L.refine64 ? Ec * bb * sizeof(cx<float>) : 0);
   L.f32tmp = a.take(L.refine64 ? Ec * bb * sizeof(cx<float>) + 4096 : 0);
-  L.perm = a.take(L.refine64 && b <= kPivotedMax ? (size_t)Ec * b * sizeof(int) : 0);
   L.n_dec = 10;
   const long nl = contacts_together(d, inverse_only) ? 2 : 1;  // contacts iterated in the same launches
   // (smaller lead blocks are iterated in shared memory; the transmission's four blocks remain)
@@ -554,7 +552,7 @@ qtx_status inverse_refined_f32(qtx_rgf_plan_s* P, cx<float>* A, int n, int batch
 // of 1e6 five).  An energy stops after the sweep whose residual norm was at most 2^-27: the next
 // residual is then its square, below FP64's resolution.  Energies still above it after kSweeps64
 // (ill-conditioned beyond FP32's reach, or non-finite) are inverted again from A by pivoted
-// elimination in FP64.  A DFMA Gauss-Jordan of a 64 x 64 leaf took 770 us on one SM (GB300's FP64 pipe
+// elimination in FP64 (n = 64, 64 blocks of kappa 1e9: 0.87 ms in all, 1.40 by DFMA leaves alone).  A DFMA Gauss-Jordan of a 64 x 64 leaf took 770 us on one SM (GB300's FP64 pipe
 // runs at 1/64 of its FP32 rate); the FP32 leaf takes 37 us.  An FP64 solve of b = 128, 12 slices and 8 energies:
 // 132 ms by DFMA products and leaves, 8.6 ms with products on the tensor cores and these inverses.
 constexpr int kSweeps64 = 5;
@@ -595,8 +593,12 @@ qtx_status inverse_f64(qtx_rgf_plan_s* P, cx<double>* A, int n, int batch, const
   }
   Term<double> tC; tC.p = Acopy; tC.s = nn; tC.alpha = 1.0;
   QTX_CK((combine<double, double>(A, nn, tC, none, none, n, batch, nullptr, 0.0, 0.0, act, st)));
+  if (n <= kLeafMax) {
+    QTX_CK(leaf_inverse<double>(A, n, nn, n, batch, act, status, st));
+    return QTX_OK;
+  }
   if (n <= kPivotedMax) {
-    QTX_CK(pivoted_inverse(A, nn, n, batch, act, status, reinterpret_cast<int*>(P->ws + P->L.perm), st));
+    QTX_CK(pivoted_inverse(A, nn, n, batch, act, status, st));
     return QTX_OK;
   }
   return inverse_refined<double>(P, A, n, batch, act, status, st);

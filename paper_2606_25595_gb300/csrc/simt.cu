@@ -7,6 +7,7 @@
 #include <type_traits>
 
 #include "df32.cuh"
+#include "gj64.cuh"
 #include "kernels.cuh"
 
 namespace qtx {
@@ -913,92 +914,110 @@ cudaError_t residual_mask(const cx<T>* R, long sR, int n, int batch, double tol,
 template cudaError_t residual_mask<df>(const cx<df>*, long, int, int, double, const int*, int*, int*, cudaStream_t);
 template cudaError_t residual_mask<double>(const cx<double>*, long, int, int, double, const int*, int*, int*, cudaStream_t);
 
-// Pivoted Gauss-Jordan of one block per CTA in global memory (L2): latency-bound, about n^3 / 0.5 G
-// complex FMAs a second per block; it only runs for blocks the refined FP32 inverse cannot resolve.
-// Row interchanges are made as the elimination goes and undone as column interchanges at the end.
-__global__ void __launch_bounds__(512) k_pivoted_inverse(cx<double>* Ag, long sA, int n, const int* active, int* status,
-                                                         int* permg) {
-  const int e = blockIdx.x, t = threadIdx.x;
-  if (active && !active[e]) return;
+// Pivoted Gauss-Jordan of a block of at most 256 in global memory (L2) by a cluster of 8 CTAs; it only runs for blocks
+// the refined FP32 inverse cannot resolve, and the clusters of the others return at once.  A warp of every CTA finds the
+// pivot and its reciprocal, the CTAs share the pivot row's columns, then each of their 64 warps takes every 64th row:
+// bound by the FP64 pipe (4 n^2 DFMA a step on 8 SMs) and, below n = 200, by a step's chain of about 10 us.  Inverses of
+// kappa 1e9 on their own, 8 blocks: 5.2 ms with a CTA a block and 2.1 so at n = 128, 31.2 and 6.0 ms at 256, where
+// the recursion by DFMA takes 4.8 and 12.2.  Row interchanges are made as
+// the elimination goes and undone as column interchanges at the end.
+constexpr int kPivT = 256, kPivC = 8;
+__global__ void __launch_bounds__(kPivT) k_pivoted_inverse(cx<double>* Ag, long sA, int n, const int* active, int* status) {
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  const int rank = (int)cl.block_rank(), e = blockIdx.x / kPivC, t = threadIdx.x, warp = t / 32, lane = t % 32;
+  if (active && !active[e]) return;  // the whole cluster
+  constexpr int PER = kPivT / 32;  // values of a row per lane
   cx<double>* A = Ag + (long)e * sA;
-  int* perm = permg + (long)e * n;
-  __shared__ double s_best[16];
-  __shared__ int s_at[16];
-  __shared__ int s_p;
+  // rows written by other SMs: loads from L2, behind the cluster's barriers
+  auto ld = [&](int i, int j) {
+    const double2 v = __ldcg(reinterpret_cast<const double2*>(A + (long)i * n + j));
+    return mk<double>(v.x, v.y);
+  };
+  auto st = [&](int i, int j, cx<double> v) { __stcg(reinterpret_cast<double2*>(A + (long)i * n + j), make_double2(v.re, v.im)); };
+  __shared__ int s_perm[kPivT], s_p;
+  __shared__ cx<double> s_r;
   for (int k = 0; k < n; ++k) {
-    double best = -1.0;
-    int at = n;
-    for (int i = k + t; i < n; i += blockDim.x) {
-      const double v = cabs1(A[(long)i * n + k]);
-      if (v > best || v != v) {  // a NaN is taken, and rejected below
-        best = v;
-        at = i;
+    if (warp == 0) {  // the first row of largest |Re| + |Im| from k on, and its entry's reciprocal
+      unsigned long long key[PER], best = 0;
+#pragma unroll
+      for (int q = 0; q < PER; ++q) {
+        const int i = lane + 32 * q;
+        key[q] = i >= k && i < n ? gj::pivot_key(ld(i, k)) : 0ull;
+        best = key[q] > best ? key[q] : best;
+      }
+      best = gj::warp_max(best);
+      int p = -1;
+#pragma unroll
+      for (int q = PER - 1; q >= 0; --q) {
+        const unsigned hit = __ballot_sync(0xffffffffu, key[q] == best);
+        if (hit) p = 32 * q + __ffs((int)hit) - 1;
+      }
+      if (best == 0 || best >= 0x7ff0000000000000ull) p = -1;
+      const cx<double> r = p < 0 ? mk<double>(0.0, 0.0) : gj::crecip_warp(ld(p, k));
+      if (lane == 0) {
+        s_p = s_perm[k] = p;
+        s_r = r;
       }
     }
-    for (int off = 16; off > 0; off >>= 1) {
-      const double ov = __shfl_down_sync(0xffffffffu, best, off);
-      const int oi = __shfl_down_sync(0xffffffffu, at, off);
-      if (ov > best || ov != ov || (ov == best && oi < at)) {
-        best = ov;
-        at = oi;
-      }
-    }
-    if (t % 32 == 0) {
-      s_best[t / 32] = best;
-      s_at[t / 32] = at;
-    }
-    __syncthreads();
-    if (t == 0) {
-      for (int w = 1; w < 16; ++w)
-        if (s_best[w] > best || s_best[w] != s_best[w] || (s_best[w] == best && s_at[w] < at)) {
-          best = s_best[w];
-          at = s_at[w];
-        }
-      s_p = (best > 0.0 && isfinite(best)) ? at : -1;
-      perm[k] = s_p;
-    }
-    __syncthreads();
+    cl.sync();  // every CTA has read column k
     const int p = s_p;
-    if (p < 0) {
-      if (t == 0 && status) atomicCAS(status + e, 0, (int)QTX_ERR_SINGULAR);
+    if (p < 0) {  // in every CTA alike
+      if (t == 0 && rank == 0 && status) atomicCAS(status + e, 0, (int)QTX_ERR_SINGULAR);
       return;
     }
-    const cx<double> r = crecip(A[(long)p * n + k]);
-    __syncthreads();
-    for (int j = t; j < n; j += blockDim.x) {  // interchange rows k and p; row k scaled by 1 / pivot
-      const cx<double> x = A[(long)p * n + j];
-      if (p != k) A[(long)p * n + j] = A[(long)k * n + j];
-      A[(long)k * n + j] = j == k ? r : x * r;
+    const cx<double> r = s_r;
+    for (int j = rank * n / kPivC + t; j < (rank + 1) * n / kPivC; j += kPivT) {  // rows k and p interchanged; row k scaled
+      const cx<double> x = ld(p, j);
+      if (p != k) st(p, j, ld(k, j));
+      st(k, j, j == k ? r : x * r);
     }
-    __syncthreads();
-    // one warp per row at a time: every lane holds the row's factor before column k is overwritten
-    for (int i = t / 32; i < n; i += (int)blockDim.x / 32) {
+    cl.sync();
+    // one warp per row at a time, which it holds before it writes
+    cx<double> a[PER], x[PER];
+#pragma unroll
+    for (int q = 0; q < PER; ++q)
+      if (lane + 32 * q < n) a[q] = ld(k, lane + 32 * q);
+    for (int i = rank + kPivC * warp; i < n; i += kPivC * PER) {
       if (i == k) continue;
-      const cx<double> f = A[(long)i * n + k];
+      const cx<double> f = ld(i, k);
+#pragma unroll
+      for (int q = 0; q < PER; ++q) {
+        const int j = lane + 32 * q;
+        if (j < n) x[q] = j == k ? mk<double>(0.0, 0.0) : ld(i, j);
+      }
       __syncwarp();
-      for (int j = t % 32; j < n; j += 32) {
-        const cx<double> x = j == k ? mk<double>(0.0, 0.0) : A[(long)i * n + j];
-        A[(long)i * n + j] = x - f * A[(long)k * n + j];
-      }
+#pragma unroll
+      for (int q = 0; q < PER; ++q)
+        if (lane + 32 * q < n) st(i, lane + 32 * q, x[q] - f * a[q]);
     }
-    __syncthreads();
+    cl.sync();
   }
-  for (int k = n - 1; k >= 0; --k) {
-    const int p = perm[k];
-    if (p != k)
-      for (int i = t; i < n; i += blockDim.x) {
-        const cx<double> x = A[(long)i * n + k];
-        A[(long)i * n + k] = A[(long)i * n + p];
-        A[(long)i * n + p] = x;
-      }
-    __syncthreads();
+  // where the column interchanges, k = n - 1 .. 0, take column j from
+  int from[PER];
+#pragma unroll
+  for (int q = 0; q < PER; ++q) from[q] = lane + 32 * q;
+  for (int k = 0; k < n; ++k) {
+    const int p = s_perm[k];
+#pragma unroll
+    for (int q = 0; q < PER; ++q) from[q] = from[q] == k ? p : (from[q] == p ? k : from[q]);
+  }
+  for (int i = rank + kPivC * warp; i < n; i += kPivC * PER) {
+    cx<double> x[PER];
+#pragma unroll
+    for (int q = 0; q < PER; ++q)
+      if (lane + 32 * q < n) x[q] = ld(i, from[q]);
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < PER; ++q)
+      if (lane + 32 * q < n) st(i, lane + 32 * q, x[q]);
   }
 }
-cudaError_t pivoted_inverse(cx<double>* A, long sA, int n, int batch, const int* active, int* status, int* perm,
-                            cudaStream_t st) {
-  k_pivoted_inverse<<<batch, 512, 0, st>>>(A, sA, n, active, status, perm);
+cudaError_t pivoted_inverse(cx<double>* A, long sA, int n, int batch, const int* active, int* status, cudaStream_t st) {
+  if (n > kPivT) return cudaErrorInvalidValue;
+  EarlyLaunches none(0);
+  const cudaError_t e = launch_after_clusters(k_pivoted_inverse, kPivC, batch * kPivC, kPivT, 0, st, A, sA, n, active, status);
   count_launch();
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 __global__ void k_set_identity(cx<double>* I, cx<df>* Idf, int b) {

@@ -164,3 +164,27 @@ def test_fp64_inverse_pivots_and_singular(q):
     assert st.cpu().tolist() == [0, 4, 4, 0]
     assert np.array_equal(X[0].cpu().numpy(), A[0].T)
     assert np.allclose(X[3].cpu().numpy() * 1e250, np.eye(n), atol=1e-15)
+
+
+# beyond FP32's reach (kappa 1e9): eliminated over a cluster's CTAs, whose column ranges and rows do not divide evenly;
+# blocks that do (kappa 10), a permutation and a singular block beside them
+@pytest.mark.parametrize("n", [33, 64, 65, 131, 255, 256])
+def test_fp64_elimination_of_ill_conditioned_blocks(q, n):
+    import torch
+    rng = np.random.default_rng(n)
+
+    def block(kappa):
+        U, _ = np.linalg.qr(_cx(rng, n, n))
+        V, _ = np.linalg.qr(_cx(rng, n, n))
+        return (U * np.geomspace(1, 1 / kappa, n)) @ V
+
+    P = np.eye(n)[rng.permutation(n)] * (1 + 2j)
+    A = np.stack([block(1e9), block(1e9) * 1e-30, P, block(1e1), np.ones((n, n)) + 0j, block(1e9)])
+    X, st = q.zinv_batched(torch.tensor(A).cuda(), "fp64")
+    X = X.cpu().numpy()
+    assert st.cpu().tolist() == [0, 0, 0, 0, 4, 0]
+    for e in (0, 1, 2, 3, 5):
+        ref = np.linalg.inv(A[e])
+        assert np.linalg.norm(X[e] - ref) <= 64 * np.linalg.cond(A[e]) * 2.0 ** -53 * np.linalg.norm(ref), e
+    alone, _ = q.zinv_batched(torch.tensor(A[5:]).cuda(), "fp64")
+    assert np.array_equal(alone[0].cpu().numpy(), X[5])
