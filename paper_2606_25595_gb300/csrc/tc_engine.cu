@@ -500,8 +500,10 @@ struct DigitJobs {
   DigitJob j[kTcMaxJobs];
 };
 
+// threads of a CTA of RPC rows: a warp per row, or eight short rows to two warps
+__host__ __device__ constexpr int digit_threads(int rpc) { return rpc == 8 ? 64 : 32 * rpc; }
 template <int S, int RPC, typename TI>
-__global__ void __launch_bounds__(32 * RPC) k_digitize_rows(const __grid_constant__ DigitJobs jobs) {
+__global__ void __launch_bounds__(digit_threads(RPC)) k_digitize_rows(const __grid_constant__ DigitJobs jobs) {
   after_previous();
   const DigitJob& job = jobs.j[blockIdx.z];
   const int e = blockIdx.y;
@@ -514,7 +516,7 @@ __global__ void __launch_bounds__(32 * RPC) k_digitize_rows(const __grid_constan
   const int ldS = strip_skew(K_pad) + 1;  // complex elements per strip row
   cx<df>* strip = reinterpret_cast<cx<df>*>(dsm);
   __shared__ int s_ex[RPC];
-  constexpr int NT = 32 * RPC;  // threads: one warp per strip row
+  constexpr int NT = digit_threads(RPC);
   const cx<TI>* Xe = static_cast<const cx<TI>*>(job.X) + (long)e * job.sX;
   // an element as df32 (FP32 inputs: lo = 0)
   auto ld = [&](long off) -> cx<df> {
@@ -694,16 +696,20 @@ cudaError_t digitize_as(const DigitJob* const* jobs, int n, cudaStream_t st) {
   }
   // fused pass: RPC rows per CTA with one warp per row -- two rows while the strip stays within
   // 48 KB of shared memory (many small CTAs per SM, so loads, digit arithmetic and stores of
-  // different CTAs overlap), else a single row up to the 200 KB the kernel is allowed
+  // different CTAs overlap), else a single row up to the 200 KB the kernel is allowed.  Rows of at most 64 k leave
+  // such CTAs little more than their launch: eight of them share one where there are more CTAs of two than the SMs hold
+  // at once, 32 each (solves of b = 8, 6 planes: 6 energies 0.55 ms in rows of two and 0.58 of eight, 25 0.66 and 0.65, 50
+  // 0.83 and 0.69; 4000 at 2 planes 20.7 and 8.5 ms, both operands of a product 424 and 123 us).
   const size_t row_bytes = (size_t)(strip_skew(K_pad) + 1) * sizeof(cx<df>);
-  const int rpc = 2 * row_bytes <= 48 * 1024 ? 2 : 1;
+  const int rpc = K_pad <= 64 && (long)R_pad / 2 * batch * n > 32L * kSms ? 8 : (2 * row_bytes <= 48 * 1024 ? 2 : 1);
   if (rpc * row_bytes > 200 * 1024) return cudaErrorInvalidValue;  // K-chunks of <= 1024 always fit
-  static std::atomic<unsigned long long> done2{0}, done1{0};
-  cudaError_t e = rpc == 2 ? allow_smem(k_digitize_rows<S, 2, TI>, 200 * 1024, done2) : allow_smem(k_digitize_rows<S, 1, TI>, 200 * 1024, done1);
+  static std::atomic<unsigned long long> done{0};
+  const cudaError_t e = rpc == 1 ? allow_smem(k_digitize_rows<S, 1, TI>, 200 * 1024, done) : cudaSuccess;
   if (e != cudaSuccess) return e;
   const size_t smem = rpc * row_bytes;
   const dim3 g((R_pad + rpc - 1) / rpc, batch, n);
-  if (rpc == 2) launch_after(k_digitize_rows<S, 2, TI>, g, 64, smem, st, all);
+  if (rpc == 8) launch_after(k_digitize_rows<S, 8, TI>, g, digit_threads(8), smem, st, all);
+  else if (rpc == 2) launch_after(k_digitize_rows<S, 2, TI>, g, 64, smem, st, all);
   else launch_after(k_digitize_rows<S, 1, TI>, g, 32, smem, st, all);
   count_launch();
   return cudaGetLastError();

@@ -61,6 +61,22 @@ def test_integer_inputs_are_exact(q, M, N, K, batch, opA, opB, prec):
     assert np.array_equal(got, ref)
 
 
+# short contractions of many entries are digitised eight rows to a CTA (K <= 64): one value, the padding's edges, the last
+# of them and the first beyond; row counts that leave CTAs partly empty; 37 entries stay below the rule's count, 39 not
+@pytest.mark.parametrize("K", [1, 31, 33, 63, 64, 65])
+@pytest.mark.parametrize("batch", [37, 39])
+@pytest.mark.parametrize("M,N", [(1, 1), (9, 50), (130, 7)])
+@pytest.mark.parametrize("ops", ["NN", "CC"])
+@pytest.mark.parametrize("prec", ["emu64", "bf16x3"])
+def test_short_contractions_are_exact(q, M, N, K, batch, ops, prec):
+    rng = np.random.default_rng(M + N + K)
+    lo, unit = (-500, 1) if prec == "emu64" else (-31, 16)
+    draw = lambda *s: unit * (rng.integers(lo, -lo + 1, s) + 1j * rng.integers(lo, -lo + 1, s))  # noqa: E731
+    A, B = draw(batch, *((M, K) if ops[0] == "N" else (K, M))), draw(batch, *((K, N) if ops[1] == "N" else (N, K)))
+    got = q.zgemm_batched(_t(A), _t(B), prec, ops[0], ops[1]).cpu().numpy()
+    assert np.array_equal(got, _op(A, ops[0]) @ _op(B, ops[1]))
+
+
 def test_emu64_shared_operand_and_zero_rows(q):
     """A 2-D operand is shared across the batch (digitised once); an all-zero row stays zero."""
     rng = np.random.default_rng(5)
