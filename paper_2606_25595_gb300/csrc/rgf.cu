@@ -1910,8 +1910,8 @@ qtx_status qtx_zinv_batched(int precision, int n, void* A, long sA, int batch, i
   if (precision == QTX_FP32) s = zinv_via<float>(P, n, A, sA, batch, stat, st);
   else if (precision == QTX_FP64) s = zinv_via<double>(P, n, A, sA, batch, stat, st);
   else s = zinv_via<df>(P, n, A, sA, batch, stat, st);
-  int hflag = 0;  // raised by a product whose bounded wait expired
-  if (s == QTX_OK && cudaMemcpyAsync(&hflag, P->d_err_flag, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) s = QTX_ERR_CUDA;
+  int hflag = 0;  // raised by a tensor-core product whose bounded wait expired
+  if (s == QTX_OK && P->L.tc_bytes && cudaMemcpyAsync(&hflag, P->d_err_flag, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) s = QTX_ERR_CUDA;
   e = cudaStreamSynchronize(st);
   if (s == QTX_OK && e != cudaSuccess) s = QTX_ERR_CUDA;
   if (s == QTX_OK && hflag) {

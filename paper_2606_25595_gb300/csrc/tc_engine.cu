@@ -699,7 +699,7 @@ cudaError_t digitize_as(const DigitJob* const* jobs, int n, cudaStream_t st) {
   // different CTAs overlap), else a single row up to the 200 KB the kernel is allowed.  Rows of at most 64 k leave
   // such CTAs little more than their launch: eight of them share one where there are more CTAs of two than the SMs hold
   // at once, 32 each (solves of b = 8, 6 planes: 6 energies 0.55 ms in rows of two and 0.58 of eight, 25 0.66 and 0.65, 50
-  // 0.83 and 0.69; 4000 at 2 planes 20.7 and 8.5 ms, both operands of a product 424 and 123 us).
+  // 0.83 and 0.69; 4000 at 2 planes 20.7 and 9.2 ms, both operands of a product 424 and 123 us).
   const size_t row_bytes = (size_t)(strip_skew(K_pad) + 1) * sizeof(cx<df>);
   const int rpc = K_pad <= 64 && (long)R_pad / 2 * batch * n > 32L * kSms ? 8 : (2 * row_bytes <= 48 * 1024 ? 2 : 1);
   if (rpc * row_bytes > 200 * 1024) return cudaErrorInvalidValue;  // K-chunks of <= 1024 always fit
