@@ -42,8 +42,8 @@ qtx_status qtx_zgemm_batched(int precision, int M, int N, int K, int opA, const 
                              double beta, const void *C0, long ldc0, long strideC0, void *C, long ldc,
                              long strideC, int batch, void *stream);
 
-/* Give the device memory that the calls of this header keep between them on the current device back to the
- * driver.  Synchronises the device; not during a stream capture.  The next call takes its memory anew.
+/* Give the device memory that the calls of this header keep between them on the current device back to
+ * CUDA.  Synchronises the device; not during a stream capture.  The next call takes its memory anew.
  * Errors: QTX_ERR_CUDA. */
 qtx_status qtx_release_memory(void);
 

@@ -194,7 +194,7 @@ def kernel_launches() -> int:
 
 
 def release_memory() -> None:
-    """Give the memory that component calls keep on the current device back to the driver."""
+    """Give the memory that component calls keep on the current device back to CUDA."""
     s = load().qtx_release_memory()
     if s != 0:
         raise QtxError(s, "qtx_release_memory")

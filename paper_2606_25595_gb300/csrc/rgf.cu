@@ -552,8 +552,9 @@ qtx_status inverse_refined_f32(qtx_rgf_plan_s* P, cx<float>* A, int n, int batch
 // of 1e6 five).  An energy stops after the sweep whose residual norm was at most 2^-27: the next
 // residual is then its square, below FP64's resolution.  Energies still above it after kSweeps64
 // (ill-conditioned beyond FP32's reach, or non-finite) are inverted again from A by pivoted
-// elimination in FP64 (n = 64, 64 blocks of kappa 1e9: 0.87 ms in all, 1.40 by DFMA leaves alone).  A DFMA Gauss-Jordan of a 64 x 64 leaf took 770 us on one SM (GB300's FP64 pipe
-// runs at 1/64 of its FP32 rate); the FP32 leaf takes 37 us.  An FP64 solve of b = 128, 12 slices and 8 energies:
+// elimination in FP64 (n = 64, 64 blocks of kappa 1e9: 0.87 ms in all, 1.40 by DFMA leaves alone).  A DFMA
+// Gauss-Jordan of a 64 x 64 leaf took 770 us on one SM (GB300's FP64 pipe runs at 1/64 of its FP32 rate); the FP32
+// leaf takes 37 us.  An FP64 solve of b = 128, 12 slices and 8 energies:
 // 132 ms by DFMA products and leaves, 8.6 ms with products on the tensor cores and these inverses.
 constexpr int kSweeps64 = 5;
 qtx_status inverse_f64(qtx_rgf_plan_s* P, cx<double>* A, int n, int batch, const int* active, int* status,
@@ -1652,8 +1653,8 @@ namespace {
 // default pool returns everything to the driver at each synchronisation, and these calls synchronise, so
 // every call paid for mapping its memory again (0.9 ms of a 1.2 ms product).  The pool keeps at most kPoolKeep
 // between calls and gives the rest back; allocation and reuse are stream-ordered, so calls on several
-// streams and threads share it.  qtx_release_memory gives the rest back too, and the driver takes it for an allocation
-// of this process that would not fit beside it.
+// streams and threads share it.  qtx_release_memory gives the rest back too, and CUDA takes it for an allocation of this
+// process that would not fit beside it.
 constexpr unsigned long long kPoolKeep = 512ull << 20;
 // make = false: the pool of the current device and context if there is one, else an error
 cudaError_t component_pool(cudaMemPool_t* out, bool make = true) {
